@@ -13,6 +13,7 @@
 #include <new>
 #include <queue>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -43,6 +44,80 @@ struct DeviceGuard {
     int cur = -1;
     if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
   }
+};
+
+// Page-locked host memory of a context: the error word that a kernel with a bounded wait raises, the
+// mirrors that launches write their telemetry and (small rings) their draws to, and the staging area of
+// small read-backs.  Locking pages costs more than a small call, so blocks of destroyed contexts are kept
+// for the next ones: at most kPinnedKept of them, the rest are freed.
+constexpr size_t kPinnedBytes = (size_t)384 << 10;
+constexpr size_t kPinnedKept = 8;
+// What a block holds: the error word and netmax_measure's result; the telemetry ring, if it is short
+// enough (2,048 rounds); a mirror of the trace ring, if that is small enough; the staging area.
+constexpr size_t kPinnedTel = 256, kPinnedTrace = kPinnedTel + ((size_t)32 << 10), kPinnedStaging = kPinnedTrace + ((size_t)64 << 10);
+constexpr size_t kStagingBytes = kPinnedBytes - kPinnedStaging;
+class PinnedPool {
+ public:
+  unsigned char* get() {
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      if (!kept_.empty()) {
+        unsigned char* p = kept_.back();
+        kept_.pop_back();
+        return p;
+      }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kPinnedBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return (unsigned char*)p;
+  }
+  void put(unsigned char* p) {  // the caller has waited for everything that writes to it
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      if (kept_.size() < kPinnedKept) {
+        kept_.push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+    cudaGetLastError();
+  }
+
+ private:
+  std::mutex mu_;
+  std::vector<unsigned char*> kept_;
+};
+PinnedPool& pinned_pool() {
+  static PinnedPool* pool = new PinnedPool();  // never destroyed: contexts may outlive static destructors
+  return *pool;
+}
+
+// Raises a kernel's limit of dynamic shared memory on the current device, once: the attribute belongs to
+// the kernel and setting it costs microseconds, so what has been set is remembered (it is never lowered).
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  static std::mutex mu;
+  static auto* set = new std::unordered_map<uint64_t, size_t>();
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t key = (uint64_t)(uintptr_t)kernel * 64u + (uint64_t)(dev & 63);
+  std::lock_guard<std::mutex> lock(mu);
+  size_t& have = (*set)[key];
+  if (bytes <= have) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) have = bytes;
+  return e;
+}
+
+struct RoundPlan {  // launch shape of round_kernel and multi_round_kernel
+  int cg = kThreads, rl = 1, rg = 1, rows_per_group = 0;
+  bool short_vectors = false;  // fewer than two streaming tiles per SM: the L2-resident shape
+  int grid = 1;
+  size_t smem = 0;
+  int64_t n_tiles = 0;
 };
 
 struct ResidentPlan {  // launch shape of resident_rounds_kernel
@@ -126,6 +201,9 @@ struct netmax_ctx {
   cudaStream_t stream = nullptr;
   bool own_memory = false;
   unsigned char* base = nullptr;
+  unsigned char* pinned = nullptr;  // block of the pinned pool: see kPinnedTel and the rest
+  bool host_writes = false;         // launches that may still write to `pinned` have been enqueued since the last synchronisation
+  int32_t* trace_mirror = nullptr;  // host copy of the trace ring, written by the sampler (small rings only)
   int storage = NETMAX_STORAGE_F32;
   unsigned char *x[2] = {nullptr, nullptr}, *c = nullptr;  // [M][ld] fp32 or bfloat16, as `storage` says
   uint32_t* thr = nullptr;
@@ -133,15 +211,16 @@ struct netmax_ctx {
   float* wtab = nullptr;
   int32_t* trace = nullptr;
   float* wring = nullptr;
-  double* tel = nullptr;
+  double* tel = nullptr;  // telemetry ring: in page-locked host memory (tel_on_host) or, when it is long, on the device
+  bool tel_on_host = false;
   double* partials = nullptr;
   unsigned int* ticket = nullptr;
   float4* colpart = nullptr;
   unsigned int* grid_barrier = nullptr;  // arrival counter of multi-round launches
-  unsigned int* dev_error = nullptr;     // raised by a kernel whose bounded wait gave up
+  volatile unsigned int* dev_error = nullptr;  // raised by a kernel whose bounded wait gave up (page-locked host memory)
   bool cooperative = false;              // device supports cooperative launches
   uint32_t inject_absent_ctas = 0;       // test hook: applied to the next multi-round launch, then cleared
-  double* measure_out = nullptr;         // device: (consensus, loss) of netmax_measure
+  double* measure_out = nullptr;         // (consensus, loss) of netmax_measure (page-locked host memory)
   // host copies of the tables in force (the asynchronous timeline draws peers on the host)
   std::vector<uint32_t> h_thr;
   std::vector<int32_t> h_last;
@@ -181,6 +260,8 @@ struct netmax_ctx {
   int policy_K = 20, policy_R = 20;
   double policy_rho_upper = 0.0;
   int fuse_rounds = 0;  // 0: automatic, 1: one launch per round, 2..kFusedMaxRounds: rounds per fused launch
+  bool round_planned[2] = {false, false};  // [0]: the context's objective, [1]: measuring
+  RoundPlan round_plan[2];
   bool fused_planned = false;
   FusedPlan fused;
   bool resident_planned = false;
@@ -426,6 +507,7 @@ int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int3
   p.last_nz = ctx->last_nz;
   p.out = out;
   p.w_out = w_out;
+  p.host_out = w_out ? ctx->trace_mirror : nullptr;  // (draws into the context's own ring)
   p.wtab = ctx->wtab;
   p.slot0 = slot0;
   p.ring = ring;
@@ -440,14 +522,6 @@ int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int3
   NM_CUDA(ctx, cudaGetLastError());
   return NETMAX_OK;
 }
-
-struct RoundPlan {
-  int cg = kThreads, rl = 1, rg = 1, rows_per_group = 0;
-  bool short_vectors = false;  // fewer than two streaming tiles per SM: the L2-resident shape
-  int grid = 1;
-  size_t smem = 0;
-  int64_t n_tiles = 0;
-};
 
 using RoundKernel = void (*)(const RoundParams);
 
@@ -523,7 +597,7 @@ int floor_pow2(int64_t v) {
 // 64- or 16-byte pieces costs more than peer rows that come from L2 instead of L1 (4096 x 4096
 // elements: 135 us per round with 16-byte pieces, 34 with 128-byte pieces and two row groups;
 // 1024 x 65536: 250 against 184).
-int plan_round(netmax_ctx* ctx, RoundPlan& plan, int objective) {
+int plan_round_uncached(netmax_ctx* ctx, RoundPlan& plan, int objective) {
   const int64_t M = ctx->M, nq = ctx->L.nq;
   const int64_t target = 2 * (int64_t)ctx->sm_count;  // the short-vector kernel runs 2 CTAs per SM
   int cg = kThreads;
@@ -570,20 +644,35 @@ int plan_round(netmax_ctx* ctx, RoundPlan& plan, int objective) {
   RoundKernel k = pick_kernel(objective, plan.short_vectors, ctx->L.halves);
   // (the kernels also hold a little static shared memory, so the opt-in is needed somewhat below 48 KB of dynamic)
   if (plan.smem > 40 * 1024)
-    NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem));
+    NM_CUDA(ctx, allow_smem((const void*)k, plan.smem));
   int per_sm = 0;
   NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, plan.smem));
   if (per_sm < 1) return fail(ctx, NETMAX_CUDA_ERROR, "round kernel does not fit on an SM (smem %zu)", plan.smem);
   if (plan.short_vectors && ctx->cooperative) {  // the multi-round kernel needs all of its CTAs resident
     MultiRoundKernel mk = pick_multi_kernel(objective == 2 ? 0 : objective, ctx->L.halves);
     if (plan.smem > 40 * 1024)
-      NM_CUDA(ctx, cudaFuncSetAttribute(mk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem));
+      NM_CUDA(ctx, allow_smem((const void*)mk, plan.smem));
     int per_sm_multi = 0;
     NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_multi, mk, kThreads, plan.smem));
     per_sm = std::min(per_sm, per_sm_multi);
     if (per_sm < 1) return fail(ctx, NETMAX_CUDA_ERROR, "multi-round kernel does not fit on an SM (smem %zu)", plan.smem);
   }
   plan.grid = (int)std::min<int64_t>(plan.n_tiles, std::min<int64_t>((int64_t)per_sm * ctx->sm_count, kMaxGrid));
+  return NETMAX_OK;
+}
+
+// The plan depends only on sizes fixed at creation; asking the driver for occupancies again on every
+// call took longer than the launches of a small call.
+int plan_round(netmax_ctx* ctx, RoundPlan& plan, int objective) {
+  const int k = objective == 2 ? 1 : 0;
+  if (!ctx->round_planned[k]) {
+    RoundPlan fresh;
+    int rc = plan_round_uncached(ctx, fresh, objective);
+    if (rc) return rc;
+    ctx->round_plan[k] = fresh;
+    ctx->round_planned[k] = true;
+  }
+  plan = ctx->round_plan[k];
   return NETMAX_OK;
 }
 
@@ -649,7 +738,7 @@ int plan_resident_uncached(netmax_ctx* ctx, const RoundPlan& plan, ResidentPlan&
   f.min_rounds = elements <= ((int64_t)1 << 20) ? 2 : elements <= ((int64_t)1 << 22) ? 6 : elements <= ((int64_t)1 << 24) ? 8 : 16;
   ResidentKernel k = pick_resident_kernel(ctx->objective, ctx->L.halves);
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
-  NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+  NM_CUDA(ctx, allow_smem((const void*)k, f.smem));
   int per_sm = 0;
   NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, f.smem));
   if (per_sm < 1) return NETMAX_OK;
@@ -702,7 +791,7 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
     for (int cand : {256, 128, 64}) {
       const size_t smem = fixed_r + (size_t)48 * M * cand;
       if (smem > (size_t)227 * 1024) continue;
-      NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      NM_CUDA(ctx, allow_smem((const void*)k, smem));
       int n = 0;
       NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, cand, smem));
       const bool better = (n >= 2) != (per_sm_r >= 2) ? n >= 2 : n * cand > per_sm_r * threads_r;
@@ -721,7 +810,7 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   f.smem = fixed + (size_t)48 * M * threads;
   f.max_rounds = slots;
   f.n_tiles = ((ctx->d + 3) / 4 + threads - 1) / threads;
-  NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+  NM_CUDA(ctx, allow_smem((const void*)k, f.smem));
   f.grid = (int)std::min<int64_t>(f.n_tiles, std::min<int64_t>((int64_t)per_sm * ctx->sm_count, kMaxGrid));
   f.ok = true;
   return NETMAX_OK;
@@ -811,7 +900,7 @@ int plan_cluster_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPla
     if (NETMAX_CLUSTER_THREADS != 0 && cand != NETMAX_CLUSTER_THREADS) continue;
     const size_t smem = cluster_smem(rpc, cand);
     if (smem > (size_t)113 * 1024) continue;  // at least two CTAs per SM
-    NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NM_CUDA(ctx, allow_smem((const void*)k, smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(C * ctx->sm_count));
     cfg.blockDim = dim3((unsigned)cand);
@@ -948,7 +1037,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
         cpar.f = fp;
         cpar.rpc = cluster.rpc;
         ClusterKernel ck = pick_cluster_kernel(ctx->objective);
-        NM_CUDA(ctx, cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster.smem));
+        NM_CUDA(ctx, allow_smem((const void*)ck, cluster.smem));
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3((unsigned)(std::min<int64_t>(cluster.grid / cluster.C, fp.n_tiles) * cluster.C));
         lc.blockDim = dim3((unsigned)cluster.threads);
@@ -966,7 +1055,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
         // (the attribute belongs to the kernel, not to this context: another context may have lowered it)
         // (one instance for all launches of the call: the larger one unless the whole call is four rounds or fewer)
         FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, (int)std::min<int64_t>(n, fused.max_rounds));
-        NM_CUDA(ctx, cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused.smem));
+        NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
         fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
       }
       ctx->launches += 1;
@@ -1088,11 +1177,11 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
   if (cfg->device >= ndev) { ctx->error = "device ordinal out of range"; return bail(NETMAX_INVALID_ARG); }
   DeviceGuard guard(cfg->device);
   if (!guard.ok) { ctx->error = "cudaSetDevice failed"; return bail(NETMAX_CUDA_ERROR); }
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, cfg->device) == cudaSuccess) {
-    ctx->sm_count = prop.multiProcessorCount;
-    ctx->cooperative = prop.cooperativeLaunch != 0;
-  }
+  int attr = 0;
+  if (cudaDeviceGetAttribute(&attr, cudaDevAttrMultiProcessorCount, cfg->device) == cudaSuccess) ctx->sm_count = attr;
+  if (cudaDeviceGetAttribute(&attr, cudaDevAttrCooperativeLaunch, cfg->device) == cudaSuccess) ctx->cooperative = attr != 0;
+  ctx->pinned = pinned_pool().get();
+  if (!ctx->pinned) { ctx->error = "cudaHostAlloc failed"; return bail(NETMAX_OOM); }
   if (cfg->workspace) {
     if (((uintptr_t)cfg->workspace & 255) != 0) { ctx->error = "workspace is not 256-byte aligned"; return bail(NETMAX_INVALID_ARG); }
     if (cfg->workspace_bytes < ctx->L.total) {
@@ -1129,8 +1218,14 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
   ctx->ticket = (unsigned int*)(ctx->base + L.off_ticket);
   ctx->colpart = (float4*)(ctx->base + L.off_colpart);
   ctx->grid_barrier = ctx->ticket + 16;
-  ctx->dev_error = ctx->ticket + 32;
-  ctx->measure_out = (double*)(ctx->ticket + 48);
+  std::memset(ctx->pinned, 0, kPinnedStaging);
+  ctx->dev_error = (volatile unsigned int*)ctx->pinned;
+  ctx->measure_out = (double*)(ctx->pinned + 64);
+  if ((size_t)ctx->trace_rounds * 16 <= kPinnedTrace - kPinnedTel) {
+    ctx->tel = (double*)(ctx->pinned + kPinnedTel);
+    ctx->tel_on_host = true;
+  }
+  if ((size_t)ctx->trace_rounds * ctx->M * 4 <= kPinnedStaging - kPinnedTrace) ctx->trace_mirror = (int32_t*)(ctx->pinned + kPinnedTrace);
   ctx->coltick = (unsigned int*)(ctx->base + L.off_coltick);
   ctx->pipe_tel = (double*)(ctx->base + L.off_pipe_tel);
 
@@ -1142,7 +1237,7 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
   if (!step(cudaMemsetAsync(ctx->ticket, 0, 256, ctx->stream), "cudaMemsetAsync(ticket)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->coltick, 0, (size_t)kMaxGrid * sizeof(unsigned int), ctx->stream), "cudaMemsetAsync(coltick)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->x[1], 0, L.plane, ctx->stream), "cudaMemsetAsync(x)")) return bail(NETMAX_CUDA_ERROR);
-  if (!step(cudaMemsetAsync(ctx->tel, 0, (size_t)ctx->trace_rounds * 2 * sizeof(double), ctx->stream), "cudaMemsetAsync(tel)")) return bail(NETMAX_CUDA_ERROR);
+  if (!ctx->tel_on_host && !step(cudaMemsetAsync(ctx->tel, 0, (size_t)ctx->trace_rounds * 2 * sizeof(double), ctx->stream), "cudaMemsetAsync(tel)")) return bail(NETMAX_CUDA_ERROR);
   rc = upload_policy(ctx);
   if (rc) return bail(rc);
   rc = launch_init(ctx, ctx->x[0], cfg->x0_std, kTagX0);
@@ -1185,6 +1280,14 @@ void netmax_destroy(netmax_ctx* ctx) {
     cudaFree(ctx->base);
     cudaGetLastError();
   }
+  if (ctx->pinned) {
+    if (ctx->host_writes) {  // (the whole device: the caller may have destroyed the stream already)
+      DeviceGuard guard(ctx->device);
+      cudaDeviceSynchronize();
+      cudaGetLastError();
+    }
+    pinned_pool().put(ctx->pinned);
+  }
   delete ctx;
 }
 
@@ -1217,13 +1320,25 @@ int netmax_get_policy(netmax_ctx* ctx, double* prob_out, double* rho_out) {
   return NETMAX_OK;
 }
 
-// After a synchronisation: has a kernel's bounded wait given up since the last check?
-static int check_device_error(netmax_ctx* ctx) {
-  unsigned int flag = 0;
-  NM_CUDA(ctx, cudaMemcpy(&flag, ctx->dev_error, sizeof flag, cudaMemcpyDeviceToHost));
-  if (flag == 0) return NETMAX_OK;
-  cudaMemset(ctx->dev_error, 0, sizeof flag);
+// Waits for the context's stream; reports a bounded wait of a kernel that has given up since the last check.
+static int synchronise(netmax_ctx* ctx) {
+  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  ctx->host_writes = false;
+  if (*ctx->dev_error == 0u) return NETMAX_OK;
+  *ctx->dev_error = 0u;
   return fail(ctx, NETMAX_CUDA_ERROR, "a multi-round launch gave up waiting at its grid barrier; replicas are not valid");
+}
+
+// Copies `bytes` of device memory to the host and synchronises.  Small copies go through the page-locked
+// staging area: a copy to pageable memory costs the driver about as much again.
+static int read_back(netmax_ctx* ctx, void* host, const void* dev, size_t bytes) {
+  const bool staged = bytes <= kStagingBytes;
+  unsigned char* stage = ctx->pinned + kPinnedStaging;
+  NM_CUDA(ctx, cudaMemcpyAsync(staged ? stage : host, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+  int rc = synchronise(ctx);
+  if (rc) return rc;
+  if (staged) std::memcpy(host, stage, bytes);
+  return NETMAX_OK;
 }
 
 // Host transfers of a bfloat16 context go through fp32 on the device: the buffer of the double
@@ -1276,13 +1391,20 @@ static int copy_out(netmax_ctx* ctx, const unsigned char* src, float* host) {
       NM_CUDA(ctx, cudaMemcpyAsync(host + (size_t)r0 * ctx->d, stage, (size_t)rows * ctx->d * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     }
     NM_CUDA(ctx, cudaMemsetAsync(stage, 0, ctx->L.plane, ctx->stream));
-    NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return check_device_error(ctx);
+    return synchronise(ctx);
+  }
+  if (ctx->L.ld == ctx->d) return read_back(ctx, host, src, ctx->L.plane);
+  if (ctx->L.plane <= kStagingBytes) {  // the padded rows as they are, taken apart on the host
+    NM_CUDA(ctx, cudaMemcpyAsync(ctx->pinned + kPinnedStaging, src, ctx->L.plane, cudaMemcpyDeviceToHost, ctx->stream));
+    int rc = synchronise(ctx);
+    if (rc) return rc;
+    const float* rows = reinterpret_cast<const float*>(ctx->pinned + kPinnedStaging);
+    for (int64_t i = 0; i < ctx->M; ++i) std::memcpy(host + i * ctx->d, rows + i * ctx->L.ld, (size_t)ctx->d * sizeof(float));
+    return NETMAX_OK;
   }
   NM_CUDA(ctx, cudaMemcpy2DAsync(host, (size_t)ctx->d * sizeof(float), src, (size_t)ctx->L.ld * sizeof(float),
                                  (size_t)ctx->d * sizeof(float), (size_t)ctx->M, cudaMemcpyDeviceToHost, ctx->stream));
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  return check_device_error(ctx);
+  return synchronise(ctx);
 }
 
 int netmax_set_replicas(netmax_ctx* ctx, const float* host_x) { return copy_in(ctx, ctx ? ctx->x[ctx->cur] : nullptr, host_x); }
@@ -1300,6 +1422,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
   RoundPlan plan;
   int rc = plan_round(ctx, plan, ctx->objective);
   if (rc) return rc;
+  ctx->host_writes = true;
   FusedPlan fused;
   rc = plan_fused(ctx, plan, fused);
   if (rc) return rc;
@@ -1351,7 +1474,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
         rp.inv_M = p.inv_M;
         rp.q_offset = p.q_offset;
         rp.keys = p.keys;
-        NM_CUDA(ctx, cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident.smem));
+        NM_CUDA(ctx, allow_smem((const void*)rk, resident.smem));
         rk<<<resident.grid, resident.threads, resident.smem, ctx->stream>>>(rp);
         const int warps_per_block = kThreads / 32;
         sum_tile_partials_kernel<<<(unsigned)((chunk + warps_per_block - 1) / warps_per_block), kThreads, 0, ctx->stream>>>(
@@ -1380,7 +1503,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
         mp.tel = ctx->tel;
         mp.partials2 = ctx->partials;
         mp.barrier = ctx->grid_barrier;
-        mp.error = ctx->dev_error;
+        mp.error = const_cast<unsigned int*>(ctx->dev_error);
         mp.slot0 = ctx->rounds % ctx->trace_rounds;
         mp.ring = ctx->trace_rounds;
         mp.first_round = (uint64_t)ctx->rounds;
@@ -1480,6 +1603,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   } while (0)
 
   const uint64_t first = (uint64_t)ctx->rounds;
+  ctx->host_writes = true;
   rc = launch_sampler(ctx, first, n_rounds, ctx->trace, ctx->wring, ctx->rounds % ctx->trace_rounds, ctx->trace_rounds);
   if (rc) return bail(rc);
   // uploads must not overtake earlier work of the context that still reads the buffers
@@ -1522,10 +1646,10 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   ctx->cur = cur_end;
   ctx->rounds += n_rounds;
   NM_PIPE(cudaStreamSynchronize(ctx->down_stream));
-  NM_PIPE(cudaStreamSynchronize(ctx->stream));
 #undef NM_PIPE
+  rc = synchronise(ctx);
   cleanup();
-  return check_device_error(ctx);
+  return rc;
 }
 
 int netmax_set_fuse_rounds(netmax_ctx* ctx, int32_t fuse_rounds) {
@@ -1560,11 +1684,11 @@ int netmax_read_columns(netmax_ctx* ctx, const int64_t* host_cols, int64_t n_col
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, d_out, (size_t)total * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) rc = fail(ctx, NETMAX_CUDA_ERROR, "read_columns: %s", cudaGetErrorString(e));
+  const int rs = synchronise(ctx);
   cudaFree(d_cols);
   cudaFree(d_out);
-  return rc ? rc : check_device_error(ctx);
+  return rc ? rc : rs;
 }
 
 // ---- sampled read-back that allocates nothing -------------------------------------------
@@ -1621,10 +1745,9 @@ int netmax_read_columns_static(netmax_ctx* ctx, const int64_t* host_cols, int64_
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, scratch->values, (size_t)total * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);
   // whatever happened, leave the shared array idle: the next call, perhaps on another stream, reuses it
-  const cudaError_t es = cudaStreamSynchronize(ctx->stream);
-  if (e == cudaSuccess) e = es;
+  const int rs = synchronise(ctx);
   if (e != cudaSuccess) return fail(ctx, NETMAX_CUDA_ERROR, "read_columns_static: %s", cudaGetErrorString(e));
-  return check_device_error(ctx);
+  return rs;
 }
 
 static int ring_range(netmax_ctx* ctx, int64_t first, int64_t n) {
@@ -1641,15 +1764,18 @@ int netmax_peer_trace(netmax_ctx* ctx, int64_t first_round, int64_t n, int32_t* 
   if (n == 0) return NETMAX_OK;
   if (!host_out) return fail(ctx, NETMAX_INVALID_ARG, "host_out is NULL");
   DeviceGuard guard(ctx->device);
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  rc = check_device_error(ctx);
-  if (rc) return rc;
+  if (ctx->trace_mirror) {
+    rc = synchronise(ctx);
+    if (rc) return rc;
+  }
   const size_t row = (size_t)ctx->M * sizeof(int32_t);
   int64_t r = first_round;
   while (r < first_round + n) {  // at most two contiguous pieces of the ring
     const int64_t slot = r % ctx->trace_rounds;
     const int64_t piece = std::min<int64_t>(first_round + n - r, ctx->trace_rounds - slot);
-    NM_CUDA(ctx, cudaMemcpy(host_out + (size_t)(r - first_round) * ctx->M, ctx->trace + (size_t)slot * ctx->M, piece * row, cudaMemcpyDeviceToHost));
+    int32_t* out = host_out + (size_t)(r - first_round) * ctx->M;
+    if (ctx->trace_mirror) std::memcpy(out, ctx->trace_mirror + (size_t)slot * ctx->M, piece * row);
+    else if ((rc = read_back(ctx, out, ctx->trace + (size_t)slot * ctx->M, piece * row)) != NETMAX_OK) return rc;
     r += piece;
   }
   return NETMAX_OK;
@@ -1661,11 +1787,16 @@ int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* ho
   if (rc) return rc;
   if (n == 0) return NETMAX_OK;
   DeviceGuard guard(ctx->device);
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  rc = check_device_error(ctx);
+  std::vector<double> copy;
+  const double* ring = ctx->tel;
+  if (ctx->tel_on_host) {
+    rc = synchronise(ctx);
+  } else {
+    copy.resize((size_t)ctx->trace_rounds * 2);
+    rc = read_back(ctx, copy.data(), ctx->tel, copy.size() * sizeof(double));
+    ring = copy.data();
+  }
   if (rc) return rc;
-  std::vector<double> ring((size_t)ctx->trace_rounds * 2);
-  NM_CUDA(ctx, cudaMemcpy(ring.data(), ctx->tel, ring.size() * sizeof(double), cudaMemcpyDeviceToHost));
   for (int64_t k = 0; k < n; ++k) {
     const int64_t slot = (first_round + k) % ctx->trace_rounds;
     if (host_consensus) host_consensus[k] = ring[2 * slot];
@@ -1721,15 +1852,14 @@ int netmax_measure(netmax_ctx* ctx, double* consensus, double* loss) {
   p.coltick = ctx->coltick;
   p.inv_M = 1.0f / (float)ctx->M;
   p.keys = ctx->keys;
+  ctx->host_writes = true;
   kernel<<<plan.grid, kThreads, plan.smem, ctx->stream>>>(p);
   ctx->launches += 1;
   NM_CUDA(ctx, cudaGetLastError());
-  double out[2] = {0.0, 0.0};
-  NM_CUDA(ctx, cudaMemcpyAsync(out, ctx->measure_out, sizeof out, cudaMemcpyDeviceToHost, ctx->stream));
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  if (consensus) *consensus = out[0];
-  if (loss) *loss = out[1];
-  return check_device_error(ctx);
+  rc = synchronise(ctx);
+  if (consensus) *consensus = ctx->measure_out[0];
+  if (loss) *loss = ctx->measure_out[1];
+  return rc;
 }
 
 // ---- asynchronous timeline --------------------------------------------------------------------

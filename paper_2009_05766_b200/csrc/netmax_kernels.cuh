@@ -34,6 +34,7 @@ struct SampleParams {
   const int32_t* last_nz;      // [M] last index with p > 0
   int32_t* out;                // slot s of round r is out + ((slot0 + r) % ring) * M
   float* w_out;                // same indexing: pull weight of the draw (0 on a self-draw); may be NULL
+  int32_t* host_out;           // same indexing: mirror in page-locked host memory; may be NULL
   const float* wtab;           // [M][M] pull weights (read when w_out is given)
   int64_t slot0, ring;
   uint64_t first_round;
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(256) sample_peers_kernel(const SampleParams p)
     const int32_t m = min(lo, __ldg(p.last_nz + i));
     const int64_t at = ((p.slot0 + r) % p.ring) * p.M + i;
     p.out[at] = m;
+    if (p.host_out) p.host_out[at] = m;
     if (p.w_out) p.w_out[at] = (m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m);
   }
 }
@@ -620,7 +622,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int
       }
       __nanosleep(32);
     }
-    if (!ok) atomicExch(error, 1u);
+    if (!ok) *reinterpret_cast<volatile unsigned int*>(error) = 1u;  // (page-locked host memory)
     __threadfence();
     s_ok = ok;
   }
