@@ -33,6 +33,7 @@
 #include <cmath>
 #include <cstdio>
 #include <functional>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -62,81 +63,185 @@ void parallel_for(int n, int min_parallel, const std::function<void(int, int)>& 
   for (auto& th : pool) th.join();
 }
 
+// ---- vector helpers: eight doubles at a time, compiled for the instruction sets a host may have -----
+typedef double vec8 __attribute__((vector_size(64)));
+typedef int64_t ivec8 __attribute__((vector_size(64)));
+#if defined(__x86_64__) && defined(__GNUC__)
+#define NM_CLONES __attribute__((target_clones("avx512f", "avx2", "default")))
+#else
+#define NM_CLONES
+#endif
+
+// Sums over j < n (n a multiple of 8) of w, w s and w s^2 with w_j = g_j exp(-eta s_j); w is kept in q.
+// The exponential is Cody and Waite's: x = k ln 2 + r with the multiple taken off in two parts, a Taylor
+// polynomial of degree 13 on |r| <= ln 2 / 2 (remainder below 5e-18), and k added to the exponent
+// (|eta s| <= 600 keeps the result a normal number).  The row solves spend their time here.
+NM_CLONES void tilt_sums(const double* s, const double* g, int n, double eta, double* q, double* z, double* a, double* b) {
+  vec8 vz = {}, va = {}, vb = {};
+  const double kLog2e = 1.4426950408889634074, kLn2Hi = 6.93147180369123816490e-01, kLn2Lo = 1.90821492927058770002e-10;
+  const double kShift = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer in the low mantissa bits
+  for (int j = 0; j < n; j += 8) {
+    vec8 sv, gv;
+    __builtin_memcpy(&sv, s + j, 64);
+    __builtin_memcpy(&gv, g + j, 64);
+    const vec8 x = sv * -eta;
+    const vec8 t = x * kLog2e + kShift;
+    const vec8 kf = t - kShift;
+    const vec8 r = (x - kf * kLn2Hi) - kf * kLn2Lo;
+    vec8 p = r * (1.0 / 6227020800.0) + (1.0 / 479001600.0);
+    p = p * r + (1.0 / 39916800.0);
+    p = p * r + (1.0 / 3628800.0);
+    p = p * r + (1.0 / 362880.0);
+    p = p * r + (1.0 / 40320.0);
+    p = p * r + (1.0 / 5040.0);
+    p = p * r + (1.0 / 720.0);
+    p = p * r + (1.0 / 120.0);
+    p = p * r + (1.0 / 24.0);
+    p = p * r + (1.0 / 6.0);
+    p = p * r + 0.5;
+    p = p * r + 1.0;
+    p = p * r + 1.0;
+    ivec8 e, bits;
+    __builtin_memcpy(&e, &t, 64);
+    __builtin_memcpy(&bits, &p, 64);
+    bits += e << 52;
+    vec8 w;
+    __builtin_memcpy(&w, &bits, 64);
+    w *= gv;
+    __builtin_memcpy(q + j, &w, 64);
+    const vec8 ws = w * sv;
+    vz += w;
+    va += ws;
+    vb += ws * sv;
+  }
+  double tz = 0, ta = 0, tb = 0;
+  for (int l = 0; l < 8; ++l) { tz += vz[l]; ta += va[l]; tb += vb[l]; }
+  *z = tz; *a = ta; *b = tb;
+}
+
+NM_CLONES double dot(const double* x, const double* y, int n) {
+  vec8 acc = {};
+  int j = 0;
+  for (; j + 8 <= n; j += 8) {
+    vec8 a, b;
+    __builtin_memcpy(&a, x + j, 64);
+    __builtin_memcpy(&b, y + j, 64);
+    acc += a * b;
+  }
+  double t = 0.0;
+  for (; j < n; ++j) t += x[j] * y[j];
+  for (int l = 0; l < 8; ++l) t += acc[l];
+  return t;
+}
+
+// y += c x
+NM_CLONES void axpy(double* y, const double* x, double c, int n) {
+  int j = 0;
+  for (; j + 8 <= n; j += 8) {
+    vec8 a, b;
+    __builtin_memcpy(&a, y + j, 64);
+    __builtin_memcpy(&b, x + j, 64);
+    a += b * c;
+    __builtin_memcpy(y + j, &a, 64);
+  }
+  for (; j < n; ++j) y[j] += c * x[j];
+}
+
+// One row of the LP, apart from the grid point.  s, g, q have n8 entries, n rounded up to a multiple of
+// eight: entries beyond n weigh nothing.
 struct Row {
-  std::vector<int> nb;        // neighbours m != i
-  std::vector<double> t, f1;  // their iteration times and d_im + d_mi
+  std::vector<int> nb;           // neighbours m != i
+  std::vector<double> t, f1;     // their iteration times and d_im + d_mi
+  std::vector<double> s, g;      // times mapped to [0, 1]; 1 for a neighbour, 0 for filling
   double C = 0, tmin = 0, tmax = 0, sum_f1 = 0, sum_f1t = 0;
+  double mean_lo = 0, mean_hi = 0;  // mean s at the ends of the bracket, eta = -+kEtaCap
+  bool flat = false;             // all links equally fast
 };
 
-// Exponential tilt: q_m ~ exp(-eta s_m), s in [0,1], with mean s equal to sig.  The mean is
-// decreasing in eta; Newton steps are kept inside a shrinking bracket.
-bool tilt(const std::vector<double>& s, double sig, std::vector<double>& q) {
-  const size_t n = s.size();
-  q.resize(n);
-  auto stats = [&](double eta, double& mean, double& var) {
-    double z = 0, a = 0, b = 0;
-    for (size_t j = 0; j < n; ++j) {
-      const double w = std::exp(-eta * s[j]);
-      q[j] = w;
-      z += w;
-      a += w * s[j];
-      b += w * s[j] * s[j];
-    }
+void finish_row(Row& r) {
+  const size_t n = r.nb.size(), n8 = (n + 7) / 8 * 8;
+  const double scale = r.tmax - r.tmin;
+  r.flat = !(scale > kTie * r.tmax);
+  if (r.flat) return;
+  r.s.assign(n8, 0.0);
+  r.g.assign(n8, 0.0);
+  for (size_t j = 0; j < n; ++j) {
+    r.s[j] = (r.t[j] - r.tmin) / scale;
+    r.g[j] = 1.0;
+  }
+  std::vector<double> q(n8);
+  double z, a, b;
+  tilt_sums(r.s.data(), r.g.data(), (int)n8, -kEtaCap, q.data(), &z, &a, &b);
+  r.mean_lo = a / z;
+  tilt_sums(r.s.data(), r.g.data(), (int)n8, kEtaCap, q.data(), &z, &a, &b);
+  r.mean_hi = a / z;
+}
+
+// Exponential tilt: q_m ~ exp(-eta s_m), s in [0,1], with mean s equal to sig.  The mean is decreasing
+// in eta; Newton steps are kept inside a shrinking bracket.  *eta is the start (the neighbouring grid
+// point's solution: two or three steps from this one's) and receives the solution; q holds the
+// unnormalised weights and *z their sum.
+bool tilt(const Row& row, double sig, double* eta_io, double* q, double* z_out) {
+  const int n8 = (int)row.s.size();
+  double z = 1.0, mean = 0.0, var = 0.0;
+  auto stats = [&](double eta) {
+    double a, b;
+    tilt_sums(row.s.data(), row.g.data(), n8, eta, q, &z, &a, &b);
     mean = a / z;
     var = b / z - mean * mean;
-    for (size_t j = 0; j < n; ++j) q[j] /= z;
   };
-  double mean, var;
-  double lo = -kEtaCap, hi = kEtaCap, eta = 0.0;
-  stats(lo, mean, var);
-  if (sig >= mean) {
-    eta = lo;
+  double lo = -kEtaCap, hi = kEtaCap, eta = *eta_io;
+  if (sig >= row.mean_lo) {
+    stats(eta = lo);
+  } else if (sig <= row.mean_hi) {
+    stats(eta = hi);
   } else {
-    stats(hi, mean, var);
-    if (sig <= mean) {
-      eta = hi;
-    } else {
-      stats(eta, mean, var);
-      for (int it = 0; it < 200; ++it) {
-        const double gap = mean - sig;
-        if (std::fabs(gap) <= 1e-15) break;
-        if (gap > 0) lo = eta; else hi = eta;
-        double next = (var > 1e-300) ? eta + gap / var : 0.5 * (lo + hi);
-        if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
-        if (next == eta || hi - lo <= 1e-15 * (1.0 + std::fabs(eta))) break;
-        eta = next;
-        stats(eta, mean, var);
-      }
+    if (!(eta > lo && eta < hi)) eta = 0.0;
+    stats(eta);
+    for (int it = 0; it < 200; ++it) {
+      const double gap = mean - sig;
+      if (std::fabs(gap) <= 1e-15) break;
+      if (gap > 0) lo = eta; else hi = eta;
+      double next = (var > 1e-300) ? eta + gap / var : 0.5 * (lo + hi);
+      if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
+      if (next == eta || hi - lo <= 1e-15 * (1.0 + std::fabs(eta))) break;
+      // a Newton step this short leaves an error of its square: below the rounding of the sums
+      const bool last = std::fabs(next - eta) <= 1e-9 * (1.0 + std::fabs(eta)) && std::fabs(gap) <= 1e-9;
+      eta = next;
+      stats(eta);
+      if (last) break;
     }
   }
-  stats(eta, mean, var);
+  *eta_io = eta;
+  *z_out = z;
   return std::fabs(mean - sig) <= 1e-9;
 }
 
 // One row of the LP at (rho, T = M t_bar).  Returns false when the row is infeasible.
-bool solve_row(const Row& row, int i, int M, double ar /* alpha rho */, double T, double* out) {
+bool solve_row(const Row& row, int i, int M, double ar /* alpha rho */, double T, double* eta, double* q, double* out) {
   const size_t n = row.nb.size();
   const double F = ar * row.sum_f1;
   if (F > 1.0) return false;
   const double free_mass = 1.0 - F;
   const double A = ar * row.sum_f1t;
   const double lo = A + free_mass * row.tmin, hi = A + free_mass * row.tmax;
-  std::fill(out, out + M, 0.0);
   if (T > hi * (1.0 + kTie)) return false;
+  if (n + 1 < (size_t)M) std::fill(out, out + M, 0.0);
+  out[i] = 0.0;
   if (T >= lo * (1.0 - kTie)) {
     if (free_mass <= 0.0) {
       for (size_t j = 0; j < n; ++j) out[row.nb[j]] = ar * row.f1[j];
       return true;
     }
-    const double target = std::min(std::max((T - A) / free_mass, row.tmin), row.tmax);
-    const double scale = row.tmax - row.tmin;
-    std::vector<double> q(n, 1.0 / (double)n);
-    if (scale > kTie * row.tmax) {
-      std::vector<double> s(n);
-      for (size_t j = 0; j < n; ++j) s[j] = (row.t[j] - row.tmin) / scale;
-      if (!tilt(s, (target - row.tmin) / scale, q)) return false;
+    if (row.flat) {
+      for (size_t j = 0; j < n; ++j) out[row.nb[j]] = ar * row.f1[j] + free_mass * (1.0 / (double)n);
+      return true;
     }
-    for (size_t j = 0; j < n; ++j) out[row.nb[j]] = ar * row.f1[j] + free_mass * q[j];
+    const double target = std::min(std::max((T - A) / free_mass, row.tmin), row.tmax);
+    double z = 1.0;
+    if (!tilt(row, (target - row.tmin) / (row.tmax - row.tmin), eta, q, &z)) return false;
+    const double f = free_mass / z;
+    for (size_t j = 0; j < n; ++j) out[row.nb[j]] = ar * row.f1[j] + f * q[j];
     return true;
   }
   double pii = (lo - T) / (row.tmin - row.C);
@@ -152,101 +257,171 @@ bool solve_row(const Row& row, int i, int M, double ar /* alpha rho */, double T
   return true;
 }
 
-// Eigenvalues of a small dense symmetric matrix by cyclic Jacobi rotations (in place).
-void jacobi_eigenvalues(std::vector<double>& a, int n, std::vector<double>& eig) {
-  for (int sweep = 0; sweep < 60; ++sweep) {
-    double off = 0.0, diag = 0.0;
-    for (int p = 0; p < n; ++p) {
-      diag += a[(size_t)p * n + p] * a[(size_t)p * n + p];
-      for (int q = p + 1; q < n; ++q) off += a[(size_t)p * n + q] * a[(size_t)p * n + q];
-    }
-    if (off <= 1e-30 * (diag + 1e-300)) break;
-    for (int p = 0; p < n - 1; ++p)
-      for (int q = p + 1; q < n; ++q) {
-        const double apq = a[(size_t)p * n + q];
-        if (apq == 0.0) continue;
-        const double theta = (a[(size_t)q * n + q] - a[(size_t)p * n + p]) / (2.0 * apq);
-        const double t = (theta >= 0 ? 1.0 : -1.0) / (std::fabs(theta) + std::sqrt(theta * theta + 1.0));
-        const double c = 1.0 / std::sqrt(t * t + 1.0), s = t * c;
-        for (int k = 0; k < n; ++k) {  // columns p, q
-          const double akp = a[(size_t)k * n + p], akq = a[(size_t)k * n + q];
-          a[(size_t)k * n + p] = c * akp - s * akq;
-          a[(size_t)k * n + q] = s * akp + c * akq;
-        }
-        for (int k = 0; k < n; ++k) {  // rows p, q
-          const double apk = a[(size_t)p * n + k], aqk = a[(size_t)q * n + k];
-          a[(size_t)p * n + k] = c * apk - s * aqk;
-          a[(size_t)q * n + k] = s * apk + c * aqk;
-        }
-      }
+// ---- eigenvalues of symmetric tridiagonal matrices ------------------------------------------------
+// How many eigenvalues of the tridiagonal matrix (diagonal d[0..m), squares of the off-diagonal e2) lie
+// below x: the negative pivots of T - x I (Sturm's sequence).
+int count_below(const double* d, const double* e2, int m, double x) {
+  int count = 0;
+  double q = d[0] - x;
+  for (int i = 0;;) {
+    if (std::fabs(q) < 1e-300) q = -1e-300;
+    count += q < 0.0;
+    if (++i == m) break;
+    q = d[i] - x - e2[i - 1] / q;
   }
-  eig.resize(n);
-  for (int p = 0; p < n; ++p) eig[p] = a[(size_t)p * n + p];
-  std::sort(eig.begin(), eig.end());
+  return count;
 }
 
-// Second largest eigenvalue of the symmetric doubly stochastic Y: the largest eigenvalue of
-// Y restricted to the complement of the all-ones vector.  Dense Jacobi for small M; Lanczos
-// with full reorthogonalisation (Ritz values by Jacobi) otherwise.
-double second_eigenvalue(const std::vector<double>& Y, int M) {
+// The eigenvalue number `index` (ascending, from 0), by bisection to neighbouring doubles.
+double tridiagonal_eigenvalue(const double* d, const double* e, int m, int index) {
+  std::vector<double> e2(m);
+  double lo = INFINITY, hi = -INFINITY;
+  for (int i = 0; i < m; ++i) {
+    const double off = (i > 0 ? std::fabs(e[i - 1]) : 0.0) + (i + 1 < m ? std::fabs(e[i]) : 0.0);
+    lo = std::min(lo, d[i] - off);
+    hi = std::max(hi, d[i] + off);
+    if (i + 1 < m) e2[i] = e[i] * e[i];
+  }
+  const double pad = 1e-15 * std::max(std::fabs(lo), std::fabs(hi)) + 1e-300;
+  lo -= pad;
+  hi += pad;
+  for (int it = 0; it < 200; ++it) {
+    const double mid = 0.5 * (lo + hi);
+    if (!(mid > lo && mid < hi) || hi - lo <= 4e-17) break;
+    if (count_below(d, e2.data(), m, mid) > index) hi = mid; else lo = mid;
+  }
+  return 0.5 * (lo + hi);
+}
+
+// An eigenvector of the tridiagonal matrix for the eigenvalue lambda: inverse iteration, two steps, with
+// row exchanges in the elimination.
+void tridiagonal_eigenvector(const double* d, const double* e, int m, double lambda, std::vector<double>& z) {
+  z.assign(m, 0.0);
+  if (m == 1) { z[0] = 1.0; return; }
+  std::vector<double> u0(m), u1(m, 0.0), u2(m, 0.0), l(m, 0.0);
+  std::vector<uint8_t> swapped(m, 0);
+  const double tiny = 1e-16;
+  double a = d[0] - lambda, b = e[0];  // the current row: diagonal, superdiagonal
+  for (int i = 0; i + 1 < m; ++i) {
+    const double c = e[i], dn = d[i + 1] - lambda, bn = i + 2 < m ? e[i + 1] : 0.0;
+    if (std::fabs(c) > std::fabs(a)) {
+      swapped[i] = 1;
+      l[i] = a / c;
+      u0[i] = c; u1[i] = dn; u2[i] = bn;
+      a = b - l[i] * dn;
+      b = -l[i] * bn;
+    } else {
+      if (std::fabs(a) < tiny) a = tiny;
+      l[i] = c / a;
+      u0[i] = a; u1[i] = b;
+      a = dn - l[i] * b;
+      b = bn;
+    }
+  }
+  u0[m - 1] = std::fabs(a) < tiny ? tiny : a;
+  for (int j = 0; j < m; ++j) z[j] = 1.0 + 0.37 * (j % 5);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i = 0; i + 1 < m; ++i) {
+      if (swapped[i]) std::swap(z[i], z[i + 1]);
+      z[i + 1] -= l[i] * z[i];
+    }
+    for (int i = m - 1; i >= 0; --i) {
+      double v = z[i];
+      if (i + 1 < m) v -= u1[i] * z[i + 1];
+      if (i + 2 < m) v -= u2[i] * z[i + 2];
+      z[i] = v / u0[i];
+    }
+    double big = 0.0;
+    for (double v : z) big = std::max(big, std::fabs(v));
+    for (double& v : z) v /= big;
+  }
+}
+
+// Takes the component along the all-ones vector out of v and normalises it.
+void centre(std::vector<double>& v) {
+  const int M = (int)v.size();
+  double mean = 0.0, nrm = 0.0;
+  for (double x : v) mean += x;
+  mean /= M;
+  for (double& x : v) { x -= mean; nrm += x * x; }
+  nrm = std::sqrt(nrm);
+  if (!(nrm > 0.0)) { v.clear(); return; }
+  for (double& x : v) x /= nrm;
+}
+
+// Second largest eigenvalue of the symmetric doubly stochastic Y: the largest eigenvalue of Y
+// restricted to the complement of the all-ones vector.  Householder's reduction to tridiagonal form and
+// bisection for small M; Lanczos with full reorthogonalisation otherwise.  vec (may be NULL) receives an
+// approximate eigenvector in that complement.
+double second_eigenvalue(const std::vector<double>& Y, int M, std::vector<double>* vec, bool parallel) {
   if (M <= 96) {
-    std::vector<double> a(Y), eig;
-    jacobi_eigenvalues(a, M, eig);
-    return eig[M - 2];
+    std::vector<double> A(Y), d(M), e(M, 0.0), w(M), scale(M, 0.0);
+    // column k is reduced with the reflection I - scale[k] v v^T; v stays in row k of A, from k + 1 on
+    for (int k = 0; k + 2 < M; ++k) {
+      double* v = A.data() + (size_t)k * M;  // row k = column k of the symmetric matrix
+      const int n = M - k - 1;
+      const double norm = std::sqrt(dot(v + k + 1, v + k + 1, n));
+      d[k] = v[k];
+      if (!(norm > 0.0)) continue;
+      const double alpha = v[k + 1] > 0.0 ? -norm : norm;
+      e[k] = alpha;
+      const double beta = 1.0 / (norm * norm - alpha * v[k + 1]);  // 2 / v^T v once alpha is taken off
+      v[k + 1] -= alpha;
+      scale[k] = beta;
+      for (int i = k + 1; i < M; ++i) w[i] = beta * dot(A.data() + (size_t)i * M + k + 1, v + k + 1, n);
+      const double half = 0.5 * beta * dot(w.data() + k + 1, v + k + 1, n);
+      axpy(w.data() + k + 1, v + k + 1, -half, n);
+      for (int i = k + 1; i < M; ++i) {
+        double* row = A.data() + (size_t)i * M;
+        axpy(row + k + 1, w.data() + k + 1, -v[i], n);
+        axpy(row + k + 1, v + k + 1, -w[i], n);
+      }
+    }
+    if (M >= 2) {
+      d[M - 2] = A[(size_t)(M - 2) * M + M - 2];
+      e[M - 2] = A[(size_t)(M - 2) * M + M - 1];
+    }
+    d[M - 1] = A[(size_t)(M - 1) * M + M - 1];
+    const double lam = tridiagonal_eigenvalue(d.data(), e.data(), M, M - 2);
+    if (vec) {
+      std::vector<double>& z = *vec;
+      tridiagonal_eigenvector(d.data(), e.data(), M, lam, z);
+      for (int k = M - 3; k >= 0; --k) {
+        const double* v = A.data() + (size_t)k * M + k + 1;
+        axpy(z.data() + k + 1, v, -scale[k] * dot(v, z.data() + k + 1, M - k - 1), M - k - 1);
+      }
+      centre(z);
+    }
+    return lam;
   }
   auto matvec = [&](const std::vector<double>& v, std::vector<double>& out) {
     double mean = 0.0;
     for (int j = 0; j < M; ++j) mean += v[j];
     mean /= M;
-    parallel_for(M, 512, [&](int a, int b) {
-      for (int i = a; i < b; ++i) {
-        const double* row = Y.data() + (size_t)i * M;
-        double acc = 0.0;
-        for (int j = 0; j < M; ++j) acc += row[j] * v[j];
-        out[i] = acc - mean;  // (Y - 11^T/M) v
-      }
+    parallel_for(M, parallel ? 512 : M + 1, [&](int a, int b) {
+      for (int i = a; i < b; ++i) out[i] = dot(Y.data() + (size_t)i * M, v.data(), M) - mean;  // (Y - 11^T/M) v
     });
   };
   const int max_steps = std::min(M - 1, 300);
   std::vector<std::vector<double>> V;
   std::vector<double> alpha, beta, v(M), wv(M);
   uint64_t lcg = 0x9E3779B97F4A7C15ull;
-  double mean = 0.0;
   for (int j = 0; j < M; ++j) {
     lcg = lcg * 6364136223846793005ull + 1442695040888963407ull;
     v[j] = (double)(lcg >> 11) / 9007199254740992.0 - 0.5;
-    mean += v[j];
   }
-  mean /= M;
-  double nrm = 0.0;
-  for (int j = 0; j < M; ++j) { v[j] -= mean; nrm += v[j] * v[j]; }
-  nrm = std::sqrt(nrm);
-  for (int j = 0; j < M; ++j) v[j] /= nrm;
+  centre(v);
   double best = 0.0;
   for (int step = 0; step < max_steps; ++step) {
     V.push_back(v);
     matvec(v, wv);
-    double a = 0.0;
-    for (int j = 0; j < M; ++j) a += wv[j] * v[j];
-    alpha.push_back(a);
+    alpha.push_back(dot(wv.data(), v.data(), M));
     for (int pass = 0; pass < 2; ++pass)  // full reorthogonalisation, twice
-      for (const auto& u : V) {
-        double dot = 0.0;
-        for (int j = 0; j < M; ++j) dot += wv[j] * u[j];
-        for (int j = 0; j < M; ++j) wv[j] -= dot * u[j];
-      }
-    double b = 0.0;
-    for (int j = 0; j < M; ++j) b += wv[j] * wv[j];
-    b = std::sqrt(b);
+      for (const auto& u : V) axpy(wv.data(), u.data(), -dot(wv.data(), u.data(), M), M);
+    const double b = std::sqrt(dot(wv.data(), wv.data(), M));
     const int m = (int)alpha.size();
     if ((m % 10 == 0) || b < 1e-13 || step == max_steps - 1) {
-      std::vector<double> Tm((size_t)m * m, 0.0), eig;
-      for (int k = 0; k < m; ++k) {
-        Tm[(size_t)k * m + k] = alpha[k];
-        if (k + 1 < m) Tm[(size_t)k * m + k + 1] = Tm[(size_t)(k + 1) * m + k] = beta[k];
-      }
-      jacobi_eigenvalues(Tm, m, eig);
-      const double top = eig[m - 1];
+      const double top = tridiagonal_eigenvalue(alpha.data(), beta.data(), m, m - 1);
       const bool settled = std::fabs(top - best) <= 1e-13 * std::max(1.0, std::fabs(top));
       best = top;
       if (b < 1e-13 || (settled && m >= 20)) break;
@@ -254,23 +429,21 @@ double second_eigenvalue(const std::vector<double>& Y, int M) {
     beta.push_back(b);
     for (int j = 0; j < M; ++j) v[j] = wv[j] / b;
   }
+  if (vec) {
+    std::vector<double> z;
+    tridiagonal_eigenvector(alpha.data(), beta.data(), (int)alpha.size(), best, z);
+    vec->assign(M, 0.0);
+    for (size_t k = 0; k < z.size(); ++k) axpy(vec->data(), V[k].data(), z[k], M);
+    centre(*vec);
+  }
   return best;
 }
 
 }  // namespace
 
 namespace netmax {
-// Largest eigenvalue of the symmetric tridiagonal matrix with diagonal alpha[0..m) and
-// off-diagonal beta[0..m-1) (the Ritz values of a Lanczos run).
 double tridiagonal_top_eigenvalue(const std::vector<double>& alpha, const std::vector<double>& beta) {
-  const int m = (int)alpha.size();
-  std::vector<double> Tm((size_t)m * m, 0.0), eig;
-  for (int k = 0; k < m; ++k) {
-    Tm[(size_t)k * m + k] = alpha[k];
-    if (k + 1 < m) Tm[(size_t)k * m + k + 1] = Tm[(size_t)(k + 1) * m + k] = beta[k];
-  }
-  jacobi_eigenvalues(Tm, m, eig);
-  return eig[m - 1];
+  return tridiagonal_eigenvalue(alpha.data(), beta.data(), (int)alpha.size(), (int)alpha.size() - 1);
 }
 }  // namespace netmax
 
@@ -336,63 +509,147 @@ int netmax_policy_generate_ex(int32_t M, const double* t, const uint8_t* adj, do
   }
   const double U_rho = rho_upper > 0.0 ? rho_upper : std::min(0.5 / lr, (1.0 - 1e-6) / (lr * max_f1));
 
-  std::vector<double> P((size_t)M * M), Y((size_t)M * M), bestP;
-  double best_tconv = INFINITY, best_rho = 0, best_lam = 0, best_tbar = 0;
-  int best_k = 0, best_r = 0;
-  for (int k = 1; k <= K; ++k) {
-    const double rho = k * U_rho / K, ar = lr * rho;
-    double L = 0.0;
-    for (int i = 0; i < M; ++i) L = std::max(L, ar / M * rows[i].sum_f1t);
-    if (!(U_time > L)) continue;
-    const double delta = (U_time - L) / R;
-    for (int r = 1; r <= R; ++r) {
-      const double tbar = U_time - (R - r) * delta, T = M * tbar;
-      std::vector<uint8_t> ok(M, 1);
-      parallel_for(M, 256, [&](int a, int b) {
-        for (int i = a; i < b; ++i) ok[i] = solve_row(rows[i], i, M, ar, T, P.data() + (size_t)i * M) ? 1 : 0;
-      });
-      if (std::find(ok.begin(), ok.end(), (uint8_t)0) != ok.end()) continue;
-      // Y_P (Eq. 22) with p_i = 1/M: p_im gamma_im = (d_im+d_mi)/2, p_im gamma_im^2 = (d_im+d_mi)^2/(4 p_im)
-      parallel_for(M, 256, [&](int a, int b) {
-        for (int i = a; i < b; ++i) {
-          double rowsum = 0.0;
-          for (int m = 0; m < M; ++m) {
-            if (m == i) continue;
-            const double pim = P[(size_t)i * M + m], pmi = P[(size_t)m * M + i];
-            const double ds = (double)adj[(size_t)i * M + m] + (double)adj[(size_t)m * M + i];
-            double lin = 0.0, quad = 0.0;
-            if (pim > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pim); }
-            if (pmi > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pmi); }
-            const double y = (ar * lin - ar * ar * quad) / M;
-            Y[(size_t)i * M + m] = y;
-            rowsum += y;
-          }
-          Y[(size_t)i * M + i] = 1.0 - rowsum;
+  for (Row& r : rows) finish_row(r);
+
+  // The grid.  lambda_2 is what costs: it is only computed where it can matter.  With v orthogonal to the
+  // all-ones vector the Rayleigh quotient v^T Y v = 1 - sum_{i<m} y_im (v_i - v_m)^2 bounds lambda_2 from
+  // below, and t_conv grows with lambda_2; with v the eigenvector of the best point so far nearly every
+  // other point is ruled out by that bound (with a margin far above its rounding).  The values of rho are
+  // shared out over threads, each of which walks its t_bar grid in order, every row starting from the
+  // solution of the previous grid point; the outcome does not depend on how the threads are timed.
+  struct Best {
+    std::vector<double> P;
+    double tconv = INFINITY, rho = 0, lam = 0, tbar = 0;
+    int k = 0, r = 0;
+  };
+  const double work_ns = (double)K * R * M * M * 12.0;
+  const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
+  const bool by_rows = M >= 1024;  // a copy of P and Y per thread would be too much: threads share a grid point instead
+  int n_threads = by_rows ? 1 : (int)std::min<double>(std::min<double>(std::min<unsigned>(hw, 16), K), 1.0 + work_ns / 4e5);
+  std::mutex mu;
+  std::vector<double> probe;             // eigenvector of the best point so far (guarded by mu)
+  double probe_tconv = INFINITY;
+  int next_k = 1;
+  auto walk = [&](std::vector<Best>& found) {
+    std::vector<double> P((size_t)M * M), Y, eta(M), v, vec;
+    std::vector<std::vector<double>> q(by_rows ? M : 1);  // scratch of solve_row
+    for (auto& buf : q) buf.resize((size_t)M + 8);
+    double v_tconv = INFINITY;
+    std::vector<uint8_t> ok(M);
+    std::vector<double> share(M);
+    for (;;) {
+      int k;
+      {
+        std::lock_guard<std::mutex> lock(mu);
+        k = next_k++;
+      }
+      if (k > K) return;
+      const double rho = k * U_rho / K, ar = lr * rho;
+      double L = 0.0;
+      for (int i = 0; i < M; ++i) L = std::max(L, ar / M * rows[i].sum_f1t);
+      if (!(U_time > L)) continue;
+      const double delta = (U_time - L) / R;
+      std::fill(eta.begin(), eta.end(), 0.0);
+      Best best;
+      for (int r = 1; r <= R; ++r) {
+        const double tbar = U_time - (R - r) * delta, T = M * tbar;
+        bool feasible = true;
+        if (by_rows) {
+          parallel_for(M, 256, [&](int a, int b) {
+            for (int i = a; i < b; ++i)
+              ok[i] = solve_row(rows[i], i, M, ar, T, &eta[i], q[i].data(), P.data() + (size_t)i * M) ? 1 : 0;
+          });
+          feasible = std::find(ok.begin(), ok.end(), (uint8_t)0) == ok.end();
+        } else {
+          for (int i = 0; i < M && feasible; ++i)
+            feasible = solve_row(rows[i], i, M, ar, T, &eta[i], q[0].data(), P.data() + (size_t)i * M);
         }
-      });
-      const double lam2 = second_eigenvalue(Y, M);
-      if (!(lam2 > 0.0 && lam2 < 1.0)) continue;
-      const double tconv = tbar * std::log(kEps) / std::log(lam2);
-      if (bestP.empty() || tconv < best_tconv * (1.0 - 1e-12)) {
-        bestP = P;
-        best_tconv = tconv;
-        best_rho = rho;
-        best_lam = lam2;
-        best_tbar = tbar;
-        best_k = k;
-        best_r = r;
+        if (!feasible) continue;
+        {
+          std::lock_guard<std::mutex> lock(mu);
+          if (probe_tconv < v_tconv) { v = probe; v_tconv = probe_tconv; }
+        }
+        // Y_P (Eq. 22) with p_i = 1/M: p_im gamma_im = (d_im+d_mi)/2, p_im gamma_im^2 = (d_im+d_mi)^2/(4 p_im)
+        auto y_of = [&](int i, int m) {
+          const double pim = P[(size_t)i * M + m], pmi = P[(size_t)m * M + i];
+          const double ds = (double)adj[(size_t)i * M + m] + (double)adj[(size_t)m * M + i];
+          double lin = 0.0, quad = 0.0;
+          if (pim > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pim); }
+          if (pmi > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pmi); }
+          return (ar * lin - ar * ar * quad) / M;
+        };
+        if (!v.empty()) {
+          parallel_for(M, by_rows ? 256 : M + 1, [&](int a, int b) {
+            for (int i = a; i < b; ++i) {
+              double acc = 0.0;
+              for (int m = i + 1; m < M; ++m) acc += y_of(i, m) * ((v[i] - v[m]) * (v[i] - v[m]));
+              share[i] = acc;
+            }
+          });
+          double rq = 1.0;
+          for (int i = 0; i < M; ++i) rq -= share[i];
+          if (rq > 0.0 && rq < 1.0 && tbar * std::log(kEps) / std::log(rq) > v_tconv * (1.0 + 1e-9)) continue;
+        }
+        Y.resize((size_t)M * M);
+        parallel_for(M, by_rows ? 256 : M + 1, [&](int a, int b) {
+          for (int i = a; i < b; ++i) {
+            double rowsum = 0.0;
+            for (int m = 0; m < M; ++m) {
+              if (m == i) continue;
+              const double y = y_of(i, m);
+              Y[(size_t)i * M + m] = y;
+              rowsum += y;
+            }
+            Y[(size_t)i * M + i] = 1.0 - rowsum;
+          }
+        });
+        const double lam2 = second_eigenvalue(Y, M, &vec, by_rows);
+        if (!(lam2 > 0.0 && lam2 < 1.0)) continue;
+        const double tconv = tbar * std::log(kEps) / std::log(lam2);
+        if (!vec.empty() && tconv < v_tconv) {
+          v = vec;
+          v_tconv = tconv;
+          std::lock_guard<std::mutex> lock(mu);
+          if (tconv < probe_tconv) { probe = vec; probe_tconv = tconv; }
+        }
+        if (best.P.empty() || tconv < best.tconv * (1.0 - 1e-12)) {
+          best.P = P;
+          best.tconv = tconv;
+          best.rho = rho;
+          best.lam = lam2;
+          best.tbar = tbar;
+          best.k = k;
+          best.r = r;
+        }
+      }
+      if (!best.P.empty()) {
+        // (of the thread's own rhos only candidates are kept: none that an earlier one of them beats)
+        if (found.empty() || best.tconv < found.back().tconv * (1.0 - 1e-12)) found.push_back(std::move(best));
+        if (found.size() > 2) found.erase(found.begin(), found.end() - 2);
       }
     }
-  }
-  if (bestP.empty()) return fail(NETMAX_INFEASIBLE, "policy_generate: no feasible (rho, t_bar) grid point");
-  std::copy(bestP.begin(), bestP.end(), prob_out);
-  *rho_out = best_rho;
+  };
+  std::vector<std::vector<Best>> found(n_threads);
+  std::vector<std::thread> pool;
+  for (int th = 1; th < n_threads; ++th) pool.emplace_back([&, th] { walk(found[th]); });
+  walk(found[0]);
+  for (auto& th : pool) th.join();
+  std::vector<const Best*> order;
+  for (const auto& list : found)
+    for (const Best& b : list) order.push_back(&b);
+  std::sort(order.begin(), order.end(), [](const Best* a, const Best* b) { return a->k < b->k; });
+  const Best* best = nullptr;
+  for (const Best* b : order)  // grid order: ties keep the earlier point
+    if (!best || b->tconv < best->tconv * (1.0 - 1e-12)) best = b;
+  if (!best) return fail(NETMAX_INFEASIBLE, "policy_generate: no feasible (rho, t_bar) grid point");
+  std::copy(best->P.begin(), best->P.end(), prob_out);
+  *rho_out = best->rho;
   if (info_out) {
-    info_out[0] = best_lam;
-    info_out[1] = best_tbar;
-    info_out[2] = best_tconv;
-    info_out[3] = best_k;
-    info_out[4] = best_r;
+    info_out[0] = best->lam;
+    info_out[1] = best->tbar;
+    info_out[2] = best->tconv;
+    info_out[3] = best->k;
+    info_out[4] = best->r;
   }
   return NETMAX_OK;
 }
@@ -600,7 +857,7 @@ int netmax_policy_generate_fixed_weight(int32_t M, const double* t, const uint8_
         }
         Y[(size_t)i * M + i] = 1.0 - (2.0 * w - w * w) * pulls / M + w * w * pulled / M;
       }
-      const double lam2 = second_eigenvalue(Y, M);
+      const double lam2 = second_eigenvalue(Y, M, nullptr, true);
       if (!(lam2 > 0.0 && lam2 < 1.0)) continue;
       const double tconv = tbar * std::log(kEps) / std::log(lam2);
       if (bestP.empty() || tconv < best_tconv * (1.0 - 1e-12)) {
