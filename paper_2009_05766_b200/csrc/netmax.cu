@@ -5,6 +5,7 @@
 #include "../../include/netmax.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -222,6 +223,8 @@ struct netmax_ctx {
   uint32_t inject_absent_ctas = 0;       // test hook: applied to the next multi-round launch, then cleared
   double* measure_out = nullptr;         // (consensus, loss) of netmax_measure (page-locked host memory)
   // host copies of the tables in force (the asynchronous timeline draws peers on the host)
+  bool host_tables = false;  // are they those of the policy in force? (need_host_tables)
+  BulkCopier bulk;           // transfers of whole M x M matrices
   std::vector<uint32_t> h_thr;
   std::vector<int32_t> h_last;
   std::vector<float> h_w;
@@ -296,23 +299,34 @@ int fail(netmax_ctx* ctx, int code, const char* fmt, ...) {
                   #call, cudaGetErrorString(e_));                                                  \
   } while (0)
 
+// From here on whole M x M matrices are worked on by threads or on the device (256 workers: 5.4 ms for a policy on
+// the host, 4.7 on the device; 512: 22 and 7).
+constexpr int32_t kManyWorkers = 320;
+
 // Link graph from speeds: d_im = 1 iff i != m and the speed is positive (symmetrised).
 int build_adjacency(netmax_ctx* ctx, int32_t M, const double* speed, std::vector<uint8_t>& adj) {
-  adj.assign((size_t)M * M, 0);
-  for (int i = 0; i < M; ++i)
-    for (int m = 0; m < M; ++m) {
-      if (i == m) continue;
-      if (!speed) { adj[(size_t)i * M + m] = 1; continue; }
-      const double a = speed[(size_t)i * M + m], b = speed[(size_t)m * M + i];
-      if (!std::isfinite(a) || !std::isfinite(b)) return fail(ctx, NETMAX_INVALID_ARG, "link speed (%d,%d) is not finite", i, m);
-      adj[(size_t)i * M + m] = (a > 0.0 && b > 0.0) ? 1 : 0;
-    }
+  adj.assign((size_t)M * M, 1);
+  std::atomic<int64_t> bad{-1};
+  constexpr int64_t kBlock = 64;  // the transposed entries are read a cache line at a time
+  parallel_rows(M, kManyWorkers, [&](int64_t r0, int64_t r1) {
+    for (int64_t ib = r0; ib < r1; ib += kBlock)
+      for (int64_t mb = 0; mb < M; mb += kBlock)
+        for (int64_t i = ib; i < std::min(r1, ib + kBlock); ++i)
+          for (int64_t m = mb; m < std::min<int64_t>(M, mb + kBlock); ++m) {
+            if (i == m) { adj[(size_t)i * M + m] = 0; continue; }
+            if (!speed) continue;
+            const double a = speed[(size_t)i * M + m], b = speed[(size_t)m * M + i];
+            if (!std::isfinite(a)) bad = i * M + m;
+            adj[(size_t)i * M + m] = (a > 0.0 && b > 0.0) ? 1 : 0;
+          }
+  });
+  if (bad >= 0) return fail(ctx, NETMAX_INVALID_ARG, "link speed (%d,%d) is not finite", (int)(bad / M), (int)(bad % M));
   // connectivity (Assumption 1) by a depth-first walk from worker 0
   std::vector<int> stack{0};
   std::vector<uint8_t> seen(M, 0);
   seen[0] = 1;
   int count = 1;
-  while (!stack.empty()) {
+  while (!stack.empty() && count < M) {
     const int v = stack.back();
     stack.pop_back();
     for (int m = 0; m < M; ++m)
@@ -323,30 +337,46 @@ int build_adjacency(netmax_ctx* ctx, int32_t M, const double* speed, std::vector
 }
 
 int validate_policy(netmax_ctx* ctx, int32_t M, const double* P, const std::vector<uint8_t>& adj) {
-  for (int i = 0; i < M; ++i) {
+  auto row = [&](int i, bool report) -> int {  // the checks of one row; the message only when asked for
     double sum = 0.0;
     for (int m = 0; m < M; ++m) {
       const double p = P[(size_t)i * M + m];
-      if (!(p >= 0.0) || !std::isfinite(p)) return fail(ctx, NETMAX_BAD_PROB_ROW, "P[%d,%d] = %g is negative or not finite", i, m, p);
+      if (!(p >= 0.0) || !std::isfinite(p))
+        return report ? fail(ctx, NETMAX_BAD_PROB_ROW, "P[%d,%d] = %g is negative or not finite", i, m, p) : NETMAX_BAD_PROB_ROW;
       if (p > 0.0 && m != i && !adj[(size_t)i * M + m])
-        return fail(ctx, NETMAX_BAD_PROB_ROW, "P[%d,%d] > 0 on a missing link (Eq. 12)", i, m);
+        return report ? fail(ctx, NETMAX_BAD_PROB_ROW, "P[%d,%d] > 0 on a missing link (Eq. 12)", i, m) : NETMAX_BAD_PROB_ROW;
       sum += p;
     }
-    if (std::fabs(sum - 1.0) > 1e-9) return fail(ctx, NETMAX_BAD_PROB_ROW, "row %d of P sums to %.12g", i, sum);
-  }
-  return NETMAX_OK;
+    if (std::fabs(sum - 1.0) > 1e-9) return report ? fail(ctx, NETMAX_BAD_PROB_ROW, "row %d of P sums to %.12g", i, sum) : NETMAX_BAD_PROB_ROW;
+    return NETMAX_OK;
+  };
+  std::atomic<int> first_bad{M};
+  parallel_rows(M, kManyWorkers, [&](int64_t a, int64_t b) {
+    for (int64_t i = a; i < b; ++i)
+      if (row((int)i, false) != NETMAX_OK) {
+        int seen = first_bad;
+        while ((int)i < seen && !first_bad.compare_exchange_weak(seen, (int)i)) {}
+        return;
+      }
+  });
+  return first_bad < M ? row(first_bad, true) : NETMAX_OK;
 }
 
 // rho <= 0: the largest rho that keeps Eq. 11 (p_im > alpha rho (d_im + d_mi)) with a 1e-6 margin.
 double default_rho(int32_t M, const double* P, const std::vector<uint8_t>& adj, double alpha) {
-  double best = INFINITY;
-  for (int i = 0; i < M; ++i)
-    for (int m = 0; m < M; ++m) {
-      const double p = P[(size_t)i * M + m];
-      if (i == m || !(p > 0.0)) continue;
-      const double dsum = (double)adj[(size_t)i * M + m] + (double)adj[(size_t)m * M + i];
-      best = std::min(best, p / (alpha * dsum));
+  std::vector<double> row_best(M, INFINITY);
+  parallel_rows(M, kManyWorkers, [&](int64_t a, int64_t b) {
+    for (int64_t i = a; i < b; ++i) {
+      double best = INFINITY;
+      for (int64_t m = 0; m < M; ++m) {
+        const double p = P[(size_t)i * M + m];
+        if (i == m || !(p > 0.0)) continue;
+        best = std::min(best, p / (alpha * (2.0 * (double)adj[(size_t)i * M + m])));  // (the graph is symmetric)
+      }
+      row_best[i] = best;
     }
+  });
+  const double best = *std::min_element(row_best.begin(), row_best.end());
   return std::isfinite(best) ? (1.0 - 1e-6) * best : 0.0;
 }
 
@@ -401,11 +431,49 @@ void build_tables(int32_t M, const double* P, const std::vector<uint8_t>& adj, d
   }
 }
 
+// Tables from P and the link graph on the device, into the context's own; waits for them (the caller's
+// buffers may go).  The asynchronous timeline draws on the host and fetches its copies (need_host_tables).
+int device_tables(netmax_ctx* ctx, const double* d_P, const uint8_t* d_adj) {
+  NM_CUDA(ctx, build_tables_device(ctx->M, d_P, d_adj, (double)(float)ctx->alpha * ctx->rho, ctx->pull_weight, ctx->thr, ctx->last_nz,
+                                   ctx->wtab, ctx->stream));
+  ctx->host_tables = false;
+  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  return NETMAX_OK;
+}
+
+int need_host_tables(netmax_ctx* ctx) {
+  if (ctx->host_tables) return NETMAX_OK;
+  const size_t MM = (size_t)ctx->M * ctx->M;
+  ctx->h_thr.resize(MM);
+  ctx->h_last.resize(ctx->M);
+  ctx->h_w.resize(MM);
+  NM_CUDA(ctx, ctx->bulk.to_host(ctx->h_thr.data(), ctx->thr, MM * sizeof(uint32_t), ctx->device, ctx->stream));
+  NM_CUDA(ctx, ctx->bulk.to_host(ctx->h_w.data(), ctx->wtab, MM * sizeof(float), ctx->device, ctx->stream));
+  NM_CUDA(ctx, cudaMemcpyAsync(ctx->h_last.data(), ctx->last_nz, ctx->M * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  ctx->host_tables = true;
+  return NETMAX_OK;
+}
+
+// Puts the tables of the policy in force on the device.  Many workers: they are built there, from P.
 int upload_policy(netmax_ctx* ctx) {
+  if (ctx->M >= kManyWorkers) {
+    const size_t MM = (size_t)ctx->M * ctx->M;
+    DeviceBuffers buf;
+    double* d_P = nullptr;
+    uint8_t* d_adj = nullptr;
+    if (buf.get(&d_P, MM) && buf.get(&d_adj, MM)) {
+      NM_CUDA(ctx, ctx->bulk.to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
+      NM_CUDA(ctx, ctx->bulk.to_device(d_adj, ctx->adj.data(), MM, ctx->device, ctx->stream));
+      return device_tables(ctx, d_P, d_adj);
+    }
+    // (no device memory to spare beside the caller's workspace: on the host, as for few workers)
+  }
   std::vector<uint32_t>& thr = ctx->h_thr;
   std::vector<int32_t>& last = ctx->h_last;
   std::vector<float>& w = ctx->h_w;
   build_tables(ctx->M, ctx->P.data(), ctx->adj, (double)(float)ctx->alpha, ctx->rho, ctx->pull_weight, thr, last, w);
+  ctx->host_tables = true;
   // pageable sources: the copies are complete (staged) when these calls return
   NM_CUDA(ctx, cudaMemcpyAsync(ctx->thr, thr.data(), thr.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
   NM_CUDA(ctx, cudaMemcpyAsync(ctx->last_nz, last.data(), last.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
@@ -423,7 +491,7 @@ int refresh_iteration_times(netmax_ctx* ctx, const double* speed) {
     speed = flat.data();
   }
   std::vector<uint8_t> adj2((size_t)M * M);
-  ctx->t_iter.assign((size_t)M * M, 0.0);
+  ctx->t_iter.resize((size_t)M * M);
   int rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_iter.data(), adj2.data());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
   return NETMAX_OK;
@@ -444,7 +512,8 @@ int resolve_policy(netmax_ctx* ctx, const double* speed, const double* prob, dou
       rc = check_rho(ctx, M, prob, ctx->adj, ctx->alpha, rho, ctx->pull_weight);
       if (rc) return rc;
     }
-    ctx->P.assign(prob, prob + (size_t)M * M);
+    ctx->P.resize((size_t)M * M);
+    parallel_copy(ctx->P.data(), prob, (size_t)M * M * sizeof(double));
     ctx->rho = rho > 0.0 ? rho : default_rho(M, prob, ctx->adj, ctx->alpha);
     return NETMAX_OK;
   }
@@ -460,9 +529,9 @@ int resolve_policy(netmax_ctx* ctx, const double* speed, const double* prob, dou
     ctx->rho = rho > 0.0 ? rho : 0.0;
     return NETMAX_OK;
   }
-  // Algorithm 3: on the device from 512 workers up (where the host generator takes seconds)
+  // Algorithm 3: on the device for many workers
   int ndev = 0;
-  const bool on_device = M >= 512 && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
+  const bool on_device = M >= kManyWorkers && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
   if (!on_device) cudaGetLastError();
   int rc = on_device ? netmax_policy_generate_device(M, ctx->t_iter.data(), ctx->adj.data(), ctx->alpha, ctx->policy_K,
                                                      ctx->policy_R, ctx->policy_rho_upper, ctx->device, ctx->stream, ctx->P.data(), &rho_sel, nullptr)
@@ -1291,31 +1360,81 @@ void netmax_destroy(netmax_ctx* ctx) {
   delete ctx;
 }
 
+// New link speeds and Algorithm 3's policy for them, for many workers: everything that is M x M is worked
+// on on the device, from the speeds to the sampler's tables; the host checks the graph meanwhile and keeps
+// the iteration times and P.  Nothing of the context changes before the search has succeeded.
+static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
+  const int32_t M = ctx->M;
+  std::vector<uint8_t> adj;
+  int graph_rc = NETMAX_OK;
+  std::string graph_error;
+  std::thread graph([&] {
+    netmax_ctx* none = nullptr;  // (messages of this thread go to its own g_error)
+    graph_rc = build_adjacency(none, M, speed, adj);
+    graph_error = g_error;
+  });
+  DeviceBuffers buf;
+  double* d_P = nullptr;
+  uint8_t* d_adj = nullptr;
+  double rho = 0.0;
+  const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
+                                          ctx->device, ctx->stream, ctx->bulk, buf, &d_P, &d_adj, &rho);
+  graph.join();
+  if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
+  if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
+  int times_rc = NETMAX_OK;
+  ctx->t_iter.resize((size_t)M * M);
+  std::thread times([&] { times_rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_iter.data(), adj.data()); });
+  ctx->rho = rho;
+  int done = device_tables(ctx, d_P, d_adj);
+  if (!done) {
+    const cudaError_t e = ctx->bulk.to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
+    if (e != cudaSuccess) done = fail(ctx, NETMAX_CUDA_ERROR, "reading P back: %s", cudaGetErrorString(e));
+  }
+  times.join();
+  ctx->adj.swap(adj);
+  if (!done && times_rc) done = fail(ctx, times_rc, "iteration times of the new speeds");
+  return done;
+}
+
 int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const double* prob, double rho) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!std::isfinite(rho)) return fail(ctx, NETMAX_INVALID_ARG, "rho is not finite");
   DeviceGuard guard(ctx->device);
-  std::vector<uint8_t> old_adj = ctx->adj;
-  std::vector<double> old_P = ctx->P, old_t = ctx->t_iter;
+  if (ctx->M >= kManyWorkers && link_speed_gbps && !prob && ctx->pull_weight <= 0.0 && rho <= 0.0) {
+    int rc = set_policy_from_links(ctx, link_speed_gbps);
+    if (!rc && ctx->async_on) rc = need_host_tables(ctx);
+    return rc;
+  }
+  std::vector<uint8_t> old_adj;
+  std::vector<double> old_P, old_t;
+  if (!prob) old_P = ctx->P;  // (a caller's P is checked before it replaces the one in force)
   const double old_rho = ctx->rho;
   int rc = NETMAX_OK;
-  if (link_speed_gbps) rc = build_adjacency(ctx, ctx->M, link_speed_gbps, ctx->adj);
+  if (link_speed_gbps) {
+    old_t = ctx->t_iter;
+    old_adj.swap(ctx->adj);
+    rc = build_adjacency(ctx, ctx->M, link_speed_gbps, ctx->adj);
+  }
   if (!rc) rc = resolve_policy(ctx, link_speed_gbps, prob, rho);
   if (rc) {  // leave the policy in force untouched
-    ctx->adj.swap(old_adj);
-    ctx->P.swap(old_P);
-    ctx->t_iter.swap(old_t);
+    if (link_speed_gbps) {
+      ctx->adj.swap(old_adj);
+      ctx->t_iter.swap(old_t);
+    }
+    if (!prob) ctx->P.swap(old_P);
     ctx->rho = old_rho;
     return rc;
   }
-  // rounds already enqueued still read the old tables: wait for them before overwriting
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  return upload_policy(ctx);
+  // rounds already enqueued still read the old tables: the new ones are written behind them on the stream
+  rc = upload_policy(ctx);
+  if (!rc && ctx->async_on) rc = need_host_tables(ctx);
+  return rc;
 }
 
 int netmax_get_policy(netmax_ctx* ctx, double* prob_out, double* rho_out) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
-  if (prob_out) std::memcpy(prob_out, ctx->P.data(), ctx->P.size() * sizeof(double));
+  if (prob_out) parallel_copy(prob_out, ctx->P.data(), ctx->P.size() * sizeof(double));
   if (rho_out) *rho_out = ctx->rho;
   return NETMAX_OK;
 }
@@ -1910,6 +2029,11 @@ int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) {
     }
     ctx->t_iter.assign(t_iter, t_iter + (size_t)M * M);
   }
+  {
+    DeviceGuard guard(ctx->device);
+    int rc = need_host_tables(ctx);
+    if (rc) return rc;
+  }
   ctx->async_on = true;
   ctx->beta = beta;
   ctx->now = 0.0;
@@ -1958,7 +2082,7 @@ static int monitor_refresh(netmax_ctx* ctx) {
   double rho = 0.0;
   int ndev = 0;
   const bool fixed = ctx->pull_weight > 0.0;  // constant pull weight: the extension section's form of Algorithm 3
-  const bool on_device = !fixed && M >= 512 && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
+  const bool on_device = !fixed && M >= kManyWorkers && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
   double floor_sel = 0.0;
   int rc = fixed ? netmax_policy_generate_fixed_weight(M, t.data(), ctx->adj.data(), ctx->pull_weight, ctx->policy_K, ctx->policy_R,
                                                        ctx->policy_rho_upper, P.data(), &floor_sel, nullptr)
@@ -1971,8 +2095,8 @@ static int monitor_refresh(netmax_ctx* ctx) {
   ctx->P.swap(P);
   if (!fixed) ctx->rho = rho;
   ctx->monitor_refreshes += 1;
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  return upload_policy(ctx);
+  rc = upload_policy(ctx);
+  return rc ? rc : need_host_tables(ctx);
 }
 
 int netmax_async_monitor(netmax_ctx* ctx, double period_s) {

@@ -30,6 +30,7 @@
 #include "../../include/netmax.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <functional>
@@ -51,16 +52,7 @@ int fail(int code, const std::string& msg) {
 }
 
 void parallel_for(int n, int min_parallel, const std::function<void(int, int)>& body) {
-  unsigned hw = std::thread::hardware_concurrency();
-  int threads = (n >= min_parallel && hw > 1) ? (int)std::min<unsigned>(hw, 16) : 1;
-  if (threads <= 1) { body(0, n); return; }
-  std::vector<std::thread> pool;
-  const int per = (n + threads - 1) / threads;
-  for (int t = 0; t < threads; ++t) {
-    const int a = std::min(n, t * per), b = std::min(n, a + per);
-    if (a < b) pool.emplace_back(body, a, b);
-  }
-  for (auto& th : pool) th.join();
+  netmax::parallel_rows(n, min_parallel, [&](int64_t a, int64_t b) { body((int)a, (int)b); });
 }
 
 // ---- vector helpers: eight doubles at a time, compiled for the instruction sets a host may have -----
@@ -287,7 +279,7 @@ double tridiagonal_eigenvalue(const double* d, const double* e, int m, int index
   hi += pad;
   for (int it = 0; it < 200; ++it) {
     const double mid = 0.5 * (lo + hi);
-    if (!(mid > lo && mid < hi) || hi - lo <= 4e-17) break;
+    if (!(mid > lo && mid < hi)) break;
     if (count_below(d, e2.data(), m, mid) > index) hi = mid; else lo = mid;
   }
   return 0.5 * (lo + hi);
@@ -300,7 +292,9 @@ void tridiagonal_eigenvector(const double* d, const double* e, int m, double lam
   if (m == 1) { z[0] = 1.0; return; }
   std::vector<double> u0(m), u1(m, 0.0), u2(m, 0.0), l(m, 0.0);
   std::vector<uint8_t> swapped(m, 0);
-  const double tiny = 1e-16;
+  double tiny = 0.0;  // a pivot that stands for zero: the matrix's rounding
+  for (int i = 0; i < m; ++i) tiny = std::max(tiny, std::fabs(d[i]) + (i + 1 < m ? std::fabs(e[i]) : 0.0));
+  tiny = 1e-16 * tiny + 1e-300;
   double a = d[0] - lambda, b = e[0];  // the current row: diagonal, superdiagonal
   for (int i = 0; i + 1 < m; ++i) {
     const double c = e[i], dn = d[i + 1] - lambda, bn = i + 2 < m ? e[i + 1] : 0.0;
@@ -445,31 +439,45 @@ namespace netmax {
 double tridiagonal_top_eigenvalue(const std::vector<double>& alpha, const std::vector<double>& beta) {
   return tridiagonal_eigenvalue(alpha.data(), beta.data(), (int)alpha.size(), (int)alpha.size() - 1);
 }
+void tridiagonal_top_vector(const std::vector<double>& alpha, const std::vector<double>& beta, double lambda, std::vector<double>& z) {
+  tridiagonal_eigenvector(alpha.data(), beta.data(), (int)alpha.size(), lambda, z);
+}
 }  // namespace netmax
 
 extern "C" {
 
 int netmax_iteration_times(int32_t M, int64_t d, const double* speed, double* t_out, uint8_t* adj_out) {
   if (M < 2 || d < 1 || !speed || !t_out || !adj_out) return fail(NETMAX_INVALID_ARG, "iteration_times: bad argument");
-  double nmin = INFINITY;
-  for (int i = 0; i < M; ++i)
-    for (int m = 0; m < M; ++m) {
-      const size_t at = (size_t)i * M + m;
-      const double a = speed[at], b = speed[(size_t)m * M + i];
-      if (!std::isfinite(a)) return fail(NETMAX_INVALID_ARG, "iteration_times: link speed is not finite");
-      const bool link = (i != m) && a > 0.0 && b > 0.0;
-      adj_out[at] = link ? 1 : 0;
-      t_out[at] = link ? 32.0 * (double)d / (a * 1e9) : 0.0;   // N_im: a full fp32 replica over the link
-      if (link) nmin = std::min(nmin, t_out[at]);
-    }
+  // (by blocks of columns, so that the transposed entries are read a cache line at a time; rows over threads)
+  constexpr int kBlock = 64;
+  std::vector<double> row_min(M, INFINITY);
+  std::atomic<bool> finite{true};
+  netmax::parallel_rows(M, 512, [&](int64_t r0, int64_t r1) {
+    for (int64_t ib = r0; ib < r1; ib += kBlock)
+      for (int64_t mb = 0; mb < M; mb += kBlock)
+        for (int64_t i = ib; i < std::min(r1, ib + kBlock); ++i)
+          for (int64_t m = mb; m < std::min<int64_t>(M, mb + kBlock); ++m) {
+            const size_t at = (size_t)i * M + m;
+            const double a = speed[at], b = speed[(size_t)m * M + i];
+            if (!std::isfinite(a)) finite = false;
+            const bool link = (i != m) && a > 0.0 && b > 0.0;
+            adj_out[at] = link ? 1 : 0;
+            t_out[at] = link ? 32.0 * (double)d / (a * 1e9) : 0.0;   // N_im: a full fp32 replica over the link
+            if (link) row_min[i] = std::min(row_min[i], t_out[at]);
+          }
+  });
+  if (!finite) return fail(NETMAX_INVALID_ARG, "iteration_times: link speed is not finite");
+  const double nmin = *std::min_element(row_min.begin(), row_min.end());
   if (!std::isfinite(nmin)) return fail(NETMAX_NOT_CONNECTED, "iteration_times: no link has a positive speed");
   const double C = 0.25 * nmin;   // C_i: computation is the short part of an iteration
-  for (int i = 0; i < M; ++i)
-    for (int m = 0; m < M; ++m) {
-      const size_t at = (size_t)i * M + m;
-      if (i == m) t_out[at] = C;
-      else if (adj_out[at]) t_out[at] = std::max(C, t_out[at]);   // t_im = max{C_i, N_im}
-    }
+  netmax::parallel_rows(M, 512, [&](int64_t r0, int64_t r1) {
+    for (int64_t i = r0; i < r1; ++i)
+      for (int64_t m = 0; m < M; ++m) {
+        const size_t at = (size_t)i * M + m;
+        if (i == m) t_out[at] = C;
+        else if (adj_out[at]) t_out[at] = std::max(C, t_out[at]);   // t_im = max{C_i, N_im}
+      }
+  });
   return NETMAX_OK;
 }
 
