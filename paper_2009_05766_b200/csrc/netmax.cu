@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "netmax_kernels.cuh"
+#include "netmax_tiles.cuh"
 #include "netmax_policy.h"
 
 using namespace netmax;
@@ -121,14 +122,6 @@ struct RoundPlan {  // launch shape of round_kernel and multi_round_kernel
   int64_t n_tiles = 0;
 };
 
-struct ResidentPlan {  // launch shape of resident_rounds_kernel
-  bool ok = false;
-  int threads = 0, grid = 0, G = 0, log2G = 0, draw_chunk = 0;
-  size_t smem = 0;
-  int64_t n_tiles = 0, max_rounds = 0;
-  int64_t min_rounds = 1;  // rounds a call must run to repay loading and storing the tiles
-};
-
 struct FusedPlan {  // launch shape of fused_rounds_kernel
   bool ok = false;
   int threads = 0, grid = 0, max_rounds = 0;
@@ -137,18 +130,20 @@ struct FusedPlan {  // launch shape of fused_rounds_kernel
   int64_t n_tiles = 0;
 };
 
-struct ClusterPlan {  // launch shape of cluster_rounds_kernel
+struct TilePlan {  // launch shape of tile_rounds_kernel
   bool ok = false;
-  int threads = 0, grid = 0, C = 0, rpc = 0, max_rounds = 0;
+  int threads = 0, grid = 0, G = 0, log2G = 0, rows = 0;  // rows: per thread
+  bool pre_reduce = false;
   size_t smem = 0;
-  int64_t n_tiles = 0;
+  int64_t n_tiles = 0, max_rounds = 0;
+  int64_t min_rounds = 1;  // rounds a call must run to repay loading and storing the tiles
 };
 
 struct Layout {
   int64_t ld = 0, ldq = 0, nq = 0;  // row stride in elements / in 16-byte column groups; column groups in use
   int elem = 4, halves = 1;         // bytes per stored element; Philox blocks (4 elements) per column group
   size_t plane = 0;                 // bytes of one [M][ld] array
-  size_t off_x0 = 0, off_x1 = 0, off_c = 0, off_thr = 0, off_last = 0, off_w = 0, off_trace = 0, off_wring = 0, off_tel = 0,
+  size_t off_x0 = 0, off_x1 = 0, off_c = 0, off_thr = 0, off_last = 0, off_w = 0, off_trace = 0, off_draws = 0, off_tel = 0,
          off_partials = 0, off_ticket = 0, off_colpart = 0, off_coltick = 0, off_pipe_tel = 0, total = 0;
 };
 
@@ -176,7 +171,7 @@ Layout make_layout(int64_t M, int64_t d, int64_t trace_rounds, int storage) {
   L.off_last = take((size_t)M * sizeof(int32_t));
   L.off_w = take((size_t)M * M * sizeof(float));
   L.off_trace = take((size_t)trace_rounds * M * sizeof(int32_t));
-  L.off_wring = take((size_t)trace_rounds * M * sizeof(float));  // pull weight of every draw in the trace ring
+  L.off_draws = take((size_t)trace_rounds * M * sizeof(int2));  // (peer, pull weight) of every draw in the trace ring
   L.off_tel = take((size_t)trace_rounds * 2 * sizeof(double));
   L.off_partials = take((size_t)kMaxGrid * 2 * sizeof(double) * kFusedMaxRounds);  // per round of a fused launch; two sets for multi-round launches
   L.off_ticket = take(256);
@@ -211,7 +206,7 @@ struct netmax_ctx {
   int32_t* last_nz = nullptr;
   float* wtab = nullptr;
   int32_t* trace = nullptr;
-  float* wring = nullptr;
+  int2* draws = nullptr;  // (peer, bits of the pull weight) of every draw in the trace ring
   double* tel = nullptr;  // telemetry ring: in page-locked host memory (tel_on_host) or, when it is long, on the device
   bool tel_on_host = false;
   double* partials = nullptr;
@@ -267,10 +262,8 @@ struct netmax_ctx {
   RoundPlan round_plan[2];
   bool fused_planned = false;
   FusedPlan fused;
-  bool resident_planned = false;
-  ResidentPlan resident;
-  bool cluster_planned = false;
-  ClusterPlan cluster;
+  bool tiles_planned = false;
+  TilePlan tiles;
   PhiloxKeys keys;
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
@@ -568,15 +561,15 @@ int launch_init(netmax_ctx* ctx, unsigned char* dst, double stddev, uint32_t tag
   return NETMAX_OK;
 }
 
-int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int32_t* out, float* w_out, int64_t slot0,
+int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int32_t* out, int2* draws, int64_t slot0,
                    int64_t ring) {
   if (n_rounds <= 0) return NETMAX_OK;
   SampleParams p;
   p.thresholds = ctx->thr;
   p.last_nz = ctx->last_nz;
   p.out = out;
-  p.w_out = w_out;
-  p.host_out = w_out ? ctx->trace_mirror : nullptr;  // (draws into the context's own ring)
+  p.draws = draws;
+  p.host_out = draws ? ctx->trace_mirror : nullptr;  // (draws into the context's own ring)
   p.wtab = ctx->wtab;
   p.slot0 = slot0;
   p.ring = ring;
@@ -599,7 +592,7 @@ using StepKernel = void (*)(const StepParams);
 // halves: 1 for fp32 state, 2 for bfloat16 state (Philox blocks per 16-byte column group)
 template <int kHalves>
 StepKernel pick_step_kernel_h(int objective) {
-  return objective == 1 ? step_kernel<1, true, kHalves> : step_kernel<0, true, kHalves>;
+  return objective == 1 ? step_kernel<1, kHalves> : step_kernel<0, kHalves>;
 }
 StepKernel pick_step_kernel(int objective, int halves) {
   return halves == 2 ? pick_step_kernel_h<2>(objective) : pick_step_kernel_h<1>(objective);
@@ -607,12 +600,12 @@ StepKernel pick_step_kernel(int objective, int halves) {
 
 template <int kHalves>
 RoundKernel pick_kernel_h(int objective, bool short_vectors) {
-  if (objective == 2) return short_vectors ? round_kernel<2, true, 4, kHalves> : round_kernel<2, true, 1, kHalves>;
-  if (short_vectors) return objective == 1 ? round_kernel<1, true, 4, kHalves> : round_kernel<0, true, 4, kHalves>;
+  if (objective == 2) return short_vectors ? round_kernel<2, 4, kHalves> : round_kernel<2, 1, kHalves>;
+  if (short_vectors) return objective == 1 ? round_kernel<1, 4, kHalves> : round_kernel<0, 4, kHalves>;
 #ifdef NETMAX_BF16_LONG_RIF
-  if (kHalves == 2) return objective == 1 ? round_kernel<1, true, NETMAX_BF16_LONG_RIF, kHalves> : round_kernel<0, true, NETMAX_BF16_LONG_RIF, kHalves>;
+  if (kHalves == 2) return objective == 1 ? round_kernel<1, NETMAX_BF16_LONG_RIF, kHalves> : round_kernel<0, NETMAX_BF16_LONG_RIF, kHalves>;
 #endif
-  return objective == 1 ? round_kernel<1, true, 1, kHalves> : round_kernel<0, true, 1, kHalves>;
+  return objective == 1 ? round_kernel<1, 1, kHalves> : round_kernel<0, 1, kHalves>;
 }
 RoundKernel pick_kernel(int objective, bool short_vectors, int halves) {
   return halves == 2 ? pick_kernel_h<2>(objective, short_vectors) : pick_kernel_h<1>(objective, short_vectors);
@@ -621,27 +614,42 @@ RoundKernel pick_kernel(int objective, bool short_vectors, int halves) {
 using MultiRoundKernel = void (*)(const MultiRoundParams);
 
 MultiRoundKernel pick_multi_kernel(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? multi_round_kernel<1, true, 2> : multi_round_kernel<0, true, 2>;
-  return objective == 1 ? multi_round_kernel<1, true, 1> : multi_round_kernel<0, true, 1>;
+  if (halves == 2) return objective == 1 ? multi_round_kernel<1, 2> : multi_round_kernel<0, 2>;
+  return objective == 1 ? multi_round_kernel<1, 1> : multi_round_kernel<0, 1>;
 }
 
 using FusedKernel = void (*)(const FusedParams);
 
 template <int kRounds>
 FusedKernel pick_fused_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, true, kRounds> : fused_rounds_kernel<0, true, true, kRounds>;
-  return objective == 1 ? fused_rounds_kernel<1, true, false, kRounds> : fused_rounds_kernel<0, true, false, kRounds>;
+  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kRounds> : fused_rounds_kernel<0, true, kRounds>;
+  return objective == 1 ? fused_rounds_kernel<1, false, kRounds> : fused_rounds_kernel<0, false, kRounds>;
 }
 // The instance for launches of `rounds` rounds (both instances share one shared-memory layout, FusedParams::slots).
 FusedKernel pick_fused_kernel(int objective, int halves, int rounds) {
   return rounds <= 4 ? pick_fused_kernel_r<4>(objective, halves) : pick_fused_kernel_r<kFusedMaxRounds>(objective, halves);
 }
 
-using ResidentKernel = void (*)(const ResidentParams);
+using TileKernel = void (*)(const TileParams);
 
-ResidentKernel pick_resident_kernel(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? resident_rounds_kernel<1, true, true> : resident_rounds_kernel<0, true, true>;
-  return objective == 1 ? resident_rounds_kernel<1, true, false> : resident_rounds_kernel<0, true, false>;
+template <int kRows>
+TileKernel pick_tile_kernel_r(int objective, int halves) {
+  if (halves == 2) return objective == 1 ? tile_rounds_kernel<1, true, kRows> : tile_rounds_kernel<0, true, kRows>;
+  return objective == 1 ? tile_rounds_kernel<1, false, kRows> : tile_rounds_kernel<0, false, kRows>;
+}
+TileKernel pick_tile_kernel(int objective, int halves, int rows) {
+  switch (rows) {
+    case 1: return pick_tile_kernel_r<1>(objective, halves);
+    case 2: return pick_tile_kernel_r<2>(objective, halves);
+    case 3: return pick_tile_kernel_r<3>(objective, halves);
+    case 4: return pick_tile_kernel_r<4>(objective, halves);
+    case 5: return pick_tile_kernel_r<5>(objective, halves);
+    case 6: return pick_tile_kernel_r<6>(objective, halves);
+    case 7: return pick_tile_kernel_r<7>(objective, halves);
+    case 8: return pick_tile_kernel_r<8>(objective, halves);
+    case 9: return pick_tile_kernel_r<9>(objective, halves);
+    default: return pick_tile_kernel_r<10>(objective, halves);
+  }
 }
 
 // The kernels' noise scale: sigma (at its fp32 rounding, the value the update is defined with)
@@ -745,88 +753,99 @@ int plan_round(netmax_ctx* ctx, RoundPlan& plan, int objective) {
   return NETMAX_OK;
 }
 
-// Rounds whose draws the resident kernel stages in shared memory at a time: about 8 KB worth
-// for up to 512 workers, none beyond (threads then fetch the draws of their own rows).
-int resident_draw_chunk(int64_t M) { return M <= 512 ? (int)std::max<int64_t>(2, 1024 / M) : 0; }
-
-size_t resident_smem(int64_t M, int threads, int G) {
-  return (size_t)48 * M * G + 2 * sizeof(float) * resident_scratch_floats(threads, G) + 128 * sizeof(float) +
-         (size_t)resident_draw_chunk(M) * M * 8;
-}
-
-// Short vectors whose M rows of at least one column group fit in a CTA's shared memory run all
-// rounds of a call on resident columns (resident_rounds_kernel).  Small M: a thread per column
-// group, as few threads per CTA as keep the CTA count within a few per SM (the problem is
-// latency-bound: spread it over the SMs).  Larger M: G column groups per CTA, the rows of each
-// split over the threads; G as large as fits, but no larger than leaves every SM a tile.
-int plan_resident_uncached(netmax_ctx* ctx, const RoundPlan& plan, ResidentPlan& f) {
-  f = ResidentPlan();
-  if (!plan.short_vectors) return NETMAX_OK;
+// Launch shape of tile_rounds_kernel: G column groups per tile, W warps per CTA.  Modelled from what was
+// measured: a row of a column group costs its scheduler about 190 cycles, a round at least 600 cycles plus
+// 230 for every row of a thread however little else runs, and an SM holds 16 warps (128 registers) as far as
+// its shared memory goes.  Wider tiles win ties (longer pieces of a row per load).  A thread keeps the noise of
+// its rows in registers, so it gets at most eight (ten where nothing else fits: 4097 to 4700 workers).
+int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, TilePlan& f) {
+  f = TilePlan();
+  if (ctx->fuse_rounds == 1 || fused.ok) return NETMAX_OK;
   const int64_t M = ctx->M, nq = (ctx->d + 3) / 4;
-  const size_t limit = (size_t)224 * 1024;
-  int threads = 0, G = 0;
-  if (resident_smem(M, 32, 32) <= (size_t)100 * 1024) {
-    // small M.  The problem is latency-bound: give a thread as few rows as still leaves about two
-    // warps per scheduler busy, i.e. split the rows of a group over RL lanes (a power of two)
-    const int64_t target_threads = (int64_t)ctx->sm_count * 256;
-    const int64_t rows_per_thread = std::max<int64_t>(1, M * nq / target_threads);
-    int RL = 1;
-    while (RL < 32 && RL < M && (M + RL - 1) / RL > rows_per_thread) RL <<= 1;
-    for (int cand : {32, 64, 128, 256}) {
-      const int g = cand / RL;
-      if (g < 1 || (RL > 1 && g > 32)) break;
-      if (resident_smem(M, cand, g) > (size_t)100 * 1024) break;
-      threads = cand;
-      G = g;
-      if ((nq + g - 1) / g <= (int64_t)8 * ctx->sm_count) break;
+  const bool f32 = ctx->storage == NETMAX_STORAGE_F32;
+  if (!plan.short_vectors && ctx->fuse_rounds >= 2 && M > 144) return NETMAX_OK;  // (fuse_rounds: see the C header)
+  const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)227 * 1024;
+  double best = 0.0;
+  int best_c = 0;
+  for (int row_limit : {8, 10}) {
+    for (int G = 32, log2G = 5; G >= 1; G >>= 1, --log2G) {
+      for (int W = 1; W <= 16; ++W) {
+        const int RL = W * 32 / G;
+        const int K = (int)((M + RL - 1) / RL);
+        if (K > row_limit || (RL > M && W > 1)) continue;
+        bool pre = false;
+        size_t smem = tile_smem(M, W * 32, G, false);
+        const size_t small = tile_smem(M, W * 32, G, true);
+        if (smem > per_cta || (smem > small && per_sm / (smem + 1024) < std::min<size_t>(16 / W, per_sm / (small + 1024)))) {
+          pre = true;
+          smem = small;
+        }
+        if (smem > per_cta) continue;
+        const int64_t fit = std::min<int64_t>(16 / W, (int64_t)(per_sm / (smem + 1024)));
+        if (fit < 1) continue;
+        const int64_t n_tiles = (nq + G - 1) / G;
+        const int64_t c = std::min<int64_t>(fit, (n_tiles + ctx->sm_count - 1) / ctx->sm_count);
+        const double passes = n_tiles > (int64_t)ctx->sm_count * c * 8 ? (double)n_tiles / (double)(ctx->sm_count * c)
+                                                                        : (double)((n_tiles + ctx->sm_count * c - 1) / (ctx->sm_count * c));
+        const double cycles = passes * std::max((double)(c * K * W) * 190.0 / 4.0, 600.0 + 230.0 * K) * (pre ? 1.03 : 1.0);
+        if (best == 0.0 || cycles < best * 0.999) {
+          best = cycles;
+          best_c = (int)c;
+          f.threads = W * 32;
+          f.G = G;
+          f.log2G = log2G;
+          f.rows = K;
+          f.pre_reduce = pre;
+          f.smem = smem;
+          f.n_tiles = n_tiles;
+        }
+      }
     }
+    if (best > 0.0) break;
   }
-  if (threads == 0) {  // rows of a group split over the threads
-    G = 32;
-    while (G > 1 && (size_t)48 * M * G > (size_t)190 * 1024) G >>= 1;
-    while (G > 1 && (nq + G - 1) / G < ctx->sm_count) G >>= 1;
-    threads = (int)std::min<int64_t>(512, std::max<int64_t>(64, floor_pow2(M * G / 2)));
-    threads = std::max(threads, G);
-    if (resident_smem(M, threads, G) > limit) return NETMAX_OK;
-  }
-  f.threads = threads;
-  f.G = G;
-  f.log2G = 0;
-  while ((1 << f.log2G) < G) ++f.log2G;
-  f.draw_chunk = (int)std::min<int64_t>(resident_draw_chunk(M), ctx->trace_rounds);
-  f.smem = resident_smem(M, threads, G);
-  f.n_tiles = (nq + G - 1) / G;
-  f.max_rounds = std::max<int64_t>(1, std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.n_tiles));
-  // A call pays once for bringing its tiles on chip and back -- narrow columns of all M rows, which stream
-  // badly (about 1.1 TB/s with one column group per tile) -- and then saves on every round.  Rounds from
-  // which that paid in measurements (us per round, resident columns against the per-round kernels, calls of
-  // 1 / 2 / 4 / many rounds): 4 x 4096 elements 13.4 / 7.0 / 4.1 / 0.9 against 10.3 / 8.2 / 6.0 / 3.8;
-  // 4096 x 1024: 57 / 33 / 21 / 9.5 against 29 / 23 / 19 / 16; 4096 x 4096: 219 / 128 / 80 / 33 against
-  // 66 / 61 / 58 / 54; 4096 x 16384: 837 / 492 / 310 / 136 against 195 / 192 / 190 / 188.
-  const int64_t elements = M * ctx->d;
-  f.min_rounds = elements <= ((int64_t)1 << 20) ? 2 : elements <= ((int64_t)1 << 22) ? 6 : elements <= ((int64_t)1 << 24) ? 8 : 16;
-  ResidentKernel k = pick_resident_kernel(ctx->objective, ctx->L.halves);
+  if (best == 0.0) return NETMAX_OK;
+  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, f.rows);
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   NM_CUDA(ctx, allow_smem((const void*)k, f.smem));
-  int per_sm = 0;
-  NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, f.smem));
-  if (per_sm < 1) return NETMAX_OK;
-  f.grid = (int)std::min<int64_t>(f.n_tiles, (int64_t)per_sm * ctx->sm_count);
+  int fit = 0;
+  NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k, f.threads, f.smem));
+  if (fit < 1) return NETMAX_OK;
+  f.grid = (int)std::min<int64_t>(f.n_tiles, std::min<int64_t>((int64_t)std::max(best_c, fit) * ctx->sm_count, kMaxGrid));
+  f.grid = (int)std::min<int64_t>(f.grid, (int64_t)fit * ctx->sm_count);
+  f.max_rounds = std::max<int64_t>(1, std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.grid));
+  if (plan.short_vectors) {
+    // A call pays once for bringing its tiles on chip and back -- narrow columns of all M rows, which stream
+    // badly -- and then saves on every round.  Rounds from which that paid in measurements (us per round,
+    // resident columns against the per-round kernels, calls of 1 / 2 / 4 / many rounds): 4 x 4096 elements
+    // 13.4 / 7.0 / 4.1 / 0.9 against 10.3 / 8.2 / 6.0 / 3.8; 4096 x 1024: 57 / 33 / 21 / 9.5 against
+    // 29 / 23 / 19 / 16; 4096 x 4096: 219 / 128 / 80 / 33 against 66 / 61 / 58 / 54; 4096 x 16384:
+    // 837 / 492 / 310 / 136 against 195 / 192 / 190 / 188.
+    const int64_t elements = M * ctx->d;
+    f.min_rounds = elements <= ((int64_t)1 << 20) ? 2 : elements <= ((int64_t)1 << 22) ? 6 : elements <= ((int64_t)1 << 24) ? 8 : 16;
+  } else if (ctx->fuse_rounds >= 2) {
+    f.min_rounds = 2;
+    f.max_rounds = std::min<int64_t>(f.max_rounds, ctx->fuse_rounds);
+  } else {
+    // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the
+    // worker counts for which the header has always said so; longer ones are where resident tiles gain most.
+    static const unsigned char fused_short[22] = {0, 1, 1, 1, 0, 1, 1, 1, 1, 1, 1, 0, 0, 1, 0, 0, 0, 1, 1, 1, 1, 1};  // M = 67 ... 88
+    const bool short_calls = !f32 || M <= 66 || (M <= 88 && fused_short[M - 67]);
+    f.min_rounds = short_calls ? 2 : 9;
+  }
   f.ok = true;
   return NETMAX_OK;
 }
 
-int plan_resident(netmax_ctx* ctx, const RoundPlan& plan, ResidentPlan& f) {
-  if (ctx->resident_planned) {
-    f = ctx->resident;
-    return NETMAX_OK;
+int plan_tiles(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, TilePlan& f) {
+  if (!ctx->tiles_planned) {
+    TilePlan fresh;
+    int rc = plan_tiles_uncached(ctx, plan, fused, fresh);
+    if (rc) return rc;
+    ctx->tiles = fresh;
+    ctx->tiles_planned = true;
   }
-  int rc = plan_resident_uncached(ctx, plan, f);
-  if (rc == NETMAX_OK) {
-    ctx->resident = f;
-    ctx->resident_planned = true;
-  }
-  return rc;
+  f = ctx->tiles;
+  return NETMAX_OK;
 }
 
 int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
@@ -849,13 +868,13 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   NM_CUDA(ctx, cudaFuncSetAttribute(pick_fused_kernel(ctx->objective, ctx->L.halves, 4), cudaFuncAttributePreferredSharedMemoryCarveout,
                                     (int)cudaSharedmemCarveoutMaxShared));
-  // The table of draws at the head of the shared memory takes 16 M bytes per round of the launch: room for
+  // The table of draws at the head of the shared memory takes 8 M bytes per round of the launch: room for
   // as many rounds as were asked for, unless the smaller table of four rounds lets more threads live on an SM
   // (M = 36: the last kilobytes decide between two CTAs and one).
   int threads = 0, per_sm = 0, slots = 0;
   size_t fixed = 0;
   for (int rounds : {want_rounds, std::min(want_rounds, 4)}) {
-    const size_t fixed_r = align_up((size_t)rounds * M * 16, 128) + 64 * sizeof(double);
+    const size_t fixed_r = align_up((size_t)rounds * M * 8, 128) + 64 * sizeof(double);
     int threads_r = 0, per_sm_r = 0;
     for (int cand : {256, 128, 64}) {
       const size_t smem = fixed_r + (size_t)48 * M * cand;
@@ -901,115 +920,6 @@ int plan_fused(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   return rc;
 }
 
-using ClusterKernel = void (*)(const ClusterParams);
-
-ClusterKernel pick_cluster_kernel(int objective) {
-  return objective == 1 ? cluster_rounds_kernel<1, true> : cluster_rounds_kernel<0, true>;
-}
-
-#ifndef NETMAX_CLUSTER_SIZE
-#define NETMAX_CLUSTER_SIZE 0  // 0: chosen from the number of workers (cluster_size below); 2, 4, 8: fixed
-#endif
-#ifndef NETMAX_CLUSTER_THREADS
-#define NETMAX_CLUSTER_THREADS 0  // 0: the smallest of 64, 128, 256 threads per CTA whose slabs fit
-#endif
-
-size_t cluster_smem(int rpc, int threads) {
-  return align_up((size_t)kClusterMaxRounds * rpc * 16, 128) + (size_t)3 * rpc * threads * 16 + (size_t)2 * threads * 16 +
-         64 * sizeof(double);
-}
-
-// CTAs per cluster for M workers, 0 for "one launch per round instead".  A CTA needs enough rows between
-// two cluster barriers to pay for them (a barrier costs about 1,500 cycles even for the last CTA to arrive)
-// and few enough that eight CTAs of 64 threads still fit on an SM; a ragged last CTA makes the others
-// wait; smaller clusters have cheaper barriers and more pulls that stay in the CTA.  The sweet spot is
-// eight rows per CTA in as few CTAs as possible, but the details do not follow a formula, so the size is
-// the one measured fastest: every size from 2 to 8, M x 2,000,002 elements, four rounds per launch against
-// one launch per round (profiles/cluster_rounds_kernel_cfg4.md has the sweep).  Entered only where the
-// cluster shape took less than 0.97 of the per-round time: 0.83-0.93 for M = 37 ... 66, 0.92-0.97 for most
-// of 68 ... 88, nothing beyond.  Clusters of 16 (not portable) fit too few at a time: 1.3-2.1 x slower.
-// `forced` (the caller asked for fused rounds): any M up to 8 x 18 rows gets the table's size or else the
-// one whose CTAs hold closest to eight rows.
-int cluster_size(int64_t M, bool forced) {
-  if (NETMAX_CLUSTER_SIZE != 0) return NETMAX_CLUSTER_SIZE;
-  static const unsigned char by_workers[] = {
-      // M = 37 ... 88 (up to 36 workers fused_rounds_kernel holds all rows in one CTA)
-      5, 5, 5, 5, 4, 4, 4, 4, 5, 6, 6, 6, 5, 5, 5, 5, 5, 5, 5, 7, 6, 6, 6, 6, 8, 8,
-      8, 8, 6, 6, 0, 4, 7, 7, 0, 7, 7, 7, 7, 7, 7, 0, 0, 8, 0, 0, 0, 8, 8, 8, 8, 8};
-  if (M >= 37 && M < 37 + (int64_t)sizeof by_workers && by_workers[M - 37] != 0) return by_workers[M - 37];
-  if (!forced) return 0;
-  int best = 0;
-  int64_t best_gap = 0;
-  for (int c = 2; c <= 8; ++c) {
-    const int64_t rpc = (M + c - 1) / c, gap = rpc > 8 ? rpc - 8 : 8 - rpc;
-    if (rpc <= 18 && (best == 0 || gap < best_gap)) {
-      best = c;
-      best_gap = gap;
-    }
-  }
-  return best;
-}
-
-// Long fp32 vectors with more workers than fused_rounds_kernel can hold per thread (M > 36): the rows
-// of a tile are split over the CTAs of a cluster (cluster_rounds_kernel), up to 18 rows per CTA.
-int plan_cluster_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, ClusterPlan& f) {
-  f = ClusterPlan();
-  if (ctx->fuse_rounds == 1 || plan.short_vectors || fused.ok || ctx->storage != NETMAX_STORAGE_F32) return NETMAX_OK;
-  const int64_t M = ctx->M;
-  const int C = cluster_size(M, ctx->fuse_rounds >= 2);
-  if (C == 0) return NETMAX_OK;
-  const int rpc = (int)((M + C - 1) / C);
-  if (rpc > 18) return NETMAX_OK;
-  ClusterKernel k = pick_cluster_kernel(ctx->objective);
-  NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
-  // Small CTAs, many per SM: a CTA that waits at the cluster barrier leaves its SM to the others.  Measured
-  // on 64 x 11.2 M elements, clusters of 8: 64 threads (8 CTAs per SM) 1.39 ms per round, 128 threads 1.43,
-  // 256 threads 1.69, 32 threads 2.08; clusters of 4 with 64 threads 1.54 (one launch per round: 1.62).
-  for (int cand : {64, 128, 256}) {
-    if (NETMAX_CLUSTER_THREADS != 0 && cand != NETMAX_CLUSTER_THREADS) continue;
-    const size_t smem = cluster_smem(rpc, cand);
-    if (smem > (size_t)113 * 1024) continue;  // at least two CTAs per SM
-    NM_CUDA(ctx, allow_smem((const void*)k, smem));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(C * ctx->sm_count));
-    cfg.blockDim = dim3((unsigned)cand);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)C;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
-    if (clusters < 1) continue;
-    f.threads = cand;
-    f.C = C;
-    f.rpc = rpc;
-    f.smem = smem;
-    f.n_tiles = ((ctx->d + 3) / 4 + cand - 1) / cand;
-    f.max_rounds = ctx->fuse_rounds >= 2 ? std::min(ctx->fuse_rounds, kClusterMaxRounds) : kClusterMaxRounds;
-    f.grid = (int)std::min<int64_t>(f.n_tiles, (int64_t)clusters) * C;
-    f.ok = true;
-    break;
-  }
-  return NETMAX_OK;
-}
-
-int plan_cluster(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, ClusterPlan& f) {
-  if (ctx->cluster_planned) {
-    f = ctx->cluster;
-    return NETMAX_OK;
-  }
-  int rc = plan_cluster_uncached(ctx, plan, fused, f);
-  if (rc == NETMAX_OK) {
-    ctx->cluster = f;
-    ctx->cluster_planned = true;
-  }
-  return rc;
-}
-
 // What every launch of the round kernels shares: buffers, tile shape, step sizes, keys.
 RoundParams make_round_params(const netmax_ctx* ctx, const RoundPlan& plan) {
   RoundParams p;
@@ -1048,13 +958,60 @@ struct ColumnRange {
   bool whole = true;        // the whole vector (the only form bfloat16 state takes)
 };
 
+// One launch of tile_rounds_kernel: `chunk` rounds from round r over a column range; the telemetry of its
+// rounds is added up by the last CTA (finalize), or by a launch of its own when there are many rounds.
+int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, const RoundParams& p, const ColumnRange& range,
+                 const unsigned char* xin, unsigned char* xout, const unsigned char* cbase, double* tel, uint64_t r, int chunk,
+                 bool finalize) {
+  TileParams tp;
+  tp.x_cur = reinterpret_cast<const char*>(xin);
+  tp.x_nxt = reinterpret_cast<char*>(xout);
+  tp.c = reinterpret_cast<const char*>(cbase);
+  tp.draws = ctx->draws;
+  tp.partials = reinterpret_cast<double*>(ctx->colpart);
+  tp.tel = tel;
+  tp.ticket = ctx->ticket;
+  tp.error = const_cast<unsigned int*>(ctx->dev_error);
+  tp.slot0 = (int64_t)(r % (uint64_t)ctx->trace_rounds);
+  tp.ring = ctx->trace_rounds;
+  tp.first_round = r;
+  tp.n_rounds = chunk;
+  tp.nq = range.nq4;
+  tp.n_tiles = (range.nq4 + tiles.G - 1) / tiles.G;
+  tp.row_bytes = p.row_bytes;
+  tp.M = p.M;
+  tp.tail = range.tail4;
+  tp.G = tiles.G;
+  tp.log2G = tiles.log2G;
+  tp.pre_reduce = tiles.pre_reduce ? 1 : 0;
+  tp.finalize = finalize ? 1 : 0;
+  tp.alpha = p.alpha;
+  tp.sigma = p.sigma;
+  tp.inv_M = p.inv_M;
+  tp.q_offset = ctx->q_offset + (uint32_t)range.q0;
+  tp.keys = p.keys;
+  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, tiles.rows);
+  NM_CUDA(ctx, allow_smem((const void*)k, tiles.smem));
+  const int64_t grid = std::min<int64_t>(tiles.grid, tp.n_tiles);
+  k<<<(unsigned)grid, tiles.threads, tiles.smem, stream>>>(tp);
+  ctx->launches += 1;
+  if (!finalize) {
+    const int warps_per_block = kThreads / 32;
+    sum_tile_partials_kernel<<<(unsigned)((chunk + warps_per_block - 1) / warps_per_block), kThreads, 0, stream>>>(
+        tp.partials, grid, chunk, (double)p.inv_M, tel, tp.slot0, tp.ring);
+    ctx->launches += 1;
+  }
+  NM_CUDA(ctx, cudaGetLastError());
+  return NETMAX_OK;
+}
+
 // Enqueues rounds [first, first + n) -- their draws are in the trace ring -- for one column range on
 // `stream`: up to four rounds per launch where tiles stay resident (fused_rounds_kernel, or
 // cluster_rounds_kernel for more workers), else one launch per round.  `cur` is the buffer that holds
 // the range's values at round `first`; it is flipped launch by launch.  Telemetry of the range goes
 // to tel (ring-indexed like the context's).
 int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& plan, const FusedPlan& fused,
-                       const ClusterPlan& cluster, RoundParams p, const ColumnRange& range, double* tel, uint64_t first,
+                       const TilePlan& tiles, RoundParams p, const ColumnRange& range, double* tel, uint64_t first,
                        int64_t n, int& cur) {
   RoundKernel kernel = pick_kernel(ctx->objective, plan.short_vectors, ctx->L.halves);
   const size_t shift = range.whole ? 0 : (size_t)range.q0 * 16;  // bytes into every row (fp32 state when not whole)
@@ -1071,12 +1028,20 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
   for (int64_t b = 0; b < n;) {
     const unsigned char* xin = ctx->x[cur] + shift;
     unsigned char* xout = ctx->x[cur ^ 1] + shift;
-    if ((fused.ok || cluster.ok) && n - b >= 2) {  // the next rounds in one launch over resident tiles
+    if (tiles.ok && n >= tiles.min_rounds && n - b >= 2) {
+      const int64_t launches_left = (n - b + tiles.max_rounds - 1) / tiles.max_rounds;
+      const int64_t chunk = (n - b + launches_left - 1) / launches_left;
+      int rc = launch_tiles(ctx, stream, tiles, p, range, xin, xout, cbase, tel, r, (int)chunk, true);
+      if (rc) return rc;
+      cur ^= 1;
+      r += (uint64_t)chunk;
+      b += chunk;
+      continue;
+    }
+    if (fused.ok && n - b >= 2) {  // the next rounds in one launch over resident tiles
       // launches of even length (20 rounds at 8 per launch: 7 + 7 + 6, not 8 + 8 + 4)
-      const int64_t per_launch = fused.ok ? fused.max_rounds : cluster.max_rounds;
-      const int64_t launches_left = (n - b + per_launch - 1) / per_launch;
+      const int64_t launches_left = (n - b + fused.max_rounds - 1) / fused.max_rounds;
       const int chunk = (int)((n - b + launches_left - 1) / launches_left);
-      const int threads = fused.ok ? fused.threads : cluster.threads;
       FusedParams fp;
       fp.x_cur = reinterpret_cast<const float4*>(xin);
       fp.x_nxt = reinterpret_cast<float4*>(xout);
@@ -1090,9 +1055,9 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
       fp.ring = ctx->trace_rounds;
       fp.first_round = r;
       fp.n_rounds = chunk;
-      fp.slots = fused.ok ? fused.slots : kClusterMaxRounds;
+      fp.slots = fused.slots;
       fp.nq = range.nq4;
-      fp.n_tiles = (range.nq4 + threads - 1) / threads;
+      fp.n_tiles = (range.nq4 + fused.threads - 1) / fused.threads;
       fp.row_bytes = p.row_bytes;
       fp.M = p.M;
       fp.tail = range.tail4;
@@ -1101,32 +1066,10 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
       fp.inv_M = p.inv_M;
       fp.q_offset = ctx->q_offset + (uint32_t)range.q0;
       fp.keys = p.keys;
-      if (!fused.ok) {  // rows split over the CTAs of a cluster
-        ClusterParams cpar;
-        cpar.f = fp;
-        cpar.rpc = cluster.rpc;
-        ClusterKernel ck = pick_cluster_kernel(ctx->objective);
-        NM_CUDA(ctx, allow_smem((const void*)ck, cluster.smem));
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)(std::min<int64_t>(cluster.grid / cluster.C, fp.n_tiles) * cluster.C));
-        lc.blockDim = dim3((unsigned)cluster.threads);
-        lc.dynamicSmemBytes = cluster.smem;
-        lc.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)cluster.C;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        lc.attrs = &attr;
-        lc.numAttrs = 1;
-        NM_CUDA(ctx, cudaLaunchKernelEx(&lc, ck, cpar));
-      } else {
-        // (the attribute belongs to the kernel, not to this context: another context may have lowered it)
-        // (one instance for all launches of the call: the larger one unless the whole call is four rounds or fewer)
-        FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, (int)std::min<int64_t>(n, fused.max_rounds));
-        NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
-        fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
-      }
+      // (one instance for all launches of the call: the larger one unless the whole call is four rounds or fewer)
+      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, (int)std::min<int64_t>(n, fused.max_rounds));
+      NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
+      fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
       ctx->launches += 1;
       cur ^= 1;
       r += (uint64_t)chunk;
@@ -1281,7 +1224,7 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
   ctx->last_nz = (int32_t*)(ctx->base + L.off_last);
   ctx->wtab = (float*)(ctx->base + L.off_w);
   ctx->trace = (int32_t*)(ctx->base + L.off_trace);
-  ctx->wring = (float*)(ctx->base + L.off_wring);
+  ctx->draws = (int2*)(ctx->base + L.off_draws);
   ctx->tel = (double*)(ctx->base + L.off_tel);
   ctx->partials = (double*)(ctx->base + L.off_partials);
   ctx->ticket = (unsigned int*)(ctx->base + L.off_ticket);
@@ -1445,7 +1388,7 @@ static int synchronise(netmax_ctx* ctx) {
   ctx->host_writes = false;
   if (*ctx->dev_error == 0u) return NETMAX_OK;
   *ctx->dev_error = 0u;
-  return fail(ctx, NETMAX_CUDA_ERROR, "a multi-round launch gave up waiting at its grid barrier; replicas are not valid");
+  return fail(ctx, NETMAX_CUDA_ERROR, "a multi-round launch gave up waiting at a barrier; replicas are not valid");
 }
 
 // Copies `bytes` of device memory to the host and synchronises.  Small copies go through the page-locked
@@ -1545,12 +1488,8 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
   FusedPlan fused;
   rc = plan_fused(ctx, plan, fused);
   if (rc) return rc;
-  ResidentPlan resident;
-  rc = plan_resident(ctx, plan, resident);
-  if (rc) return rc;
-  if (ctx->fuse_rounds == 1) resident.ok = false;  // one launch per round was asked for
-  ClusterPlan cluster;
-  rc = plan_cluster(ctx, plan, fused, cluster);
+  TilePlan tiles;
+  rc = plan_tiles(ctx, plan, fused, tiles);
   if (rc) return rc;
 
   RoundParams p = make_round_params(ctx, plan);
@@ -1560,46 +1499,19 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
     // peers of a batch of rounds in one launch (counter-based draws do not depend on x),
     // at most one lap of the ring at a time
     const int64_t batch = std::min<int64_t>(n_rounds - done, ctx->trace_rounds);
-    rc = launch_sampler(ctx, (uint64_t)ctx->rounds, batch, ctx->trace, ctx->wring, ctx->rounds % ctx->trace_rounds,
+    rc = launch_sampler(ctx, (uint64_t)ctx->rounds, batch, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds,
                         ctx->trace_rounds);
     if (rc) return rc;
-    if (resident.ok && batch >= resident.min_rounds) {
+    if (plan.short_vectors && tiles.ok && batch >= tiles.min_rounds) {
       // short vectors: every round of the batch on shared-memory-resident columns
-      ResidentKernel rk = pick_resident_kernel(ctx->objective, ctx->L.halves);
-      int64_t b = 0;
-      while (b < batch) {
-        const int64_t chunk = std::min<int64_t>(batch - b, resident.max_rounds);
-        ResidentParams rp;
-        rp.x_cur = reinterpret_cast<const char*>(ctx->x[ctx->cur]);
-        rp.x_nxt = reinterpret_cast<char*>(ctx->x[ctx->cur ^ 1]);
-        rp.c = reinterpret_cast<const char*>(ctx->c);
-        rp.trace = ctx->trace;
-        rp.wring = ctx->wring;
-        rp.partials = reinterpret_cast<double*>(ctx->colpart);
-        rp.slot0 = ctx->rounds % ctx->trace_rounds;
-        rp.ring = ctx->trace_rounds;
-        rp.first_round = (uint64_t)ctx->rounds;
-        rp.n_rounds = (int32_t)chunk;
-        rp.nq = (ctx->d + 3) / 4;
-        rp.n_tiles = resident.n_tiles;
-        rp.row_bytes = p.row_bytes;
-        rp.M = p.M;
-        rp.tail = (int32_t)(ctx->d % 4);
-        rp.G = resident.G;
-        rp.log2G = resident.log2G;
-        rp.draw_chunk = resident.draw_chunk;
-        rp.alpha = p.alpha;
-        rp.sigma = p.sigma;
-        rp.inv_M = p.inv_M;
-        rp.q_offset = p.q_offset;
-        rp.keys = p.keys;
-        NM_CUDA(ctx, allow_smem((const void*)rk, resident.smem));
-        rk<<<resident.grid, resident.threads, resident.smem, ctx->stream>>>(rp);
-        const int warps_per_block = kThreads / 32;
-        sum_tile_partials_kernel<<<(unsigned)((chunk + warps_per_block - 1) / warps_per_block), kThreads, 0, ctx->stream>>>(
-            rp.partials, rp.n_tiles, rp.n_rounds, (double)p.inv_M, ctx->tel, rp.slot0, rp.ring);
-        ctx->launches += 2;
-        NM_CUDA(ctx, cudaGetLastError());
+      ColumnRange all;
+      all.nq4 = (ctx->d + 3) / 4;
+      all.tail4 = (int32_t)(ctx->d % 4);
+      for (int64_t b = 0; b < batch;) {
+        const int64_t chunk = std::min<int64_t>(batch - b, tiles.max_rounds);
+        rc = launch_tiles(ctx, ctx->stream, tiles, p, all, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], ctx->c, ctx->tel,
+                          (uint64_t)ctx->rounds, (int)chunk, false);
+        if (rc) return rc;
         ctx->cur ^= 1;
         ctx->rounds += chunk;
         b += chunk;
@@ -1648,7 +1560,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
       all.tail4 = (int32_t)(ctx->d % 4);
       all.whole = true;
       int cur = ctx->cur;
-      rc = launch_long_rounds(ctx, ctx->stream, plan, fused, cluster, p, all, ctx->tel, (uint64_t)ctx->rounds, batch, cur);
+      rc = launch_long_rounds(ctx, ctx->stream, plan, fused, tiles, p, all, ctx->tel, (uint64_t)ctx->rounds, batch, cur);
       if (rc) return rc;
       ctx->cur = cur;
       ctx->rounds += batch;
@@ -1690,8 +1602,8 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   FusedPlan fused;
   rc = plan_fused(ctx, plan, fused);
   if (rc) return rc;
-  ClusterPlan cluster;
-  rc = plan_cluster(ctx, plan, fused, cluster);
+  TilePlan tiles;
+  rc = plan_tiles(ctx, plan, fused, tiles);
   if (rc) return rc;
   if (!ctx->up_stream) NM_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->up_stream, cudaStreamNonBlocking));
   if (!ctx->down_stream) NM_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->down_stream, cudaStreamNonBlocking));
@@ -1723,7 +1635,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
 
   const uint64_t first = (uint64_t)ctx->rounds;
   ctx->host_writes = true;
-  rc = launch_sampler(ctx, first, n_rounds, ctx->trace, ctx->wring, ctx->rounds % ctx->trace_rounds, ctx->trace_rounds);
+  rc = launch_sampler(ctx, first, n_rounds, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds, ctx->trace_rounds);
   if (rc) return bail(rc);
   // uploads must not overtake earlier work of the context that still reads the buffers
   NM_PIPE(cudaEventRecord(events[2 * chunks], ctx->stream));
@@ -1748,7 +1660,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
     NM_PIPE(cudaEventRecord(events[2 * k], ctx->up_stream));
     NM_PIPE(cudaStreamWaitEvent(ctx->stream, events[2 * k], 0));
     int cur = ctx->cur;
-    rc = launch_long_rounds(ctx, ctx->stream, plan, fused, cluster, p, range, ctx->pipe_tel + (size_t)k * ctx->trace_rounds * 2,
+    rc = launch_long_rounds(ctx, ctx->stream, plan, fused, tiles, p, range, ctx->pipe_tel + (size_t)k * ctx->trace_rounds * 2,
                             first, n_rounds, cur);
     if (rc) return bail(rc);
     cur_end = cur;
@@ -1777,7 +1689,7 @@ int netmax_set_fuse_rounds(netmax_ctx* ctx, int32_t fuse_rounds) {
     return fail(ctx, NETMAX_INVALID_ARG, "fuse_rounds = %d outside [0, %d]", fuse_rounds, kFusedMaxRounds);
   ctx->fuse_rounds = fuse_rounds;
   ctx->fused_planned = false;
-  ctx->cluster_planned = false;
+  ctx->tiles_planned = false;
   return NETMAX_OK;
 }
 

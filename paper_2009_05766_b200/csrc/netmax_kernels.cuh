@@ -33,9 +33,9 @@ struct SampleParams {
   const uint32_t* thresholds;  // [M][M] non-decreasing per row
   const int32_t* last_nz;      // [M] last index with p > 0
   int32_t* out;                // slot s of round r is out + ((slot0 + r) % ring) * M
-  float* w_out;                // same indexing: pull weight of the draw (0 on a self-draw); may be NULL
+  int2* draws;                 // same indexing: (peer, bits of the pull weight, 0 on a self-draw); may be NULL
   int32_t* host_out;           // same indexing: mirror in page-locked host memory; may be NULL
-  const float* wtab;           // [M][M] pull weights (read when w_out is given)
+  const float* wtab;           // [M][M] pull weights (read when draws is given)
   int64_t slot0, ring;
   uint64_t first_round;
   int64_t n_rounds;
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) sample_peers_kernel(const SampleParams p)
     const int64_t at = ((p.slot0 + r) % p.ring) * p.M + i;
     p.out[at] = m;
     if (p.host_out) p.host_out[at] = m;
-    if (p.w_out) p.w_out[at] = (m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m);
+    if (p.draws) p.draws[at] = make_int2(m, __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m)));
   }
 }
 
@@ -132,151 +132,55 @@ __device__ __forceinline__ int live_lanes(bool ragged, int tail, int h) {
   return ragged ? min(4, max(0, tail - 4 * h)) : 4;
 }
 
-// Per-lane noise scale of one column group (fused_rounds_kernel): sigma_s on real elements, 0 on the padding lanes of a
-// row's last, ragged group.  Padding lanes hold x = c = 0 in every row; with no noise Eq. 15-16
-// keep them at exactly +0 (every product and sum below is +0 or -0 + +0), so nothing has to be
-// masked after the update.
-struct NoiseLanes {
-  pair_t a, b;
-};
-__device__ __forceinline__ NoiseLanes noise_lanes(float sigma_s, int live) {
-  NoiseLanes n;
-  n.a = pack2(live > 0 ? sigma_s : 0.0f, live > 1 ? sigma_s : 0.0f);
-  n.b = pack2(live > 2 ? sigma_s : 0.0f, live > 3 ? sigma_s : 0.0f);
-  return n;
-}
-
 // Eq. 15 and Eq. 16 on one column group of one worker, on packed fp32 pairs:
-//   g = (x - c) + sigma z,  h = x - alpha g                                       (Eq. 15)
+//   g = (x - c) + n,      h = x - alpha g                                          (Eq. 15)
 //   x' = h - w (h - x_m),   w = alpha rho gamma_im  (w = 0 on a self-draw)          (Eq. 16)
-// rnd is the Philox block of the four elements (counter: global index of the block, worker,
-// round or -- on the asynchronous timeline -- the worker's local iteration); ns holds, per lane,
-// sigma sqrt(2 ln 2), the noise scale with the constant factor of the Box-Muller radius folded in
-// (fast path; the accurate path takes it out again), or 0 on padding lanes; nw2 is (-w, -w).
-// ta, tb return x - c for the caller's loss statistic.
-template <int kObjective, bool kFastNoise>
-__device__ __forceinline__ ulonglong2 update_core_rnd(float alpha, const NoiseLanes& ns, uint4 rnd, ulonglong2 xv, ulonglong2 cv,
-                                                      ulonglong2 xm, pair_t nw2, pair_t& ta, pair_t& tb) {
-  const pair_t neg1 = pack2(-1.0f, -1.0f);
-  ta = fma2(cv.x, neg1, xv.x);  // x - c
-  tb = fma2(cv.y, neg1, xv.y);
-  pair_t ha = xv.x, hb = xv.y;
-  if (kObjective == 1) {
-    const pair_t nalpha2 = pack2(-alpha, -alpha);
-    pair_t za, zb, sa = ns.a, sb = ns.b;
-    if (kFastNoise) {
-      za = normal_pair_fast_unscaled(rnd.x, rnd.y);
-      zb = normal_pair_fast_unscaled(rnd.z, rnd.w);
-    } else {
-      const pair_t inv = pack2((float)(1.0 / kNormalScale), (float)(1.0 / kNormalScale));
-      sa = mul2(sa, inv);
-      sb = mul2(sb, inv);
-      const float4 z = normals4<false>(rnd);
-      za = pack2(z.x, z.y);
-      zb = pack2(z.z, z.w);
-    }
-    ha = fma2(nalpha2, fma2(sa, za, ta), xv.x);
-    hb = fma2(nalpha2, fma2(sb, zb, tb), xv.y);
-  }
-  const pair_t oa = fma2(nw2, fma2(xm.x, neg1, ha), ha);
-  const pair_t ob = fma2(nw2, fma2(xm.y, neg1, hb), hb);
-  return make_ulonglong2(oa, ob);
-}
-
-// The Philox block of the noise of one column group of one worker (only drawn when there is noise).
+// n is sigma times the normals (scaled_normals4; +0 on padding lanes of a row's last, ragged group, which
+// hold x = c = 0 and so stay at exactly +0).  ta, tb return x - c for the caller's loss statistic.
+// Operand counts matter here: a packed instruction with three distinct register pairs issues every 3.2
+// cycles, one with two every 2.2 -- hence subtractions instead of multiply-adds with -1, and the product
+// with alpha as two scalar multiply-adds that take alpha from the constant bank.
 template <int kObjective>
-__device__ __forceinline__ uint4 noise_block(const PhiloxKeys& keys, uint32_t iter_lo, uint32_t ctr3, uint32_t q32, uint32_t worker) {
-  if (kObjective != 1) return make_uint4(0u, 0u, 0u, 0u);
-  return philox4x32_10(q32, worker, iter_lo, ctr3, keys);
-}
-
-// The same update with the Philox block drawn inside, for the kernels that stream rows through
-// registers (round_kernel, step_kernel) or walk them one at a time (resident_rounds_kernel).  One
-// noise scale serves all four lanes and the padding lanes of a ragged group (`live` < 4 real
-// elements) are cleared after the update: the streaming kernel runs at its register limit, and
-// this form -- one scale pair instead of NoiseLanes' two, the masking behind a branch that is
-// almost never taken -- measured 191 us per round against 223 on 8 x 11.2 M elements.  Real lanes
-// see exactly the arithmetic of update_core_rnd, so all kernels agree bit for bit.
-template <int kObjective, bool kFastNoise>
-__device__ __forceinline__ ulonglong2 update_core(float alpha, float sigma_s, const PhiloxKeys& keys,
-                                                  uint32_t iter_lo, uint32_t ctr3, uint32_t q32, uint32_t worker,
-                                                  ulonglong2 xv, ulonglong2 cv, ulonglong2 xm, float w, int live,
+__device__ __forceinline__ ulonglong2 update_core(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm, float w,
                                                   pair_t& ta, pair_t& tb) {
-  const pair_t neg1 = pack2(-1.0f, -1.0f);
-  const pair_t nw2 = pack2(-w, -w);
-  ta = fma2(cv.x, neg1, xv.x);  // x - c
-  tb = fma2(cv.y, neg1, xv.y);
+  ta = sub2(xv.x, cv.x);
+  tb = sub2(xv.y, cv.y);
   pair_t ha = xv.x, hb = xv.y;
   if (kObjective == 1) {
-    pair_t sig2 = pack2(sigma_s, sigma_s);
-    const pair_t nalpha2 = pack2(-alpha, -alpha);
-    const uint4 rnd = philox4x32_10(q32, worker, iter_lo, ctr3, keys);
-    pair_t za, zb;
-    if (kFastNoise) {
-      za = normal_pair_fast_unscaled(rnd.x, rnd.y);
-      zb = normal_pair_fast_unscaled(rnd.z, rnd.w);
-    } else {
-      sig2 = mul2(sig2, pack2((float)(1.0 / kNormalScale), (float)(1.0 / kNormalScale)));
-      const float4 z = normals4<false>(rnd);
-      za = pack2(z.x, z.y);
-      zb = pack2(z.z, z.w);
-    }
-    ha = fma2(nalpha2, fma2(sig2, za, ta), xv.x);
-    hb = fma2(nalpha2, fma2(sig2, zb, tb), xv.y);
+    float g0, g1, g2, g3, x0, x1, x2, x3;
+    unpack2(add2(ta, n.x), g0, g1);
+    unpack2(add2(tb, n.y), g2, g3);
+    unpack2(xv.x, x0, x1);
+    unpack2(xv.y, x2, x3);
+    ha = pack2(fmaf(-alpha, g0, x0), fmaf(-alpha, g1, x1));
+    hb = pack2(fmaf(-alpha, g2, x2), fmaf(-alpha, g3, x3));
   }
-  pair_t oa = fma2(nw2, fma2(xm.x, neg1, ha), ha);
-  pair_t ob = fma2(nw2, fma2(xm.y, neg1, hb), hb);
-  if (live < 4) {  // keep the padding lanes of the last group at zero
-    float o0, o1, o2, o3;
-    unpack2(oa, o0, o1);
-    unpack2(ob, o2, o3);
-    if (live < 1) o0 = 0.f;
-    if (live < 2) o1 = 0.f;
-    if (live < 3) o2 = 0.f;
-    oa = pack2(o0, o1);
-    ob = pack2(o2, 0.f);
-  }
-  return make_ulonglong2(oa, ob);
+  const pair_t nw2 = pack2(-w, -w);
+  return make_ulonglong2(fma2(nw2, sub2(ha, xm.x), ha), fma2(nw2, sub2(hb, xm.y), hb));
+}
+
+// The noise of one column group of one worker, with its Philox block drawn on the spot.
+template <int kObjective>
+__device__ __forceinline__ ulonglong2 draw_noise(float sigma_s, const PhiloxKeys& keys, uint32_t iter_lo, uint32_t ctr3, uint32_t q32,
+                                                 uint32_t worker, int live) {
+  if (kObjective != 1) return make_ulonglong2(0ull, 0ull);
+  const ulonglong2 n = scaled_normals4(philox4x32_10(q32, worker, iter_lo, ctr3, keys), sigma_s);
+  return live < 4 ? mask_lanes(n, live) : n;
 }
 
 // update_core plus the telemetry sums of the round-start values.  kObjective == 2 measures only.
-template <int kObjective, bool kFastNoise>
-__device__ __forceinline__ ulonglong2 row_update_rnd(float alpha, const NoiseLanes& ns, uint4 rnd, ulonglong2 xv, ulonglong2 cv,
-                                                     ulonglong2 xm, ulonglong2 pivot, pair_t nw2, ColAcc& acc, LossAcc& lacc) {
-  const pair_t neg1 = pack2(-1.0f, -1.0f);
+template <int kObjective>
+__device__ __forceinline__ ulonglong2 row_update(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm,
+                                                 ulonglong2 pivot, float w, ColAcc& acc, LossAcc& lacc) {
   pair_t ta, tb;
   ulonglong2 o = xv;
   if (kObjective == 2) {
-    ta = fma2(cv.x, neg1, xv.x);
-    tb = fma2(cv.y, neg1, xv.y);
+    ta = sub2(xv.x, cv.x);
+    tb = sub2(xv.y, cv.y);
   } else {
-    o = update_core_rnd<kObjective, kFastNoise>(alpha, ns, rnd, xv, cv, xm, nw2, ta, tb);
+    o = update_core<kObjective>(alpha, n, xv, cv, xm, w, ta, tb);
   }
-  const pair_t da = fma2(pivot.x, neg1, xv.x), db = fma2(pivot.y, neg1, xv.y);  // x - pivot
-  acc.s1a = add2(acc.s1a, da);
-  acc.s1b = add2(acc.s1b, db);
-  acc.s2a = fma2(da, da, acc.s2a);
-  acc.s2b = fma2(db, db, acc.s2b);
-  lacc.la = fma2(ta, ta, lacc.la);
-  lacc.lb = fma2(tb, tb, lacc.lb);
-  return o;
-}
-
-template <int kObjective, bool kFastNoise>
-__device__ __forceinline__ ulonglong2 row_update(float alpha, float sigma_s, const PhiloxKeys& keys, uint32_t round_lo,
-                                                 uint32_t ctr3, uint32_t q32, uint32_t worker, ulonglong2 xv, ulonglong2 cv,
-                                                 ulonglong2 xm, ulonglong2 pivot, float w, int live, ColAcc& acc,
-                                                 LossAcc& lacc) {
-  const pair_t neg1 = pack2(-1.0f, -1.0f);
-  pair_t ta, tb;
-  ulonglong2 o = xv;
-  if (kObjective == 2) {
-    ta = fma2(cv.x, neg1, xv.x);
-    tb = fma2(cv.y, neg1, xv.y);
-  } else {
-    o = update_core<kObjective, kFastNoise>(alpha, sigma_s, keys, round_lo, ctr3, q32, worker, xv, cv, xm, w, live, ta, tb);
-  }
-  const pair_t da = fma2(pivot.x, neg1, xv.x), db = fma2(pivot.y, neg1, xv.y);  // x - pivot
+  const pair_t da = sub2(xv.x, pivot.x), db = sub2(xv.y, pivot.y);
   acc.s1a = add2(acc.s1a, da);
   acc.s1b = add2(acc.s1b, db);
   acc.s2a = fma2(da, da, acc.s2a);
@@ -410,7 +314,7 @@ __device__ __forceinline__ ulonglong2 ld_x(const char* ptr) {
 }
 
 // All tiles of this CTA for one round.  Every thread of the CTA must call this.
-template <int kObjective, bool kFastNoise, int kRowsInFlight, bool kCoherent, int kHalves>
+template <int kObjective, int kRowsInFlight, bool kCoherent, int kHalves>
 __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* x_cur, float4* x_nxt, const int32_t* peers,
                                             uint32_t round_lo, uint32_t ctr3, int2* s_pw, float4* s_col,
                                             double& acc_cons, double& acc_loss) {
@@ -479,10 +383,11 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
             ulonglong2 o;
 #pragma unroll
             for (int h = 0; h < kHalves; ++h) {
-              const ulonglong2 oh = row_update<kObjective, kFastNoise>(
-                  p.alpha, p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
-                  group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h), __int_as_float(pw[u].y),
-                  live_lanes(ragged, p.tail, h), acc[h], lacc);
+              const ulonglong2 noise = draw_noise<kObjective>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i,
+                                                              live_lanes(ragged, p.tail, h));
+              const ulonglong2 oh = row_update<kObjective>(p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
+                                                           group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h),
+                                                           __int_as_float(pw[u].y), acc[h], lacc);
               if (kHalves == 1) o = oh;
               else if (h == 0) o.x = narrow_bf16x4(oh);
               else o.y = narrow_bf16x4(oh);
@@ -570,7 +475,7 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
 // kRowsInFlight = 1 (64 registers, 4 CTAs/SM) is the streaming shape for long vectors, where
 // occupancy hides the HBM latency; kRowsInFlight = 4 (2 CTAs/SM) serves short, L2-resident
 // problems, where a thread's chain of dependent row loads is what takes the time.
-template <int kObjective, bool kFastNoise, int kRowsInFlight, int kHalves>
+template <int kObjective, int kRowsInFlight, int kHalves>
 __global__ void __launch_bounds__(256, kRowsInFlight != 1 ? 2 : kHalves == 1 ? NETMAX_ROUND_MIN_CTAS : NETMAX_ROUND_MIN_CTAS_BF16)
     round_kernel(const RoundParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -579,7 +484,7 @@ __global__ void __launch_bounds__(256, kRowsInFlight != 1 ? 2 : kHalves == 1 ? N
   float4* s_col = reinterpret_cast<float4*>(smem_raw + head);
   double* s_red = reinterpret_cast<double*>(smem_raw + head + (p.rl > 1 ? (size_t)blockDim.x * 32 * kHalves : 0));
   double acc_cons = 0.0, acc_loss = 0.0;
-  round_tiles<kObjective, kFastNoise, kRowsInFlight, false, kHalves>(p, p.x_cur, p.x_nxt, p.peers, p.round_lo, p.ctr3, s_pw,
+  round_tiles<kObjective, kRowsInFlight, false, kHalves>(p, p.x_cur, p.x_nxt, p.peers, p.round_lo, p.ctr3, s_pw,
                                                                      s_col, acc_cons, acc_loss);
   finalize_telemetry(p, acc_cons, acc_loss, s_red);
 }
@@ -630,7 +535,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int
   return s_ok != 0;
 }
 
-template <int kObjective, bool kFastNoise, int kHalves>
+template <int kObjective, int kHalves>
 __global__ void __launch_bounds__(256, 2) multi_round_kernel(const MultiRoundParams mp) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const RoundParams& p = mp.r;
@@ -645,7 +550,7 @@ __global__ void __launch_bounds__(256, 2) multi_round_kernel(const MultiRoundPar
     const int64_t slot = (mp.slot0 + k) % mp.ring;
     double* partials = mp.partials2 + (size_t)(k & 1) * 2 * gridDim.x;
     double acc_cons = 0.0, acc_loss = 0.0;
-    round_tiles<kObjective, kFastNoise, 4, true, kHalves>(p, x_cur, x_nxt, mp.trace + slot * p.M, (uint32_t)round,
+    round_tiles<kObjective, 4, true, kHalves>(p, x_cur, x_nxt, mp.trace + slot * p.M, (uint32_t)round,
                                                           philox_ctr3(kTagNoise, round), s_pw, s_col, acc_cons, acc_loss);
     block_partials(partials, acc_cons, acc_loss, s_red);
     if (!grid_barrier(mp.barrier, (unsigned int)(k + 1), mp.error, mp.absent_ctas)) return;
@@ -712,18 +617,18 @@ struct FusedParams {
   PhiloxKeys keys;
 };
 
-// Dynamic shared memory: (peer row offset, -, -weight, -weight) int4[slots][M], then the slabs
+// Dynamic shared memory: (peer row offset, weight) int2[slots][M], then the slabs
 // float4[3][M][blockDim] (replicas of even rounds, of odd rounds, centres), then 64 doubles.
 // Any block size that is a multiple of 32 up to 256 works.
 // kRounds: rounds a launch runs at most (4 or kFusedMaxRounds); a thread keeps two double accumulators per round,
 // and a launch of up to four rounds runs 4 % faster on the instance that holds eight instead of sixteen of them.
-template <int kObjective, bool kFastNoise, bool kBf16, int kRounds>
+template <int kObjective, bool kBf16, int kRounds>
 __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int tid = threadIdx.x, T = blockDim.x, M = p.M;
-  int4* s_pw = reinterpret_cast<int4*>(smem_raw);  // (byte offset of the peer's row in a slab, unused, -w, -w)
-  const uint32_t head = ((uint32_t)(p.slots * M * 16) + 127u) & ~127u;
+  int2* s_pw = reinterpret_cast<int2*>(smem_raw);  // (byte offset of the peer's row in a slab, pull weight)
+  const uint32_t head = ((uint32_t)(p.slots * M * 8) + 127u) & ~127u;
   const uint32_t stride = (uint32_t)T * 16u;     // bytes between consecutive rows of a slab
   const uint32_t plane = (uint32_t)M * stride;   // bytes of one [M][T] slab
   unsigned char* slab = smem_raw + head + (uint32_t)tid * 16u;  // this thread's column: slabs 0, 1 (replicas), 2 (centres)
@@ -733,8 +638,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     const int32_t* peers = p.trace + ((p.slot0 + k) % p.ring) * M;
     for (int i = tid; i < M; i += T) {
       const int32_t m = __ldg(peers + i);
-      const int nw = __float_as_int((m == i) ? -0.0f : -__ldg(p.wtab + (size_t)i * M + m));
-      s_pw[k * M + i] = make_int4((int)((uint32_t)m * stride), 0, nw, nw);
+      s_pw[k * M + i] = make_int2((int)((uint32_t)m * stride), __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * M + m)));
     }
   }
   __syncthreads();
@@ -758,7 +662,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
     const int64_t q = tile * T + tid;
     if (q >= p.nq) continue;  // no barrier below: threads are independent (and later tiles only have larger q)
-    const NoiseLanes ns = noise_lanes(p.sigma, live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0));
+    const int live = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
     const uint32_t q32 = (uint32_t)q + p.q_offset;
     const int64_t q_next = q + (int64_t)gridDim.x * T;
     const bool have_next = kPrefetch && tile + gridDim.x < p.n_tiles && q_next < p.nq;
@@ -800,8 +704,9 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     const char* const cq_next = reinterpret_cast<const char*>(p.c) + (uint64_t)q_next * kGroupBytes;
 
     // one round over the thread's column group; kLast: the tile's last round (see above)
-    auto run_round = [&](int k, auto last_tag) {
+    auto run_round = [&](int k, auto last_tag, auto ragged_tag) {
       constexpr bool kLast = decltype(last_tag)::value;
+      constexpr bool kRagged = decltype(ragged_tag)::value;
       const uint64_t round = p.first_round + (uint64_t)k;
       const uint32_t round_lo = (uint32_t)round, ctr3 = philox_ctr3(kTagNoise, round);
       const unsigned char* cur = slab + ((base + (uint32_t)k) & 1u) * plane;
@@ -817,19 +722,19 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
           sx += stride;
         }
       }
-      const int4* pw = s_pw + k * M;
+      const int2* pw = s_pw + k * M;
       const ulonglong2 pivot = *reinterpret_cast<const ulonglong2*>(cur);
       ColAcc acc;
       LossAcc lacc;
       uint32_t off = 0;
       uint64_t goff = 0;
       auto do_row = [&](int i, uint4 rnd) {
-        const int4 d = pw[i];
-        const pair_t nw2 = ((pair_t)(uint32_t)d.w << 32) | (uint32_t)d.z;
-        const ulonglong2 o = row_update_rnd<kObjective, kFastNoise>(
-            p.alpha, ns, rnd, *reinterpret_cast<const ulonglong2*>(cur + off),
-            *reinterpret_cast<const ulonglong2*>(cen + off), *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x), pivot,
-            nw2, acc, lacc);
+        const int2 d = pw[i];
+        ulonglong2 noise = kObjective == 1 ? scaled_normals4(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
+        if (kRagged) noise = mask_lanes(noise, live);
+        const ulonglong2 o = row_update<kObjective>(
+            p.alpha, noise, *reinterpret_cast<const ulonglong2*>(cur + off), *reinterpret_cast<const ulonglong2*>(cen + off),
+            *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x), pivot, __int_as_float(d.y), acc, lacc);
         if (kLast) {
           if (kBf16) *reinterpret_cast<unsigned long long*>(oq + goff) = narrow_bf16x4(o);
           else *reinterpret_cast<ulonglong2*>(oq + goff) = o;
@@ -845,10 +750,11 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       };
       // the Philox block of row i + 1 is drawn while row i goes through Box-Muller and Eq. 15-16:
       // the two are independent, so the integer multiplies of the one fill the latencies of the other
-      uint4 rnd = noise_block<kObjective>(p.keys, round_lo, ctr3, q32, 0u);
+      const NoiseBase nb = noise_base(q32, round_lo, ctr3, p.keys);
+      uint4 rnd = noise_words(nb, 0u, p.keys);
 #pragma unroll kFusedUnroll
       for (int i = 0; i + 1 < M; ++i) {
-        const uint4 rnd_next = noise_block<kObjective>(p.keys, round_lo, ctr3, q32, (uint32_t)(i + 1));
+        const uint4 rnd_next = noise_words(nb, (uint32_t)(i + 1), p.keys);
         do_row(i, rnd);
         rnd = rnd_next;
       }
@@ -872,8 +778,15 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
         }
       }
     };
-    for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type());
-    run_round(p.n_rounds - 1, std::true_type());
+    // (a test for padding lanes in every row would keep the rows' instructions apart: the one warp that has
+    // any runs its own instance of the round)
+    if (live == 4) {
+      for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type(), std::false_type());
+      run_round(p.n_rounds - 1, std::true_type(), std::false_type());
+    } else {
+      for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type(), std::true_type());
+      run_round(p.n_rounds - 1, std::true_type(), std::true_type());
+    }
     base = (base + (uint32_t)p.n_rounds) & 1u;
     fetched = have_next;
   }
@@ -894,505 +807,6 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     for (int k = 0; k < p.n_rounds; ++k)
       sum_partials(p.partials + (size_t)k * 2 * gridDim.x, (double)p.inv_M, p.tel + 2 * ((p.slot0 + k) % p.ring), s_red);
     if (tid == 0) *p.ticket = 0u;
-  }
-}
-
-// ---- several rounds over a tile that is resident across a thread-block cluster ----------------
-// More workers than a thread's slab can hold (48 M bytes per column group: M = 64 would leave two
-// warps per SM): the rows of a tile are split over the CTAs of a cluster.  CTA `rank` keeps rows
-// [rank * rpc, rank * rpc + rpc) of T column groups in its shared memory exactly as
-// fused_rounds_kernel keeps all of them, a thread still owns one column group, and the peer's
-// value -- the same column group of a row that may live in another CTA of the cluster -- is read
-// through distributed shared memory (mapa + ld.shared::cluster: plain loads, no multicast).  All
-// CTAs of a cluster advance round by round: a cluster barrier (the hardware's
-// barrier.cluster, not a spin) ends every round, which orders this round's remote reads of a slab
-// before the next round's writes to it and keeps a CTA's shared memory alive while others read it.
-// The consensus statistic needs the column sums over ALL rows: every CTA measures its rows against
-// the common pivot (row 0 of the tile, read from rank 0), sum (x - a)^2 adds up CTA by CTA like
-// the loss does, and the per-column sums of (x - a) go to a small double-buffered exchange area
-// that rank 0 collects after the barrier.  Prefetch, direct store of the last round and the
-// arithmetic are fused_rounds_kernel's, so replicas agree with every other launch shape bit for bit.
-struct ClusterParams {
-  FusedParams f;       // n_tiles: tiles of blockDim column groups
-  int32_t rpc;         // rows per CTA = ceil(M / cluster size)
-};
-
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_nctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-// All threads of all CTAs of the cluster; release / acquire order shared-memory accesses across it.
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// 16 bytes at the same shared-memory offset in CTA `rank` of the cluster.
-__device__ __forceinline__ ulonglong2 ld_cluster_16(uint32_t smem_addr, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_addr), "r"(rank));
-  ulonglong2 v;
-  asm volatile("ld.shared::cluster.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(remote) : "memory");
-  return v;
-}
-
-// Dynamic shared memory: (peer's local row offset, peer's CTA, -weight, -weight) int4[kClusterMaxRounds][rpc],
-// then the slabs float4[3][rpc][blockDim], then the exchange area float4[2][blockDim], then 64 doubles.
-template <int kObjective, bool kFastNoise>
-__global__ void __launch_bounds__(256, 2) cluster_rounds_kernel(const ClusterParams cp) {
-  const FusedParams& p = cp.f;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int tid = threadIdx.x, T = blockDim.x, M = p.M, rpc = cp.rpc;
-  const uint32_t rank = cluster_ctarank(), C = cluster_nctarank();
-  const int r0 = min(M, (int)rank * rpc), rows = min(M, r0 + rpc) - r0;  // this CTA's rows [r0, r0 + rows)
-  int4* s_pw = reinterpret_cast<int4*>(smem_raw);
-  const uint32_t head = ((uint32_t)(kClusterMaxRounds * rpc * 16) + 127u) & ~127u;
-  const uint32_t stride = (uint32_t)T * 16u;
-  const uint32_t plane = (uint32_t)rpc * stride;
-  unsigned char* slab = smem_raw + head + (uint32_t)tid * 16u;
-  float4* s_xchg = reinterpret_cast<float4*>(smem_raw + head + 3u * plane);  // [2][T] column sums of (x - pivot) over this CTA's rows
-  double* s_red = reinterpret_cast<double*>(smem_raw + head + 3u * plane + 2u * stride);
-  const uint32_t slab_addr = (uint32_t)__cvta_generic_to_shared(slab);
-  const uint32_t xchg_addr = (uint32_t)__cvta_generic_to_shared(s_xchg + tid);
-
-  for (int k = 0; k < p.n_rounds; ++k) {
-    const int32_t* peers = p.trace + ((p.slot0 + k) % p.ring) * M;
-    for (int j = tid; j < rows; j += T) {
-      const int i = r0 + j;
-      const int32_t m = __ldg(peers + i);
-      const int nw = __float_as_int((m == i) ? -0.0f : -__ldg(p.wtab + (size_t)i * M + m));
-      const int pm = m / rpc;
-      s_pw[k * rpc + j] = make_int4((int)((uint32_t)(m - pm * rpc) * stride), pm, nw, nw);
-    }
-  }
-  __syncthreads();
-
-  double acc_cons[kClusterMaxRounds], acc_loss[kClusterMaxRounds];
-#pragma unroll
-  for (int k = 0; k < kClusterMaxRounds; ++k) acc_cons[k] = acc_loss[k] = 0.0;
-
-  const int64_t n_clusters = gridDim.x / C, cluster_id = blockIdx.x / C;
-  const uint64_t row0_bytes = (uint64_t)(uint32_t)r0 * p.row_bytes;
-  uint32_t base = 0;
-  bool fetched = false;
-  uint32_t epoch = 0;  // rounds done by this cluster: parity selects the exchange buffer
-  // every CTA of a cluster runs the same tiles and rounds, so all of them meet at every barrier
-  for (int64_t tile = cluster_id; tile < p.n_tiles; tile += n_clusters) {
-    const int64_t q = tile * T + tid;
-    const bool live = q < p.nq;
-    const NoiseLanes ns = noise_lanes(p.sigma, live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0));
-    const uint32_t q32 = (uint32_t)q + p.q_offset;
-    const int64_t q_next = q + n_clusters * T;
-    const bool tile_has_next = NETMAX_FUSED_PREFETCH != 0 && tile + n_clusters < p.n_tiles;  // the same in every CTA of the cluster
-    const bool have_next = tile_has_next && q_next < p.nq;
-    if (!fetched && live) {
-      const char* xq = reinterpret_cast<const char*>(p.x_cur) + row0_bytes + (uint64_t)q * 16u;
-      const char* cq = reinterpret_cast<const char*>(p.c) + row0_bytes + (uint64_t)q * 16u;
-      unsigned char* sx = slab + base * plane;
-      unsigned char* sc = slab + 2u * plane;
-#pragma unroll 4
-      for (int j = 0; j < rows; ++j) {
-        *reinterpret_cast<ulonglong2*>(sx) = __ldg(reinterpret_cast<const ulonglong2*>(xq));
-        *reinterpret_cast<ulonglong2*>(sc) = __ldg(reinterpret_cast<const ulonglong2*>(cq));
-        xq += p.row_bytes;
-        cq += p.row_bytes;
-        sx += stride;
-        sc += stride;
-      }
-    }
-    // every CTA's rows of the tile are in place before anyone pulls from them (a fetched tile was
-    // published by the barrier that ended its predecessor's last round)
-    if (!fetched) cluster_barrier();
-    unsigned char* const cen = slab + 2u * plane;
-    char* const oq = reinterpret_cast<char*>(p.x_nxt) + row0_bytes + (uint64_t)q * 16u;
-    const char* const cq_next = reinterpret_cast<const char*>(p.c) + row0_bytes + (uint64_t)q_next * 16u;
-
-    auto run_round = [&](int k, auto last_tag) {
-      constexpr bool kLast = decltype(last_tag)::value;
-      const uint64_t round = p.first_round + (uint64_t)k;
-      const uint32_t round_lo = (uint32_t)round, ctr3 = philox_ctr3(kTagNoise, round);
-      const uint32_t cur_off = ((base + (uint32_t)k) & 1u) * plane;
-      const unsigned char* cur = slab + cur_off;
-      unsigned char* nxt = slab + ((base + (uint32_t)k + 1u) & 1u) * plane;
-      if (kLast && have_next) {
-        const char* xq = reinterpret_cast<const char*>(p.x_cur) + row0_bytes + (uint64_t)q_next * 16u;
-        unsigned char* sx = nxt;
-#pragma unroll 4
-        for (int j = 0; j < rows; ++j) {
-          cp_async_16_stream(sx, xq);
-          xq += p.row_bytes;
-          sx += stride;
-        }
-      }
-      ColAcc acc;
-      LossAcc lacc;
-      if (live) {
-        const int4* pw = s_pw + k * rpc;
-        const ulonglong2 pivot = ld_cluster_16(slab_addr + cur_off, 0u);  // row 0 of the tile lives in CTA 0
-        uint32_t off = 0;
-        uint64_t goff = 0;
-        auto pull = [&](int j) {  // the peer's value for local row j, from whichever CTA holds that row
-          const int4 d = pw[j];
-          return ld_cluster_16(slab_addr + cur_off + (uint32_t)d.x, (uint32_t)d.y);
-        };
-        auto do_row = [&](int j, uint4 rnd, ulonglong2 xm) {
-          const int4 d = pw[j];
-          const pair_t nw2 = ((pair_t)(uint32_t)d.w << 32) | (uint32_t)d.z;
-          const ulonglong2 o = row_update_rnd<kObjective, kFastNoise>(p.alpha, ns, rnd, *reinterpret_cast<const ulonglong2*>(cur + off),
-                                                                      *reinterpret_cast<const ulonglong2*>(cen + off), xm, pivot, nw2, acc,
-                                                                      lacc);
-          if (kLast) {
-            *reinterpret_cast<ulonglong2*>(oq + goff) = o;
-            if (have_next) cp_async_16_stream(cen + off, cq_next + goff);
-            goff += p.row_bytes;
-          } else {
-            *reinterpret_cast<ulonglong2*>(nxt + off) = o;
-          }
-          off += stride;
-        };
-        if (rows > 0) {
-          // one row ahead: the next row's Philox block (integer work that fills this row's latencies) and
-          // its pull, whose trip through the cluster's shared-memory network takes several hundred cycles
-          // (two rows ahead measured slower: 1.43 against 1.39 ms per round of 64 x 11.2 M elements)
-          uint4 rnd = noise_block<kObjective>(p.keys, round_lo, ctr3, q32, (uint32_t)r0);
-          ulonglong2 xm = pull(0);
-#pragma unroll kFusedUnroll
-          for (int j = 0; j + 1 < rows; ++j) {
-            const ulonglong2 xm_next = pull(j + 1);
-            const uint4 rnd_next = noise_block<kObjective>(p.keys, round_lo, ctr3, q32, (uint32_t)(r0 + j + 1));
-            do_row(j, rnd, xm);
-            rnd = rnd_next;
-            xm = xm_next;
-          }
-          do_row(rows - 1, rnd, xm);
-        }
-      }
-      float4 s1, s2;
-      unpack2(acc.s1a, s1.x, s1.y);
-      unpack2(acc.s1b, s1.z, s1.w);
-      unpack2(acc.s2a, s2.x, s2.y);
-      unpack2(acc.s2b, s2.z, s2.w);
-      float l0, l1, l2, l3;
-      unpack2(lacc.la, l0, l1);
-      unpack2(lacc.lb, l2, l3);
-      const uint32_t buf = epoch & 1u;
-      s_xchg[buf * T + tid] = s1;
-      if (kLast) cp_async_wait_all();  // the next tile's rows have landed: the barrier below publishes them too
-      cluster_barrier();  // the round is complete everywhere; the column sums of all CTAs are published
-      ++epoch;
-      double cons = (double)((s2.x + s2.y) + (s2.z + s2.w));  // this CTA's share of sum (x - a)^2
-      if (rank == 0) {
-        // sum_i (x_i - xbar)^2 = sum_i (x_i - a)^2 - (sum_i (x_i - a))^2 / M per column: rank 0 subtracts the second term
-        float4 tot = s1;
-        for (uint32_t r = 1; r < C; ++r) {
-          const ulonglong2 v = ld_cluster_16(xchg_addr + buf * stride, r);
-          float a, b, c2, d2;
-          unpack2(v.x, a, b);
-          unpack2(v.y, c2, d2);
-          tot.x += a;
-          tot.y += b;
-          tot.z += c2;
-          tot.w += d2;
-        }
-        cons -= (double)((tot.x * tot.x + tot.y * tot.y + tot.z * tot.z + tot.w * tot.w) * p.inv_M);
-      }
-      const double loss = (double)((l0 + l1) + (l2 + l3));
-#pragma unroll
-      for (int kk = 0; kk < kClusterMaxRounds; ++kk) {
-        if (kk == k) {
-          acc_cons[kk] += cons;
-          acc_loss[kk] += loss;
-        }
-      }
-    };
-    for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type());
-    run_round(p.n_rounds - 1, std::true_type());
-    base = (base + (uint32_t)p.n_rounds) & 1u;
-    fetched = tile_has_next;
-  }
-  cluster_barrier();  // no CTA leaves while another may still read its exchange area
-
-#pragma unroll
-  for (int k = 0; k < kClusterMaxRounds; ++k)
-    if (k < p.n_rounds) block_partials(p.partials + (size_t)k * 2 * gridDim.x, acc_cons[k], acc_loss[k], s_red);
-  __shared__ bool s_last;
-  if (tid == 0) {
-    __threadfence();
-    const unsigned int t = atomicAdd(p.ticket, 1u);
-    s_last = (t == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    for (int k = 0; k < p.n_rounds; ++k)
-      sum_partials(p.partials + (size_t)k * 2 * gridDim.x, (double)p.inv_M, p.tel + 2 * ((p.slot0 + k) % p.ring), s_red);
-    if (tid == 0) *p.ticket = 0u;
-  }
-}
-
-// ---- all rounds of a call over resident columns (short vectors) -------------------------------
-// The same independence of columns serves the opposite shape: when the whole problem is a few
-// megabytes, a round takes microseconds and what costs time is every launch and every grid-wide
-// exchange.  Here a CTA keeps ALL M rows of G column groups (four elements each) in shared
-// memory, fp32, double-buffered by round, together with their centres, and runs every round of
-// the call on them; CTAs never talk to each other.  Two thread mappings:
-//   G == blockDim  a thread owns a column group and walks all M rows (small M): no barrier is
-//                  needed for the data, only the per-round telemetry reduction synchronises
-//                  (and not even that in a CTA of a single warp);
-//   G <= 32        thread (g, r) owns the rows r, r + blockDim / G, ... of group g (large M):
-//                  a peer's row belongs to another thread, so rounds are separated by ONE barrier
-//                  (a warp-level one in a single-warp CTA); the column sums of the round are
-//                  added over the lanes of each warp before it and over the warps after it, by
-//                  one warp that changes from round to round while the others carry on.
-// Per round every CTA writes its two telemetry sums to partials[round][tile]; a second small
-// kernel adds the tiles of each round in index order.  Arithmetic per element is row_update's,
-// so replicas are bit-identical to the other launch shapes.
-struct ResidentParams {
-  const char* x_cur;      // replicas at the start of the first round, row stride row_bytes
-  char* x_nxt;            // replicas after the last round
-  const char* c;
-  const int32_t* trace;   // peer-trace ring [ring][M]
-  const float* wring;     // pull weight of every draw, same ring
-  double* partials;       // [n_rounds][n_tiles][2]
-  int64_t slot0, ring;
-  uint64_t first_round;
-  int32_t n_rounds;
-  int64_t nq, n_tiles;    // column groups of four elements per row; tiles of G of them
-  uint32_t row_bytes;
-  int32_t M, tail;        // tail = d % 4
-  int32_t G, log2G;       // column groups per tile (a power of two)
-  int32_t draw_chunk;     // > 0: the (peer, weight) pairs of this many rounds at a time are staged in shared
-                          // memory; 0 (large M): every thread loads the draws of its own rows, a round ahead
-  float alpha, sigma, inv_M;
-  uint32_t q_offset;
-  PhiloxKeys keys;
-};
-
-// Dynamic shared memory: slabs float4[3][M][G]; then (G < blockDim) two reduction scratch
-// buffers float[warps][G][9] (padded to 16 bytes); then 2 x 64 floats; then int2[draw_chunk][M].
-constexpr int kDrawRegs = 8;  // large M: draws of a thread's first rows that are fetched a round ahead
-#ifndef NETMAX_RESIDENT_UNROLL
-#define NETMAX_RESIDENT_UNROLL 2
-#endif
-constexpr int kResidentUnroll = NETMAX_RESIDENT_UNROLL;  // rows of a round in flight per thread
-__host__ __device__ inline uint32_t resident_scratch_floats(int threads, int G) {
-  return G < threads ? (uint32_t)(((threads >> 5) * G * 9 + 3) & ~3) : 0u;
-}
-template <int kObjective, bool kFastNoise, bool kBf16>
-__global__ void __launch_bounds__(512) resident_rounds_kernel(const ResidentParams p) {
-  constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int tid = threadIdx.x, T = blockDim.x, M = p.M, G = p.G;
-  const int g = tid & (G - 1), r = tid >> p.log2G, RL = T >> p.log2G;
-  const int lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
-  const uint32_t stride = (uint32_t)G * 16u;    // bytes between consecutive rows of a slab
-  const uint32_t plane = (uint32_t)M * stride;
-  unsigned char* slab = smem_raw + (uint32_t)g * 16u;
-  float* s_scratch = reinterpret_cast<float*>(smem_raw + 3u * plane);
-  const uint32_t scratch_floats = resident_scratch_floats(T, G);
-  float* s_red = s_scratch + 2 * scratch_floats;  // 2 x 64 floats
-  int2* s_pw = reinterpret_cast<int2*>(s_red + 128);
-
-  for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
-    const int64_t q = tile * G + g;
-    const bool live = q < p.nq;
-    const int live_lo = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
-    const uint32_t q32 = (uint32_t)q + p.q_offset;
-    __syncthreads();  // the previous tile is stored
-    for (int i = r; i < M; i += RL) {
-      ulonglong2 xv = make_ulonglong2(0ull, 0ull), cv = xv;
-      if (live) {
-        const char* xq = p.x_cur + (uint64_t)(uint32_t)i * p.row_bytes + (uint64_t)q * kGroupBytes;
-        const char* cq = p.c + (uint64_t)(uint32_t)i * p.row_bytes + (uint64_t)q * kGroupBytes;
-        if (kBf16) {
-          xv = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(xq)));
-          cv = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(cq)));
-        } else {
-          xv = __ldg(reinterpret_cast<const ulonglong2*>(xq));
-          cv = __ldg(reinterpret_cast<const ulonglong2*>(cq));
-        }
-      }
-      *reinterpret_cast<ulonglong2*>(slab + (uint32_t)i * stride) = xv;
-      *reinterpret_cast<ulonglong2*>(slab + 2u * plane + (uint32_t)i * stride) = cv;
-    }
-    int64_t slot = p.slot0 % p.ring;  // ring slot of round k, stepped along with k
-    const int KC = p.draw_chunk;      // rounds whose draws are staged in shared memory at a time (0: none)
-    int2 dreg[kDrawRegs];             // KC == 0: the draws of this thread's first rows, loaded a round ahead
-    if (KC == 0 && live) {
-#pragma unroll
-      for (int j = 0; j < kDrawRegs; ++j) {
-        const int i = r + j * RL;
-        if (i < M) dreg[j] = make_int2(__ldg(p.trace + slot * M + i), __float_as_int(__ldg(p.wring + slot * M + i)));
-      }
-    }
-    __syncthreads();
-
-    for (int k = 0; k < p.n_rounds; ++k) {
-      const uint64_t round = p.first_round + (uint64_t)k;
-      const uint32_t round_lo = (uint32_t)round, ctr3 = philox_ctr3(kTagNoise, round);
-      const int kc = KC > 0 ? k % KC : 0;
-      if (KC > 0 && kc == 0) {
-        // stage the draws of the next KC rounds (the previous round's barrier has retired their predecessors)
-        const int n = min(KC, p.n_rounds - k) * M;
-#pragma unroll 4
-        for (int idx = tid; idx < n; idx += T) {
-          const int ahead = idx / M;  // rounds ahead of round k
-          int64_t s2 = slot + ahead;
-          if (s2 >= p.ring) s2 -= p.ring;  // (a chunk is never longer than the ring)
-          const int64_t src = s2 * M + (idx - ahead * M);
-          s_pw[idx] = make_int2(__ldg(p.trace + src), __float_as_int(__ldg(p.wring + src)));
-        }
-        __syncthreads();
-      }
-      const int64_t at = slot * M;
-      slot = slot + 1 == p.ring ? 0 : slot + 1;
-      const unsigned char* cur = slab + (uint32_t)(k & 1) * plane;
-      unsigned char* nxt = slab + (uint32_t)((k & 1) ^ 1) * plane;
-      const unsigned char* cen = slab + 2u * plane;
-      ColAcc acc;
-      LossAcc lacc;
-      if (live) {
-        const ulonglong2 pivot = *reinterpret_cast<const ulonglong2*>(cur);
-        auto do_row = [&](int i, int2 d) {
-          const uint32_t off = (uint32_t)i * stride;
-          ulonglong2 o = row_update<kObjective, kFastNoise>(
-              p.alpha, p.sigma, p.keys, round_lo, ctr3, q32, (uint32_t)i, *reinterpret_cast<const ulonglong2*>(cur + off),
-              *reinterpret_cast<const ulonglong2*>(cen + off), *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x * stride),
-              pivot, __int_as_float(d.y), live_lo, acc, lacc);
-          if (kBf16) o = widen_bf16x4(narrow_bf16x4(o));
-          *reinterpret_cast<ulonglong2*>(nxt + off) = o;
-        };
-        if (KC > 0) {
-          const int2* pw = s_pw + kc * M;
-#pragma unroll kResidentUnroll
-          for (int i = r; i < M; i += RL) do_row(i, pw[i]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < kDrawRegs; ++j) {
-            const int i = r + j * RL;
-            if (i < M) do_row(i, dreg[j]);
-          }
-          for (int i = r + kDrawRegs * RL; i < M; i += RL)
-            do_row(i, make_int2(__ldg(p.trace + at + i), __float_as_int(__ldg(p.wring + at + i))));
-          if (k + 1 < p.n_rounds) {  // next round's draws: in flight during the reduction below
-#pragma unroll
-            for (int j = 0; j < kDrawRegs; ++j) {
-              const int i = r + j * RL;
-              if (i < M) dreg[j] = make_int2(__ldg(p.trace + slot * M + i), __float_as_int(__ldg(p.wring + slot * M + i)));
-            }
-          }
-        }
-      }
-      // ---- telemetry of the round: column sums over the row lanes, then over the tile
-      float v[9];
-      unpack2(acc.s1a, v[0], v[1]);
-      unpack2(acc.s1b, v[2], v[3]);
-      unpack2(acc.s2a, v[4], v[5]);
-      unpack2(acc.s2b, v[6], v[7]);
-      {
-        float l0, l1, l2, l3;
-        unpack2(lacc.la, l0, l1);
-        unpack2(lacc.lb, l2, l3);
-        v[8] = (l0 + l1) + (l2 + l3);
-      }
-      double* out = p.partials + ((size_t)k * p.n_tiles + tile) * 2;
-      if (RL > 1) {
-        // the rows of a column group are spread over row lanes: first over those of this warp ...
-        for (int off = 16; off >= G; off >>= 1) {
-#pragma unroll
-          for (int a = 0; a < 9; ++a) v[a] += __shfl_xor_sync(0xffffffffu, v[a], off);
-        }
-        if (nwarps > 1) {
-          float* scratch = s_scratch + (k & 1) * scratch_floats;
-          if (lane < G) {
-#pragma unroll
-            for (int a = 0; a < 9; ++a) scratch[(warp * G + lane) * 9 + a] = v[a];
-          }
-          __syncthreads();  // the round's one barrier: every row is written before the next round reads it, every warp's sums are out
-          // ... then over the warps, by ONE warp (a different one every round) while the others go on with
-          // the next round: its buffer is not written again before the barrier after next.  (With a second
-          // barrier and one thread adding the warps' sums, a round of 4096 x 4 elements spent 2,900 of its
-          // 9,800 cycles here.)
-          if (warp == k % nwarps) {
-#pragma unroll
-            for (int a = 0; a < 9; ++a) v[a] = 0.f;
-            for (int e = lane; e < nwarps * G; e += 32) {  // entry e = (warp, group e % G); G divides 32
-#pragma unroll
-              for (int a = 0; a < 9; ++a) v[a] += scratch[e * 9 + a];
-            }
-            for (int off = 16; off >= G; off >>= 1) {
-#pragma unroll
-              for (int a = 0; a < 9; ++a) v[a] += __shfl_xor_sync(0xffffffffu, v[a], off);
-            }
-          }
-        } else {
-          __syncwarp();  // a single warp: its lanes are all the threads that exchange rows
-        }
-        if (nwarps == 1 || warp == k % nwarps) {  // lanes 0 .. G-1 hold the sums of their groups
-          float cons = 0.f, loss = 0.f;
-          if (lane < G) {
-            cons = (v[4] - v[0] * v[0] * p.inv_M) + (v[5] - v[1] * v[1] * p.inv_M) + (v[6] - v[2] * v[2] * p.inv_M) +
-                   (v[7] - v[3] * v[3] * p.inv_M);
-            loss = v[8];
-          }
-          for (int off = 16; off > 0; off >>= 1) {
-            cons += __shfl_down_sync(0xffffffffu, cons, off);
-            loss += __shfl_down_sync(0xffffffffu, loss, off);
-          }
-          if (lane == 0) {
-            out[0] = (double)cons;
-            out[1] = 0.5 * (double)loss;
-          }
-        }
-      } else {
-        // a thread holds the complete sums of its column group; no thread reads another's rows
-        float cons = (v[4] - v[0] * v[0] * p.inv_M) + (v[5] - v[1] * v[1] * p.inv_M) + (v[6] - v[2] * v[2] * p.inv_M) +
-                     (v[7] - v[3] * v[3] * p.inv_M);
-        float loss = v[8];
-        for (int off = 16; off > 0; off >>= 1) {
-          cons += __shfl_down_sync(0xffffffffu, cons, off);
-          loss += __shfl_down_sync(0xffffffffu, loss, off);
-        }
-        if (nwarps == 1) {
-          if (lane == 0) {
-            out[0] = (double)cons;
-            out[1] = 0.5 * (double)loss;
-          }
-          __syncwarp();  // (the staged draws are overwritten by whichever lane gets there first)
-        } else {
-          float* red = s_red + (k & 1) * 64;
-          if (lane == 0) {
-            red[warp] = cons;
-            red[32 + warp] = loss;
-          }
-          __syncthreads();
-          if (tid == 0) {
-            double a = 0.0, b = 0.0;
-            for (int w = 0; w < nwarps; ++w) {
-              a += (double)red[w];
-              b += (double)red[32 + w];
-            }
-            out[0] = a;
-            out[1] = 0.5 * b;
-          }
-        }
-      }
-    }
-
-    if (live) {
-      const unsigned char* fin = slab + (uint32_t)(p.n_rounds & 1) * plane;
-      for (int i = r; i < M; i += RL) {
-        char* oq = p.x_nxt + (uint64_t)(uint32_t)i * p.row_bytes + (uint64_t)q * kGroupBytes;
-        const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(fin + (uint32_t)i * stride);
-        if (kBf16) *reinterpret_cast<unsigned long long*>(oq) = narrow_bf16x4(o);
-        else *reinterpret_cast<ulonglong2*>(oq) = o;
-      }
-    }
   }
 }
 
@@ -1461,7 +875,7 @@ struct StepParams {
   PhiloxKeys keys;
 };
 
-template <int kObjective, bool kFastNoise, int kHalves>
+template <int kObjective, int kHalves>
 __global__ void __launch_bounds__(256) step_kernel(const StepParams p) {
   const StepEvent& e = p.ev[blockIdx.y];
   const uint64_t row_i = (uint64_t)(uint32_t)e.worker * p.row_bytes;
@@ -1479,10 +893,10 @@ __global__ void __launch_bounds__(256) step_kernel(const StepParams p) {
 #pragma unroll
     for (int h = 0; h < kHalves; ++h) {
       pair_t ta, tb;
-      const ulonglong2 oh = update_core<kObjective, kFastNoise>(
-          p.alpha, p.sigma, p.keys, e.iter_lo, e.ctr3, (uint32_t)q * kHalves + h + p.q_offset, (uint32_t)e.worker,
-          group_half<kHalves>(xv, h), group_half<kHalves>(cv, h), group_half<kHalves>(xm, h), e.w,
-          live_lanes(ragged, p.tail, h), ta, tb);
+      const ulonglong2 noise = draw_noise<kObjective>(p.sigma, p.keys, e.iter_lo, e.ctr3, (uint32_t)q * kHalves + h + p.q_offset,
+                                                      (uint32_t)e.worker, live_lanes(ragged, p.tail, h));
+      const ulonglong2 oh = update_core<kObjective>(p.alpha, noise, group_half<kHalves>(xv, h), group_half<kHalves>(cv, h),
+                                                    group_half<kHalves>(xm, h), e.w, ta, tb);
       if (kHalves == 1) o = oh;
       else if (h == 0) o.x = narrow_bf16x4(oh);
       else o.y = narrow_bf16x4(oh);
@@ -1512,7 +926,7 @@ __global__ void __launch_bounds__(256) init_normal_kernel(const InitParams p) {
     ulonglong2 o;
 #pragma unroll
     for (int h = 0; h < kHalves; ++h) {
-      float4 z = normals4<false>(philox4x32_10((uint32_t)q * kHalves + h + p.q_offset, (uint32_t)i, 0u, p.tag, p.keys));
+      float4 z = normals4(philox4x32_10((uint32_t)q * kHalves + h + p.q_offset, (uint32_t)i, 0u, p.tag, p.keys));
       z.x *= p.stddev; z.y *= p.stddev; z.z *= p.stddev; z.w *= p.stddev;
       const int live = live_lanes(ragged, p.tail, h);
       if (live < 1) z.x = 0.f;

@@ -114,35 +114,85 @@ __device__ __forceinline__ pair_t add2(pair_t a, pair_t b) {
   return d;
 }
 
-// The two normals of one Box-Muller pair, packed, fast path, WITHOUT the constant factor of the
-// radius: returns sqrt(-log2 u1) (cos 2 pi u2, sin 2 pi u2), i.e. the pair of normals divided by
-// kNormalScale = sqrt(2 ln 2); the caller folds that constant into its noise scale.
+// sub.rn.f32x2 is a - b in each lane.
+__device__ __forceinline__ pair_t sub2(pair_t a, pair_t b) {
+  pair_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// A Box-Muller pair times sigma, fast path: (sigma_s rad) (cos, sin) of 2 pi u2 with rad = sqrt(-log2 u1);
+// sigma_s is sigma times the constant factor kNormalScale = sqrt(2 ln 2) that rad leaves out.
 // u1 < 1, so log2 u1 < 0; the hardware logarithm has an absolute error of about 2^-22 and may
 // return +0 or a tiny positive value for u1 next to 1, hence |.| (an operand modifier, not an
 // instruction) instead of a negation under the square root.
 constexpr double kNormalScale = 1.17741002251547469101;  // sqrt(2 ln 2)
-__device__ __forceinline__ pair_t normal_pair_fast_unscaled(uint32_t a, uint32_t b) {
+__device__ __forceinline__ pair_t scaled_pair(uint32_t a, uint32_t b, float sigma_s) {
   const float u1 = radius_uniform(a);
   const float ang = (float)((int32_t)b >> 8) * 3.74507028e-07f;  // 2 pi / 2^24
   float rad;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rad) : "f"(fabsf(log2_fast(u1))));
+  rad *= sigma_s;
   float s, c;
   __sincosf(ang, &s, &c);
-  return mul2(pack2(rad, rad), pack2(c, s));
+  return pack2(rad * c, rad * s);
+}
+// sigma times the four normals of a Philox block.
+__device__ __forceinline__ ulonglong2 scaled_normals4(uint4 r, float sigma_s) {
+  return make_ulonglong2(scaled_pair(r.x, r.y, sigma_s), scaled_pair(r.z, r.w, sigma_s));
+}
+// Clears the lanes from `live` on (padding of a row's last, ragged group).
+__device__ __forceinline__ ulonglong2 mask_lanes(ulonglong2 v, int live) {
+  float v0, v1, v2, v3;
+  unpack2(v.x, v0, v1);
+  unpack2(v.y, v2, v3);
+  return make_ulonglong2(pack2(live > 0 ? v0 : 0.f, live > 1 ? v1 : 0.f), pack2(live > 2 ? v2 : 0.f, live > 3 ? v3 : 0.f));
 }
 
-template <bool kFast>
+// The four normals of a Philox block, accurate (initial state).
 __device__ __forceinline__ float4 normals4(uint4 r) {
   float4 z;
-  if (kFast) {  // (the update kernels use normal_pair_fast_unscaled directly and fold the constant into their noise scale)
-    unpack2(normal_pair_fast_unscaled(r.x, r.y), z.x, z.y);
-    unpack2(normal_pair_fast_unscaled(r.z, r.w), z.z, z.w);
-    z.x *= (float)kNormalScale; z.y *= (float)kNormalScale; z.z *= (float)kNormalScale; z.w *= (float)kNormalScale;
-  } else {
-    normal_pair_accurate(r.x, r.y, z.x, z.y);
-    normal_pair_accurate(r.z, r.w, z.z, z.w);
-  }
+  normal_pair_accurate(r.x, r.y, z.x, z.y);
+  normal_pair_accurate(r.z, r.w, z.z, z.w);
   return z;
+}
+
+// ---- noise blocks of many workers at one (column group, round) --------------------------------------
+// Philox4x32-10 at counter (q, worker, round, tag).  The parts of its first three rounds that do not depend
+// on the worker are worked out once per (column group, round): of the twenty 32 x 32 -> 64 multiplies of a
+// block sixteen remain per worker.  (What these multiplies cost: a stream of them issues one per 5 cycles
+// and scheduler, and the blocks alone take 76 of the 104 cycles of four normals.)
+struct NoiseBase {
+  uint32_t a0, c3, c1, h0, l0;
+};
+__device__ __forceinline__ NoiseBase noise_base(uint32_t q, uint32_t round_lo, uint32_t ctr3, const PhiloxKeys& keys) {
+  NoiseBase b;
+  const uint64_t p0 = (uint64_t)kPhiloxMul0 * q, p1 = (uint64_t)kPhiloxMul1 * round_lo;
+  b.a0 = (uint32_t)(p1 >> 32) ^ keys.k0[0];                       // with the worker word: word 0 after round 0
+  const uint32_t c2 = (uint32_t)(p0 >> 32) ^ ctr3 ^ keys.k1[0];
+  b.c3 = (uint32_t)p0 ^ keys.k1[1];
+  const uint64_t q1 = (uint64_t)kPhiloxMul1 * c2;
+  const uint32_t c0 = (uint32_t)(q1 >> 32) ^ (uint32_t)p1 ^ keys.k0[1];
+  b.c1 = (uint32_t)q1 ^ keys.k0[2];
+  const uint64_t p2 = (uint64_t)kPhiloxMul0 * c0;
+  b.h0 = (uint32_t)(p2 >> 32) ^ keys.k1[2];
+  b.l0 = (uint32_t)p2;
+  return b;
+}
+__device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint32_t worker, const PhiloxKeys& keys) {
+  const uint64_t e = (uint64_t)kPhiloxMul0 * (b.a0 ^ worker);
+  const uint64_t p = (uint64_t)kPhiloxMul1 * ((uint32_t)(e >> 32) ^ b.c3);
+  uint32_t c0 = (uint32_t)(p >> 32) ^ b.c1, c1 = (uint32_t)p, c2 = b.h0 ^ (uint32_t)e, c3 = b.l0;
+#pragma unroll
+  for (int r = 3; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)kPhiloxMul0 * c0, p1 = (uint64_t)kPhiloxMul1 * c2;
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ keys.k0[r], n2 = (uint32_t)(p0 >> 32) ^ c3 ^ keys.k1[r];
+    c0 = n0;
+    c1 = (uint32_t)p1;
+    c2 = n2;
+    c3 = (uint32_t)p0;
+  }
+  return make_uint4(c0, c1, c2, c3);
 }
 
 }  // namespace netmax

@@ -1,0 +1,320 @@
+// Rounds on resident tiles whose rows are shared out over the threads of a CTA (any number of workers
+// that fits on chip: 48 bytes per worker and column group).
+//
+// Given the peer draws, every column of the M x d state evolves on its own (Eq. 16 is elementwise), so a
+// CTA that holds ALL M rows of G column groups (four elements each) in shared memory can run any number
+// of rounds on them.  Thread (g, r) owns the rows r, r + RL, ... of group g; a pull reads the peer's row of
+// the same group, which another thread wrote a round earlier, so rounds are separated by a barrier.
+//
+// What bounds it, and why it is laid out this way.  Three quarters of a round's instructions draw the
+// gradient noise, which depends on no replica: a thread draws the noise of its rows for the NEXT round
+// between arriving at the round's barrier and waiting for it (an mbarrier, so that the two are apart), and
+// carries it over in registers (4 per row; at most kRows rows per thread).  The barrier, the slowest warp
+// and the telemetry sums then hide behind work that has to be done anyway.  On 64 x 11.2 M elements the
+// same tile with noise drawn inside the round and a CTA barrier measured 1,685 us per round, rows over a
+// cluster of eight CTAs 1,380.
+#pragma once
+#include "netmax_kernels.cuh"
+
+namespace netmax {
+
+// ---- mbarrier ----------------------------------------------------------------------------------------
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.shared::cta.b64 t, [%0];\n}" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok)
+               : "r"(bar), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
+// Every warp of the CTA arrives unconditionally, so the wait ends; it is bounded all the same, and one that
+// runs out is reported (the replicas are then not valid).
+constexpr uint32_t kTileSpinLimit = 1u << 22;
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, unsigned int* error) {
+  for (uint32_t it = 0; it < kTileSpinLimit; ++it)
+    if (mbar_try_wait(bar, parity)) return;
+  *reinterpret_cast<volatile unsigned int*>(error) = 1u;
+}
+
+struct TileParams {
+  const char* x_cur;      // replicas at the start of the first round, row stride row_bytes
+  char* x_nxt;            // replicas after the last round
+  const char* c;
+  const int2* draws;      // ring of (peer, bits of the pull weight), [ring][M]
+  double* partials;       // [n_rounds][gridDim.x][2]: telemetry shares of every CTA
+  double* tel;            // telemetry ring; written by the last CTA when finalize is set
+  unsigned int* ticket;   // last-CTA-done counter (0 between launches)
+  unsigned int* error;
+  int64_t slot0, ring;
+  uint64_t first_round;
+  int32_t n_rounds;
+  int64_t nq, n_tiles;    // column groups of four elements per row; tiles of G of them
+  uint32_t row_bytes;
+  int32_t M, tail;        // tail = d % 4
+  int32_t G, log2G;       // column groups per tile (a power of two, at most 32)
+  int32_t pre_reduce;     // sums are added over the lanes of a warp first (scratch for G entries per warp, not 32)
+  int32_t finalize;
+  float alpha, sigma, inv_M;   // sigma: the noise scale sigma sqrt(2 ln 2)
+  uint32_t q_offset;
+  PhiloxKeys keys;
+};
+
+// Dynamic shared memory: slabs float4[3][M][G] (replicas of even and of odd rounds, centres), then two
+// buffers of telemetry shares, each float4[E] + float2[E] with E = warps x (pre_reduce ? G : 32).
+__host__ __device__ inline uint32_t tile_share_entries(int threads, int G, bool pre_reduce) {
+  return (uint32_t)(threads >> 5) * (uint32_t)(pre_reduce ? G : 32);
+}
+__host__ __device__ inline size_t tile_smem(int64_t M, int threads, int G, bool pre_reduce) {
+  return (size_t)48 * M * G + (size_t)48 * tile_share_entries(threads, G, pre_reduce);
+}
+
+// kRows: rows per thread, ceil(M / RL).  Exact, so that only a thread's LAST row can be missing: rows before it
+// run without a test between them and the scheduler can mix their instructions (with a test per row the same
+// rows took 282 cycles each instead of 195).
+template <int kObjective, bool kBf16, int kRows>
+__global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p) {
+  constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long s_bar;
+  const int tid = threadIdx.x, T = blockDim.x, M = p.M, G = p.G;
+  const int lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
+  const int g = tid & (G - 1), r = tid >> p.log2G, RL = T >> p.log2G;
+  const uint32_t stride = (uint32_t)G * 16u;    // bytes between consecutive rows of a slab
+  const uint32_t plane = (uint32_t)M * stride;
+  const uint32_t step = (uint32_t)RL * stride;  // bytes between consecutive rows of a thread
+  const bool full = r + (kRows - 1) * RL < M;   // has this thread a last row?
+  const uint64_t row_step = (uint64_t)(uint32_t)RL * p.row_bytes, row_first = (uint64_t)(uint32_t)r * p.row_bytes;
+  unsigned char* const col = smem_raw + (uint32_t)g * 16u;
+  unsigned char* const own = col + (uint32_t)r * stride;
+  const uint32_t E = tile_share_entries(T, G, p.pre_reduce != 0);
+  float4* const s_sum = reinterpret_cast<float4*>(smem_raw + 3u * plane);     // [2][E]
+  float2* const s_two = reinterpret_cast<float2*>(s_sum + 2u * E);            // [2][E]
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_bar);
+  if (tid == 0) mbar_init(bar, (uint32_t)nwarps);
+  __syncthreads();
+
+  int2 draw[kRows];
+  ulonglong2 noise[kRows];
+  int64_t tile = blockIdx.x;
+
+  // body(j) for the rows of this thread
+  auto rows = [&](auto body) {
+#pragma unroll
+    for (int j = 0; j < kRows - 1; ++j) body(j);
+    if (full) body(kRows - 1);
+  };
+  int64_t slot = p.slot0;  // ring slot of the next draws to load
+  auto next_draws = [&](int k) {
+    if (k == 0) slot = p.slot0;
+    const int2* src = p.draws + slot * M + r;
+    rows([&](int j) { draw[j] = __ldg(src + j * RL); });
+    slot = slot + 1 == p.ring ? 0 : slot + 1;
+  };
+  auto next_noise = [&](int64_t q, int k) {
+    if (kObjective != 1) return;
+    const uint64_t round = p.first_round + (uint64_t)k;
+    const NoiseBase nb = noise_base((uint32_t)q + p.q_offset, (uint32_t)round, philox_ctr3(kTagNoise, round), p.keys);
+    rows([&](int j) { noise[j] = scaled_normals4(noise_words(nb, (uint32_t)(r + j * RL), p.keys), p.sigma); });
+    if (p.tail != 0 && q == p.nq - 1)
+      rows([&](int j) { noise[j] = mask_lanes(noise[j], p.tail); });
+  };
+  // telemetry of one round: this warp adds the shares of all threads (lane -> entries lane, lane + 32, ...,
+  // which belong to column group lane % G) and leaves the CTA's two sums
+  auto add_shares = [&](uint32_t buf, int k, bool first) {
+    float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float s2 = 0.f, loss = 0.f;
+    for (uint32_t e = lane; e < E; e += 32) {
+      const float4 a = s_sum[buf * E + e];
+      const float2 b = s_two[buf * E + e];
+      s1.x += a.x; s1.y += a.y; s1.z += a.z; s1.w += a.w;
+      s2 += b.x;
+      loss += b.y;
+    }
+    for (int off = 16; off >= G; off >>= 1) {
+      s1.x += __shfl_xor_sync(0xffffffffu, s1.x, off);
+      s1.y += __shfl_xor_sync(0xffffffffu, s1.y, off);
+      s1.z += __shfl_xor_sync(0xffffffffu, s1.z, off);
+      s1.w += __shfl_xor_sync(0xffffffffu, s1.w, off);
+    }
+    // sum_i (x_i - xbar)^2 = sum_i (x_i - a)^2 - (sum_i (x_i - a))^2 / M per column
+    if (lane < G) s2 -= (s1.x * s1.x + s1.y * s1.y + s1.z * s1.z + s1.w * s1.w) * p.inv_M;
+    for (int off = 16; off > 0; off >>= 1) {
+      s2 += __shfl_down_sync(0xffffffffu, s2, off);
+      loss += __shfl_down_sync(0xffffffffu, loss, off);
+    }
+    if (lane == 0) {
+      double* out = p.partials + ((size_t)k * gridDim.x + blockIdx.x) * 2;
+      const double a = (double)s2, b = 0.5 * (double)loss;
+      if (first) {
+        out[0] = a;
+        out[1] = b;
+      } else {  // this CTA's share of an earlier tile is there, written by this very thread
+        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out), "d"(a) : "memory");
+        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + 1), "d"(b) : "memory");
+      }
+    }
+  };
+
+  // the first tile
+  int64_t q = tile * G + g;
+  bool live = q < p.nq;
+  if (tile < p.n_tiles) {
+    if (live) {
+      const char* xq = p.x_cur + (uint64_t)q * kGroupBytes + row_first;
+      const char* cq = p.c + (uint64_t)q * kGroupBytes + row_first;
+      rows([&](int j) {
+        unsigned char* sx = own + (uint32_t)j * step;
+        if (kBf16) {
+          *reinterpret_cast<ulonglong2*>(sx) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(xq + j * row_step)));
+          *reinterpret_cast<ulonglong2*>(sx + 2u * plane) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(cq + j * row_step)));
+        } else {
+          cp_async_16_stream(sx, xq + j * row_step);
+          cp_async_16_stream(sx + 2u * plane, cq + j * row_step);
+        }
+      });
+    }
+    next_draws(0);
+    next_noise(q, 0);
+    cp_async_wait_all();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+  }
+
+  uint32_t base = 0, phase = 0, buf = 0;
+  int turn = 0;             // the warp that adds the shares of the round before the current one
+  int summed = 0;           // round whose shares are due
+  bool due = false, due_first = true;
+  for (; tile < p.n_tiles; tile += gridDim.x) {
+    const int64_t q_next = q + (int64_t)gridDim.x * G;
+    const bool tile_next = tile + gridDim.x < p.n_tiles;
+    const bool have_next = tile_next && q_next < p.nq;
+    const bool first_tile = tile == blockIdx.x;
+
+    auto run_round = [&](int k, auto last_tag) {
+      constexpr bool kLast = decltype(last_tag)::value;
+      mbar_wait(bar, phase, p.error);  // all rows of the previous round are written
+      phase ^= 1u;
+      if (due && warp == turn) add_shares(buf ^ 1u, summed, due_first);
+      turn = turn + 1 == nwarps ? 0 : turn + 1;
+      const uint32_t cur_off = ((base + (uint32_t)k) & 1u) * plane, nxt_off = plane - cur_off;
+      ColAcc acc;
+      LossAcc lacc;
+      if (kLast && have_next) {  // the next tile's replicas into the slab this round does not write
+        const char* xq = p.x_cur + (uint64_t)q_next * kGroupBytes + row_first;
+        rows([&](int j) {
+          unsigned char* sx = own + nxt_off + (uint32_t)j * step;
+          if (kBf16) cp_async_8(sx, xq + j * row_step);
+          else cp_async_16_stream(sx, xq + j * row_step);
+        });
+      }
+      if (live) {
+        const unsigned char* cur = col + cur_off;
+        const ulonglong2 pivot = *reinterpret_cast<const ulonglong2*>(cur);  // row 0
+        char* oq = p.x_nxt + (uint64_t)q * kGroupBytes + row_first;
+        rows([&](int j) {
+          unsigned char* sx = own + (uint32_t)j * step;
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sx + cur_off);
+          const ulonglong2 cv = *reinterpret_cast<const ulonglong2*>(sx + 2u * plane);
+          const ulonglong2 xm = *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)draw[j].x * stride);
+          const ulonglong2 o = row_update<kObjective>(p.alpha, noise[j], xv, cv, xm, pivot, __int_as_float(draw[j].y), acc, lacc);
+          if (kLast) {
+            if (kBf16) *reinterpret_cast<unsigned long long*>(oq + j * row_step) = narrow_bf16x4(o);
+            else *reinterpret_cast<ulonglong2*>(oq + j * row_step) = o;
+          } else {
+            *reinterpret_cast<ulonglong2*>(sx + nxt_off) = kBf16 ? widen_bf16x4(narrow_bf16x4(o)) : o;
+          }
+        });
+      }
+      if (kLast && have_next) {  // the centres of this tile have been read for the last time
+        const char* cq = p.c + (uint64_t)q_next * kGroupBytes + row_first;
+        rows([&](int j) {
+          unsigned char* sc = own + 2u * plane + (uint32_t)j * step;
+          if (kBf16) cp_async_8(sc, cq + j * row_step);
+          else cp_async_16_stream(sc, cq + j * row_step);
+        });
+      }
+      // this thread's shares of the round's sums
+      float4 s1;
+      float a0, a1, l0, l1;
+      unpack2(acc.s1a, s1.x, s1.y);
+      unpack2(acc.s1b, s1.z, s1.w);
+      unpack2(add2(acc.s2a, acc.s2b), a0, a1);
+      unpack2(add2(lacc.la, lacc.lb), l0, l1);
+      float2 two = make_float2(a0 + a1, l0 + l1);
+      if (p.pre_reduce) {
+        for (int off = 16; off >= G; off >>= 1) {
+          s1.x += __shfl_xor_sync(0xffffffffu, s1.x, off);
+          s1.y += __shfl_xor_sync(0xffffffffu, s1.y, off);
+          s1.z += __shfl_xor_sync(0xffffffffu, s1.z, off);
+          s1.w += __shfl_xor_sync(0xffffffffu, s1.w, off);
+          two.x += __shfl_xor_sync(0xffffffffu, two.x, off);
+          two.y += __shfl_xor_sync(0xffffffffu, two.y, off);
+        }
+        if (lane < G) {
+          s_sum[buf * E + warp * G + lane] = s1;
+          s_two[buf * E + warp * G + lane] = two;
+        }
+      } else {
+        s_sum[buf * E + tid] = s1;
+        s_two[buf * E + tid] = two;
+      }
+      if (kLast && tile_next) {
+        cp_async_wait_all();  // the next tile's rows have landed: the barrier publishes them too
+        if (kBf16 && have_next) {
+          rows([&](int j) {
+            unsigned char* sx = own + nxt_off + (uint32_t)j * step;
+            unsigned char* sc = own + 2u * plane + (uint32_t)j * step;
+            *reinterpret_cast<ulonglong2*>(sx) = widen_bf16x4(*reinterpret_cast<const unsigned long long*>(sx));
+            *reinterpret_cast<ulonglong2*>(sc) = widen_bf16x4(*reinterpret_cast<const unsigned long long*>(sc));
+          });
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar);
+      buf ^= 1u;
+      due = true;
+      due_first = first_tile;
+      summed = k;
+      // while the others finish: the draws and the noise of the next round
+      if (!kLast) {
+        next_draws(k + 1);
+        next_noise(q, k + 1);
+      } else if (tile_next) {
+        next_draws(0);
+        next_noise(q_next, 0);
+      }
+    };
+    for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type());
+    run_round(p.n_rounds - 1, std::true_type());
+    base = (base + (uint32_t)p.n_rounds) & 1u;
+    q = q_next;
+    live = q < p.nq;
+  }
+  if (due) {
+    mbar_wait(bar, phase, p.error);
+    if (warp == turn) add_shares(buf ^ 1u, summed, due_first);
+  }
+  if (!p.finalize) return;
+  __shared__ bool s_last;
+  __shared__ double s_red[64];
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    for (int k = 0; k < p.n_rounds; ++k)
+      sum_partials(p.partials + (size_t)k * 2 * gridDim.x, (double)p.inv_M, p.tel + 2 * ((p.slot0 + k) % p.ring), s_red);
+    if (tid == 0) *p.ticket = 0u;
+  }
+}
+
+}  // namespace netmax
