@@ -147,8 +147,10 @@ struct Layout {
          off_partials = 0, off_ticket = 0, off_colpart = 0, off_coltick = 0, off_pipe_tel = 0, total = 0;
 };
 
+constexpr int kFuseRoundsLimit = 8;  // largest netmax_config.fuse_rounds
 constexpr int kMaxGrid = 148 * 16;  // upper bound on resident CTAs of the round kernel
 constexpr int64_t kMaxRoundsPerLaunch = 4096;  // rounds one cooperative launch runs at most
+constexpr size_t kPartialsBytes = (size_t)kMaxGrid * 2 * sizeof(double) * 8;  // per CTA and round of a fused launch; two sets for multi-round launches
 constexpr size_t kColPartBytes = (size_t)8 << 20;  // column partials of the row-split (short vector) shape
 constexpr int kMaxChunks = 32;  // column chunks of a pipelined host round trip
 
@@ -173,7 +175,7 @@ Layout make_layout(int64_t M, int64_t d, int64_t trace_rounds, int storage) {
   L.off_trace = take((size_t)trace_rounds * M * sizeof(int32_t));
   L.off_draws = take((size_t)trace_rounds * M * sizeof(int2));  // (peer, pull weight) of every draw in the trace ring
   L.off_tel = take((size_t)trace_rounds * 2 * sizeof(double));
-  L.off_partials = take((size_t)kMaxGrid * 2 * sizeof(double) * kFusedMaxRounds);  // per round of a fused launch; two sets for multi-round launches
+  L.off_partials = take(kPartialsBytes);
   L.off_ticket = take(256);
   L.off_colpart = take(kColPartBytes);
   L.off_coltick = take((size_t)kMaxGrid * sizeof(unsigned int));
@@ -257,7 +259,7 @@ struct netmax_ctx {
   uint64_t seed = 0;
   int policy_K = 20, policy_R = 20;
   double policy_rho_upper = 0.0;
-  int fuse_rounds = 0;  // 0: automatic, 1: one launch per round, 2..kFusedMaxRounds: rounds per fused launch
+  int fuse_rounds = 0;  // 0: automatic, 1: one launch per round, 2..kFuseRoundsLimit: rounds per fused launch
   bool round_planned[2] = {false, false};  // [0]: the context's objective, [1]: measuring
   RoundPlan round_plan[2];
   bool fused_planned = false;
@@ -620,14 +622,9 @@ MultiRoundKernel pick_multi_kernel(int objective, int halves) {
 
 using FusedKernel = void (*)(const FusedParams);
 
-template <int kRounds>
-FusedKernel pick_fused_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kRounds> : fused_rounds_kernel<0, true, kRounds>;
-  return objective == 1 ? fused_rounds_kernel<1, false, kRounds> : fused_rounds_kernel<0, false, kRounds>;
-}
-// The instance for launches of `rounds` rounds (both instances share one shared-memory layout, FusedParams::slots).
-FusedKernel pick_fused_kernel(int objective, int halves, int rounds) {
-  return rounds <= 4 ? pick_fused_kernel_r<4>(objective, halves) : pick_fused_kernel_r<kFusedMaxRounds>(objective, halves);
+FusedKernel pick_fused_kernel(int objective, int halves) {
+  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true> : fused_rounds_kernel<0, true>;
+  return objective == 1 ? fused_rounds_kernel<1, false> : fused_rounds_kernel<0, false>;
 }
 
 using TileKernel = void (*)(const TileParams);
@@ -764,7 +761,7 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
   const int64_t M = ctx->M, nq = (ctx->d + 3) / 4;
   const bool f32 = ctx->storage == NETMAX_STORAGE_F32;
   if (!plan.short_vectors && ctx->fuse_rounds >= 2 && M > 144) return NETMAX_OK;  // (fuse_rounds: see the C header)
-  const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)227 * 1024;
+  const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)226 * 1024;
   double best = 0.0;
   int best_c = 0;
   for (int row_limit : {8, 10}) {
@@ -851,6 +848,9 @@ int plan_tiles(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, T
 int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   f = FusedPlan();
   if (ctx->fuse_rounds == 1 || plan.short_vectors) return NETMAX_OK;
+#ifdef NETMAX_FUSED_MAX_M
+  if (ctx->M > NETMAX_FUSED_MAX_M) return NETMAX_OK;
+#endif
   const int64_t M = ctx->M;
   const int want_rounds = ctx->fuse_rounds >= 2 ? std::min(ctx->fuse_rounds, kFusedMaxRounds) : kFusedMaxRounds;
   // 256 or 128 threads per CTA (a multiple of four warps keeps the SM's four schedulers evenly
@@ -864,21 +864,17 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   // M = 20: 132 against 144, 28: 182 against 214, 36: 227 against 287) -- no barrier, no pull that leaves
   // the CTA.  A single such CTA per SM (M = 37 ... 73) is slower than the cluster shape (M = 40: 330
   // against 309), so the kernel is used down to 128 threads per SM.
-  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves, kFusedMaxRounds);  // (the instance with more registers)
+  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves);
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
-  NM_CUDA(ctx, cudaFuncSetAttribute(pick_fused_kernel(ctx->objective, ctx->L.halves, 4), cudaFuncAttributePreferredSharedMemoryCarveout,
-                                    (int)cudaSharedmemCarveoutMaxShared));
-  // The table of draws at the head of the shared memory takes 8 M bytes per round of the launch: room for
-  // as many rounds as were asked for, unless the smaller table of four rounds lets more threads live on an SM
-  // (M = 36: the last kilobytes decide between two CTAs and one).
+  // The head of the shared memory (draws and telemetry sums) grows with the rounds of a launch: room for as
+  // many as were asked for, unless fewer let more threads live on an SM (M = 36: the last kilobytes decide
+  // between two CTAs and one).
   int threads = 0, per_sm = 0, slots = 0;
-  size_t fixed = 0;
-  for (int rounds : {want_rounds, std::min(want_rounds, 4)}) {
-    const size_t fixed_r = align_up((size_t)rounds * M * 8, 128) + 64 * sizeof(double);
+  for (int rounds = want_rounds;; rounds = std::max(2, rounds / 2)) {
     int threads_r = 0, per_sm_r = 0;
     for (int cand : {256, 128, 64}) {
-      const size_t smem = fixed_r + (size_t)48 * M * cand;
-      if (smem > (size_t)227 * 1024) continue;
+      const size_t smem = fused_head(rounds, M, cand) + (size_t)48 * M * cand;
+      if (smem > (size_t)226 * 1024) continue;  // (227 KB less the static part)
       NM_CUDA(ctx, allow_smem((const void*)k, smem));
       int n = 0;
       NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, cand, smem));
@@ -889,17 +885,18 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
       threads = threads_r;
       per_sm = per_sm_r;
       slots = rounds;
-      fixed = fixed_r;
     }
+    if (rounds <= 4) break;
   }
   if (threads == 0 || per_sm * threads < 128) return NETMAX_OK;  // too few warps to hide the arithmetic latency
   f.threads = threads;
   f.slots = slots;
-  f.smem = fixed + (size_t)48 * M * threads;
+  f.smem = fused_head(slots, M, threads) + (size_t)48 * M * threads;
   f.max_rounds = slots;
   f.n_tiles = ((ctx->d + 3) / 4 + threads - 1) / threads;
   NM_CUDA(ctx, allow_smem((const void*)k, f.smem));
   f.grid = (int)std::min<int64_t>(f.n_tiles, std::min<int64_t>((int64_t)per_sm * ctx->sm_count, kMaxGrid));
+  f.max_rounds = (int)std::min<int64_t>(f.max_rounds, (int64_t)(kPartialsBytes / 16) / f.grid);
   f.ok = true;
   return NETMAX_OK;
 }
@@ -1066,8 +1063,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
       fp.inv_M = p.inv_M;
       fp.q_offset = ctx->q_offset + (uint32_t)range.q0;
       fp.keys = p.keys;
-      // (one instance for all launches of the call: the larger one unless the whole call is four rounds or fewer)
-      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, (int)std::min<int64_t>(n, fused.max_rounds));
+      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves);
       NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
       fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
       ctx->launches += 1;
@@ -1118,8 +1114,8 @@ static int check_sizes(const netmax_config* cfg) {
   if (cfg->element_offset < 0 || cfg->element_offset % 4 != 0 || cfg->element_offset + cfg->d >= kMaxD)
     return fail(nullptr, NETMAX_INVALID_ARG, "element_offset = %lld must be a non-negative multiple of 4 with offset + d < 2^30 - 32", (long long)cfg->element_offset);
   if (cfg->trace_rounds < 1) return fail(nullptr, NETMAX_INVALID_ARG, "trace_rounds = %lld < 1", (long long)cfg->trace_rounds);
-  if (cfg->fuse_rounds < 0 || cfg->fuse_rounds > kFusedMaxRounds)
-    return fail(nullptr, NETMAX_INVALID_ARG, "fuse_rounds = %d outside [0, %d]", cfg->fuse_rounds, kFusedMaxRounds);
+  if (cfg->fuse_rounds < 0 || cfg->fuse_rounds > kFuseRoundsLimit)
+    return fail(nullptr, NETMAX_INVALID_ARG, "fuse_rounds = %d outside [0, %d]", cfg->fuse_rounds, kFuseRoundsLimit);
   if (cfg->first_round < 0 || cfg->first_round >= ((int64_t)1 << 56))
     return fail(nullptr, NETMAX_INVALID_ARG, "first_round = %lld outside [0, 2^56)", (long long)cfg->first_round);
   return NETMAX_OK;
@@ -1685,8 +1681,8 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
 
 int netmax_set_fuse_rounds(netmax_ctx* ctx, int32_t fuse_rounds) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
-  if (fuse_rounds < 0 || fuse_rounds > kFusedMaxRounds)
-    return fail(ctx, NETMAX_INVALID_ARG, "fuse_rounds = %d outside [0, %d]", fuse_rounds, kFusedMaxRounds);
+  if (fuse_rounds < 0 || fuse_rounds > kFuseRoundsLimit)
+    return fail(ctx, NETMAX_INVALID_ARG, "fuse_rounds = %d outside [0, %d]", fuse_rounds, kFuseRoundsLimit);
   ctx->fuse_rounds = fuse_rounds;
   ctx->fused_planned = false;
   ctx->tiles_planned = false;

@@ -266,6 +266,38 @@ __device__ __forceinline__ void finalize_telemetry(const RoundParams& p, double 
   }
 }
 
+// A launch of several rounds: the last CTA of the grid to publish its partials [n_rounds][gridDim.x][2] adds
+// them, a warp per round, in a fixed order.  Every thread must call this.
+__device__ __forceinline__ void finalize_rounds(const double* partials, int n_rounds, double inv_M, double* tel, int64_t slot0,
+                                                int64_t ring, unsigned int* ticket) {
+  __shared__ bool s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < n_rounds; k += blockDim.x >> 5) {
+    double a = 0.0, b = 0.0;
+    for (unsigned int j = lane; j < gridDim.x; j += 32) {
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(partials) + (size_t)k * gridDim.x + j);
+      a += v.x;
+      b += v.y;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, off);
+      b += __shfl_down_sync(0xffffffffu, b, off);
+    }
+    if (lane == 0) {
+      double* out = tel + 2 * ((slot0 + k) % ring);
+      out[0] = a * inv_M;
+      out[1] = b * inv_M;
+    }
+  }
+  if (threadIdx.x == 0) *ticket = 0u;
+}
+
 // Direct-load round kernel (any M).  One tile = all M rows (or, for short vectors with many
 // workers, one of rg row groups) x cg column groups.  Thread (cgi, rli) owns column group cgi
 // of the tile and the rows rli, rli + rl, ... of its row group; tiles are taken round-robin by
@@ -580,20 +612,13 @@ __global__ void __launch_bounds__(256, 2) multi_round_kernel(const MultiRoundPar
 // thread's column group is four bfloat16 values (8 bytes of global memory), widened on the way
 // in, and every round's result is rounded to bfloat16 before it is written to the slab, exactly
 // as a store to and a load from the bfloat16 state would.
-#ifndef NETMAX_FUSED_MAX_ROUNDS
-#define NETMAX_FUSED_MAX_ROUNDS 8
-#endif
-#ifndef NETMAX_CLUSTER_MAX_ROUNDS
-#define NETMAX_CLUSTER_MAX_ROUNDS 4
-#endif
 #ifndef NETMAX_FUSED_UNROLL
 #define NETMAX_FUSED_UNROLL 2
 #endif
 #ifndef NETMAX_FUSED_PREFETCH
 #define NETMAX_FUSED_PREFETCH 1  // fetch the next tile under the last round of the current one (fp32 state)
 #endif
-constexpr int kFusedMaxRounds = NETMAX_FUSED_MAX_ROUNDS;      // rounds per launch of fused_rounds_kernel, at most
-constexpr int kClusterMaxRounds = NETMAX_CLUSTER_MAX_ROUNDS;  // of cluster_rounds_kernel (16 accumulator registers per four rounds: it has none to spare)
+constexpr int kFusedMaxRounds = 32;  // rounds per launch of fused_rounds_kernel, at most
 constexpr int kFusedUnroll = NETMAX_FUSED_UNROLL;  // rows of a round in flight per thread
 
 struct FusedParams {
@@ -603,7 +628,7 @@ struct FusedParams {
   const int32_t* trace;  // peer-trace ring [ring][M], filled for these rounds
   const float* wtab;     // [M][M]
   double* tel;           // telemetry ring [ring][2]
-  double* partials;      // [kFusedMaxRounds][gridDim.x][2]
+  double* partials;      // [n_rounds][gridDim.x][2]
   unsigned int* ticket;  // last-CTA-done counter (0 between launches)
   int64_t slot0, ring;   // ring slot of the first round
   uint64_t first_round;
@@ -617,23 +642,29 @@ struct FusedParams {
   PhiloxKeys keys;
 };
 
-// Dynamic shared memory: (peer row offset, weight) int2[slots][M], then the slabs
-// float4[3][M][blockDim] (replicas of even rounds, of odd rounds, centres), then 64 doubles.
-// Any block size that is a multiple of 32 up to 256 works.
-// kRounds: rounds a launch runs at most (4 or kFusedMaxRounds); a thread keeps two double accumulators per round,
-// and a launch of up to four rounds runs 4 % faster on the instance that holds eight instead of sixteen of them.
-template <int kObjective, bool kBf16, int kRounds>
+// Dynamic shared memory: (peer row offset, weight) int2[slots][M], the warps' telemetry sums
+// double[slots][warps][2], then the slabs float4[3][M][blockDim] (replicas of even rounds, of odd rounds,
+// centres).  Any block size that is a multiple of 32 up to 256 works.
+// The telemetry of a round is added over the lanes of a warp at its end (in double, as every sum across threads
+// is) and kept per warp in shared memory: with a thread's own sums in registers a launch was limited to eight
+// rounds, and 32 registers a thread went into them.
+__host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {
+  return (uint32_t)(((uint64_t)slots * (uint64_t)(M * 8 + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);
+}
+template <int kObjective, bool kBf16>
 __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int tid = threadIdx.x, T = blockDim.x, M = p.M;
   int2* s_pw = reinterpret_cast<int2*>(smem_raw);  // (byte offset of the peer's row in a slab, pull weight)
-  const uint32_t head = ((uint32_t)(p.slots * M * 8) + 127u) & ~127u;
+  const uint32_t head = fused_head(p.slots, M, T);
+  double* s_tel = reinterpret_cast<double*>(smem_raw + (size_t)p.slots * M * 8);
+  const int lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
   const uint32_t stride = (uint32_t)T * 16u;     // bytes between consecutive rows of a slab
   const uint32_t plane = (uint32_t)M * stride;   // bytes of one [M][T] slab
   unsigned char* slab = smem_raw + head + (uint32_t)tid * 16u;  // this thread's column: slabs 0, 1 (replicas), 2 (centres)
-  double* s_red = reinterpret_cast<double*>(smem_raw + head + 3u * plane);
 
+  for (int k = tid; k < p.n_rounds * nwarps * 2; k += T) s_tel[k] = 0.0;
   for (int k = 0; k < p.n_rounds; ++k) {
     const int32_t* peers = p.trace + ((p.slot0 + k) % p.ring) * M;
     for (int i = tid; i < M; i += T) {
@@ -642,10 +673,6 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     }
   }
   __syncthreads();
-
-  double acc_cons[kRounds], acc_loss[kRounds];
-#pragma unroll
-  for (int k = 0; k < kRounds; ++k) acc_cons[k] = acc_loss[k] = 0.0;
 
   // Slab `base` (0 or 1) holds the tile's values at the start of the first round; round k reads
   // slab (base + k) & 1 and writes the other one.  The LAST round of a tile writes its results
@@ -661,8 +688,8 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   bool fetched = false;  // has this tile been fetched by the previous one?
   for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
     const int64_t q = tile * T + tid;
-    if (q >= p.nq) continue;  // no barrier below: threads are independent (and later tiles only have larger q)
-    const int live = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
+    const bool live = q < p.nq;  // (no barrier below: warps are independent)
+    const int lanes = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
     const uint32_t q32 = (uint32_t)q + p.q_offset;
     const int64_t q_next = q + (int64_t)gridDim.x * T;
     const bool have_next = kPrefetch && tile + gridDim.x < p.n_tiles && q_next < p.nq;
@@ -679,7 +706,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
           sc += stride;
         }
       }
-    } else {  // all rows of this column group into the thread's slabs
+    } else if (live) {  // all rows of this column group into the thread's slabs
       const char* xq = reinterpret_cast<const char*>(p.x_cur) + (uint64_t)q * kGroupBytes;
       const char* cq = reinterpret_cast<const char*>(p.c) + (uint64_t)q * kGroupBytes;
       unsigned char* sx = slab + base * plane;
@@ -731,7 +758,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       auto do_row = [&](int i, uint4 rnd) {
         const int2 d = pw[i];
         ulonglong2 noise = kObjective == 1 ? scaled_normals4(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
-        if (kRagged) noise = mask_lanes(noise, live);
+        if (kRagged) noise = mask_lanes(noise, lanes);
         const ulonglong2 o = row_update<kObjective>(
             p.alpha, noise, *reinterpret_cast<const ulonglong2*>(cur + off), *reinterpret_cast<const ulonglong2*>(cen + off),
             *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x), pivot, __int_as_float(d.y), acc, lacc);
@@ -750,6 +777,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       };
       // the Philox block of row i + 1 is drawn while row i goes through Box-Muller and Eq. 15-16:
       // the two are independent, so the integer multiplies of the one fill the latencies of the other
+      if (live) {
       const NoiseBase nb = noise_base(q32, round_lo, ctr3, p.keys);
       uint4 rnd = noise_words(nb, 0u, p.keys);
 #pragma unroll kFusedUnroll
@@ -759,6 +787,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
         rnd = rnd_next;
       }
       do_row(M - 1, rnd);
+      }
       float4 s1, s2;
       unpack2(acc.s1a, s1.x, s1.y);
       unpack2(acc.s1b, s1.z, s1.w);
@@ -770,17 +799,16 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       const double cons = (double)((s2.x - s1.x * s1.x * p.inv_M) + (s2.y - s1.y * s1.y * p.inv_M) +
                                    (s2.z - s1.z * s1.z * p.inv_M) + (s2.w - s1.w * s1.w * p.inv_M));
       const double loss = (double)((l0 + l1) + (l2 + l3));
+      // lanes 0-15 go on with the one sum, lanes 16-31 with the other
+      const bool low = lane < 16;
+      double keep = (low ? cons : loss) + __shfl_xor_sync(0xffffffffu, low ? loss : cons, 16);
 #pragma unroll
-      for (int kk = 0; kk < kRounds; ++kk) {  // acc[k] with k known only at run time: predicated adds keep it in registers
-        if (kk == k) {
-          acc_cons[kk] += cons;
-          acc_loss[kk] += loss;
-        }
-      }
+      for (int off = 8; off > 0; off >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, off);
+      if ((lane & 15) == 0) s_tel[(k * nwarps + warp) * 2 + (lane >> 4)] += keep;
     };
     // (a test for padding lanes in every row would keep the rows' instructions apart: the one warp that has
     // any runs its own instance of the round)
-    if (live == 4) {
+    if (__all_sync(0xffffffffu, lanes == 4)) {
       for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type(), std::false_type());
       run_round(p.n_rounds - 1, std::true_type(), std::false_type());
     } else {
@@ -791,23 +819,15 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     fetched = have_next;
   }
 
-  // telemetry: per round, CTA partials; the last CTA to finish sums them in index order
-#pragma unroll
-  for (int k = 0; k < kRounds; ++k)
-    if (k < p.n_rounds) block_partials(p.partials + (size_t)k * 2 * gridDim.x, acc_cons[k], acc_loss[k], s_red);
-  __shared__ bool s_last;
-  if (tid == 0) {
-    __threadfence();
-    const unsigned int t = atomicAdd(p.ticket, 1u);
-    s_last = (t == gridDim.x - 1);
-  }
+  // telemetry: per round, CTA partials; the last CTA to finish sums them
   __syncthreads();
-  if (s_last) {
-    __threadfence();
-    for (int k = 0; k < p.n_rounds; ++k)
-      sum_partials(p.partials + (size_t)k * 2 * gridDim.x, (double)p.inv_M, p.tel + 2 * ((p.slot0 + k) % p.ring), s_red);
-    if (tid == 0) *p.ticket = 0u;
+  for (int e = tid; e < p.n_rounds * 2; e += T) {
+    const int k = e >> 1;
+    double a = 0.0;
+    for (int w = 0; w < nwarps; ++w) a += s_tel[(k * nwarps + w) * 2 + (e & 1)];
+    p.partials[((size_t)k * gridDim.x + blockIdx.x) * 2 + (e & 1)] = (e & 1) ? 0.5 * a : a;
   }
+  finalize_rounds(p.partials, p.n_rounds, (double)p.inv_M, p.tel, p.slot0, p.ring, p.ticket);
 }
 
 // tel[slot of round k] = (sum over tiles of partials[k][tile]) / M, one warp per round, tiles in a fixed order.

@@ -61,7 +61,8 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 // u1 = (top23(a) + 1/2) / 2^23 in (0,1), exactly representable in fp32:
 // bits 0x3F800000 | top23 are the float 1 + top23 / 2^23; subtracting 1 - 2^-24 is exact.
 __device__ __forceinline__ float radius_uniform(uint32_t a) {
-  return __uint_as_float(0x3F800000u | (a >> 9)) - 0.99999994039535522461f;
+  // (those bits are the funnel shift of 0x7F : a by 9, one instruction)
+  return __uint_as_float(__funnelshift_r(a, 0x7Fu, 9)) - 0.99999994039535522461f;
 }
 
 // Hardware log2 of a normal number (u1 >= 2^-24 here, so flushing subnormals changes nothing
@@ -160,8 +161,9 @@ __device__ __forceinline__ float4 normals4(uint4 r) {
 // ---- noise blocks of many workers at one (column group, round) --------------------------------------
 // Philox4x32-10 at counter (q, worker, round, tag).  The parts of its first three rounds that do not depend
 // on the worker are worked out once per (column group, round): of the twenty 32 x 32 -> 64 multiplies of a
-// block sixteen remain per worker.  (What these multiplies cost: a stream of them issues one per 5 cycles
-// and scheduler, and the blocks alone take 76 of the 104 cycles of four normals.)
+// block sixteen remain per worker.  (A stream of such multiplies issues one per 5 cycles and
+// scheduler; a block takes 65 of the 190 cycles of a row of a column group.  High halves by fp64 multiply-adds, whose
+// pipe idles, took as long with 14 instructions more.)
 struct NoiseBase {
   uint32_t a0, c3, c1, h0, l0;
 };

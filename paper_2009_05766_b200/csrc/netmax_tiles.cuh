@@ -301,20 +301,7 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
     if (warp == turn) add_shares(buf ^ 1u, summed, due_first);
   }
   if (!p.finalize) return;
-  __shared__ bool s_last;
-  __shared__ double s_red[64];
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    for (int k = 0; k < p.n_rounds; ++k)
-      sum_partials(p.partials + (size_t)k * 2 * gridDim.x, (double)p.inv_M, p.tel + 2 * ((p.slot0 + k) % p.ring), s_red);
-    if (tid == 0) *p.ticket = 0u;
-  }
+  finalize_rounds(p.partials, p.n_rounds, (double)p.inv_M, p.tel, p.slot0, p.ring, p.ticket);
 }
 
 }  // namespace netmax
