@@ -149,6 +149,7 @@ struct Layout {
 
 constexpr int kFuseRoundsLimit = 8;  // largest netmax_config.fuse_rounds
 constexpr int kMaxGrid = 148 * 16;  // upper bound on resident CTAs of the round kernel
+constexpr int64_t kCutLaps = 16, kCutRounds = 16;  // tiles are cut for up to this many tiles per CTA, from this many rounds on
 constexpr int64_t kMaxRoundsPerLaunch = 4096;  // rounds one cooperative launch runs at most
 constexpr size_t kPartialsBytes = (size_t)kMaxGrid * 2 * sizeof(double) * 8;  // per CTA and round of a fused launch; two sets for multi-round launches
 constexpr size_t kColPartBytes = (size_t)8 << 20;  // column partials of the row-split (short vector) shape
@@ -645,7 +646,13 @@ TileKernel pick_tile_kernel(int objective, int halves, int rows) {
     case 7: return pick_tile_kernel_r<7>(objective, halves);
     case 8: return pick_tile_kernel_r<8>(objective, halves);
     case 9: return pick_tile_kernel_r<9>(objective, halves);
-    default: return pick_tile_kernel_r<10>(objective, halves);
+    case 10: return pick_tile_kernel_r<10>(objective, halves);
+    case 11: return pick_tile_kernel_r<11>(objective, halves);
+    case 12: return pick_tile_kernel_r<12>(objective, halves);
+    case 13: return pick_tile_kernel_r<13>(objective, halves);
+    case 14: return pick_tile_kernel_r<14>(objective, halves);
+    case 15: return pick_tile_kernel_r<15>(objective, halves);
+    default: return pick_tile_kernel_r<16>(objective, halves);
   }
 }
 
@@ -750,41 +757,44 @@ int plan_round(netmax_ctx* ctx, RoundPlan& plan, int objective) {
   return NETMAX_OK;
 }
 
-// Launch shape of tile_rounds_kernel: G column groups per tile, W warps per CTA.  Modelled from what was
-// measured: a row of a column group costs its scheduler about 190 cycles, a round at least 600 cycles plus
-// 230 for every row of a thread however little else runs, and an SM holds 16 warps (128 registers) as far as
-// its shared memory goes.  Wider tiles win ties (longer pieces of a row per load).  A thread keeps the noise of
-// its rows in registers, so it gets at most eight (ten where nothing else fits: 4097 to 4700 workers).
+// Launch shape of tile_rounds_kernel: G column groups per tile, W warps per CTA, K rows per thread.  Modelled on
+// measurements of every shape for 32 sizes (2 to 4600 workers): a row costs its scheduler 224 cycles and the rest
+// of a thread's round as much as a row (so many rows per thread are better than many threads); a round takes at
+// least 1,000 cycles and 450 more for every row of a thread, however little else runs; warp counts that four does
+// not divide lose 10 %.  An SM holds 12 to 16 warps (by the registers of the instance) as far as its shared memory
+// goes.  The shape chosen is within 2 % of the best one on average.
 int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, TilePlan& f) {
   f = TilePlan();
   if (ctx->fuse_rounds == 1 || fused.ok) return NETMAX_OK;
   const int64_t M = ctx->M, nq = (ctx->d + 3) / 4;
   const bool f32 = ctx->storage == NETMAX_STORAGE_F32;
   if (!plan.short_vectors && ctx->fuse_rounds >= 2 && M > 144) return NETMAX_OK;  // (fuse_rounds: see the C header)
-  const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)226 * 1024;
+  const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)226 * 1024;  // (227 KB less the static part)
   double best = 0.0;
   int best_c = 0;
-  for (int row_limit : {8, 10}) {
+  {
     for (int G = 32, log2G = 5; G >= 1; G >>= 1, --log2G) {
       for (int W = 1; W <= 16; ++W) {
         const int RL = W * 32 / G;
         const int K = (int)((M + RL - 1) / RL);
-        if (K > row_limit || (RL > M && W > 1)) continue;
+        if (K > kTileMaxRows || (RL > M && W > 1) || W * 32 > tile_max_threads(K)) continue;
+        const int warps = tile_max_threads(K) / 32;  // that an SM's registers hold
         bool pre = false;
-        size_t smem = tile_smem(M, W * 32, G, false);
-        const size_t small = tile_smem(M, W * 32, G, true);
-        if (smem > per_cta || (smem > small && per_sm / (smem + 1024) < std::min<size_t>(16 / W, per_sm / (small + 1024)))) {
+        size_t smem = tile_smem(M, W * 32, G, false, K);
+        const size_t small = tile_smem(M, W * 32, G, true, K);
+        if (smem > per_cta || (smem > small && per_sm / (smem + 1024) < std::min<size_t>(warps / W, per_sm / (small + 1024)))) {
           pre = true;
           smem = small;
         }
         if (smem > per_cta) continue;
-        const int64_t fit = std::min<int64_t>(16 / W, (int64_t)(per_sm / (smem + 1024)));
+        const int64_t fit = std::min<int64_t>(warps / W, (int64_t)(per_sm / (smem + 1024)));
         if (fit < 1) continue;
         const int64_t n_tiles = (nq + G - 1) / G;
         const int64_t c = std::min<int64_t>(fit, (n_tiles + ctx->sm_count - 1) / ctx->sm_count);
-        const double passes = n_tiles > (int64_t)ctx->sm_count * c * 8 ? (double)n_tiles / (double)(ctx->sm_count * c)
-                                                                        : (double)((n_tiles + ctx->sm_count * c - 1) / (ctx->sm_count * c));
-        const double cycles = passes * std::max((double)(c * K * W) * 190.0 / 4.0, 600.0 + 230.0 * K) * (pre ? 1.03 : 1.0);
+        const double laps = (double)n_tiles / (double)(ctx->sm_count * c);
+        const double passes = laps > 8.0 || (laps > 1.0 && plan.short_vectors) ? laps : std::ceil(laps);  // (few tiles are cut)
+        const double cycles = passes * std::max((double)((c * W + 3) / 4) * (224.0 * K + 224.0), 1000.0 + 450.0 * K) *
+                              (W % 4 != 0 ? 1.1 : 1.0) * (pre ? 1.03 : 1.0);
         if (best == 0.0 || cycles < best * 0.999) {
           best = cycles;
           best_c = (int)c;
@@ -798,7 +808,6 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
         }
       }
     }
-    if (best > 0.0) break;
   }
   if (best == 0.0) return NETMAX_OK;
   TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, f.rows);
@@ -878,6 +887,7 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
       NM_CUDA(ctx, allow_smem((const void*)k, smem));
       int n = 0;
       NM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, cand, smem));
+      if (cand == 64 && per_sm_r >= 2) continue;  // (two-warp CTAs load two of an SM's four schedulers: M = 10, 235 cycles a row against 197)
       const bool better = (n >= 2) != (per_sm_r >= 2) ? n >= 2 : n * cand > per_sm_r * threads_r;
       if (n >= 1 && (threads_r == 0 || better)) { threads_r = cand; per_sm_r = n; }
     }
@@ -990,7 +1000,20 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
   TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, tiles.rows);
   NM_CUDA(ctx, allow_smem((const void*)k, tiles.smem));
   const int64_t grid = std::min<int64_t>(tiles.grid, tp.n_tiles);
-  k<<<(unsigned)grid, tiles.threads, tiles.smem, stream>>>(tp);
+  // Few tiles per CTA and enough rounds: equal lengths of cut tiles instead of whole ones, where the last lap
+  // would leave more than 3 % of the CTAs' time unused (a cut costs one more load of the tile's rows).
+  const int64_t laps = (tp.n_tiles + grid - 1) / grid;
+  tp.cut = reinterpret_cast<unsigned int*>(ctx->partials);  // (this kernel keeps its partials in colpart)
+  tp.units = 0;
+  if (ctx->cooperative && laps >= 2 && laps <= kCutLaps && chunk >= kCutRounds && laps * grid * 100 > tp.n_tiles * 103)
+    tp.units = (tp.n_tiles * chunk + grid - 1) / grid;
+  if (tp.units > 0) {
+    NM_CUDA(ctx, cudaMemsetAsync(tp.cut, 0, (size_t)grid * sizeof(unsigned int), stream));
+    void* args[] = {&tp};
+    NM_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k, dim3((unsigned)grid), dim3((unsigned)tiles.threads), args, tiles.smem, stream));
+  } else {
+    k<<<(unsigned)grid, tiles.threads, tiles.smem, stream>>>(tp);
+  }
   ctx->launches += 1;
   if (!finalize) {
     const int warps_per_block = kThreads / 32;

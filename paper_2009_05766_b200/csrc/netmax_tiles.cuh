@@ -60,26 +60,84 @@ struct TileParams {
   int32_t G, log2G;       // column groups per tile (a power of two, at most 32)
   int32_t pre_reduce;     // sums are added over the lanes of a warp first (scratch for G entries per warp, not 32)
   int32_t finalize;
+  int64_t units;          // > 0: tiles are cut, every CTA runs this many rounds of tiles (see Piece)
+  unsigned int* cut;      // [gridDim.x]: raised by a CTA that has run its share of a cut tile (0 before the launch)
   float alpha, sigma, inv_M;   // sigma: the noise scale sigma sqrt(2 ln 2)
   uint32_t q_offset;
   PhiloxKeys keys;
 };
 
-// Dynamic shared memory: slabs float4[3][M][G] (replicas of even and of odd rounds, centres), then two
+// What a CTA runs: rounds [k0, k1) of a tile.  With many tiles a CTA takes every gridDim.x-th one, all rounds.
+// With few of them (units > 0) that leaves some CTAs a whole tile more than others -- 256 tiles on 148 CTAs
+// take as long as 296 -- so tiles are cut: laid end to end, tile by tile and round by round, the work is dealt
+// out in equal lengths, each at least one tile's.  A cut tile's first rounds are the END of CTA b - 1's length
+// and its last rounds the BEGINNING of CTA b's; every CTA runs its length from the far end, so that b - 1
+// starts with its share and b finishes with the rest, long after the share is there.  The state between them
+// goes through x_nxt; b waits (bounded) for a flag of b - 1, which by then waits for nobody, and the launch is
+// cooperative, so that both are resident.  4096 x 1024 elements: 8.7 -> 7.5 us per round.
+struct Piece {
+  int64_t tile;
+  int32_t k0, k1;
+};
+// The n-th piece of this CTA; false: there is none.
+__device__ __forceinline__ bool tile_piece(const TileParams& p, int n, Piece& out) {
+  const int64_t b = blockIdx.x, R = p.n_rounds;
+  out.k0 = 0;
+  out.k1 = p.n_rounds;
+  if (p.units == 0) {
+    out.tile = b + (int64_t)n * gridDim.x;
+    return out.tile < p.n_tiles;
+  }
+  const int64_t all = p.n_tiles * R;
+  const int64_t lo = min(all, b * p.units), hi = min(all, lo + p.units);
+  const int32_t k_lo = (int32_t)(lo % R), k_hi = (int32_t)(hi % R);
+  const int64_t first = (lo + R - 1) / R, last = hi / R;  // whole tiles [first, last)
+  if (k_hi > 0) {  // the share of tile `last` (a length is at least one tile's, so it begins in this one)
+    if (n == 0) {
+      out.tile = last;
+      out.k1 = k_hi;
+      return true;
+    }
+    --n;
+  }
+  if (n < last - first) {
+    out.tile = first + n;
+    return true;
+  }
+  if (n == last - first && k_lo > 0) {  // the rest of the tile that CTA b - 1 begins
+    out.tile = first - 1;
+    out.k0 = k_lo;
+    return true;
+  }
+  return false;
+}
+
+// Threads a CTA of the instance with `rows` rows per thread may have (and an SM holds): the registers of a row
+// decide.
+__host__ __device__ constexpr int tile_max_threads(int rows) { return rows <= 8 ? 512 : rows <= 10 ? 448 : 384; }
+constexpr int kTileMaxRows = 16;
+// Few rows per thread make a round short, and what is not the round itself counts: draws are fetched two rounds
+// ahead, and the sums of a round are added after the NEXT round's arrival, beside its noise, which takes a third
+// buffer (32 x 1000 elements: 0.79 -> 0.68 us per round).  With more rows the buffer is better kept for slabs.
+__host__ __device__ constexpr bool tile_far(int rows) { return rows <= 4; }
+
+// Dynamic shared memory: slabs float4[3][M][G] (replicas of even and of odd rounds, centres), then two or three
 // buffers of telemetry shares, each float4[E] + float2[E] with E = warps x (pre_reduce ? G : 32).
 __host__ __device__ inline uint32_t tile_share_entries(int threads, int G, bool pre_reduce) {
   return (uint32_t)(threads >> 5) * (uint32_t)(pre_reduce ? G : 32);
 }
-__host__ __device__ inline size_t tile_smem(int64_t M, int threads, int G, bool pre_reduce) {
-  return (size_t)48 * M * G + (size_t)48 * tile_share_entries(threads, G, pre_reduce);
+__host__ __device__ inline size_t tile_smem(int64_t M, int threads, int G, bool pre_reduce, int rows) {
+  return (size_t)48 * M * G + (size_t)(tile_far(rows) ? 72 : 48) * tile_share_entries(threads, G, pre_reduce);
 }
 
 // kRows: rows per thread, ceil(M / RL).  Exact, so that only a thread's LAST row can be missing: rows before it
 // run without a test between them and the scheduler can mix their instructions (with a test per row the same
 // rows took 282 cycles each instead of 195).
 template <int kObjective, bool kBf16, int kRows>
-__global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p) {
+__global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel(const TileParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
+  constexpr bool kFar = tile_far(kRows);
+  constexpr uint32_t kBuffers = kFar ? 3u : 2u;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long s_bar;
   const int tid = threadIdx.x, T = blockDim.x, M = p.M, G = p.G;
@@ -93,15 +151,14 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
   unsigned char* const col = smem_raw + (uint32_t)g * 16u;
   unsigned char* const own = col + (uint32_t)r * stride;
   const uint32_t E = tile_share_entries(T, G, p.pre_reduce != 0);
-  float4* const s_sum = reinterpret_cast<float4*>(smem_raw + 3u * plane);     // [2][E]
-  float2* const s_two = reinterpret_cast<float2*>(s_sum + 2u * E);            // [2][E]
+  float4* const s_sum = reinterpret_cast<float4*>(smem_raw + 3u * plane);     // [kBuffers][E]
+  float2* const s_two = reinterpret_cast<float2*>(s_sum + kBuffers * E);      // [kBuffers][E]
   const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_bar);
   if (tid == 0) mbar_init(bar, (uint32_t)nwarps);
   __syncthreads();
 
-  int2 draw[kRows];
+  int2 draw[kRows], draw_far[kFar ? kRows : 1];
   ulonglong2 noise[kRows];
-  int64_t tile = blockIdx.x;
 
   // body(j) for the rows of this thread
   auto rows = [&](auto body) {
@@ -109,12 +166,24 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
     for (int j = 0; j < kRows - 1; ++j) body(j);
     if (full) body(kRows - 1);
   };
-  int64_t slot = p.slot0;  // ring slot of the next draws to load
-  auto next_draws = [&](int k) {
-    if (k == 0) slot = p.slot0;
+  int64_t slot = 0;  // ring slot of the draws to be loaded next
+  auto load_draws = [&](int2* into) {
     const int2* src = p.draws + slot * M + r;
-    rows([&](int j) { draw[j] = __ldg(src + j * RL); });
+    rows([&](int j) { into[j] = __ldg(src + j * RL); });
     slot = slot + 1 == p.ring ? 0 : slot + 1;
+  };
+  auto first_draws = [&](int k) {  // of a piece that starts at round k
+    slot = (p.slot0 + k) % p.ring;
+    load_draws(draw);
+    if (kFar) load_draws(draw_far);
+  };
+  auto next_draws = [&]() {  // (past the last round what comes is not used)
+    if (kFar) {
+      rows([&](int j) { draw[j] = draw_far[j]; });
+      load_draws(draw_far);
+    } else {
+      load_draws(draw);
+    }
   };
   auto next_noise = [&](int64_t q, int k) {
     if (kObjective != 1) return;
@@ -126,7 +195,7 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
   };
   // telemetry of one round: this warp adds the shares of all threads (lane -> entries lane, lane + 32, ...,
   // which belong to column group lane % G) and leaves the CTA's two sums
-  auto add_shares = [&](uint32_t buf, int k, bool first) {
+  auto add_shares = [&](uint32_t buf, int k) {
     float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f);
     float s2 = 0.f, loss = 0.f;
     for (uint32_t e = lane; e < E; e += 32) {
@@ -150,59 +219,69 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
     }
     if (lane == 0) {
       double* out = p.partials + ((size_t)k * gridDim.x + blockIdx.x) * 2;
-      const double a = (double)s2, b = 0.5 * (double)loss;
-      if (first) {
-        out[0] = a;
-        out[1] = b;
-      } else {  // this CTA's share of an earlier tile is there, written by this very thread
-        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out), "d"(a) : "memory");
-        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + 1), "d"(b) : "memory");
-      }
+      asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out), "d"((double)s2) : "memory");
+      asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + 1), "d"(0.5 * (double)loss) : "memory");
     }
   };
+  for (int k = tid; k < p.n_rounds; k += T)
+    reinterpret_cast<double2*>(p.partials)[(size_t)k * gridDim.x + blockIdx.x] = make_double2(0.0, 0.0);
+  __syncthreads();
 
-  // the first tile
-  int64_t q = tile * G + g;
-  bool live = q < p.nq;
-  if (tile < p.n_tiles) {
-    if (live) {
-      const char* xq = p.x_cur + (uint64_t)q * kGroupBytes + row_first;
+  // a piece's rows into slab `base` (once CTA b - 1 has done its share of a cut tile), the draws and the noise of
+  // its first round; then arrives
+  auto load_piece = [&](const Piece& pc, uint32_t base) {
+    if (pc.k0 > 0) {
+      if (tid == 0) {
+        uint32_t it = 0;
+        while (*reinterpret_cast<volatile unsigned int*>(p.cut + blockIdx.x - 1) == 0u && ++it < kTileSpinLimit) __nanosleep(64);
+        if (it == kTileSpinLimit) *reinterpret_cast<volatile unsigned int*>(p.error) = 1u;
+        __threadfence();
+      }
+      __syncthreads();
+    }
+    const int64_t q = pc.tile * G + g;
+    if (q < p.nq) {
+      const char* xq = (pc.k0 == 0 ? p.x_cur : p.x_nxt) + (uint64_t)q * kGroupBytes + row_first;
       const char* cq = p.c + (uint64_t)q * kGroupBytes + row_first;
       rows([&](int j) {
-        unsigned char* sx = own + (uint32_t)j * step;
+        unsigned char* sx = own + base * plane + (uint32_t)j * step;
+        unsigned char* sc = own + 2u * plane + (uint32_t)j * step;
         if (kBf16) {
-          *reinterpret_cast<ulonglong2*>(sx) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(xq + j * row_step)));
-          *reinterpret_cast<ulonglong2*>(sx + 2u * plane) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(cq + j * row_step)));
+          *reinterpret_cast<ulonglong2*>(sx) = widen_bf16x4(__ldcg(reinterpret_cast<const unsigned long long*>(xq + j * row_step)));
+          *reinterpret_cast<ulonglong2*>(sc) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(cq + j * row_step)));
         } else {
           cp_async_16_stream(sx, xq + j * row_step);
-          cp_async_16_stream(sx + 2u * plane, cq + j * row_step);
+          cp_async_16_stream(sc, cq + j * row_step);
         }
       });
     }
-    next_draws(0);
-    next_noise(q, 0);
+    first_draws(pc.k0);
+    next_noise(q, pc.k0);
     cp_async_wait_all();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);
-  }
+  };
 
   uint32_t base = 0, phase = 0, buf = 0;
-  int turn = 0;             // the warp that adds the shares of the round before the current one
-  int summed = 0;           // round whose shares are due
-  bool due = false, due_first = true;
-  for (; tile < p.n_tiles; tile += gridDim.x) {
-    const int64_t q_next = q + (int64_t)gridDim.x * G;
-    const bool tile_next = tile + gridDim.x < p.n_tiles;
-    const bool have_next = tile_next && q_next < p.nq;
-    const bool first_tile = tile == blockIdx.x;
+  // the last round whose shares have not been added, and the warp -- a different one every round -- that does it
+  int turn = 0, last_k = -1;
+  Piece pc = {0, 0, 0}, next = {0, 0, 0};
+  bool more = tile_piece(p, 0, pc);
+  if (more) load_piece(pc, 0);
+  for (int n = 1; more; ++n) {
+    const int64_t q = pc.tile * G + g;
+    const bool live = q < p.nq;
+    more = tile_piece(p, n, next);
+    const bool ahead = more && next.k0 == 0;  // the next piece's rows are fetched under this one's last round
+    const int64_t q_next = next.tile * G + g;
+    const bool have_next = ahead && q_next < p.nq;
 
     auto run_round = [&](int k, auto last_tag) {
       constexpr bool kLast = decltype(last_tag)::value;
       mbar_wait(bar, phase, p.error);  // all rows of the previous round are written
       phase ^= 1u;
-      if (due && warp == turn) add_shares(buf ^ 1u, summed, due_first);
-      turn = turn + 1 == nwarps ? 0 : turn + 1;
-      const uint32_t cur_off = ((base + (uint32_t)k) & 1u) * plane, nxt_off = plane - cur_off;
+      if (!kFar && last_k >= 0 && warp == turn) add_shares(buf ^ 1u, last_k);
+      const uint32_t cur_off = ((base + (uint32_t)(k - pc.k0)) & 1u) * plane, nxt_off = plane - cur_off;
       ColAcc acc;
       LossAcc lacc;
       if (kLast && have_next) {  // the next tile's replicas into the slab this round does not write
@@ -264,7 +343,7 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
         s_sum[buf * E + tid] = s1;
         s_two[buf * E + tid] = two;
       }
-      if (kLast && tile_next) {
+      if (kLast && ahead) {
         cp_async_wait_all();  // the next tile's rows have landed: the barrier publishes them too
         if (kBf16 && have_next) {
           rows([&](int j) {
@@ -277,28 +356,37 @@ __global__ void __launch_bounds__(512, 1) tile_rounds_kernel(const TileParams p)
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar);
-      buf ^= 1u;
-      due = true;
-      due_first = first_tile;
-      summed = k;
-      // while the others finish: the draws and the noise of the next round
+      // while the others finish: the draws and the noise of the next round, the sums of the previous one
       if (!kLast) {
-        next_draws(k + 1);
+        next_draws();
         next_noise(q, k + 1);
-      } else if (tile_next) {
-        next_draws(0);
+      } else if (ahead) {
+        first_draws(0);
         next_noise(q_next, 0);
       }
+      if (kFar && last_k >= 0 && warp == turn) add_shares(buf == 0 ? 2u : buf - 1u, last_k);  // (not written again before two more barriers)
+      turn = turn + 1 == nwarps ? 0 : turn + 1;
+      buf = buf == kBuffers - 1u ? 0 : buf + 1;
+      last_k = k;
     };
-    for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type());
-    run_round(p.n_rounds - 1, std::true_type());
-    base = (base + (uint32_t)p.n_rounds) & 1u;
-    q = q_next;
-    live = q < p.nq;
+    for (int k = pc.k0; k + 1 < pc.k1; ++k) run_round(k, std::false_type());
+    run_round(pc.k1 - 1, std::true_type());
+    base = (base + (uint32_t)(pc.k1 - pc.k0)) & 1u;
+    if (pc.k1 < p.n_rounds) {  // this CTA's share of a cut tile is in x_nxt
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) *reinterpret_cast<volatile unsigned int*>(p.cut + blockIdx.x) = 1u;
+    }
+    if (more && !ahead) {  // the rest of the tile that CTA b - 1 has begun
+      mbar_wait(bar, phase, p.error);  // (this piece's last round: its slabs are free)
+      phase ^= 1u;
+      load_piece(next, base);
+    }
+    pc = next;
   }
-  if (due) {
+  if (last_k >= 0) {
     mbar_wait(bar, phase, p.error);
-    if (warp == turn) add_shares(buf ^ 1u, summed, due_first);
+    if (warp == turn) add_shares(buf == 0 ? kBuffers - 1u : buf - 1u, last_k);
   }
   if (!p.finalize) return;
   finalize_rounds(p.partials, p.n_rounds, (double)p.inv_M, p.tel, p.slot0, p.ring, p.ticket);

@@ -153,3 +153,23 @@ def test_split_calls_change_no_bit_of_replicas_trace_or_telemetry(nm):
     assert (ta[0] == tb[0]).all() and (ta[1] == tb[1]).all()
     a.close()
     b.close()
+
+
+# cut tiles (few tiles per CTA, 16 rounds and more): one tile more than CTAs; a last CTA with only the rest of a tile;
+# two CTAs per SM; long vectors; instances with 1, 4, 11 and 12 rows per thread, the largest number of workers
+@pytest.mark.parametrize("M,d,rounds,storage", [(4096, 149 * 4, 16, "f32"), (4096, 1024, 37, "bf16"), (2100, 1801, 20, "f32"),
+                                                (4700, 603, 17, "f32"), (350, 50_002, 16, "f32"), (93, 90_003, 23, "bf16"),
+                                                (64, 77_001, 16, "f32"), (1000, 4_001, 40, "f32"), (13, 100_003, 18, "f32")])
+def test_cut_tiles_change_no_bit(nm, M, d, rounds, storage):
+    rng = np.random.default_rng(M + d)
+    P = random_policy(M, rng)
+    kw = dict(M=M, d=d, lr=0.05, prob=P, sigma=0.1, x0_std=1.0, c_std=1.0, objective=1, seed=d + M, trace_rounds=64, storage=storage)
+    plain, res = nm.Netmax(fuse_rounds=1, **kw), nm.Netmax(**kw)
+    plain.round(rounds)
+    res.round(rounds)
+    assert (plain.read_replicas().view(np.uint32) == res.read_replicas().view(np.uint32)).all()
+    (ca, la), (cb, lb) = plain.telemetry(), res.telemetry()
+    np.testing.assert_allclose(cb, ca, rtol=2e-5)      # fp32 partial sums in another order: M up to 4700 of them, 2e-5 as above
+    np.testing.assert_allclose(lb, la, rtol=2e-5)
+    plain.close()
+    res.close()
