@@ -580,10 +580,36 @@ int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int3
   p.n_rounds = n_rounds;
   p.M = ctx->M;
   p.keys = ctx->keys;
-  const int64_t total = n_rounds * (int64_t)ctx->M;
-  const int grid = (int)std::min<int64_t>((total + kThreads - 1) / kThreads, (int64_t)ctx->sm_count * 32);
-  sample_peers_kernel<<<grid, kThreads, 0, ctx->stream>>>(p);
-  ctx->launches += 1;
+  const int64_t M = ctx->M;
+  // Rows in shared memory pay where there is much to draw and a row is drawn from often enough to repay reading it
+  // whole (us for thresholds through the caches against rows: 4096 x 64 draws 19 / 19, x 128 32 / 22, x 1024 177 / 45;
+  // 1024 x 256 17 / 12, x 4096 141 / 43; 256 x 1024 15 / 12).  Four rows per CTA as long as three CTAs share an SM,
+  // else two (8192 x 1024: 160 against 109).
+  const int rows = sample_smem((uint32_t)M, 4) <= (size_t)75 * 1024 ? 4 : 2;
+  const size_t smem = sample_smem((uint32_t)M, rows);
+  if (M >= 128 && n_rounds * M >= ((int64_t)1 << 17) && n_rounds * 40 >= M && n_rounds <= (int64_t)1 << 30 && smem <= (size_t)220 * 1024) {
+    auto kernel = rows == 4 ? sample_rows_kernel<4> : sample_rows_kernel<2>;
+    NM_CUDA(ctx, allow_smem((const void*)kernel, smem));
+    const int64_t groups = (M + rows - 1) / rows;
+    // rounds are shared out over CTAs as well where the workers alone would not give every SM three of them
+    const int64_t splits = std::max<int64_t>(1, std::min<int64_t>(3 * (int64_t)ctx->sm_count / groups, n_rounds / 256));
+    const int64_t per_cta = (n_rounds + splits - 1) / splits;
+    kernel<<<dim3((unsigned)groups, (unsigned)((n_rounds + per_cta - 1) / per_cta)), kSampleThreads, smem, ctx->stream>>>(
+        p, (uint32_t)per_cta);
+    ctx->launches += 1;
+    NM_CUDA(ctx, cudaGetLastError());
+    return NETMAX_OK;
+  }
+  const int64_t most = std::max<int64_t>(1, (((int64_t)1 << 31) - 1) / M);  // rounds of one launch: its indices are 32 bits wide
+  for (int64_t done = 0; done < n_rounds; done += most) {
+    p.n_rounds = std::min<int64_t>(most, n_rounds - done);
+    p.first_round = first_round + (uint64_t)done;
+    p.slot0 = (slot0 + done) % ring;
+    const int64_t total = p.n_rounds * M;
+    const int grid = (int)std::min<int64_t>((total + kThreads - 1) / kThreads, (int64_t)ctx->sm_count * 32);
+    sample_peers_kernel<<<grid, kThreads, 0, ctx->stream>>>(p);
+    ctx->launches += 1;
+  }
   NM_CUDA(ctx, cudaGetLastError());
   return NETMAX_OK;
 }

@@ -28,6 +28,19 @@
 
 namespace netmax {
 
+// 16 bytes from global to shared memory without passing through registers or L1 (data that no other
+// thread of the SM will ask for); completion is awaited by the same thread with cp_async_wait_all.
+__device__ __forceinline__ void cp_async_16_stream(void* smem_dst, const void* gmem_src) {
+  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gmem_src) : "memory");
+}
+// The same for 8 bytes (four bfloat16 values; copies below 16 bytes go through L1).
+__device__ __forceinline__ void cp_async_8(void* smem_dst, const void* gmem_src) {
+  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ------------------------------------------------------------------------- sampler
 struct SampleParams {
   const uint32_t* thresholds;  // [M][M] non-decreasing per row
@@ -43,26 +56,111 @@ struct SampleParams {
   PhiloxKeys keys;
 };
 
-// m = min(#{j : T[j] <= u}, last_nz): the count is found by bisection (T is sorted).
+__device__ __forceinline__ uint32_t peer_word(const SampleParams& p, uint32_t worker, uint64_t round) {
+  return philox4x32_10(0u, worker, (uint32_t)round, philox_ctr3(kTagPeer, round), p.keys).x;
+}
+__device__ __forceinline__ void put_draw(const SampleParams& p, uint32_t r, uint32_t i, int32_t m) {
+  int64_t slot = p.slot0 + r;  // (a batch is never longer than the ring)
+  if (slot >= p.ring) slot -= p.ring;
+  const int64_t at = slot * p.M + i;
+  p.out[at] = m;
+  if (p.host_out) p.host_out[at] = m;
+  if (p.draws) p.draws[at] = make_int2(m, __float_as_int((m == (int32_t)i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m)));
+}
+
+// m = min(#{j : T[j] <= u}, last_nz): the count is found by bisection (T is sorted).  One thread per draw,
+// thresholds through the caches: for few rounds or few workers.  At most 2^31 draws per launch.
 __global__ void __launch_bounds__(256) sample_peers_kernel(const SampleParams p) {
-  const int64_t total = p.n_rounds * (int64_t)p.M;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = idx / p.M;
-    const int32_t i = (int32_t)(idx - r * p.M);
-    const uint64_t round = p.first_round + (uint64_t)r;
-    const uint32_t u = philox4x32_10(0u, (uint32_t)i, (uint32_t)round, philox_ctr3(kTagPeer, round), p.keys).x;
-    const uint32_t* __restrict__ row = p.thresholds + (size_t)i * p.M;
+  const uint32_t M = (uint32_t)p.M, total = (uint32_t)p.n_rounds * M;
+  for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
+    const uint32_t r = idx / M, i = idx - r * M;
+    const uint32_t u = peer_word(p, i, p.first_round + r);
+    const uint32_t* __restrict__ row = p.thresholds + (size_t)i * M;
     int32_t lo = 0, hi = p.M;
     while (lo < hi) {
       const int32_t mid = (lo + hi) >> 1;
       if (__ldg(row + mid) <= u) lo = mid + 1; else hi = mid;
     }
-    const int32_t m = min(lo, __ldg(p.last_nz + i));
-    const int64_t at = ((p.slot0 + r) % p.ring) * p.M + i;
-    p.out[at] = m;
-    if (p.host_out) p.host_out[at] = m;
-    if (p.draws) p.draws[at] = make_int2(m, __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m)));
+    put_draw(p, r, i, min(lo, __ldg(p.last_nz + i)));
+  }
+}
+
+// The same for many rounds of many workers: bisection through the caches is twelve dependent trips to L2 per draw
+// (177 us for 1,024 rounds of 4,096 workers).  Here a CTA brings the rows of kSampleRows workers into shared
+// memory, once and in whole lines, and draws for them in all rounds of its share.  Lanes run over workers first, so
+// that a round's draws leave as segments.  In sorted order the probes of a bisection are a power of two apart, all in
+// one bank (42 us of conflicts and waiting); so every sixteenth threshold is copied into an implicit search tree, level
+// after level (the middle, the quartiles, ...), and only the last four probes go to the row itself.  Rows are filled up
+// to a multiple of sixteen with the top; the last block needs no node, as its last threshold only ever counts for
+// u = 2^32 - 1, where `last` decides all the same.
+constexpr int kSampleThreads = 256;
+__host__ __device__ inline uint32_t sample_levels(uint32_t M) {  // of the tree: 2^levels >= blocks of sixteen
+  uint32_t h = 0;
+  while ((16u << h) < M) ++h;
+  return h;
+}
+// Words between the rows and between the trees of a CTA: rows start in different banks.
+__host__ __device__ inline uint32_t sample_stride(uint32_t M, int rows) { return ((M + 31u) & ~31u) + 32u / rows; }
+__host__ __device__ inline uint32_t sample_tree(uint32_t M, int rows) { return (1u << sample_levels(M)) + 32u / rows; }
+__host__ __device__ inline size_t sample_smem(uint32_t M, int rows) { return (size_t)rows * (sample_stride(M, rows) + sample_tree(M, rows)) * 4u; }
+
+template <int kSampleRows>
+__global__ void __launch_bounds__(kSampleThreads) sample_rows_kernel(const SampleParams p, const uint32_t rounds_per_cta) {
+  extern __shared__ __align__(16) uint32_t s_thr[];
+  const uint32_t M = (uint32_t)p.M, stride = sample_stride(M, kSampleRows), h = sample_levels(M), tree_stride = sample_tree(M, kSampleRows);
+  uint32_t* s_tree = s_thr + kSampleRows * stride;
+  const uint32_t i0 = blockIdx.x * kSampleRows;
+  const uint32_t rows = min((uint32_t)kSampleRows, M - i0);
+  for (uint32_t w = 0; w < rows; ++w) {
+    const uint32_t* src = p.thresholds + (size_t)(i0 + w) * M;
+    uint32_t* dst = s_thr + w * stride;
+    if ((M & 3u) == 0u) {
+      for (uint32_t j = 4u * threadIdx.x; j < M; j += 4u * kSampleThreads) cp_async_16_stream(dst + j, src + j);
+    } else {
+#pragma unroll 8
+      for (uint32_t j = threadIdx.x; j < M; j += kSampleThreads) dst[j] = __ldg(src + j);
+    }
+    for (uint32_t j = M + threadIdx.x; j < ((M + 15u) & ~15u); j += kSampleThreads) dst[j] = 0xFFFFFFFFu;
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  for (uint32_t e = threadIdx.x; e < rows << h; e += kSampleThreads) {
+    const uint32_t w = e >> h, j = e & ((1u << h) - 1u);  // block j - 1 -> node
+    if (j == 0) continue;
+    const uint32_t z = __ffs(j) - 1;
+    s_tree[w * tree_stride + (1u << (h - 1 - z)) + (j >> (z + 1))] = 16u * j <= M ? s_thr[w * stride + 16u * j - 1u] : 0xFFFFFFFFu;
+  }
+  __syncthreads();
+  const uint32_t w = threadIdx.x & (kSampleRows - 1);
+  if (w >= rows) return;
+  const uint32_t i = i0 + w;
+  const uint32_t *row = s_thr + w * stride, *tree = s_tree + w * tree_stride;
+  const int32_t last = __ldg(p.last_nz + i);
+  const uint32_t begin = blockIdx.y * rounds_per_cta, end = min((uint32_t)p.n_rounds, begin + rounds_per_cta);
+  constexpr uint32_t kPerPass = kSampleThreads / kSampleRows;
+  constexpr int kAtOnce = 4;  // draws of a thread in flight: a probe's latency is what a single one waits for
+  for (uint32_t r = begin + threadIdx.x / kSampleRows; r < end; r += kAtOnce * kPerPass) {
+    uint32_t u[kAtOnce], at[kAtOnce];
+#pragma unroll
+    for (int a = 0; a < kAtOnce; ++a) {
+      u[a] = peer_word(p, i, p.first_round + r + a * kPerPass);
+      at[a] = 1;
+    }
+    for (uint32_t l = 0; l < h; ++l) {
+#pragma unroll
+      for (int a = 0; a < kAtOnce; ++a) at[a] = 2u * at[a] + (tree[at[a]] <= u[a] ? 1u : 0u);
+    }
+#pragma unroll
+    for (int a = 0; a < kAtOnce; ++a) at[a] = 16u * (at[a] - (1u << h));  // thresholds of whole blocks <= u
+#pragma unroll
+    for (int s = 8; s > 0; s >>= 1) {
+#pragma unroll
+      for (int a = 0; a < kAtOnce; ++a)
+        if (row[at[a] + s - 1] <= u[a]) at[a] += s;
+    }
+#pragma unroll
+    for (int a = 0; a < kAtOnce; ++a)
+      if (r + a * kPerPass < end) put_draw(p, r + a * kPerPass, i, min((int32_t)at[a], last));
   }
 }
 
@@ -323,19 +421,6 @@ __device__ __forceinline__ void load_draws(const RoundParams& p, const int32_t* 
     s_pw[i] = make_int2(m, __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * p.M + m)));
   }
 }
-
-// 16 bytes from global to shared memory without passing through registers or L1 (data that no other
-// thread of the SM will ask for); completion is awaited by the same thread with cp_async_wait_all.
-__device__ __forceinline__ void cp_async_16_stream(void* smem_dst, const void* gmem_src) {
-  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-// The same for 8 bytes (four bfloat16 values; copies below 16 bytes go through L1).
-__device__ __forceinline__ void cp_async_8(void* smem_dst, const void* gmem_src) {
-  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Loads of replica data.  Inside one launch per round the round-start buffer is read-only
 // (non-coherent path); a launch that runs several rounds reads what other SMs wrote a round

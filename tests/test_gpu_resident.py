@@ -173,3 +173,19 @@ def test_cut_tiles_change_no_bit(nm, M, d, rounds, storage):
     np.testing.assert_allclose(lb, la, rtol=2e-5)
     plain.close()
     res.close()
+
+
+# both samplers (thresholds through the caches, rows in shared memory) around the rule's borders: M not a multiple of
+# four, of sixteen, of the rows of a CTA; rounds that fill no pass; two rows per CTA; a row whose last entries are zero
+@pytest.mark.parametrize("M,rounds", [(127, 1100), (128, 1024), (131, 1001), (1025, 129), (4095, 103), (4096, 70), (5003, 127), (8200, 210)])
+def test_peer_draws_equal_the_oracle(nm, M, rounds):
+    import torch
+    rng = np.random.default_rng(M)
+    P = rng.random((M, M)) + 0.05
+    P[:, M - 5:] *= rng.random((M, 1)) < 0.5           # in half of the rows the last five workers are never drawn
+    P /= P.sum(axis=1, keepdims=True)
+    g = nm.Netmax(M=M, d=8, lr=0.05, prob=P, seed=M, trace_rounds=4)
+    out = torch.full((rounds, M), -1, dtype=torch.int32, device="cuda")
+    g.sample_peers(7, rounds, out.data_ptr())
+    assert (out.cpu().numpy() == oracle.peer_draws(P, M, 7, rounds)).all()
+    g.close()
