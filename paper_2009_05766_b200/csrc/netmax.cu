@@ -10,9 +10,9 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <new>
-#include <queue>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -238,7 +238,7 @@ struct netmax_ctx {
   std::vector<double> pending_duration; // t_im of the pending iteration, under the times it started with
   std::vector<double> finish;
   // pending iterations ordered by (finish time, worker): exactly one entry per worker
-  std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<std::pair<double, int>>> queue;
+  std::vector<std::pair<double, int>> queue;  // a binary heap, the earliest on top
   std::vector<double> ema;
   std::vector<int64_t> ema_count;
   double monitor_period = 0.0, monitor_next = 0.0;  // Network Monitor on the simulated clock (0: off)
@@ -2007,11 +2007,12 @@ int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) {
   ctx->ev_peer.assign(ctx->ev_cap, 0);
   ctx->ev_n.assign(ctx->ev_cap, 0);
   ctx->ev_time.assign(ctx->ev_cap, 0.0);
-  ctx->queue = decltype(ctx->queue)();
+  ctx->queue.clear();
   for (int i = 0; i < M; ++i) {
     async_start_iteration(ctx, i, 0.0);
-    ctx->queue.emplace(ctx->finish[i], i);
+    ctx->queue.emplace_back(ctx->finish[i], i);
   }
+  std::make_heap(ctx->queue.begin(), ctx->queue.end(), std::greater<std::pair<double, int>>());
   return NETMAX_OK;
 }
 
@@ -2067,12 +2068,26 @@ int netmax_async_monitor(netmax_ctx* ctx, double period_s) {
 
 int64_t netmax_async_monitor_refreshes(const netmax_ctx* ctx) { return ctx ? ctx->monitor_refreshes : -1; }
 
-int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
-  if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
-  if (!ctx->async_on) return fail(ctx, NETMAX_INVALID_ARG, "call netmax_async_begin first");
-  if (n_steps < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_steps = %lld < 0", (long long)n_steps);
-  DeviceGuard guard(ctx->device);
-  const int32_t M = ctx->M;
+// Replaces the smallest entry of a binary heap (one way down instead of a pop and a push).
+static void replace_top(std::vector<std::pair<double, int>>& heap, std::pair<double, int> entry) {
+  const size_t n = heap.size();
+  size_t at = 0;
+  for (;;) {
+    size_t child = 2 * at + 1;
+    if (child >= n) break;
+    if (child + 1 < n && heap[child + 1] < heap[child]) ++child;
+    if (!(heap[child] < entry)) break;
+    heap[at] = heap[child];
+    at = child;
+  }
+  heap[at] = entry;
+}
+
+constexpr int64_t kEventsAhead = 4 * kStepTileEvents;
+
+// Consecutive global steps, one launch for as many as touch disjoint replicas.  *used: how many were enqueued -- with
+// more events to come (!last) a launch that could still take some waits for them.
+static int enqueue_disjoint_steps(netmax_ctx* ctx, const StepEvent* events, int64_t n, bool last, int64_t* used) {
   StepKernel kernel = pick_step_kernel(ctx->objective, ctx->L.halves);
   StepParams p;
   p.x = reinterpret_cast<float4*>(ctx->x[ctx->cur]);
@@ -2083,55 +2098,155 @@ int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
   p.alpha = (float)ctx->alpha;
   p.sigma = noise_scale(ctx);
   p.q_offset = ctx->q_offset;
-  p.n_events = 0;
   p.keys = ctx->keys;
-  std::vector<uint8_t> writes(M, 0), reads(M, 0);
-  auto flush = [&]() -> int {
-    if (p.n_events == 0) return NETMAX_OK;
+  std::vector<uint8_t> writes(ctx->M, 0), reads(ctx->M, 0);
+  *used = 0;
+  for (int64_t done = 0; done < n;) {
+    p.n_events = 0;
+    // a step must not write a row that an earlier step of the launch reads or writes, nor read a row that one writes
+    while (done < n && p.n_events < kMaxStepEvents) {
+      const StepEvent& e = events[done];
+      if (writes[e.worker] || reads[e.worker] || writes[e.peer]) break;
+      writes[e.worker] = reads[e.worker] = reads[e.peer] = 1;
+      p.ev[p.n_events++] = e;
+      ++done;
+    }
+    if (!last && done == n && p.n_events < kMaxStepEvents) break;
+    *used = done;
     const int64_t want = (ctx->L.nq + kThreads - 1) / kThreads;
     const int64_t cap = std::max<int64_t>(1, (int64_t)8 * ctx->sm_count / p.n_events);
     dim3 grid((unsigned)std::min<int64_t>(want, cap), (unsigned)p.n_events);
     kernel<<<grid, kThreads, 0, ctx->stream>>>(p);
     ctx->launches += 1;
-    NM_CUDA(ctx, cudaGetLastError());
-    for (int e = 0; e < p.n_events; ++e) {
-      writes[p.ev[e].worker] = 0;
-      reads[p.ev[e].worker] = 0;
-      reads[p.ev[e].peer] = 0;
+    for (int e = 0; e < p.n_events; ++e) writes[p.ev[e].worker] = reads[p.ev[e].worker] = reads[p.ev[e].peer] = 0;
+  }
+  NM_CUDA(ctx, cudaGetLastError());
+  return NETMAX_OK;
+}
+
+using StepTileKernel = void (*)(const StepTileParams);
+static StepTileKernel pick_step_tile_kernel(int objective, int halves) {
+  if (halves == 2) return objective == 1 ? step_tiles_kernel<1, true> : step_tiles_kernel<0, true>;
+  return objective == 1 ? step_tiles_kernel<1, false> : step_tiles_kernel<0, false>;
+}
+
+// Launch shape of step_tiles_kernel, and whether it pays: microseconds of a step in either kernel and of bringing the
+// columns on chip.  A thread takes 32 M bytes of shared memory.  Measured: a step of a column group takes a scheduler
+// 172 cycles with warps enough (8 workers: 12.8 us per step of 11.2 M elements against 27.1) and 480 with a single one
+// (32 workers, 1.5 warps: 4.3 us of 2 M elements against 5.2; 36 workers, one warp: 6.4 by this rule, not taken);
+// step_kernel moves 16 bytes per element at 6.2 TB/s, but a step takes half a microsecond of launches at least.
+struct StepTilePlan {
+  int threads = 0;
+  int64_t per_sm = 0;
+  double tile_us = 0, step_us = 0, load_us = 0;
+  bool pays(int64_t steps) const { return threads > 0 && (double)steps * (step_us - tile_us) > load_us; }
+};
+static StepTilePlan plan_step_tiles(const netmax_ctx* ctx) {
+  StepTilePlan f;
+  const int64_t M = ctx->M, nq = (ctx->d + 3) / 4;
+  const size_t head = step_tile_head(kStepTileEvents, M);
+  int64_t best_warps = 0;
+  for (int threads : {256, 128, 64, 32}) {
+    const size_t smem = head + (size_t)32 * M * threads;
+    if (smem > (size_t)226 * 1024) continue;
+    const int64_t fit = std::min<int64_t>(512 / threads, (int64_t)((size_t)228 * 1024 / (smem + 1024)));
+    // no more warps than the column groups fill; narrow CTAs only where they bring more of them (fewer than four warps
+    // do not spread over the four schedulers by themselves), or where everything is resident in them
+    const int64_t warps = std::min<int64_t>(fit * threads / 32, std::max<int64_t>(1, (nq / 32 + ctx->sm_count - 1) / ctx->sm_count));
+    const bool spread = threads == 32 && (nq + 31) / 32 <= fit * ctx->sm_count;
+    if (warps > best_warps || (spread && warps >= best_warps)) {
+      best_warps = warps;
+      f.threads = threads;
+      f.per_sm = fit;
     }
-    p.n_events = 0;
-    return NETMAX_OK;
+  }
+  if (f.threads == 0) return f;
+  const double items = (double)nq / 32.0 / (4.0 * ctx->sm_count), bytes = (double)ctx->d * ctx->L.elem;
+  f.tile_us = std::max(1.0, items) * std::max(172.0, 480.0 / std::min(1.0 * std::max(1.0, best_warps / 4.0), std::max(1.0, items))) / 1965.0;
+  if (best_warps < 4 && items > 1.0) f.tile_us *= 4.0 / (double)best_warps;  // (schedulers without a warp)
+  f.step_us = std::max(0.5, 4.0 * bytes / 6.2e6);
+  f.load_us = 3.0 + 2.2 * (double)M * bytes / 6.2e6;  // (12 M bytes, a quarter of it beside the steps)
+  return f;
+}
+
+// Enqueues the collected events and takes them out of the list (see enqueue_disjoint_steps).
+static int enqueue_steps(netmax_ctx* ctx, std::vector<StepEvent>& events, const StepTilePlan& plan, bool last) {
+  const int64_t n = (int64_t)events.size();
+  const int threads = plan.threads;
+  int64_t done = 0;
+  if (plan.pays(n)) {
+    StepTileKernel kernel = pick_step_tile_kernel(ctx->objective, ctx->L.halves);
+    StepTileParams p;
+    p.x = reinterpret_cast<char*>(ctx->x[ctx->cur]);
+    p.c = reinterpret_cast<const char*>(ctx->c);
+    p.nq = (ctx->d + 3) / 4;
+    p.n_tiles = (p.nq + threads - 1) / threads;
+    p.row_bytes = (uint32_t)(ctx->L.ld * ctx->L.elem);
+    p.M = ctx->M;
+    p.tail = (int32_t)(ctx->d % 4);
+    p.alpha = (float)ctx->alpha;
+    p.sigma = noise_scale(ctx);
+    p.q_offset = ctx->q_offset;
+    p.keys = ctx->keys;
+    const size_t slabs = (size_t)32 * ctx->M * threads;
+    NM_CUDA(ctx, allow_smem((const void*)kernel, step_tile_head(kStepTileEvents, ctx->M) + slabs));
+    const unsigned grid = (unsigned)std::min<int64_t>(p.n_tiles, plan.per_sm * ctx->sm_count);
+    while (plan.pays(n - done)) {
+      const int64_t launches_left = (n - done + kStepTileEvents - 1) / kStepTileEvents;  // launches of even length
+      p.n_events = (int32_t)((n - done + launches_left - 1) / launches_left);
+      std::memcpy(p.ev, events.data() + done, p.n_events * sizeof(StepEvent));
+      kernel<<<grid, threads, step_tile_head(p.n_events, ctx->M) + slabs, ctx->stream>>>(p);
+      ctx->launches += 1;
+      done += p.n_events;
+    }
+    NM_CUDA(ctx, cudaGetLastError());
+  }
+  int64_t used = 0;
+  const int rc = enqueue_disjoint_steps(ctx, events.data() + done, n - done, last, &used);
+  events.erase(events.begin(), events.begin() + done + used);
+  return rc;
+}
+
+int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
+  if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
+  if (!ctx->async_on) return fail(ctx, NETMAX_INVALID_ARG, "call netmax_async_begin first");
+  if (n_steps < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_steps = %lld < 0", (long long)n_steps);
+  DeviceGuard guard(ctx->device);
+  const int32_t M = ctx->M;
+  // Events are collected and enqueued some hundred at a time: the GPU runs them while the clocks go on.
+  std::vector<StepEvent> events;
+  events.reserve((size_t)std::min<int64_t>(n_steps, kEventsAhead));
+  const StepTilePlan plan = plan_step_tiles(ctx);
+  // (events of single launches go out soon: the host's part is the longer one there)
+  const size_t ahead = plan.pays(kEventsAhead) ? (size_t)kEventsAhead : 8;
+  size_t due = ahead;
+  int64_t ev_slot = ctx->steps % ctx->ev_cap;
+  auto flush = [&](bool last) {
+    const int rc = enqueue_steps(ctx, events, plan, last);
+    due = events.size() + ahead;
+    return rc;
   };
   for (int64_t k = 0; k < n_steps; ++k) {
     // the next global step: the worker whose iteration finishes first (ties: lowest index)
-    const int i = ctx->queue.top().second;
+    const int i = ctx->queue[0].second;
     // the Network Monitor wakes up before any step at or after its next period boundary
     while (ctx->monitor_period > 0.0 && ctx->finish[i] >= ctx->monitor_next) {
-      int rc = flush();
+      int rc = flush(true);
       if (!rc) rc = monitor_refresh(ctx);
       if (rc) return rc;
       ctx->monitor_next += ctx->monitor_period;
     }
     const int m = ctx->pending_peer[i];
-    // a launch holds steps on disjoint replicas only: this one must not write a row that an
-    // earlier step of the launch reads or writes, nor read a row that one writes
-    if (p.n_events == kMaxStepEvents || writes[i] || reads[i] || writes[m]) {
-      int rc = flush();
+    if (events.size() >= due) {
+      int rc = flush(false);
       if (rc) return rc;
     }
     const uint64_t n = (uint64_t)ctx->local_n[i];
-    StepEvent& e = p.ev[p.n_events++];
-    e.worker = i;
-    e.peer = m;
-    e.iter_lo = (uint32_t)n;
-    e.ctr3 = philox_ctr3(kTagNoise, n);
-    e.w = ctx->pending_weight[i];
-    writes[i] = 1;
-    reads[i] = 1;
-    reads[m] = 1;
+    events.push_back(StepEvent{i, m, (uint32_t)n, philox_ctr3(kTagNoise, n), ctx->pending_weight[i]});
     // bookkeeping of Algorithm 2: the clock, the EMA of the iteration time, the next iteration
     ctx->now = ctx->finish[i];
-    const int64_t slot = ctx->steps % ctx->ev_cap;
+    const int64_t slot = ev_slot;
+    ev_slot = ev_slot + 1 == ctx->ev_cap ? 0 : ev_slot + 1;
     ctx->ev_worker[slot] = i;
     ctx->ev_peer[slot] = m;
     ctx->ev_n[slot] = (int64_t)n;
@@ -2142,10 +2257,9 @@ int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
     ctx->local_n[i] += 1;
     ctx->steps += 1;
     async_start_iteration(ctx, i, ctx->now);
-    ctx->queue.pop();
-    ctx->queue.emplace(ctx->finish[i], i);
+    replace_top(ctx->queue, {ctx->finish[i], i});
   }
-  return flush();
+  return flush(true);
 }
 
 int netmax_async_time(netmax_ctx* ctx, double* sim_time, int64_t* steps_done) {

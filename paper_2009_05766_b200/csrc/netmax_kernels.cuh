@@ -1010,6 +1010,114 @@ __global__ void __launch_bounds__(256) step_kernel(const StepParams p) {
   }
 }
 
+// Many consecutive global steps on resident columns: given who acts and whom it pulls from, every column evolves
+// on its own, so a thread that keeps one column group of ALL M rows (replicas, updated in place, and centres: 32 M
+// bytes of shared memory) runs any number of steps on it without a barrier.  step_kernel moves 16 bytes per element
+// and step and is bound by HBM at 27 us per step of 11.2 M elements; here a launch moves 12 M bytes per column
+// element for all of its steps, and the noise (drawn a step ahead) is what takes the time.  Short vectors gain more:
+// one launch for all steps instead of one for every few that touch disjoint replicas.
+constexpr int kStepTileEvents = 160;  // of one launch: they travel as a kernel argument
+struct StepTileParams {
+  char* x;          // replicas, updated in place, row stride row_bytes
+  const char* c;
+  int64_t nq, n_tiles;  // column groups of four elements per row; tiles of blockDim of them
+  uint32_t row_bytes;
+  int32_t M, tail;  // tail = d % 4
+  float alpha, sigma;
+  uint32_t q_offset;
+  int32_t n_events;
+  PhiloxKeys keys;
+  StepEvent ev[kStepTileEvents];
+};
+// Dynamic shared memory: events (offset of the worker's row, of the peer's, weight, iteration) int4[n] and (worker,
+// fourth counter word) uint2[n], what happens to each row (1: written, 2: read), slabs float4[2][M][blockDim].
+__host__ __device__ inline uint32_t step_tile_head(int events, int64_t M) { return (uint32_t)((events * 24 + M + 127) & ~(int64_t)127); }
+
+template <int kObjective, bool kBf16>
+__global__ void __launch_bounds__(256, 2) step_tiles_kernel(const __grid_constant__ StepTileParams p) {
+  constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;
+  constexpr int kAhead = 4;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int tid = threadIdx.x, T = blockDim.x, M = p.M, n = p.n_events;
+  const uint32_t stride = (uint32_t)T * 16u, plane = (uint32_t)M * stride;
+  int4* s_ev = reinterpret_cast<int4*>(smem_raw);
+  uint2* s_ctr = reinterpret_cast<uint2*>(s_ev + n);
+  unsigned char* s_use = smem_raw + (size_t)n * 24;
+  unsigned char* const x = smem_raw + step_tile_head(n, M) + (uint32_t)tid * 16u;  // this thread's column, row i at i * stride
+  unsigned char* const cen = x + plane;
+  for (int i = tid; i < M; i += T) s_use[i] = 0;
+  for (int e = tid; e < n; e += T) {
+    const StepEvent& ev = p.ev[e];
+    s_ev[e] = make_int4((int)((uint32_t)ev.worker * stride), (int)((uint32_t)ev.peer * stride), __float_as_int(ev.w), (int)ev.iter_lo);
+    s_ctr[e] = make_uint2((uint32_t)ev.worker, ev.ctr3);
+  }
+  __syncthreads();
+  for (int e = tid; e < n; e += T) s_use[p.ev[e].peer] = 2;
+  __syncthreads();
+  for (int e = tid; e < n; e += T) s_use[p.ev[e].worker] = 3;
+  __syncthreads();
+
+  for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
+    const int64_t q = tile * T + tid;
+    if (q >= p.nq) continue;  // (threads are independent)
+    char* const xq = p.x + (uint64_t)q * kGroupBytes;
+    const char* const cq = p.c + (uint64_t)q * kGroupBytes;
+#pragma unroll 4
+    for (int i = 0; i < M; ++i) {
+      const int use = s_use[i];
+      const uint64_t at = (uint64_t)(uint32_t)i * p.row_bytes;
+      const uint32_t to = (uint32_t)i * stride;
+      if (kBf16) {
+        if (use & 2) *reinterpret_cast<ulonglong2*>(x + to) = widen_bf16x4(*reinterpret_cast<const unsigned long long*>(xq + at));
+        if (use & 1) *reinterpret_cast<ulonglong2*>(cen + to) = widen_bf16x4(__ldg(reinterpret_cast<const unsigned long long*>(cq + at)));
+      } else {
+        if (use & 2) cp_async_16_stream(x + to, xq + at);
+        if (use & 1) cp_async_16_stream(cen + to, cq + at);
+      }
+    }
+    cp_async_wait_all();
+    const uint32_t q32 = (uint32_t)q + p.q_offset;
+    const int live = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
+    auto draw = [&](int e) {  // event e's noise
+      ulonglong2 v = make_ulonglong2(0ull, 0ull);
+      if (kObjective == 1) {
+        const uint2 ctr = s_ctr[e];
+        v = scaled_normals4(philox4x32_10(q32, ctr.x, (uint32_t)s_ev[e].w, ctr.y, p.keys), p.sigma);
+        if (live < 4) v = mask_lanes(v, live);
+      }
+      return v;
+    };
+    auto step = [&](int e, ulonglong2 noise) {
+      const int4 d = s_ev[e];
+      pair_t ta, tb;
+      const ulonglong2 o = update_core<kObjective>(p.alpha, noise, *reinterpret_cast<const ulonglong2*>(x + (uint32_t)d.x),
+                                                   *reinterpret_cast<const ulonglong2*>(cen + (uint32_t)d.x),
+                                                   *reinterpret_cast<const ulonglong2*>(x + (uint32_t)d.y), __int_as_float(d.z), ta, tb);
+      *reinterpret_cast<ulonglong2*>(x + (uint32_t)d.x) = kBf16 ? widen_bf16x4(narrow_bf16x4(o)) : o;
+    };
+    // The steps depend on one another, their noise does not: it is drawn kAhead events at a time, as many chains of
+    // multiplies and special functions side by side (11.2 M elements: 13.3 us per step with two at a time,
+    // 12.8 with four).
+    int e = 0;
+    for (; e + kAhead <= n; e += kAhead) {
+      ulonglong2 noise[kAhead];
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) noise[a] = draw(e + a);
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) step(e + a, noise[a]);
+    }
+    for (; e < n; ++e) step(e, draw(e));
+#pragma unroll 4
+    for (int i = 0; i < M; ++i) {
+      if (!(s_use[i] & 1)) continue;
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(x + (uint32_t)i * stride);
+      const uint64_t at = (uint64_t)(uint32_t)i * p.row_bytes;
+      if (kBf16) *reinterpret_cast<unsigned long long*>(xq + at) = narrow_bf16x4(v);
+      else *reinterpret_cast<ulonglong2*>(xq + at) = v;
+    }
+  }
+}
+
 // ------------------------------------------------------------------------- init / IO
 struct InitParams {
   float4* dst;  // [M][ldq] column groups

@@ -293,3 +293,27 @@ def test_adaptive_policy_converges_sooner_in_simulated_time(nm):
         t_un, t_ad = time_to(P_un, rho_un, level), time_to(P_ad, rho_ad, level)
         assert np.isfinite(t_un) and np.isfinite(t_ad)
         assert t_un / t_ad > 1.15, (level, t_un, t_ad)
+
+
+# steps of one call on resident columns (launches of at most 160) against the same steps call by call (one launch each):
+# lengths around a launch, ragged tails, one column group, narrow and wide CTAs, the last columns of a partial tile
+@pytest.mark.parametrize("M,d,steps,storage", [(2, 3, 160, "f32"), (3, 8_191, 161, "f32"), (8, 700_003, 321, "bf16"), (8, 1_200_001, 40, "f32"),
+                                               (16, 300_002, 159, "f32"), (40, 50_001, 162, "f32"), (150, 33, 400, "bf16")])
+@pytest.mark.parametrize("objective", [0, 1])
+def test_steps_on_resident_columns_change_no_bit(nm, M, d, steps, storage, objective):
+    rng = np.random.default_rng(M + d)
+    P, t = random_policy(M, rng), random_times(M, rng)
+    kw = dict(M=M, d=d, lr=0.05, prob=P, sigma=0.1, x0_std=1.0, c_std=1.0, objective=objective, seed=d, storage=storage)
+    a, b = nm.Netmax(**kw), nm.Netmax(**kw)
+    a.async_begin(t, beta=0.7)
+    b.async_begin(t, beta=0.7)
+    before = a.kernel_launches
+    a.async_steps(steps)
+    assert a.kernel_launches - before < steps // 4, "the steps did not run on resident columns"
+    for _ in range(steps):
+        b.async_steps(1)
+    assert (a.read_replicas().view(np.uint32) == b.read_replicas().view(np.uint32)).all()
+    for p, q in zip(a.async_trace(), b.async_trace()):
+        assert (p == q).all()
+    a.close()
+    b.close()
