@@ -115,7 +115,7 @@ def lib():
 
 
 def _p(a):
-    return None if a is None else a.ctypes.data_as(C.c_void_p)
+    return None if a is None else a.ctypes.data
 
 
 def _f64(a, shape=None):
@@ -221,6 +221,7 @@ class Netmax:
         self.storage = storage
         self.M, self.d = int(M), int(d)
         self._h = C.c_void_p()
+        self._L = L
         _check(L.netmax_create_ex(C.byref(cfg), C.byref(self._h)))
 
     @staticmethod
@@ -277,8 +278,12 @@ class Netmax:
         self._keep = a
         return _p(a)
 
+    # (the calls a program makes every round or few go to the library without detours: marshalling was a third of a
+    # small one)
     def round(self, n_rounds: int = 1):
-        _check(lib().netmax_round(self._h, int(n_rounds)), self._h)
+        code = self._L.netmax_round(self._h, int(n_rounds))
+        if code:
+            _check(code, self._h)
 
     def round_from_host(self, x, c, n_rounds: int, out, n_chunks: int = 0):
         """netmax_round_from_host: x, c, out are numpy arrays (M, d) float32 or host pointers (int); x and c may be None."""
@@ -298,14 +303,16 @@ class Netmax:
 
     @property
     def rounds_done(self) -> int:
-        return int(lib().netmax_rounds_done(self._h))
+        return self._L.netmax_rounds_done(self._h)
 
     def read_replicas(self, out=None):
         if isinstance(out, int):
             _check(lib().netmax_read_replicas(self._h, C.c_void_p(out)), self._h)
             return None
         out = np.empty((self.M, self.d), dtype=np.float32) if out is None else out
-        _check(lib().netmax_read_replicas(self._h, _p(out)), self._h)
+        code = self._L.netmax_read_replicas(self._h, out.ctypes.data)
+        if code:
+            _check(code, self._h)
         return out
 
     def read_centres(self):
@@ -331,16 +338,20 @@ class Netmax:
         first_round = self.first_round if first_round is None else first_round
         n = self.rounds_done - first_round if n is None else n
         out = np.empty((n, self.M), dtype=np.int32)
-        _check(lib().netmax_peer_trace(self._h, int(first_round), int(n), _p(out)), self._h)
+        code = self._L.netmax_peer_trace(self._h, int(first_round), int(n), out.ctypes.data)
+        if code:
+            _check(code, self._h)
         return out
 
     def telemetry(self, first_round: Optional[int] = None, n: Optional[int] = None):
         first_round = self.first_round if first_round is None else first_round
         n = self.rounds_done - first_round if n is None else n
-        cons = np.empty(n, dtype=np.float64)
-        loss = np.empty(n, dtype=np.float64)
-        _check(lib().netmax_telemetry(self._h, int(first_round), int(n), _p(cons), _p(loss)), self._h)
-        return cons, loss
+        both = np.empty((2, n), dtype=np.float64)
+        at = both.ctypes.data
+        code = self._L.netmax_telemetry(self._h, int(first_round), int(n), at, at + 8 * int(n))
+        if code:
+            _check(code, self._h)
+        return both[0], both[1]
 
     def replicas_device(self):
         ptr, ld = C.c_void_p(), C.c_int64()

@@ -202,6 +202,8 @@ struct netmax_ctx {
   unsigned char* base = nullptr;
   unsigned char* pinned = nullptr;  // block of the pinned pool: see kPinnedTel and the rest
   bool host_writes = false;         // launches that may still write to `pinned` have been enqueued since the last synchronisation
+  bool read_since_round = false;    // netmax_read_replicas has been called since the last netmax_round
+  bool staged = false;              // the staging area holds, or is about to hold, the current replicas
   int32_t* trace_mirror = nullptr;  // host copy of the trace ring, written by the sampler (small rings only)
   int storage = NETMAX_STORAGE_F32;
   unsigned char *x[2] = {nullptr, nullptr}, *c = nullptr;  // [M][ld] fp32 or bfloat16, as `storage` says
@@ -991,15 +993,34 @@ struct ColumnRange {
   bool whole = true;        // the whole vector (the only form bfloat16 state takes)
 };
 
+// Launches a kernel that waits for its predecessor itself (wait_for_previous), so that its own start-up runs beside the
+// predecessor's end: of the two short kernels of a small call the second one's launch is what is saved.
+template <typename Params>
+cudaError_t launch_behind_sampler(void (*kernel)(const Params), unsigned grid, int threads, size_t smem, cudaStream_t stream,
+                                  const Params& p) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
 // One launch of tile_rounds_kernel: `chunk` rounds from round r over a column range; the telemetry of its
 // rounds is added up by the last CTA (finalize), or by a launch of its own when there are many rounds.
 int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, const RoundParams& p, const ColumnRange& range,
                  const unsigned char* xin, unsigned char* xout, const unsigned char* cbase, double* tel, uint64_t r, int chunk,
-                 bool finalize) {
+                 bool finalize, unsigned char* mirror) {
   TileParams tp;
   tp.x_cur = reinterpret_cast<const char*>(xin);
   tp.x_nxt = reinterpret_cast<char*>(xout);
   tp.c = reinterpret_cast<const char*>(cbase);
+  tp.mirror = reinterpret_cast<char*>(mirror);
   tp.draws = ctx->draws;
   tp.partials = reinterpret_cast<double*>(ctx->colpart);
   tp.tel = tel;
@@ -1038,7 +1059,7 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
     void* args[] = {&tp};
     NM_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k, dim3((unsigned)grid), dim3((unsigned)tiles.threads), args, tiles.smem, stream));
   } else {
-    k<<<(unsigned)grid, tiles.threads, tiles.smem, stream>>>(tp);
+    NM_CUDA(ctx, launch_behind_sampler(k, (unsigned)grid, tiles.threads, tiles.smem, stream, tp));
   }
   ctx->launches += 1;
   if (!finalize) {
@@ -1077,7 +1098,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
     if (tiles.ok && n >= tiles.min_rounds && n - b >= 2) {
       const int64_t launches_left = (n - b + tiles.max_rounds - 1) / tiles.max_rounds;
       const int64_t chunk = (n - b + launches_left - 1) / launches_left;
-      int rc = launch_tiles(ctx, stream, tiles, p, range, xin, xout, cbase, tel, r, (int)chunk, true);
+      int rc = launch_tiles(ctx, stream, tiles, p, range, xin, xout, cbase, tel, r, (int)chunk, true, nullptr);
       if (rc) return rc;
       cur ^= 1;
       r += (uint64_t)chunk;
@@ -1128,7 +1149,8 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
     p.tel_out = tel + 2 * slot;
     p.round_lo = (uint32_t)r;
     p.ctr3 = philox_ctr3(kTagNoise, r);
-    kernel<<<round_grid, kThreads, plan.smem, stream>>>(p);
+    if (plan.short_vectors) NM_CUDA(ctx, launch_behind_sampler(kernel, (unsigned)round_grid, kThreads, plan.smem, stream, p));
+    else kernel<<<round_grid, kThreads, plan.smem, stream>>>(p);
     ctx->launches += 1;
     cur ^= 1;
     r += 1;
@@ -1429,7 +1451,11 @@ int netmax_get_policy(netmax_ctx* ctx, double* prob_out, double* rho_out) {
 
 // Waits for the context's stream; reports a bounded wait of a kernel that has given up since the last check.
 static int synchronise(netmax_ctx* ctx) {
-  NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  // (an idle stream, as after another read, answers a query sooner than a wait)
+  if (cudaStreamQuery(ctx->stream) != cudaSuccess) {
+    cudaGetLastError();
+    NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  }
   ctx->host_writes = false;
   if (*ctx->dev_error == 0u) return NETMAX_OK;
   *ctx->dev_error = 0u;
@@ -1441,6 +1467,7 @@ static int synchronise(netmax_ctx* ctx) {
 static int read_back(netmax_ctx* ctx, void* host, const void* dev, size_t bytes) {
   const bool staged = bytes <= kStagingBytes;
   unsigned char* stage = ctx->pinned + kPinnedStaging;
+  if (staged) ctx->staged = false;
   NM_CUDA(ctx, cudaMemcpyAsync(staged ? stage : host, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
   int rc = synchronise(ctx);
   if (rc) return rc;
@@ -1502,6 +1529,7 @@ static int copy_out(netmax_ctx* ctx, const unsigned char* src, float* host) {
   }
   if (ctx->L.ld == ctx->d) return read_back(ctx, host, src, ctx->L.plane);
   if (ctx->L.plane <= kStagingBytes) {  // the padded rows as they are, taken apart on the host
+    ctx->staged = false;
     NM_CUDA(ctx, cudaMemcpyAsync(ctx->pinned + kPinnedStaging, src, ctx->L.plane, cudaMemcpyDeviceToHost, ctx->stream));
     int rc = synchronise(ctx);
     if (rc) return rc;
@@ -1514,9 +1542,24 @@ static int copy_out(netmax_ctx* ctx, const unsigned char* src, float* host) {
   return synchronise(ctx);
 }
 
-int netmax_set_replicas(netmax_ctx* ctx, const float* host_x) { return copy_in(ctx, ctx ? ctx->x[ctx->cur] : nullptr, host_x); }
+int netmax_set_replicas(netmax_ctx* ctx, const float* host_x) {
+  if (ctx) ctx->staged = false;
+  return copy_in(ctx, ctx ? ctx->x[ctx->cur] : nullptr, host_x);
+}
 int netmax_set_centres(netmax_ctx* ctx, const float* host_c) { return copy_in(ctx, ctx ? ctx->c : nullptr, host_c); }
-int netmax_read_replicas(netmax_ctx* ctx, float* host_out) { return copy_out(ctx, ctx ? ctx->x[ctx->cur] : nullptr, host_out); }
+int netmax_read_replicas(netmax_ctx* ctx, float* host_out) {
+  if (ctx) ctx->read_since_round = true;
+  if (ctx && host_out && ctx->staged) {  // on its way since netmax_round; good for one read
+    ctx->staged = false;
+    DeviceGuard guard(ctx->device);
+    const int rc = synchronise(ctx);
+    if (rc) return rc;
+    const float* rows = reinterpret_cast<const float*>(ctx->pinned + kPinnedStaging);
+    for (int64_t i = 0; i < ctx->M; ++i) std::memcpy(host_out + i * ctx->d, rows + i * ctx->L.ld, (size_t)ctx->d * sizeof(float));
+    return NETMAX_OK;
+  }
+  return copy_out(ctx, ctx ? ctx->x[ctx->cur] : nullptr, host_out);
+}
 int netmax_read_centres(netmax_ctx* ctx, float* host_out) { return copy_out(ctx, ctx ? ctx->c : nullptr, host_out); }
 
 int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
@@ -1530,6 +1573,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
   int rc = plan_round(ctx, plan, ctx->objective);
   if (rc) return rc;
   ctx->host_writes = true;
+  ctx->staged = false;
   FusedPlan fused;
   rc = plan_fused(ctx, plan, fused);
   if (rc) return rc;
@@ -1539,6 +1583,11 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
 
   RoundParams p = make_round_params(ctx, plan);
 
+  // A program that reads small replicas after every call gets them with the rounds: the last launch writes them to
+  // the page-locked staging area as well (4 x 4096 elements: a copy and a wait of their own were 15 of 45 us).
+  unsigned char* mirror = ctx->read_since_round && ctx->storage == NETMAX_STORAGE_F32 && ctx->L.plane <= kStagingBytes
+                              ? ctx->pinned + kPinnedStaging : nullptr;
+  bool mirrored = false;
   int64_t done = 0;
   while (done < n_rounds) {
     // peers of a batch of rounds in one launch (counter-based draws do not depend on x),
@@ -1555,8 +1604,9 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
       for (int64_t b = 0; b < batch;) {
         const int64_t chunk = std::min<int64_t>(batch - b, tiles.max_rounds);
         rc = launch_tiles(ctx, ctx->stream, tiles, p, all, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], ctx->c, ctx->tel,
-                          (uint64_t)ctx->rounds, (int)chunk, false);
+                          (uint64_t)ctx->rounds, (int)chunk, false, done + b + chunk == n_rounds ? mirror : nullptr);
         if (rc) return rc;
+        mirrored = true;
         ctx->cur ^= 1;
         ctx->rounds += chunk;
         b += chunk;
@@ -1605,6 +1655,10 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
       all.tail4 = (int32_t)(ctx->d % 4);
       all.whole = true;
       int cur = ctx->cur;
+      // (the short-vector kernel mirrors a batch of one round; it is the only one that runs here on so few elements)
+      const bool one = plan.short_vectors && batch == 1 && done + batch == n_rounds;
+      p.mirror = one ? reinterpret_cast<char*>(mirror) : nullptr;
+      mirrored = one;
       rc = launch_long_rounds(ctx, ctx->stream, plan, fused, tiles, p, all, ctx->tel, (uint64_t)ctx->rounds, batch, cur);
       if (rc) return rc;
       ctx->cur = cur;
@@ -1613,6 +1667,8 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
     NM_CUDA(ctx, cudaGetLastError());
     done += batch;
   }
+  ctx->staged = mirror != nullptr && mirrored;
+  ctx->read_since_round = false;
   return NETMAX_OK;
 }
 
@@ -1680,6 +1736,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
 
   const uint64_t first = (uint64_t)ctx->rounds;
   ctx->host_writes = true;
+  ctx->staged = false;
   rc = launch_sampler(ctx, first, n_rounds, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds, ctx->trace_rounds);
   if (rc) return bail(rc);
   // uploads must not overtake earlier work of the context that still reads the buffers
@@ -2210,6 +2267,7 @@ static int enqueue_steps(netmax_ctx* ctx, std::vector<StepEvent>& events, const 
 int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!ctx->async_on) return fail(ctx, NETMAX_INVALID_ARG, "call netmax_async_begin first");
+  ctx->staged = false;
   if (n_steps < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_steps = %lld < 0", (long long)n_steps);
   DeviceGuard guard(ctx->device);
   const int32_t M = ctx->M;

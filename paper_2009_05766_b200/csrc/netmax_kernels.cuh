@@ -41,6 +41,11 @@ __device__ __forceinline__ void cp_async_8(void* smem_dst, const void* gmem_src)
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Programmatic dependent launch: the sampler lets the kernel behind it start at once; that kernel waits here for the
+// sampler to end and its writes to be visible (no-ops where a launch does not ask for it).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------- sampler
 struct SampleParams {
   const uint32_t* thresholds;  // [M][M] non-decreasing per row
@@ -71,6 +76,7 @@ __device__ __forceinline__ void put_draw(const SampleParams& p, uint32_t r, uint
 // m = min(#{j : T[j] <= u}, last_nz): the count is found by bisection (T is sorted).  One thread per draw,
 // thresholds through the caches: for few rounds or few workers.  At most 2^31 draws per launch.
 __global__ void __launch_bounds__(256) sample_peers_kernel(const SampleParams p) {
+  launch_dependents();
   const uint32_t M = (uint32_t)p.M, total = (uint32_t)p.n_rounds * M;
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
     const uint32_t r = idx / M, i = idx - r * M;
@@ -168,6 +174,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_rows_kernel(const Sampl
 struct RoundParams {
   const float4* x_cur;   // [M][ldq] round-start replicas (16-byte column groups: 4 fp32 or 8 bfloat16)
   float4* x_nxt;         // [M][ldq] next replicas
+  char* mirror;          // copy of x_nxt in page-locked host memory (short-vector kernel only); may be NULL
   const float4* c;       // [M][ldq] centres
   const int32_t* peers;  // [M] this round's draws
   const float* wtab;     // [M][M] pull weights w_im (fp32)
@@ -510,6 +517,8 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
               else o.y = narrow_bf16x4(oh);
             }
             if (kObjective != 2) *reinterpret_cast<ulonglong2*>(oq + (uint64_t)(uint32_t)i * p.row_bytes) = o;
+            if (kRowsInFlight != 1 && !kCoherent && kObjective != 2 && p.mirror)
+              *reinterpret_cast<ulonglong2*>(p.mirror + (uint64_t)q * 16u + (uint64_t)(uint32_t)i * p.row_bytes) = o;
           }
         }
       }
@@ -595,6 +604,7 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
 template <int kObjective, int kRowsInFlight, int kHalves>
 __global__ void __launch_bounds__(256, kRowsInFlight != 1 ? 2 : kHalves == 1 ? NETMAX_ROUND_MIN_CTAS : NETMAX_ROUND_MIN_CTAS_BF16)
     round_kernel(const RoundParams p) {
+  if (kRowsInFlight != 1) wait_for_previous();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   int2* s_pw = reinterpret_cast<int2*>(smem_raw);  // (peer, bits of the pull weight) per worker
   const size_t head = (((size_t)p.M * 8) + 15) & ~(size_t)15;

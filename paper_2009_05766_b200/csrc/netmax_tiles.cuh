@@ -45,6 +45,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, unsigne
 struct TileParams {
   const char* x_cur;      // replicas at the start of the first round, row stride row_bytes
   char* x_nxt;            // replicas after the last round
+  char* mirror;           // copy of them in page-locked host memory (fp32 state); may be NULL
   const char* c;
   const int2* draws;      // ring of (peer, bits of the pull weight), [ring][M]
   double* partials;       // [n_rounds][gridDim.x][2]: telemetry shares of every CTA
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
   float2* const s_two = reinterpret_cast<float2*>(s_sum + kBuffers * E);      // [kBuffers][E]
   const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_bar);
   if (tid == 0) mbar_init(bar, (uint32_t)nwarps);
+  wait_for_previous();
   __syncthreads();
 
   int2 draw[kRows], draw_far[kFar ? kRows : 1];
@@ -296,6 +298,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
         const unsigned char* cur = col + cur_off;
         const ulonglong2 pivot = *reinterpret_cast<const ulonglong2*>(cur);  // row 0
         char* oq = p.x_nxt + (uint64_t)q * kGroupBytes + row_first;
+        char* mq = !kBf16 && kLast && p.mirror && pc.k1 == p.n_rounds ? p.mirror + (uint64_t)q * kGroupBytes + row_first : nullptr;
         rows([&](int j) {
           unsigned char* sx = own + (uint32_t)j * step;
           const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sx + cur_off);
@@ -305,6 +308,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
           if (kLast) {
             if (kBf16) *reinterpret_cast<unsigned long long*>(oq + j * row_step) = narrow_bf16x4(o);
             else *reinterpret_cast<ulonglong2*>(oq + j * row_step) = o;
+            if (!kBf16 && mq) *reinterpret_cast<ulonglong2*>(mq + j * row_step) = o;
           } else {
             *reinterpret_cast<ulonglong2*>(sx + nxt_off) = kBf16 ? widen_bf16x4(narrow_bf16x4(o)) : o;
           }
