@@ -194,7 +194,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds);
  * resulting replicas to host_out -- what netmax_set_replicas, netmax_set_centres, netmax_round and
  * netmax_read_replicas do one after the other, with the same replicas, peer trace, telemetry and
  * round counter bit for bit.  Given the draws, Eq. 15-16 act on every column separately, so the work
- * is cut into n_chunks column ranges (0: automatic; at most 32) and pipelined: while the rounds of
+ * is cut into n_chunks column ranges (0: automatic: 2, 4 or 8 by size; at most 32) and pipelined: while the rounds of
  * one range run on the context's stream, the next range is uploaded and the previous one downloaded
  * on two streams of the library's own.  All arrays are dense M*d floats on the host; pinned memory
  * lets the copies overlap.  Ranges are pipelined for fp32 state, long vectors and

@@ -1688,7 +1688,10 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   if (rc) return rc;
   const int64_t nq4 = (ctx->d + 3) / 4;
   const int64_t unit = 256;  // chunk boundaries on 4 KB of every row
-  int chunks = n_chunks > 0 ? n_chunks : 8;
+  // More chunks hide more of the first upload and the last download, but every chunk has launches and copies of its own
+  // (upload of 12.8 MB: 0.37 ms with two, 0.43 with eight; 128 MB: 2.86 with four, 2.88 with eight; 715 MB: 15.1 / 14.6).
+  const int64_t upload = 8 * (int64_t)ctx->M * ctx->d;
+  int chunks = n_chunks > 0 ? n_chunks : upload <= ((int64_t)20 << 20) ? 2 : upload <= ((int64_t)200 << 20) ? 4 : 8;
   chunks = (int)std::min<int64_t>(chunks, (nq4 + unit - 1) / unit);
   const bool pipelined = ctx->storage == NETMAX_STORAGE_F32 && !plan.short_vectors && n_rounds >= 1 &&
                          n_rounds <= ctx->trace_rounds && chunks >= 2 &&
