@@ -8,8 +8,8 @@ pulls from the peer's round-start replica, over all M x d elements.  The metric 
 GB/s = 16 bytes x M x d x rounds / time (reads of x_i, x_peer and c_i plus the write of x_i',
 4 bytes each).  One JSON line is printed by rank 0.
 
-The library advances up to eight rounds per launch where all M rows of a column tile fit in
-shared memory (one CTA's up to 36 workers; four rounds over a thread-block cluster's beyond); that launch
+The library advances many rounds per launch where all M rows of a column tile fit in shared memory
+(a column per thread up to 36 workers, the rows shared out over the threads beyond); that launch
 is bound by instruction issue, not by HBM,
 and the line's `roofline` says so.  The same workload with one launch per round (the HBM-bound
 kernel) is timed as well and reported under `one_launch_per_round`.
@@ -47,36 +47,34 @@ UNIQUE_FRACTION = 0.75          # x_peer is a row the same tile reads anyway (a 
                                 # bytes (6 of 8) have to cross the DRAM pins, and the HBM roofline is taken against those
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0
-KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_rng.cuh")
+KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh")
 # Counters of one launch, from ncu captures of this file's own commands (see profiles/): DRAM bytes
 # (dram__bytes_read.sum + dram__bytes_write.sum) per element of the launch and warp instructions
 # (smsp__inst_executed.sum) per element and round.  Captured on the workload itself where that is small
 # enough to profile, else on the same M and tile shape with a shorter vector (`captured_on`); bytes and
 # instructions per element are what carries over.  Only reported while the kernel sources still hash to
 # the value the capture was taken at.
-NCU_HASH = "f3a1fa0b6db6c040"
+NCU_HASH = "e65debb22b22f859"
 NCU_COUNTERS = {
     # (workload tag, kernel): dram bytes per element-launch, warp instructions per element-round, captured on
-    ("cfg2_M8_resnet18", "round_kernel"): (1_041_843_000 / 89_391_696, 78_504_733 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_041_110_000 / 89_391_696, 612_995_880 / (89_391_696 * 8), "cfg2"),
-    ("cfg2_M8_resnet18/bf16", "round_kernel"): (507_135_000 / 89_391_696, 85_164_099 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (505_620_000 / 89_391_696, 660_744_326 / (89_391_696 * 8), "cfg2"),
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (3_805_327_000 / 320_000_000, 2_031_045_889 / (320_000_000 * 8), "cfg3"),
-    ("cfg3_M16_vgg19scale", "round_kernel"): (1_543_966_000 / (16 * 8_000_002), 101_887_293 / (16 * 8_000_002), "cfg3 at d = 8,000,002"),
-    ("cfg4_M64_resnet18", "cluster_rounds_kernel"): (1_503_694_000 / (64 * 2_000_002), 524_126_023 / (64 * 2_000_002 * 4), "cfg4 at d = 2,000,002"),
-    ("cfg4_M64_resnet18", "round_kernel"): (1_545_154_000 / (64 * 2_000_002), 104_626_918 / (64 * 2_000_002), "cfg4 at d = 2,000,002"),
-    ("cfg1_M4_d4096", "resident_rounds_kernel"): (None, 49_802_752 / (16_384 * 1024), "cfg1"),
-    ("cfg5_M4096_sampling", "resident_rounds_kernel"): (None, 5_822_930_304 / (4_194_304 * 1024), "cfg5"),
+    # (the per-round kernel's bytes on cfg2 are an earlier capture's; the latest one read 1,046,194,000)
+    ("cfg2_M8_resnet18", "round_kernel"): (1_041_843_000 / 89_391_696, 85_571_066 / 89_391_696, "cfg2"),
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_042_876_000 / 89_391_696, 670_157_455 / (89_391_696 * 8), "cfg2"),
+    ("cfg2_M8_resnet18/bf16", "round_kernel"): (507_162_000 / 89_391_696, 88_428_295 / 89_391_696, "cfg2"),
+    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (507_691_000 / 89_391_696, 722_424_204 / (89_391_696 * 8), "cfg2"),
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (1_502_230_000 / (16 * 8_000_002), 881_740_913 / (16 * 8_000_002 * 8), "cfg3 at d = 8,000,002"),
+    ("cfg3_M16_vgg19scale", "round_kernel"): (1_567_855_000 / (16 * 8_000_002), 111_945_198 / (16 * 8_000_002), "cfg3 at d = 8,000,002"),
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): (1_507_134_000 / (64 * 2_000_002), 1_239_779_448 / (64 * 2_000_002 * 10), "cfg4 at d = 2,000,002"),
+    ("cfg4_M64_resnet18", "round_kernel"): (1_557_018_000 / (64 * 2_000_002), 114_685_198 / (64 * 2_000_002), "cfg4 at d = 2,000,002"),
+    ("cfg1_M4_d4096", "tile_rounds_kernel"): (None, 31_031_584 / (16_384 * 1000), "cfg1"),
+    ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_729_561_508 / (4_194_304 * 1000), "cfg5"),
 }
-# Busy fractions (of active SM cycles) of the issue slots and of the arithmetic pipes, from the same captures on
-# shorter vectors of the same M: which unit a launch that is bound by instruction issue leans on hardest.
+# Busy fractions (of active SM cycles) of the issue slots and of the arithmetic pipes, from the same captures:
+# which unit a launch that is bound by instruction issue leans on hardest.
 NCU_PIPES = {
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.600, "fmaheavy": 0.657, "fmalite": 0.296, "alu": 0.370,
-                                                   "captured_on": "cfg2 at d = 4,000,002"},
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.557, "fmaheavy": 0.639, "fmalite": 0.292, "alu": 0.345,
-                                                      "captured_on": "cfg3 at d = 8,000,002"},
-    ("cfg4_M64_resnet18", "cluster_rounds_kernel"): {"issue": 0.486, "fmaheavy": 0.499, "fmalite": 0.197, "alu": 0.339,
-                                                      "captured_on": "cfg4 at d = 2,000,002"},
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.637, "fmaheavy": 0.643, "alu": 0.422, "captured_on": "cfg2"},
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.583, "fmaheavy": 0.620, "alu": 0.381, "captured_on": "cfg3 at d = 8,000,002"},
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.587, "fmaheavy": 0.628, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
 }
 SM_COUNT, SCHEDULERS_PER_SM = 148, 4     # one warp instruction per scheduler and clock at most
 
@@ -333,11 +331,9 @@ def launch_shape(g, rounds, ring):
     before = g.kernel_launches
     g.round(rounds)
     per = rounds / max(1, g.kernel_launches - before - (rounds + ring - 1) // ring)      # sampler launches excluded
-    if per > 8.5 or (per > 1.5 and g.M * g.d < (1 << 23)):      # (short vectors never take the tile-resident shapes)
-        return "all rounds of a call on shared-memory-resident columns", "resident_rounds_kernel", per
     if per > 1.5:
-        if g.M > 36:        # more rows than one CTA's slabs hold: the tile is resident across a cluster of CTAs
-            return "%d rounds per launch over tiles resident across a thread-block cluster" % round(per), "cluster_rounds_kernel", per
+        if g.M * g.d < (1 << 23) or g.M > 36 or per > 32.5:     # rows shared out over a CTA's threads
+            return "%d rounds per launch over tiles with the rows shared out over the threads" % round(per), "tile_rounds_kernel", per
         return "%d rounds per launch over resident tiles" % round(per), "fused_rounds_kernel", per
     return "one launch per round", "round_kernel", per
 
@@ -384,7 +380,7 @@ def measure_config(torch, binding, wk, args, local, timer, peak, peak_kind, sm_m
     timer.stop.synchronize()
     entry["sampler_only_draws_per_s"] = 10 * batch * wk.M / (timer.start.elapsed_time(timer.stop) / 1e3)
     del draws
-    if kernel in ("fused_rounds_kernel", "cluster_rounds_kernel"):
+    if kernel != "round_kernel" and elements > 1 << 22:
         g.set_fuse_rounds(1)
         g.round(20)
         one = min(timer.repeats(g, rounds, 3))
@@ -464,8 +460,8 @@ def run_ours(args, w):
     value = bytes_per_element * elements * world * args.steps / sec / 1e9
 
     rounds_per_launch = args.steps / max(1, launches - (args.steps + ring - 1) // ring)   # sampler launches excluded
-    resident = rounds_per_launch > 8.5 or (rounds_per_launch > 1.5 and elements < (1 << 23))   # short vectors: all rounds
-    fused = rounds_per_launch > 1.5 and not resident                                          # of a call on resident columns
+    resident = rounds_per_launch > 1.5 and elements < (1 << 23)      # short vectors: all rounds of a call on resident columns
+    fused = rounds_per_launch > 1.5 and not resident
     single_ms = None
     if fused:                       # the same rounds, one launch each: the HBM-bound kernel
         g.set_fuse_rounds(1)
@@ -535,8 +531,8 @@ def run_ours(args, w):
     tag = w.name + ("/bf16" if bf16 else "")
     sm_max_mhz = clocks.summary()["sm_max_mhz"]
     if fused or resident:
-        kernel = (("cluster_rounds_kernel" if w.M > 36 else "fused_rounds_kernel") if fused else
-                  ("multi_round_kernel" if args.fuse_rounds == 1 else "resident_rounds_kernel"))
+        kernel = (("tile_rounds_kernel" if w.M > 36 else "fused_rounds_kernel") if fused else
+                  ("multi_round_kernel" if args.fuse_rounds == 1 else "tile_rounds_kernel"))
         roofline = issue_roofline(tag, kernel, per_round_ms, elements, bytes_per_element, rounds_per_launch, sm_max_mhz,
                                   peak, peak_kind)
     else:
@@ -654,6 +650,8 @@ def run_async(args, w):
         "simulated_seconds": sim_time,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": None, "peak_kind": f"of {peak_kind}", "kernel": "step_kernel",
+                     "note": "achieved counts step_kernel's 16 bytes per element and step; up to 160 steps per launch run on resident "
+                             "columns (step_tiles_kernel) where that pays, and move far fewer",
                      "bytes_per_launch": bytes_per_element * w.d * args.steps / max(launches, 1)},
         "gpu_launches": int(launches), "clocks": clocks.summary(),
         "telemetry_now": {"consensus": cons, "loss": loss},
