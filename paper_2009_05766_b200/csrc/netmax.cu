@@ -860,8 +860,8 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
     f.min_rounds = 2;
     f.max_rounds = std::min<int64_t>(f.max_rounds, ctx->fuse_rounds);
   } else {
-    // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the
-    // worker counts for which the header has always said so; longer ones are where resident tiles gain most.
+    // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the worker
+    // counts the header says so for; longer ones are where resident tiles gain most.
     static const unsigned char fused_short[22] = {0, 1, 1, 1, 0, 1, 1, 1, 1, 1, 1, 0, 0, 1, 0, 0, 0, 1, 1, 1, 1, 1};  // M = 67 ... 88
     const bool short_calls = !f32 || M <= 66 || (M <= 88 && fused_short[M - 67]);
     f.min_rounds = short_calls ? 2 : 9;
@@ -897,10 +897,9 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   // and the kernel's ~100 registers cap an SM at 16 warps (capping it at 96 or 80 registers for
   // 18-20 warps measured slower: 135 and 157 us against 128 per cfg2 round).  Beyond 18 workers only
   // 64-thread CTAs fit, three per SM up to M = 24 and two up to M = 36: four to six warps per SM, and
-  // still 9 to 21 % faster than the same rows split over a cluster (M x 4,000,002 elements, us per round:
+  // faster than one launch per round (M x 4,000,002 elements, us per round, against rows over a cluster of CTAs:
   // M = 20: 132 against 144, 28: 182 against 214, 36: 227 against 287) -- no barrier, no pull that leaves
-  // the CTA.  A single such CTA per SM (M = 37 ... 73) is slower than the cluster shape (M = 40: 330
-  // against 309), so the kernel is used down to 128 threads per SM.
+  // the CTA.  A single such CTA per SM (M = 37 ... 73) is slower (M = 40: 330 against 309), so the kernel is used down to 128 threads per SM.
   FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves);
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   // The head of the shared memory (draws and telemetry sums) grows with the rounds of a launch: room for as
@@ -1073,8 +1072,8 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
 }
 
 // Enqueues rounds [first, first + n) -- their draws are in the trace ring -- for one column range on
-// `stream`: up to four rounds per launch where tiles stay resident (fused_rounds_kernel, or
-// cluster_rounds_kernel for more workers), else one launch per round.  `cur` is the buffer that holds
+// `stream`: many rounds per launch where tiles stay resident (fused_rounds_kernel, or
+// tile_rounds_kernel for more workers), else one launch per round.  `cur` is the buffer that holds
 // the range's values at round `first`; it is flipped launch by launch.  Telemetry of the range goes
 // to tel (ring-indexed like the context's).
 int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& plan, const FusedPlan& fused,
@@ -1648,7 +1647,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
       done += batch;
       continue;
     }
-    {  // long vectors: fused, cluster-resident or one launch per round, over all columns
+    {  // long vectors: resident tiles or one launch per round, over all columns
       ColumnRange all;
       all.q0 = 0;
       all.nq4 = (ctx->d + 3) / 4;

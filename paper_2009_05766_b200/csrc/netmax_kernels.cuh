@@ -1,16 +1,18 @@
 // CUDA kernels of the NetMax round simulator (sm_100a).
 //
 //   sample_peers_kernel   Algorithm 2, peer selection: one Philox draw per (round, worker)
-//                         searched in that worker's row of 32-bit cumulative thresholds.
+//                         searched in that worker's row of 32-bit cumulative thresholds
+//                         (sample_rows_kernel: many rounds of many workers).
 //   round_kernel          Eq. 15 (local SGD step with inline Gaussian gradient noise) fused
 //                         with Eq. 16 (pull from the round-start snapshot of the peer) and
 //                         with the round's telemetry; reads one buffer, writes the other.
-//   fused_rounds_kernel   the same for up to four rounds per launch on tiles that stay in a
-//                         CTA's shared memory (long vectors, up to 36 workers).
-//   cluster_rounds_kernel the same with the rows of a tile split over the CTAs of a thread-block
-//                         cluster, pulls through distributed shared memory (up to 144 workers).
-//   resident_rounds_kernel, multi_round_kernel   short vectors: all rounds of a call in one launch.
-//   step_kernel           the asynchronous timeline: one worker per global step (Eq. 17).
+//   fused_rounds_kernel   the same for many rounds per launch on tiles that stay in a CTA's shared
+//                         memory, a column per thread (long vectors, up to 36 workers).
+//   tile_rounds_kernel    (netmax_tiles.cuh) the same with the rows of a tile shared out over the
+//                         threads: more workers, and short vectors.
+//   multi_round_kernel    short vectors of more workers than fit on chip: all rounds in one launch.
+//   step_kernel           the asynchronous timeline: one worker per global step (Eq. 17);
+//                         step_tiles_kernel: many steps per launch on resident columns.
 //   init_normal_kernel    x(0) and c from the seed.
 //   gather_columns_kernel sampled read-back.
 //
