@@ -224,7 +224,6 @@ struct netmax_ctx {
   double* measure_out = nullptr;         // (consensus, loss) of netmax_measure (page-locked host memory)
   // host copies of the tables in force (the asynchronous timeline draws peers on the host)
   bool host_tables = false;  // are they those of the policy in force? (need_host_tables)
-  BulkCopier bulk;           // transfers of whole M x M matrices
   std::vector<uint32_t> h_thr;
   std::vector<int32_t> h_last;
   std::vector<float> h_w;
@@ -445,8 +444,8 @@ int need_host_tables(netmax_ctx* ctx) {
   ctx->h_thr.resize(MM);
   ctx->h_last.resize(ctx->M);
   ctx->h_w.resize(MM);
-  NM_CUDA(ctx, ctx->bulk.to_host(ctx->h_thr.data(), ctx->thr, MM * sizeof(uint32_t), ctx->device, ctx->stream));
-  NM_CUDA(ctx, ctx->bulk.to_host(ctx->h_w.data(), ctx->wtab, MM * sizeof(float), ctx->device, ctx->stream));
+  NM_CUDA(ctx, BulkPool::get().to_host(ctx->h_thr.data(), ctx->thr, MM * sizeof(uint32_t), ctx->device, ctx->stream));
+  NM_CUDA(ctx, BulkPool::get().to_host(ctx->h_w.data(), ctx->wtab, MM * sizeof(float), ctx->device, ctx->stream));
   NM_CUDA(ctx, cudaMemcpyAsync(ctx->h_last.data(), ctx->last_nz, ctx->M * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
   NM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   ctx->host_tables = true;
@@ -461,8 +460,8 @@ int upload_policy(netmax_ctx* ctx) {
     double* d_P = nullptr;
     uint8_t* d_adj = nullptr;
     if (buf.get(&d_P, MM) && buf.get(&d_adj, MM)) {
-      NM_CUDA(ctx, ctx->bulk.to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
-      NM_CUDA(ctx, ctx->bulk.to_device(d_adj, ctx->adj.data(), MM, ctx->device, ctx->stream));
+      NM_CUDA(ctx, BulkPool::get().to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
+      NM_CUDA(ctx, BulkPool::get().to_device(d_adj, ctx->adj.data(), MM, ctx->device, ctx->stream));
       return device_tables(ctx, d_P, d_adj);
     }
     // (no device memory to spare beside the caller's workspace: on the host, as for few workers)
@@ -863,8 +862,10 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
     // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the worker
     // counts the header says so for; longer ones are where resident tiles gain most.
     static const unsigned char fused_short[22] = {0, 1, 1, 1, 0, 1, 1, 1, 1, 1, 1, 0, 0, 1, 0, 0, 0, 1, 1, 1, 1, 1};  // M = 67 ... 88
-    const bool short_calls = !f32 || M <= 66 || (M <= 88 && fused_short[M - 67]);
-    f.min_rounds = short_calls ? 2 : 9;
+    const bool short_calls = M <= 66 || (M <= 88 && fused_short[M - 67]);
+    // bfloat16 state: the tiles' narrow pieces are half as long, and the per-round kernel is nearer (one launch per round
+    // against tiles, 2 / 4 / 8 / 16 rounds: 40 workers 0.73 / 0.88 / 1.06 / 1.19, 300: 0.72 / 0.87 / 1.02 / 1.19).
+    f.min_rounds = !f32 ? 8 : short_calls ? 2 : 9;
   }
   f.ok = true;
   return NETMAX_OK;
@@ -1387,7 +1388,7 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   uint8_t* d_adj = nullptr;
   double rho = 0.0;
   const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
-                                          ctx->device, ctx->stream, ctx->bulk, buf, &d_P, &d_adj, &rho);
+                                          ctx->device, ctx->stream, buf, &d_P, &d_adj, &rho);
   graph.join();
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
@@ -1397,7 +1398,7 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   ctx->rho = rho;
   int done = device_tables(ctx, d_P, d_adj);
   if (!done) {
-    const cudaError_t e = ctx->bulk.to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
+    const cudaError_t e = BulkPool::get().to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
     if (e != cudaSuccess) done = fail(ctx, NETMAX_CUDA_ERROR, "reading P back: %s", cudaGetErrorString(e));
   }
   times.join();

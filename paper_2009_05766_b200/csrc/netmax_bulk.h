@@ -6,6 +6,8 @@
 #include <cstddef>
 #include <cstring>
 #include <functional>
+#include <memory>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -42,7 +44,7 @@ inline void parallel_copy(void* dst, const void* src, size_t bytes) {
 }
 
 // Copies of pageable memory by kLanes threads, each with two page-locked chunks of its own: the driver's
-// own staging runs on one core (134 MB: about 13 ms each way; 5 ms with four).  Owned by one context.
+// own staging runs on one core (134 MB: about 13 ms each way; 5 ms with four).  For one device and one caller at a time.
 class BulkCopier {
  public:
   ~BulkCopier() {
@@ -123,6 +125,51 @@ class BulkCopier {
     for (cudaError_t r : failed)
       if (r != cudaSuccess) return r;
     return cudaSuccess;
+  }
+};
+
+// Copiers shared by all contexts: locking their pages takes milliseconds, more than most transfers, so idle ones are
+// kept for the next transfer, at most two of them.
+class BulkPool {
+ public:
+  cudaError_t to_device(void* dst, const void* src, size_t bytes, int device, cudaStream_t stream) {
+    return with(device, [&](BulkCopier& c) { return c.to_device(dst, src, bytes, device, stream); });
+  }
+  cudaError_t to_host(void* dst, const void* src, size_t bytes, int device, cudaStream_t stream) {
+    return with(device, [&](BulkCopier& c) { return c.to_host(dst, src, bytes, device, stream); });
+  }
+  static BulkPool& get() {
+    static BulkPool* pool = new BulkPool();  // never destroyed: contexts may outlive static destructors
+    return *pool;
+  }
+
+ private:
+  struct Idle {
+    int device;
+    std::unique_ptr<BulkCopier> copier;
+  };
+  std::mutex mu_;
+  std::vector<Idle> idle_;
+
+  template <typename F>
+  cudaError_t with(int device, F body) {
+    std::unique_ptr<BulkCopier> c;
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      for (size_t k = 0; k < idle_.size(); ++k)
+        if (idle_[k].device == device) {
+          c = std::move(idle_[k].copier);
+          idle_.erase(idle_.begin() + (long)k);
+          break;
+        }
+    }
+    if (!c) c.reset(new BulkCopier());
+    const cudaError_t e = body(*c);
+    if (e == cudaSuccess) {
+      std::lock_guard<std::mutex> lock(mu_);
+      if (idle_.size() < 2) idle_.push_back(Idle{device, std::move(c)});
+    }
+    return e;
   }
 };
 

@@ -41,7 +41,7 @@ class DeviceBuffers {
 // A whole policy change on the current device: link speeds (host) -> link graph and iteration times ->
 // Algorithm 3.  The matrices stay on the device; *d_P is P there, owned by `buf`.
 int policy_from_links_device(int32_t M, int64_t d, const double* speed, double lr, int32_t K, int32_t R, double rho_upper,
-                             int device, cudaStream_t stream, BulkCopier& copier, DeviceBuffers& buf, double** d_P, uint8_t** d_adj,
+                             int device, cudaStream_t stream, DeviceBuffers& buf, double** d_P, uint8_t** d_adj,
                              double* rho);
 
 // The sampler's tables from P on the device: 32-bit cumulative thresholds, last positive entry and pull
