@@ -246,18 +246,14 @@ __device__ __forceinline__ int live_lanes(bool ragged, int tail, int h) {
 // hold x = c = 0 and so stay at exactly +0).  ta, tb return x - c for the caller's loss statistic.
 // Operand counts matter here: a packed instruction with three distinct register pairs issues every 3.2
 // cycles, one with two every 2.2 -- hence subtractions instead of multiply-adds with -1, and the product
-// with alpha as two scalar multiply-adds that take alpha from the constant bank.  kPacked: see scaled_pair.
-template <int kObjective, bool kPacked = false>
+// with alpha as two scalar multiply-adds that take alpha from the constant bank.
+template <int kObjective>
 __device__ __forceinline__ ulonglong2 update_core(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm, float w,
                                                   pair_t& ta, pair_t& tb) {
   ta = sub2(xv.x, cv.x);
   tb = sub2(xv.y, cv.y);
   pair_t ha = xv.x, hb = xv.y;
-  if (kObjective == 1 && kPacked) {
-    const pair_t nalpha2 = pack2(-alpha, -alpha);
-    ha = fma2(nalpha2, add2(ta, n.x), xv.x);
-    hb = fma2(nalpha2, add2(tb, n.y), xv.y);
-  } else if (kObjective == 1) {
+  if (kObjective == 1) {
     float g0, g1, g2, g3, x0, x1, x2, x3;
     unpack2(add2(ta, n.x), g0, g1);
     unpack2(add2(tb, n.y), g2, g3);
@@ -271,16 +267,16 @@ __device__ __forceinline__ ulonglong2 update_core(float alpha, ulonglong2 n, ulo
 }
 
 // The noise of one column group of one worker, with its Philox block drawn on the spot.
-template <int kObjective, bool kPacked = false>
+template <int kObjective>
 __device__ __forceinline__ ulonglong2 draw_noise(float sigma_s, const PhiloxKeys& keys, uint32_t iter_lo, uint32_t ctr3, uint32_t q32,
                                                  uint32_t worker, int live) {
   if (kObjective != 1) return make_ulonglong2(0ull, 0ull);
-  const ulonglong2 n = scaled_normals4<kPacked>(philox4x32_10(q32, worker, iter_lo, ctr3, keys), sigma_s);
+  const ulonglong2 n = scaled_normals4(philox4x32_10(q32, worker, iter_lo, ctr3, keys), sigma_s);
   return live < 4 ? mask_lanes(n, live) : n;
 }
 
 // update_core plus the telemetry sums of the round-start values.  kObjective == 2 measures only.
-template <int kObjective, bool kPacked = false>
+template <int kObjective>
 __device__ __forceinline__ ulonglong2 row_update(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm,
                                                  ulonglong2 pivot, float w, ColAcc& acc, LossAcc& lacc) {
   pair_t ta, tb;
@@ -289,7 +285,7 @@ __device__ __forceinline__ ulonglong2 row_update(float alpha, ulonglong2 n, ulon
     ta = sub2(xv.x, cv.x);
     tb = sub2(xv.y, cv.y);
   } else {
-    o = update_core<kObjective, kPacked>(alpha, n, xv, cv, xm, w, ta, tb);
+    o = update_core<kObjective>(alpha, n, xv, cv, xm, w, ta, tb);
   }
   const pair_t da = sub2(xv.x, pivot.x), db = sub2(xv.y, pivot.y);
   acc.s1a = add2(acc.s1a, da);
@@ -513,14 +509,11 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
             ulonglong2 o;
 #pragma unroll
             for (int h = 0; h < kHalves; ++h) {
-              // (padding lanes are cleared after the update here: a test between the noise and the update keeps their
-              // instructions apart, 207 us per round of 8 x 11.2 M elements against MASK_US)
-              const ulonglong2 noise = draw_noise<kObjective, kRowsInFlight == 1>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i, 4);
-              ulonglong2 oh = row_update<kObjective, kRowsInFlight == 1>(
-                  p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h), group_half<kHalves>(xm[u], h),
-                  group_half<kHalves>(pivot, h), __int_as_float(pw[u].y), acc[h], lacc);
-              const int live = live_lanes(ragged, p.tail, h);
-              if (live < 4) oh = mask_lanes(oh, live);
+              const ulonglong2 noise = draw_noise<kObjective>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i,
+                                                              live_lanes(ragged, p.tail, h));
+              const ulonglong2 oh = row_update<kObjective>(p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
+                                                           group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h),
+                                                           __int_as_float(pw[u].y), acc[h], lacc);
               if (kHalves == 1) o = oh;
               else if (h == 0) o.x = narrow_bf16x4(oh);
               else o.y = narrow_bf16x4(oh);

@@ -128,9 +128,6 @@ __device__ __forceinline__ pair_t sub2(pair_t a, pair_t b) {
 // return +0 or a tiny positive value for u1 next to 1, hence |.| (an operand modifier, not an
 // instruction) instead of a negation under the square root.
 constexpr double kNormalScale = 1.17741002251547469101;  // sqrt(2 ln 2)
-// kPacked: the last product as one packed instruction (same results): fewer instructions, which round_kernel at its
-// register limit wants; the kernels bound by issue run as fast or faster with two scalar ones.
-template <bool kPacked>
 __device__ __forceinline__ pair_t scaled_pair(uint32_t a, uint32_t b, float sigma_s) {
   const float u1 = radius_uniform(a);
   const float ang = (float)((int32_t)b >> 8) * 3.74507028e-07f;  // 2 pi / 2^24
@@ -139,12 +136,11 @@ __device__ __forceinline__ pair_t scaled_pair(uint32_t a, uint32_t b, float sigm
   rad *= sigma_s;
   float s, c;
   __sincosf(ang, &s, &c);
-  return kPacked ? mul2(pack2(rad, rad), pack2(c, s)) : pack2(rad * c, rad * s);
+  return pack2(rad * c, rad * s);
 }
 // sigma times the four normals of a Philox block.
-template <bool kPacked = false>
 __device__ __forceinline__ ulonglong2 scaled_normals4(uint4 r, float sigma_s) {
-  return make_ulonglong2(scaled_pair<kPacked>(r.x, r.y, sigma_s), scaled_pair<kPacked>(r.z, r.w, sigma_s));
+  return make_ulonglong2(scaled_pair(r.x, r.y, sigma_s), scaled_pair(r.z, r.w, sigma_s));
 }
 // Clears the lanes from `live` on (padding of a row's last, ragged group).
 __device__ __forceinline__ ulonglong2 mask_lanes(ulonglong2 v, int live) {
