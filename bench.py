@@ -47,14 +47,14 @@ UNIQUE_FRACTION = 0.75          # x_peer is a row the same tile reads anyway (a 
                                 # bytes (6 of 8) have to cross the DRAM pins, and the HBM roofline is taken against those
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0
-KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh")
+KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh", "netmax_search.h")
 # Counters of one launch, from ncu captures of this file's own commands (see profiles/): DRAM bytes
 # (dram__bytes_read.sum + dram__bytes_write.sum) per element of the launch and warp instructions
 # (smsp__inst_executed.sum) per element and round.  Captured on the workload itself where that is small
 # enough to profile, else on the same M and tile shape with a shorter vector (`captured_on`); bytes and
 # instructions per element are what carries over.  Only reported while the kernel sources still hash to
 # the value the capture was taken at.
-NCU_HASH = "e65debb22b22f859"
+NCU_HASH = "7141458fc988a423"
 NCU_COUNTERS = {
     # (workload tag, kernel): dram bytes per element-launch, warp instructions per element-round, captured on
     # (the per-round kernel's bytes on cfg2 are an earlier capture's; the latest one read 1,046,194,000)

@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "netmax_rng.cuh"
+#include "netmax_search.h"
 
 namespace netmax {
 
@@ -99,18 +100,10 @@ __global__ void __launch_bounds__(256) sample_peers_kernel(const SampleParams p)
 // that a round's draws leave as segments.  In sorted order the probes of a bisection are a power of two apart, all in
 // one bank (42 us of conflicts and waiting); so every sixteenth threshold is copied into an implicit search tree, level
 // after level (the middle, the quartiles, ...), and only the last four probes go to the row itself.  Rows are filled up
-// to a multiple of sixteen with the top; the last block needs no node, as its last threshold only ever counts for
-// u = 2^32 - 1, where `last` decides all the same.
+// to a multiple of sixteen with the top.  No threshold is above u = 2^32 - 1, so that draw leaves the tree at its last
+// leaf, behind the row's end unless M fills the tree: sample_block keeps the probes in the row's last block (`last`
+// decides what is drawn).  The index arithmetic is in netmax_search.h.
 constexpr int kSampleThreads = 256;
-__host__ __device__ inline uint32_t sample_levels(uint32_t M) {  // of the tree: 2^levels >= blocks of sixteen
-  uint32_t h = 0;
-  while ((16u << h) < M) ++h;
-  return h;
-}
-// Words between the rows and between the trees of a CTA: rows start in different banks.
-__host__ __device__ inline uint32_t sample_stride(uint32_t M, int rows) { return ((M + 31u) & ~31u) + 32u / rows; }
-__host__ __device__ inline uint32_t sample_tree(uint32_t M, int rows) { return (1u << sample_levels(M)) + 32u / rows; }
-__host__ __device__ inline size_t sample_smem(uint32_t M, int rows) { return (size_t)rows * (sample_stride(M, rows) + sample_tree(M, rows)) * 4u; }
 
 template <int kSampleRows>
 __global__ void __launch_bounds__(kSampleThreads) sample_rows_kernel(const SampleParams p, const uint32_t rounds_per_cta) {
@@ -133,10 +126,9 @@ __global__ void __launch_bounds__(kSampleThreads) sample_rows_kernel(const Sampl
   cp_async_wait_all();
   __syncthreads();
   for (uint32_t e = threadIdx.x; e < rows << h; e += kSampleThreads) {
-    const uint32_t w = e >> h, j = e & ((1u << h) - 1u);  // block j - 1 -> node
+    const uint32_t w = e >> h, j = e & ((1u << h) - 1u);  // the last threshold before block j -> node
     if (j == 0) continue;
-    const uint32_t z = __ffs(j) - 1;
-    s_tree[w * tree_stride + (1u << (h - 1 - z)) + (j >> (z + 1))] = 16u * j <= M ? s_thr[w * stride + 16u * j - 1u] : 0xFFFFFFFFu;
+    s_tree[w * tree_stride + sample_node(j, h, __ffs(j) - 1)] = 16u * j <= M ? s_thr[w * stride + 16u * j - 1u] : 0xFFFFFFFFu;
   }
   __syncthreads();
   const uint32_t w = threadIdx.x & (kSampleRows - 1);
@@ -159,7 +151,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_rows_kernel(const Sampl
       for (int a = 0; a < kAtOnce; ++a) at[a] = 2u * at[a] + (tree[at[a]] <= u[a] ? 1u : 0u);
     }
 #pragma unroll
-    for (int a = 0; a < kAtOnce; ++a) at[a] = 16u * (at[a] - (1u << h));  // thresholds of whole blocks <= u
+    for (int a = 0; a < kAtOnce; ++a) at[a] = 16u * sample_block(at[a], h, M);  // thresholds of whole blocks <= u
 #pragma unroll
     for (int s = 8; s > 0; s >>= 1) {
 #pragma unroll
