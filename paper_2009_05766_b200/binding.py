@@ -115,6 +115,7 @@ def lib():
 
 
 def _p(a):
+    """Address of an array's memory; the caller holds the array until the call has returned."""
     return None if a is None else a.ctypes.data
 
 
@@ -263,20 +264,22 @@ class Netmax:
         return P, rho.value
 
     def set_replicas(self, x):
-        _check(lib().netmax_set_replicas(self._h, self._host_plane(x)), self._h)
+        x, at = self._host_plane(x)  # (x: keeps a converted copy alive until the call has returned)
+        _check(lib().netmax_set_replicas(self._h, at), self._h)
 
     def set_centres(self, c):
-        _check(lib().netmax_set_centres(self._h, self._host_plane(c)), self._h)
+        c, at = self._host_plane(c)
+        _check(lib().netmax_set_centres(self._h, at), self._h)
 
     def _host_plane(self, a):
-        """numpy array or host pointer (int) of M*d floats."""
+        """numpy array or host pointer (int) of M*d floats, as (array, address): the array owns the memory."""
         if isinstance(a, int):
-            return C.c_void_p(a)
+            return None, a
         a = np.ascontiguousarray(a, dtype=np.float32)
         if a.shape != (self.M, self.d):
             raise ValueError(f"expected shape {(self.M, self.d)}, got {a.shape}")
-        self._keep = a
-        return _p(a)
+        self._keep = a  # (the copy of a page-locked array may still be under way after the call)
+        return a, _p(a)
 
     # (the calls a program makes every round or few go to the library without detours: marshalling was a third of a
     # small one)
@@ -287,15 +290,14 @@ class Netmax:
 
     def round_from_host(self, x, c, n_rounds: int, out, n_chunks: int = 0):
         """netmax_round_from_host: x, c, out are numpy arrays (M, d) float32 or host pointers (int); x and c may be None."""
-        def ptr(a):
-            return None if a is None else self._host_plane(a)
-        keep = [ptr(x), ptr(c)]
+        x, px = (None, None) if x is None else self._host_plane(x)
+        c, pc = (None, None) if c is None else self._host_plane(c)
         if isinstance(out, int):
             po = C.c_void_p(out)
         else:
             assert out.dtype == np.float32 and out.shape == (self.M, self.d) and out.flags.c_contiguous
             po = _p(out)
-        _check(lib().netmax_round_from_host(self._h, keep[0], keep[1], int(n_rounds), po, int(n_chunks)), self._h)
+        _check(lib().netmax_round_from_host(self._h, px, pc, int(n_rounds), po, int(n_chunks)), self._h)
         return out
 
     def set_fuse_rounds(self, fuse_rounds: int):

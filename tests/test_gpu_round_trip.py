@@ -90,3 +90,22 @@ def test_round_trip_through_pinned_buffers_and_its_argument_checks(nm):
     assert nm.lib().netmax_round_from_host(g._h, None, None, 1, None, 0) == -1
     g.close()
     h.close()
+
+
+def test_converted_inputs_give_the_same_bits(nm):
+    """float64 and non-contiguous replicas and centres, both given: converted by the binding, same result."""
+    M, d = 6, 400_003
+    rng = np.random.default_rng(12)
+    kw = dict(M=M, d=d, lr=0.05, prob=random_policy(M, rng), sigma=0.1, seed=3)
+    x = rng.standard_normal((M, d)).astype(np.float32)
+    c = rng.standard_normal((M, d)).astype(np.float32)
+    strided = np.zeros((M, 2 * d), dtype=np.float32)
+    strided[:, ::2] = c
+    want, out = (np.empty((M, d), dtype=np.float32) for _ in range(2))
+    a, b = nm.Netmax(**kw), nm.Netmax(**kw)
+    for _ in range(2):
+        a.round_from_host(x, c, 3, want)
+        b.round_from_host(x.astype(np.float64), strided[:, ::2], 3, out)
+        assert (out.view(np.uint32) == want.view(np.uint32)).all()
+    a.close()
+    b.close()

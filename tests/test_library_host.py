@@ -154,6 +154,44 @@ def test_null_context_calls_return_errors_not_crashes():
     assert size >= 3 * 8 * 1024 * 4 and size % 256 == 0
 
 
+def test_converted_inputs_live_until_the_library_returns(monkeypatch):
+    """Inputs that are not contiguous float32 are converted, and both converted arrays must still be there when the
+    library reads them: the library is replaced by one that looks at the memory it is given."""
+    M, d = 3, 1001
+    rng = np.random.default_rng(4)
+    seen = {}
+
+    class Library:
+        @staticmethod
+        def netmax_round_from_host(handle, x, c, n, out, chunks):
+            scratch = [np.full((M, d), np.nan, dtype=np.float32) for _ in range(8)]  # takes the place of anything freed
+            for name, at in (("x", x), ("c", c)):
+                seen[name] = np.ctypeslib.as_array(C.cast(at, C.POINTER(C.c_float)), shape=(M, d)).copy()
+            del scratch
+            return 0
+
+        @staticmethod
+        def netmax_set_replicas(handle, x):
+            seen["set"] = np.ctypeslib.as_array(C.cast(x, C.POINTER(C.c_float)), shape=(M, d)).copy()
+            return 0
+
+        netmax_set_centres = netmax_set_replicas
+
+    monkeypatch.setattr(binding, "lib", lambda: Library)
+    sim = object.__new__(binding.Netmax)
+    sim.M, sim.d, sim._h = M, d, C.c_void_p()
+    out = np.empty((M, d), dtype=np.float32)
+    wide = rng.standard_normal((M, 2 * d))
+    for x, c in ((wide[:, ::2], wide[:, 1::2]), (wide[:, :d].astype(np.float32)[:, ::-1], wide[:, d:]),
+                 (wide[:, :d].copy(), wide[:, d:].astype(np.float32))):
+        sim.round_from_host(x, c, 1, out)
+        assert (seen["x"] == x.astype(np.float32)).all() and (seen["c"] == c.astype(np.float32)).all()
+        sim.set_replicas(x)
+        assert (seen["set"] == x.astype(np.float32)).all()
+        sim.set_centres(c)
+        assert (seen["set"] == c.astype(np.float32)).all()
+
+
 def test_product_path_fails_loudly_without_a_gpu(gpu_available):
     if gpu_available:
         pytest.skip("a GPU is present")
