@@ -332,6 +332,9 @@ int netmax_async_ema(netmax_ctx* ctx, double* ema_out, int64_t* samples_out);
  * valid until the next netmax_round / netmax_set_* / netmax_read_replicas call; nothing is
  * synchronised.  In a bfloat16 context the buffer holds bfloat16 values: cast the pointer;
  * ld then counts bfloat16 elements.
+ * A program that changes replicas on the device -- in order with the context's stream -- takes
+ * their address from this call, in a workspace of its own too: until then netmax_read_replicas
+ * may return small replicas that the last netmax_round has already written to the host.
  */
 int netmax_replicas_device(netmax_ctx* ctx, const float** x, int64_t* ld);
 

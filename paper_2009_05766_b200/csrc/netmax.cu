@@ -204,6 +204,7 @@ struct netmax_ctx {
   bool host_writes = false;         // launches that may still write to `pinned` have been enqueued since the last synchronisation
   bool read_since_round = false;    // netmax_read_replicas has been called since the last netmax_round
   bool staged = false;              // the staging area holds, or is about to hold, the current replicas
+  bool replicas_exposed = false;    // a program may change the replicas behind the library: reads go to the device
   int32_t* trace_mirror = nullptr;  // host copy of the trace ring, written by the sampler (small rings only)
   int storage = NETMAX_STORAGE_F32;
   unsigned char *x[2] = {nullptr, nullptr}, *c = nullptr;  // [M][ld] fp32 or bfloat16, as `storage` says
@@ -1585,7 +1586,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
 
   // A program that reads small replicas after every call gets them with the rounds: the last launch writes them to
   // the page-locked staging area as well (4 x 4096 elements: a copy and a wait of their own were 15 of 45 us).
-  unsigned char* mirror = ctx->read_since_round && ctx->storage == NETMAX_STORAGE_F32 && ctx->L.plane <= kStagingBytes
+  unsigned char* mirror = ctx->read_since_round && !ctx->replicas_exposed && ctx->storage == NETMAX_STORAGE_F32 && ctx->L.plane <= kStagingBytes
                               ? ctx->pinned + kPinnedStaging : nullptr;
   bool mirrored = false;
   int64_t done = 0;
@@ -1944,6 +1945,8 @@ int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* ho
 int netmax_replicas_device(netmax_ctx* ctx, const float** x, int64_t* ld) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!x || !ld) return fail(ctx, NETMAX_INVALID_ARG, "output pointer is NULL");
+  ctx->replicas_exposed = true;  // (the caller may write through the address: what was mirrored may be stale from now on)
+  ctx->staged = false;
   *x = reinterpret_cast<const float*>(ctx->x[ctx->cur]);
   *ld = ctx->L.ld;
   return NETMAX_OK;

@@ -189,3 +189,45 @@ def test_peer_draws_equal_the_oracle(nm, M, rounds):
     g.sample_peers(7, rounds, out.data_ptr())
     assert (out.cpu().numpy() == oracle.peer_draws(P, M, 7, rounds)).all()
     g.close()
+
+
+@pytest.mark.parametrize("when", ["address taken first", "address taken after the rounds"])
+@pytest.mark.parametrize("own_workspace", [False, True])
+@pytest.mark.parametrize("rounds", [1, 5])
+def test_replicas_changed_on_the_device_are_what_is_read(nm, when, own_workspace, rounds):
+    """A program that reads small replicas after every call gets them with the rounds -- but one that has changed them on
+    the device in between gets what it wrote, and a read after a read what is there."""
+    import torch
+    M, d = 4, 1003
+    kw = dict(M=M, d=d, lr=0.05, prob=random_policy(M, np.random.default_rng(3)), sigma=0.1, x0_std=1.0, c_std=1.0, seed=5)
+    if own_workspace:
+        size = nm.Netmax.workspace_size(M, d)
+        memory = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        kw.update(workspace=(memory.data_ptr() + 255) // 256 * 256, workspace_bytes=size)
+    g, same = nm.Netmax(**kw), nm.Netmax(**{k: v for k, v in kw.items() if not k.startswith("workspace")})
+
+    def row(i):  # row i of the current replicas, as a tensor over the context's memory
+        ptr, ld = g.replicas_device()
+        iface = {"shape": (d,), "typestr": "<f4", "data": (ptr + 4 * i * ld, False), "version": 3}
+        return torch.as_tensor(type("Row", (), {"__cuda_array_interface__": iface})(), device="cuda")
+
+    def step():
+        for s in (g, same):
+            s.round(rounds)
+
+    step()
+    assert (g.read_replicas() == same.read_replicas()).all()   # (from here on reads are expected after every call)
+    if when == "address taken first":
+        row(0)
+    for k in range(3):
+        step()
+        row(2).fill_(0.25 * (k + 1))
+        torch.cuda.synchronize()
+        x = g.read_replicas()
+        want = same.read_replicas()
+        want[2] = 0.25 * (k + 1)
+        assert (x.view(np.uint32) == want.view(np.uint32)).all()
+        assert (g.read_replicas() == want).all()
+        same.set_replicas(want)
+    g.close()
+    same.close()
