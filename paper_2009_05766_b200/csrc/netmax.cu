@@ -11,6 +11,8 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <future>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -288,6 +290,8 @@ int fail(netmax_ctx* ctx, int code, const char* fmt, ...) {
   if (ctx) ctx->error = buf; else g_error = buf;
   return code;
 }
+
+#define NM_CATCH_CTX(ctx) NM_CATCH([&](int code, const char* what) { return ::fail(ctx, code, "%s", what); })
 
 #define NM_CUDA(ctx, call)                                                                         \
   do {                                                                                             \
@@ -1201,7 +1205,7 @@ int netmax_workspace_size(const netmax_config* cfg, size_t* bytes) {
   return NETMAX_OK;
 }
 
-int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
+int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) try {
   if (!out) return fail(nullptr, NETMAX_INVALID_ARG, "out is NULL");
   *out = nullptr;
   int rc = check_sizes(cfg);
@@ -1218,9 +1222,9 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
 
   netmax_ctx* ctx = new (std::nothrow) netmax_ctx();
   if (!ctx) return fail(nullptr, NETMAX_OOM, "host allocation failed");
+  std::unique_ptr<netmax_ctx, void (*)(netmax_ctx*)> owned(ctx, netmax_destroy);
   auto bail = [&](int code) {
     g_error = ctx->error;
-    netmax_destroy(ctx);
     return code;
   };
   ctx->M = cfg->M;
@@ -1325,9 +1329,9 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) {
   rc = launch_init(ctx, ctx->c, cfg->c_std, kTagC);
   if (rc) return bail(rc);
   if (!step(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize")) return bail(NETMAX_CUDA_ERROR);
-  *out = ctx;
+  *out = owned.release();
   return NETMAX_OK;
-}
+} NM_CATCH_CTX((netmax_ctx*)nullptr)
 
 int netmax_create(int32_t M, int64_t d, const double* link_speed_gbps, const double* prob, double lr, uint64_t seed,
                   netmax_ctx** out) {
@@ -1377,12 +1381,14 @@ void netmax_destroy(netmax_ctx* ctx) {
 static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   const int32_t M = ctx->M;
   std::vector<uint8_t> adj;
-  int graph_rc = NETMAX_OK;
   std::string graph_error;
-  std::thread graph([&] {
-    netmax_ctx* none = nullptr;  // (messages of this thread go to its own g_error)
-    graph_rc = build_adjacency(none, M, speed, adj);
-    graph_error = g_error;
+  // (a future's destructor waits for its thread, whichever way this function is left; without a thread to be had
+  // the work is done at get())
+  constexpr auto kBeside = std::launch::async | std::launch::deferred;
+  std::future<int> graph = std::async(kBeside, [&] {
+    const int rc = build_adjacency(nullptr, M, speed, adj);  // (its message goes to this thread's g_error)
+    if (rc) graph_error = g_error;
+    return rc;
   });
   DeviceBuffers buf;
   double* d_P = nullptr;
@@ -1390,65 +1396,75 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   double rho = 0.0;
   const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
                                           ctx->device, ctx->stream, buf, &d_P, &d_adj, &rho);
-  graph.join();
+  const int graph_rc = graph.get();
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
-  int times_rc = NETMAX_OK;
   ctx->t_iter.resize((size_t)M * M);
-  std::thread times([&] { times_rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_iter.data(), adj.data()); });
+  std::future<int> times = std::async(kBeside, [&] { return netmax_iteration_times(M, ctx->d, speed, ctx->t_iter.data(), adj.data()); });
   ctx->rho = rho;
   int done = device_tables(ctx, d_P, d_adj);
   if (!done) {
     const cudaError_t e = BulkPool::get().to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
     if (e != cudaSuccess) done = fail(ctx, NETMAX_CUDA_ERROR, "reading P back: %s", cudaGetErrorString(e));
   }
-  times.join();
+  const int times_rc = times.get();
   ctx->adj.swap(adj);
   if (!done && times_rc) done = fail(ctx, times_rc, "iteration times of the new speeds");
   return done;
 }
 
-int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const double* prob, double rho) {
+int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const double* prob, double rho) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!std::isfinite(rho)) return fail(ctx, NETMAX_INVALID_ARG, "rho is not finite");
   DeviceGuard guard(ctx->device);
+  int rc = NETMAX_OK;
   if (ctx->M >= kManyWorkers && link_speed_gbps && !prob && ctx->pull_weight <= 0.0 && rho <= 0.0) {
-    int rc = set_policy_from_links(ctx, link_speed_gbps);
+    rc = set_policy_from_links(ctx, link_speed_gbps);
     if (!rc && ctx->async_on) rc = need_host_tables(ctx);
     return rc;
   }
-  std::vector<uint8_t> old_adj;
-  std::vector<double> old_P, old_t;
-  if (!prob) old_P = ctx->P;  // (a caller's P is checked before it replaces the one in force)
-  const double old_rho = ctx->rho;
-  int rc = NETMAX_OK;
-  if (link_speed_gbps) {
-    old_t = ctx->t_iter;
-    old_adj.swap(ctx->adj);
-    rc = build_adjacency(ctx, ctx->M, link_speed_gbps, ctx->adj);
-  }
-  if (!rc) rc = resolve_policy(ctx, link_speed_gbps, prob, rho);
-  if (rc) {  // leave the policy in force untouched
+  {
+    struct Undo {  // leaves the policy in force untouched unless all of the new one is there
+      netmax_ctx* ctx;
+      bool links, generated;  // what is replaced: link graph and times; P (a caller's P is checked before it replaces the one in force)
+      std::vector<uint8_t> adj;
+      std::vector<double> P, t;
+      double rho;
+      bool done = false;
+      ~Undo() {
+        if (done) return;
+        if (links) {
+          ctx->adj.swap(adj);
+          ctx->t_iter.swap(t);
+        }
+        if (generated) ctx->P.swap(P);
+        ctx->rho = rho;
+      }
+    };
+    std::vector<double> old_P, old_t;
+    if (!prob) old_P = ctx->P;
+    if (link_speed_gbps) old_t = ctx->t_iter;
+    Undo undo{ctx, link_speed_gbps != nullptr, prob == nullptr, {}, std::move(old_P), std::move(old_t), ctx->rho};
     if (link_speed_gbps) {
-      ctx->adj.swap(old_adj);
-      ctx->t_iter.swap(old_t);
+      undo.adj.swap(ctx->adj);
+      rc = build_adjacency(ctx, ctx->M, link_speed_gbps, ctx->adj);
     }
-    if (!prob) ctx->P.swap(old_P);
-    ctx->rho = old_rho;
-    return rc;
+    if (!rc) rc = resolve_policy(ctx, link_speed_gbps, prob, rho);
+    if (rc) return rc;
+    undo.done = true;
   }
   // rounds already enqueued still read the old tables: the new ones are written behind them on the stream
   rc = upload_policy(ctx);
   if (!rc && ctx->async_on) rc = need_host_tables(ctx);
   return rc;
-}
+} NM_CATCH_CTX(ctx)
 
-int netmax_get_policy(netmax_ctx* ctx, double* prob_out, double* rho_out) {
+int netmax_get_policy(netmax_ctx* ctx, double* prob_out, double* rho_out) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (prob_out) parallel_copy(prob_out, ctx->P.data(), ctx->P.size() * sizeof(double));
   if (rho_out) *rho_out = ctx->rho;
   return NETMAX_OK;
-}
+} NM_CATCH_CTX(ctx)
 
 // Waits for the context's stream; reports a bounded wait of a kernel that has given up since the last check.
 static int synchronise(netmax_ctx* ctx) {
@@ -1563,7 +1579,7 @@ int netmax_read_replicas(netmax_ctx* ctx, float* host_out) {
 }
 int netmax_read_centres(netmax_ctx* ctx, float* host_out) { return copy_out(ctx, ctx ? ctx->c : nullptr, host_out); }
 
-int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
+int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (n_rounds < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_rounds = %lld < 0", (long long)n_rounds);
   if (ctx->async_on) return fail(ctx, NETMAX_INVALID_ARG, "the context runs the asynchronous timeline; use netmax_async_steps");
@@ -1671,13 +1687,13 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) {
   ctx->staged = mirror != nullptr && mirrored;
   ctx->read_since_round = false;
   return NETMAX_OK;
-}
+} NM_CATCH_CTX(ctx)
 
 int64_t netmax_rounds_done(const netmax_ctx* ctx) { return ctx ? ctx->rounds : -1; }
 
 // ---- host round trip, pipelined over column chunks ----------------------------------------------
 int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* host_c, int64_t n_rounds, float* host_out,
-                           int32_t n_chunks) {
+                           int32_t n_chunks) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (n_rounds < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_rounds = %lld < 0", (long long)n_rounds);
   if (!host_out) return fail(ctx, NETMAX_INVALID_ARG, "host_out is NULL");
@@ -1787,7 +1803,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   rc = synchronise(ctx);
   cleanup();
   return rc;
-}
+} NM_CATCH_CTX(ctx)
 
 int netmax_set_fuse_rounds(netmax_ctx* ctx, int32_t fuse_rounds) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
@@ -1918,7 +1934,7 @@ int netmax_peer_trace(netmax_ctx* ctx, int64_t first_round, int64_t n, int32_t* 
   return NETMAX_OK;
 }
 
-int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* host_consensus, double* host_loss) {
+int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* host_consensus, double* host_loss) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   int rc = ring_range(ctx, first_round, n);
   if (rc) return rc;
@@ -1940,7 +1956,7 @@ int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* ho
     if (host_loss) host_loss[k] = ring[2 * slot + 1];
   }
   return NETMAX_OK;
-}
+} NM_CATCH_CTX(ctx)
 
 int netmax_replicas_device(netmax_ctx* ctx, const float** x, int64_t* ld) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
@@ -1952,12 +1968,12 @@ int netmax_replicas_device(netmax_ctx* ctx, const float** x, int64_t* ld) {
   return NETMAX_OK;
 }
 
-int netmax_sample_peers(netmax_ctx* ctx, int64_t first_round, int64_t n_rounds, int32_t* device_out) {
+int netmax_sample_peers(netmax_ctx* ctx, int64_t first_round, int64_t n_rounds, int32_t* device_out) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (first_round < 0 || n_rounds < 0 || (n_rounds > 0 && !device_out)) return fail(ctx, NETMAX_INVALID_ARG, "bad range or NULL output");
   DeviceGuard guard(ctx->device);
   return launch_sampler(ctx, (uint64_t)first_round, n_rounds, device_out, nullptr, 0, INT64_MAX);
-}
+} NM_CATCH_CTX(ctx)
 
 // ---- telemetry on demand --------------------------------------------------------------------
 int netmax_measure(netmax_ctx* ctx, double* consensus, double* loss) {
@@ -2035,7 +2051,7 @@ static void async_start_iteration(netmax_ctx* ctx, int i, double start) {
   ctx->finish[i] = start + ctx->pending_duration[i];
 }
 
-int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) {
+int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (ctx->rounds != ctx->round0) return fail(ctx, NETMAX_INVALID_ARG, "netmax_async_begin must precede any netmax_round");
   if (!(beta >= 0.0 && beta < 1.0)) return fail(ctx, NETMAX_INVALID_ARG, "beta = %g outside [0, 1)", beta);
@@ -2054,7 +2070,7 @@ int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) {
     int rc = need_host_tables(ctx);
     if (rc) return rc;
   }
-  ctx->async_on = true;
+  ctx->async_on = false;  // until all of the state below is there
   ctx->beta = beta;
   ctx->now = 0.0;
   ctx->steps = 0;
@@ -2076,15 +2092,16 @@ int netmax_async_begin(netmax_ctx* ctx, const double* t_iter, double beta) {
     ctx->queue.emplace_back(ctx->finish[i], i);
   }
   std::make_heap(ctx->queue.begin(), ctx->queue.end(), std::greater<std::pair<double, int>>());
+  ctx->async_on = true;
   return NETMAX_OK;
-}
+} NM_CATCH_CTX(ctx)
 
-int netmax_async_set_times(netmax_ctx* ctx, const double* t_iter) {
+int netmax_async_set_times(netmax_ctx* ctx, const double* t_iter) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!t_iter) return fail(ctx, NETMAX_INVALID_ARG, "t_iter is NULL");
   ctx->t_iter.assign(t_iter, t_iter + (size_t)ctx->M * ctx->M);
   return NETMAX_OK;
-}
+} NM_CATCH_CTX(ctx)
 
 // Network Monitor (Algorithm 1): collect the workers' moving averages of iteration times, run
 // Algorithm 3 on them and send P and rho back.  An average that has seen n samples is read as
@@ -2270,7 +2287,7 @@ static int enqueue_steps(netmax_ctx* ctx, std::vector<StepEvent>& events, const 
   return rc;
 }
 
-int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
+int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (!ctx->async_on) return fail(ctx, NETMAX_INVALID_ARG, "call netmax_async_begin first");
   ctx->staged = false;
@@ -2324,7 +2341,7 @@ int netmax_async_steps(netmax_ctx* ctx, int64_t n_steps) {
     replace_top(ctx->queue, {ctx->finish[i], i});
   }
   return flush(true);
-}
+} NM_CATCH_CTX(ctx)
 
 int netmax_async_time(netmax_ctx* ctx, double* sim_time, int64_t* steps_done) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");

@@ -4,8 +4,9 @@
 #include <algorithm>
 #include <atomic>
 #include <cstddef>
+#include <cstdint>
 #include <cstring>
-#include <functional>
+#include <exception>
 #include <memory>
 #include <mutex>
 #include <thread>
@@ -15,22 +16,45 @@
 
 namespace netmax {
 
+// body(t) for t = 0 ... n - 1 at the same time, body(0) on the calling thread; n at most kMaxThreads.  Where the system has
+// no thread to give, the calling one does that part as well; what a part throws is thrown here, after all have ended.
+constexpr int kMaxThreads = 16;
+template <typename Body>
+void on_threads(int n, const Body& body) {
+  std::thread pool[kMaxThreads];
+  std::exception_ptr thrown[kMaxThreads];
+  auto part = [&](int t) noexcept {
+    try {
+      body(t);
+    } catch (...) {
+      thrown[t] = std::current_exception();
+    }
+  };
+  for (int t = 1; t < n; ++t) {
+    try {
+      pool[t] = std::thread([&part, t] { part(t); });
+    } catch (...) {
+      part(t);
+    }
+  }
+  part(0);
+  for (int t = 1; t < n; ++t)
+    if (pool[t].joinable()) pool[t].join();
+  for (int t = 0; t < n; ++t)
+    if (thrown[t]) std::rethrow_exception(thrown[t]);
+}
+
 // body(begin, end) on slices of [0, n), on up to 16 threads once n reaches min_parallel.
-inline void parallel_rows(int64_t n, int64_t min_parallel, const std::function<void(int64_t, int64_t)>& body) {
-  const unsigned hw = std::thread::hardware_concurrency();
-  const int threads = (n >= min_parallel && hw > 1) ? (int)std::min<unsigned>(hw, 16) : 1;
+template <typename Body>
+void parallel_rows(int64_t n, int64_t min_parallel, const Body& body) {
+  const unsigned hw = n >= min_parallel ? std::thread::hardware_concurrency() : 1;
+  const int threads = (int)std::min<unsigned>(hw, kMaxThreads);
   if (threads <= 1) {
     body(0, n);
     return;
   }
-  std::vector<std::thread> pool;
   const int64_t per = (n + threads - 1) / threads;
-  for (int t = 1; t < threads; ++t) {
-    const int64_t a = std::min<int64_t>(n, t * per), b = std::min<int64_t>(n, a + per);
-    if (a < b) pool.emplace_back(body, a, b);
-  }
-  body(0, std::min<int64_t>(n, per));
-  for (auto& th : pool) th.join();
+  on_threads((int)((n + per - 1) / per), [&](int t) { body(t * per, std::min<int64_t>(n, (t + 1) * per)); });
 }
 
 // memcpy; from 8 MB on by several threads (one core neither reaches the memory's bandwidth nor keeps up
@@ -62,7 +86,7 @@ class BulkCopier {
   }
 
  private:
-  static constexpr int kLanes = 4;
+  static constexpr int kLanes = 4;  // (a lane that gets no thread of its own finds its work done by the others)
   static constexpr size_t kChunk = (size_t)1 << 20;
   unsigned char* stage_ = nullptr;
   cudaStream_t streams_[kLanes] = {};
@@ -118,10 +142,7 @@ class BulkCopier {
         if (ev) cudaEventDestroy(ev);
       failed[l] = r;
     };
-    std::thread pool[kLanes];
-    for (int l = 1; l < kLanes; ++l) pool[l] = std::thread(lane, l);
-    lane(0);
-    for (int l = 1; l < kLanes; ++l) pool[l].join();
+    on_threads(kLanes, lane);
     for (cudaError_t r : failed)
       if (r != cudaSuccess) return r;
     return cudaSuccess;
@@ -150,6 +171,7 @@ class BulkPool {
   };
   std::mutex mu_;
   std::vector<Idle> idle_;
+  BulkPool() { idle_.reserve(2); }  // (giving a copier back allocates nothing)
 
   template <typename F>
   cudaError_t with(int device, F body) {

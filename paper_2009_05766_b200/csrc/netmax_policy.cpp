@@ -33,7 +33,6 @@
 #include <atomic>
 #include <cmath>
 #include <cstdio>
-#include <functional>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -51,7 +50,8 @@ int fail(int code, const std::string& msg) {
   return code;
 }
 
-void parallel_for(int n, int min_parallel, const std::function<void(int, int)>& body) {
+template <typename Body>
+void parallel_for(int n, int min_parallel, const Body& body) {
   netmax::parallel_rows(n, min_parallel, [&](int64_t a, int64_t b) { body((int)a, (int)b); });
 }
 
@@ -446,7 +446,7 @@ void tridiagonal_top_vector(const std::vector<double>& alpha, const std::vector<
 
 extern "C" {
 
-int netmax_iteration_times(int32_t M, int64_t d, const double* speed, double* t_out, uint8_t* adj_out) {
+int netmax_iteration_times(int32_t M, int64_t d, const double* speed, double* t_out, uint8_t* adj_out) try {
   if (M < 2 || d < 1 || !speed || !t_out || !adj_out) return fail(NETMAX_INVALID_ARG, "iteration_times: bad argument");
   // (by blocks of columns, so that the transposed entries are read a cache line at a time; rows over threads)
   constexpr int kBlock = 64;
@@ -479,7 +479,7 @@ int netmax_iteration_times(int32_t M, int64_t d, const double* speed, double* t_
       }
   });
   return NETMAX_OK;
-}
+} NM_CATCH(fail)
 
 int netmax_policy_generate(int32_t M, const double* t, const uint8_t* adj, double lr, int32_t K, int32_t R,
                            double* prob_out, double* rho_out, double* info_out) {
@@ -487,7 +487,7 @@ int netmax_policy_generate(int32_t M, const double* t, const uint8_t* adj, doubl
 }
 
 int netmax_policy_generate_ex(int32_t M, const double* t, const uint8_t* adj, double lr, int32_t K, int32_t R,
-                              double rho_upper, double* prob_out, double* rho_out, double* info_out) {
+                              double rho_upper, double* prob_out, double* rho_out, double* info_out) try {
   if (M < 2 || !t || !adj || !prob_out || !rho_out || !(lr > 0.0) || K < 1 || R < 1)
     return fail(NETMAX_INVALID_ARG, "policy_generate: bad argument");
   std::vector<Row> rows(M);
@@ -533,7 +533,7 @@ int netmax_policy_generate_ex(int32_t M, const double* t, const uint8_t* adj, do
   const double work_ns = (double)K * R * M * M * 12.0;
   const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
   const bool by_rows = M >= 1024;  // a copy of P and Y per thread would be too much: threads share a grid point instead
-  int n_threads = by_rows ? 1 : (int)std::min<double>(std::min<double>(std::min<unsigned>(hw, 16), K), 1.0 + work_ns / 4e5);
+  int n_threads = by_rows ? 1 : (int)std::min<double>(std::min<double>(std::min<unsigned>(hw, netmax::kMaxThreads), K), 1.0 + work_ns / 4e5);
   std::mutex mu;
   std::vector<double> probe;             // eigenvector of the best point so far (guarded by mu)
   double probe_tconv = INFINITY;
@@ -638,10 +638,7 @@ int netmax_policy_generate_ex(int32_t M, const double* t, const uint8_t* adj, do
     }
   };
   std::vector<std::vector<Best>> found(n_threads);
-  std::vector<std::thread> pool;
-  for (int th = 1; th < n_threads; ++th) pool.emplace_back([&, th] { walk(found[th]); });
-  walk(found[0]);
-  for (auto& th : pool) th.join();
+  netmax::on_threads(n_threads, [&](int th) { walk(found[th]); });
   std::vector<const Best*> order;
   for (const auto& list : found)
     for (const Best& b : list) order.push_back(&b);
@@ -660,7 +657,7 @@ int netmax_policy_generate_ex(int32_t M, const double* t, const uint8_t* adj, do
     info_out[4] = best->r;
   }
   return NETMAX_OK;
-}
+} NM_CATCH(fail)
 
 }  // extern "C"
 
@@ -796,7 +793,7 @@ bool solve_fixed_weight(int M, const double* t, const uint8_t* adj, double phi, 
 
 extern "C" {
 
-int netmax_policy_fixed_weight_at(int32_t M, const double* t, const uint8_t* adj, double floor, double t_bar, double* prob_out) {
+int netmax_policy_fixed_weight_at(int32_t M, const double* t, const uint8_t* adj, double floor, double t_bar, double* prob_out) try {
   if (M < 2 || !t || !adj || !prob_out || !(floor >= 0.0) || !(t_bar > 0.0) || !std::isfinite(floor) || !std::isfinite(t_bar))
     return fail(NETMAX_INVALID_ARG, "policy_fixed_weight_at: bad argument");
   std::vector<double> P;
@@ -804,10 +801,10 @@ int netmax_policy_fixed_weight_at(int32_t M, const double* t, const uint8_t* adj
     return fail(NETMAX_INFEASIBLE, "policy_fixed_weight_at: no P meets the floors, the row and column sums and the mean iteration time");
   std::copy(P.begin(), P.end(), prob_out);
   return NETMAX_OK;
-}
+} NM_CATCH(fail)
 
 int netmax_policy_generate_fixed_weight(int32_t M, const double* t, const uint8_t* adj, double pull_weight, int32_t K,
-                                        int32_t R, double floor_upper, double* prob_out, double* floor_out, double* info_out) {
+                                        int32_t R, double floor_upper, double* prob_out, double* floor_out, double* info_out) try {
   if (M < 2 || !t || !adj || !prob_out || !floor_out || !(pull_weight > 0.0 && pull_weight < 1.0) || K < 1 || R < 1)
     return fail(NETMAX_INVALID_ARG, "policy_generate_fixed_weight: bad argument");
   int max_deg = 0;
@@ -890,6 +887,6 @@ int netmax_policy_generate_fixed_weight(int32_t M, const double* t, const uint8_
     info_out[4] = best_r;
   }
   return NETMAX_OK;
-}
+} NM_CATCH(fail)
 
 }  // extern "C"

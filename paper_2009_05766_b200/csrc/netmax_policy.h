@@ -1,6 +1,8 @@
 // Internal glue between the C-ABI translation units.
 #pragma once
 #include <cstdint>
+#include <exception>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -9,6 +11,19 @@
 #include "netmax_bulk.h"
 
 namespace netmax {
+template <typename Fail>
+int caught(const Fail& fail, int code, const char* what) noexcept {
+  try {
+    return fail(code, what);
+  } catch (...) {
+    return code;  // (no memory for the message either)
+  }
+}
+// Ends the function-try-block of a C entry, none of which throws.  fail(code, message) records the message.
+#define NM_CATCH(fail)                                                                                          \
+  catch (const std::bad_alloc&) { return netmax::caught(fail, NETMAX_OOM, "host allocation failed"); }          \
+  catch (const std::exception& e) { return netmax::caught(fail, NETMAX_OOM, e.what()); }
+
 // Records the message netmax_last_error(NULL) returns on the calling thread.
 void set_global_error(const std::string& msg);
 // Largest eigenvalue of a symmetric tridiagonal matrix (diagonal alpha, off-diagonal beta), and an

@@ -278,3 +278,63 @@ def test_fixed_weight_grid_points_match_oracle_and_report_infeasibility():
     with pytest.raises(binding.NetmaxError) as e:
         binding.netmax_policy_generate_fixed_weight(t, one_way, 0.5, 4, 4)
     assert e.value.code == -1
+
+
+# Run in a process of its own: its address space is capped before the calls, so that threads (their stacks) and then
+# memory cannot be had.
+STARVED = r"""
+import ctypes as C, resource, sys
+import numpy as np
+from paper_2009_05766_b200 import binding
+L = binding.lib()
+def matrices(M):
+    rng = np.random.default_rng(M)
+    s = np.triu(np.exp(rng.uniform(0.0, np.log(100.0), (M, M))), 1)
+    return s + s.T, np.empty((M, M)), np.empty((M, M), dtype=np.uint8), np.empty((M, M))
+def cap(more):
+    with open("/proc/self/statm") as f:
+        now = int(f.read().split()[0]) * resource.getpagesize()
+    resource.setrlimit(resource.RLIMIT_AS, (now + more, now + more))
+def at(a):
+    return a.ctypes.data
+rho = C.c_double()
+s, t, adj, P = matrices(600)
+assert L.netmax_iteration_times(600, 1000, at(s), at(t), at(adj)) == 0
+assert L.netmax_policy_generate_ex(600, at(t), at(adj), 0.1, 4, 3, 0.0, at(P), C.byref(rho), None) == 0
+want_t, want_P, want_rho = t.copy(), P.copy(), rho.value
+big = matrices(4096)
+few = np.zeros((2, 2))
+cap(48 << 20)                    # room for some matrices of 600 workers, not for the stacks of fifteen threads
+t[:] = P[:] = 0.0
+assert L.netmax_iteration_times(600, 1000, at(s), at(t), at(adj)) == 0
+code = L.netmax_policy_generate_ex(600, at(t), at(adj), 0.1, 4, 3, 0.0, at(P), C.byref(rho), None)
+assert (t == want_t).all()
+if code == 0:
+    assert (P == want_P).all() and rho.value == want_rho
+else:
+    assert code == -3, code
+cap(1 << 20)
+assert L.netmax_iteration_times(4096, 1000, at(big[0]), at(big[1]), at(big[2])) in (0, -3)
+big[1][:] = 1.0
+np.fill_diagonal(big[1], 0.25)
+big[2][:] = 1
+assert L.netmax_policy_generate_ex(4096, at(big[1]), at(big[2]), 0.1, 2, 2, 0.0, at(big[3]), C.byref(rho), None) == -3
+assert L.netmax_policy_generate_fixed_weight(4096, at(big[1]), at(big[2]), 0.5, 2, 2, 0.0, at(big[3]), C.byref(rho), None) == -3
+assert L.netmax_policy_fixed_weight_at(4096, at(big[1]), at(big[2]), 0.0, 0.5 / 4096, at(big[3])) == -3
+cfg, handle = binding.Config(), C.c_void_p()
+assert L.netmax_config_init(C.byref(cfg)) == 0
+cfg.M, cfg.d, cfg.lr = 4096, 8, 0.1
+assert L.netmax_create_ex(C.byref(cfg), C.byref(handle)) < 0 and not handle.value
+assert L.netmax_last_error(None)
+print("fine")
+"""
+
+
+def test_calls_without_threads_or_memory_return_a_status():
+    """The C functions neither throw nor abort: without threads to be had they do the work on the calling one, with the
+    same result; without memory they return NETMAX_OOM."""
+    import subprocess
+    import sys
+    done = subprocess.run([sys.executable, "-c", STARVED], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                          env=dict(os.environ, OMP_NUM_THREADS="1", OPENBLAS_NUM_THREADS="1", MALLOC_ARENA_MAX="1"))
+    assert done.returncode == 0 and done.stdout.strip() == "fine", (done.returncode, done.stdout, done.stderr[-2000:])
