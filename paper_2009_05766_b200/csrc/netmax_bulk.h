@@ -91,15 +91,22 @@ class BulkCopier {
   unsigned char* stage_ = nullptr;
   cudaStream_t streams_[kLanes] = {};
 
+  bool prepare() {
+    void* p = nullptr;
+    if (!stage_ && cudaHostAlloc(&p, 2 * kLanes * kChunk, cudaHostAllocPortable) != cudaSuccess) return false;
+    if (!stage_) stage_ = (unsigned char*)p;
+    for (auto& s : streams_)
+      if (!s && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
+    return true;
+  }
+
   cudaError_t run(char* dst, const char* src, size_t bytes, int device, cudaStream_t stream, bool up) {
     cudaError_t e;
-    if (!stage_) {
-      void* p = nullptr;
-      if ((e = cudaHostAlloc(&p, 2 * kLanes * kChunk, cudaHostAllocPortable)) != cudaSuccess) return e;
-      stage_ = (unsigned char*)p;
+    if (!prepare()) {  // no memory to be locked: one plain copy
+      cudaGetLastError();
+      if ((e = cudaMemcpyAsync(dst, src, bytes, up ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return e;
+      return cudaStreamSynchronize(stream);
     }
-    for (auto& s : streams_)
-      if (!s && (e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return e;  // the other streams start behind it
     const int64_t chunks = (int64_t)((bytes + kChunk - 1) / kChunk);
     std::atomic<int64_t> next{0};
