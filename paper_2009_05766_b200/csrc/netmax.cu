@@ -62,13 +62,15 @@ constexpr size_t kPinnedTel = 256, kPinnedTrace = kPinnedTel + ((size_t)32 << 10
 constexpr size_t kStagingBytes = kPinnedBytes - kPinnedStaging;
 class PinnedPool {
  public:
-  unsigned char* get() {
+  // For the current device, whose context has the number `context`.
+  unsigned char* get(int device, uint64_t context) {
     {
       std::lock_guard<std::mutex> lock(mu_);
-      if (!kept_.empty()) {
-        unsigned char* p = kept_.back();
-        kept_.pop_back();
-        return p;
+      for (size_t k = n_kept_; k-- > 0;) {
+        if (kept_[k].device != device) continue;
+        const Block b = kept_[k];
+        kept_[k] = kept_[--n_kept_];
+        if (b.context == context) return b.p;  // (else: it went with the context it was locked in)
       }
     }
     void* p = nullptr;
@@ -78,11 +80,11 @@ class PinnedPool {
     }
     return (unsigned char*)p;
   }
-  void put(unsigned char* p) {  // the caller has waited for everything that writes to it
+  void put(unsigned char* p, int device, uint64_t context) {  // the caller has waited for everything that writes to it
     {
       std::lock_guard<std::mutex> lock(mu_);
-      if (kept_.size() < kPinnedKept) {
-        kept_.push_back(p);
+      if (n_kept_ < kPinnedKept) {
+        kept_[n_kept_++] = Block{p, device, context};
         return;
       }
     }
@@ -91,28 +93,41 @@ class PinnedPool {
   }
 
  private:
+  struct Block {
+    unsigned char* p;
+    int device;
+    uint64_t context;
+  };
   std::mutex mu_;
-  std::vector<unsigned char*> kept_;
+  Block kept_[kPinnedKept];
+  size_t n_kept_ = 0;
 };
 PinnedPool& pinned_pool() {
   static PinnedPool* pool = new PinnedPool();  // never destroyed: contexts may outlive static destructors
   return *pool;
 }
 
-// Raises a kernel's limit of dynamic shared memory on the current device, once: the attribute belongs to
-// the kernel and setting it costs microseconds, so what has been set is remembered (it is never lowered).
+// Raises a kernel's limit of dynamic shared memory on the current device, once: the attribute belongs to the kernel in
+// the device's context and setting it costs microseconds, so what has been set there is remembered (it is never lowered).
 cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  struct Limit {
+    uint64_t context = 0;
+    size_t bytes = 0;
+  };
   static std::mutex mu;
-  static auto* set = new std::unordered_map<uint64_t, size_t>();
+  static auto* set = new std::unordered_map<uint64_t, Limit>();
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const uint64_t key = (uint64_t)(uintptr_t)kernel * 64u + (uint64_t)(dev & 63);
+  const uint64_t key = (uint64_t)(uintptr_t)kernel * 64u + (uint64_t)(dev & 63), context = context_number();
   std::lock_guard<std::mutex> lock(mu);
-  size_t& have = (*set)[key];
-  if (bytes <= have) return cudaSuccess;
+  Limit& have = (*set)[key];
+  if (have.context == context && bytes <= have.bytes) return cudaSuccess;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) have = bytes;
+  if (e == cudaSuccess) {
+    have.context = context;
+    have.bytes = bytes;
+  }
   return e;
 }
 
@@ -202,6 +217,7 @@ struct netmax_ctx {
   cudaStream_t stream = nullptr;
   bool own_memory = false;
   unsigned char* base = nullptr;
+  uint64_t context = 0;             // number of the CUDA context that everything below was made in
   unsigned char* pinned = nullptr;  // block of the pinned pool: see kPinnedTel and the rest
   bool host_writes = false;         // launches that may still write to `pinned` have been enqueued since the last synchronisation
   bool read_since_round = false;    // netmax_read_replicas has been called since the last netmax_round
@@ -1261,10 +1277,17 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) try {
   if (cfg->device >= ndev) { ctx->error = "device ordinal out of range"; return bail(NETMAX_INVALID_ARG); }
   DeviceGuard guard(cfg->device);
   if (!guard.ok) { ctx->error = "cudaSetDevice failed"; return bail(NETMAX_CUDA_ERROR); }
+  auto step = [&](cudaError_t e, const char* what) {
+    if (e == cudaSuccess) return true;
+    ctx->error = std::string(what) + ": " + cudaGetErrorString(e);
+    return false;
+  };
   int attr = 0;
   if (cudaDeviceGetAttribute(&attr, cudaDevAttrMultiProcessorCount, cfg->device) == cudaSuccess) ctx->sm_count = attr;
   if (cudaDeviceGetAttribute(&attr, cudaDevAttrCooperativeLaunch, cfg->device) == cudaSuccess) ctx->cooperative = attr != 0;
-  ctx->pinned = pinned_pool().get();
+  if (!step(cudaFree(nullptr), "initialising the device")) return bail(NETMAX_CUDA_ERROR);  // (its context, if it is not there yet)
+  ctx->context = context_number();
+  ctx->pinned = pinned_pool().get(ctx->device, ctx->context);
   if (!ctx->pinned) { ctx->error = "cudaHostAlloc failed"; return bail(NETMAX_OOM); }
   if (cfg->workspace) {
     if (((uintptr_t)cfg->workspace & 255) != 0) { ctx->error = "workspace is not 256-byte aligned"; return bail(NETMAX_INVALID_ARG); }
@@ -1313,11 +1336,6 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) try {
   ctx->coltick = (unsigned int*)(ctx->base + L.off_coltick);
   ctx->pipe_tel = (double*)(ctx->base + L.off_pipe_tel);
 
-  auto step = [&](cudaError_t e, const char* what) {
-    if (e == cudaSuccess) return true;
-    ctx->error = std::string(what) + ": " + cudaGetErrorString(e);
-    return false;
-  };
   if (!step(cudaMemsetAsync(ctx->ticket, 0, 256, ctx->stream), "cudaMemsetAsync(ticket)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->coltick, 0, (size_t)kMaxGrid * sizeof(unsigned int), ctx->stream), "cudaMemsetAsync(coltick)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->x[1], 0, L.plane, ctx->stream), "cudaMemsetAsync(x)")) return bail(NETMAX_CUDA_ERROR);
@@ -1370,7 +1388,7 @@ void netmax_destroy(netmax_ctx* ctx) {
       cudaDeviceSynchronize();
       cudaGetLastError();
     }
-    pinned_pool().put(ctx->pinned);
+    pinned_pool().put(ctx->pinned, ctx->device, ctx->context);
   }
   delete ctx;
 }
@@ -1854,22 +1872,26 @@ struct StaticGatherScratch {
 static __device__ __align__(256) unsigned char g_gather_scratch[sizeof(StaticGatherScratch)];
 
 // In host code g_gather_scratch is only a stand-in for the symbol; the address a kernel or a
-// copy can use comes from cudaGetSymbolAddress, looked up once per device (that device
-// current) and cached here.
+// copy can use comes from cudaGetSymbolAddress, looked up once per device and CUDA context (that
+// device current) and cached here.
 static std::mutex g_gather_mu;
 static StaticGatherScratch* g_gather_ptr[64] = {};
+static uint64_t g_gather_context[64] = {};
 
 static int gather_scratch_address(netmax_ctx* ctx, StaticGatherScratch** out) {
   std::lock_guard<std::mutex> lock(g_gather_mu);
   const bool cached = ctx->device >= 0 && ctx->device < 64;
-  if (cached && g_gather_ptr[ctx->device]) {
+  if (cached && g_gather_ptr[ctx->device] && g_gather_context[ctx->device] == ctx->context) {
     *out = g_gather_ptr[ctx->device];
     return NETMAX_OK;
   }
   void* ptr = nullptr;
   NM_CUDA(ctx, cudaGetSymbolAddress(&ptr, g_gather_scratch));
   if (!ptr) return fail(ctx, NETMAX_CUDA_ERROR, "cudaGetSymbolAddress returned a null address");
-  if (cached) g_gather_ptr[ctx->device] = (StaticGatherScratch*)ptr;
+  if (cached) {
+    g_gather_ptr[ctx->device] = (StaticGatherScratch*)ptr;
+    g_gather_context[ctx->device] = ctx->context;
+  }
   *out = (StaticGatherScratch*)ptr;
   return NETMAX_OK;
 }

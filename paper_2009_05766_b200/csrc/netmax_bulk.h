@@ -16,6 +16,22 @@
 
 namespace netmax {
 
+// Number of the current device's CUDA context, another one after every cudaDeviceReset (0: not known).  Whatever outlives
+// a simulator -- page-locked blocks, copiers, kernel attributes that have been set -- belongs to the context it was made
+// in and is forgotten when that is gone.
+inline uint64_t context_number() {
+  using Query = int (*)(void*, unsigned long long*);  // cuCtxGetId
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult status;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &f, cudaEnableDefault, &status) != cudaSuccess) cudaGetLastError();
+    return (Query)f;
+  }();
+  unsigned long long id = 0;
+  if (!query || query(nullptr, &id) != 0) return 0;
+  return id;
+}
+
 // body(t) for t = 0 ... n - 1 at the same time, body(0) on the calling thread; n at most kMaxThreads.  Where the system has
 // no thread to give, the calling one does that part as well; what a part throws is thrown here, after all have ended.
 constexpr int kMaxThreads = 16;
@@ -76,6 +92,11 @@ class BulkCopier {
       if (s) cudaStreamDestroy(s);
     if (stage_) cudaFreeHost(stage_);
     cudaGetLastError();
+  }
+  // Its memory and streams went with their context.
+  void forget() {
+    stage_ = nullptr;
+    for (auto& s : streams_) s = nullptr;
   }
   // Copies after everything enqueued on `stream`; has finished when it returns.
   cudaError_t to_device(void* dst, const void* src, size_t bytes, int device, cudaStream_t stream) {
@@ -174,6 +195,7 @@ class BulkPool {
  private:
   struct Idle {
     int device;
+    uint64_t context;
     std::unique_ptr<BulkCopier> copier;
   };
   std::mutex mu_;
@@ -183,20 +205,25 @@ class BulkPool {
   template <typename F>
   cudaError_t with(int device, F body) {
     std::unique_ptr<BulkCopier> c;
+    const uint64_t context = context_number();
     {
       std::lock_guard<std::mutex> lock(mu_);
-      for (size_t k = 0; k < idle_.size(); ++k)
-        if (idle_[k].device == device) {
+      for (size_t k = idle_.size(); k-- > 0;) {
+        if (idle_[k].device != device) continue;
+        if (idle_[k].context == context) {
+          if (c) continue;
           c = std::move(idle_[k].copier);
-          idle_.erase(idle_.begin() + (long)k);
-          break;
+        } else {
+          idle_[k].copier->forget();
         }
+        idle_.erase(idle_.begin() + (long)k);
+      }
     }
     if (!c) c.reset(new BulkCopier());
     const cudaError_t e = body(*c);
     if (e == cudaSuccess) {
       std::lock_guard<std::mutex> lock(mu_);
-      if (idle_.size() < 2) idle_.push_back(Idle{device, std::move(c)});
+      if (idle_.size() < 2) idle_.push_back(Idle{device, context, std::move(c)});
     }
     return e;
   }

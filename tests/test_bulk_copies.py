@@ -1,5 +1,5 @@
 """Large host transfers (netmax_bulk.h) against a CUDA runtime of a few lines on the host: whole and ragged sizes, both
-directions, and a runtime that locks no memory or creates no stream -- the copies are then made all the same."""
+directions, and a runtime that locks no memory or creates no stream (the copies are then made all the same), and a device reset in between."""
 import os
 import subprocess
 
@@ -38,6 +38,11 @@ inline cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSucce
 inline cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 inline cudaError_t cudaEventDestroy(cudaEvent_t e) { delete e; return cudaSuccess; }
 inline cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { ++copies; std::memcpy(d, s, n); return cudaSuccess; }
+typedef int cudaDriverEntryPointQueryResult;
+constexpr int cudaEnableDefault = 0;
+inline unsigned long long context = 1;
+inline int context_id(void*, unsigned long long* id) { *id = context; return 0; }
+inline cudaError_t cudaGetDriverEntryPoint(const char*, void** f, int, int*) { *f = (void*)context_id; return cudaSuccess; }
 inline cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 inline cudaError_t cudaGetLastError() { return cudaSuccess; }
 """
@@ -61,6 +66,15 @@ int main() {
         if (up != src || down != src) return std::printf("copy: %zu\n", bytes), 1;
       }
     }
+  // a device reset takes the locked memory and the streams with it: what is kept from before is not touched again
+  locked_left = streams_left = 1000;
+  std::vector<unsigned char> src(1 << 20, 7), up(1 << 20);
+  const int held = locked, open = streams;
+  if (held < 1) return std::printf("nothing was kept\n"), 1;
+  context = 2;
+  for (int k = 0; k < 3; ++k)
+    if (BulkPool::get().to_device(up.data(), src.data(), up.size(), 0, nullptr) != cudaSuccess || up != src) return std::printf("after a reset\n"), 1;
+  if (locked != held + 1 || streams != open + 4) return std::printf("%d blocks, %d streams\n", (int)locked, (int)streams), 1;
   std::printf("fine\n");
   return 0;
 }
