@@ -515,6 +515,22 @@ int refresh_iteration_times(netmax_ctx* ctx, const double* speed) {
   return NETMAX_OK;
 }
 
+// Algorithm 3 on iteration times: on the device for many workers, on the host for fewer and where the device has no memory
+// to spare beside the caller's workspace.
+int generate_policy(netmax_ctx* ctx, const double* t_iter, double* P, double* rho) {
+  int ndev = 0;
+  if (ctx->M >= kManyWorkers) {
+    if (cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev) {
+      const int rc = netmax_policy_generate_device(ctx->M, t_iter, ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R,
+                                                   ctx->policy_rho_upper, ctx->device, ctx->stream, P, rho, nullptr);
+      if (rc != NETMAX_OOM) return rc;
+    }
+    cudaGetLastError();
+  }
+  return netmax_policy_generate_ex(ctx->M, t_iter, ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper, P, rho,
+                                   nullptr);
+}
+
 // Chooses P and rho: the caller's, or Algorithm 3's.  speed == NULL keeps the iteration times
 // in force (or, at creation, takes equal speeds).
 int resolve_policy(netmax_ctx* ctx, const double* speed, const double* prob, double rho) {
@@ -547,14 +563,7 @@ int resolve_policy(netmax_ctx* ctx, const double* speed, const double* prob, dou
     ctx->rho = rho > 0.0 ? rho : 0.0;
     return NETMAX_OK;
   }
-  // Algorithm 3: on the device for many workers
-  int ndev = 0;
-  const bool on_device = M >= kManyWorkers && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
-  if (!on_device) cudaGetLastError();
-  int rc = on_device ? netmax_policy_generate_device(M, ctx->t_iter.data(), ctx->adj.data(), ctx->alpha, ctx->policy_K,
-                                                     ctx->policy_R, ctx->policy_rho_upper, ctx->device, ctx->stream, ctx->P.data(), &rho_sel, nullptr)
-                     : netmax_policy_generate_ex(M, ctx->t_iter.data(), ctx->adj.data(), ctx->alpha, ctx->policy_K,
-                                                 ctx->policy_R, ctx->policy_rho_upper, ctx->P.data(), &rho_sel, nullptr);
+  int rc = generate_policy(ctx, ctx->t_iter.data(), ctx->P.data(), &rho_sel);
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
   if (rho > 0.0) {  // the caller's rho with Algorithm 3's P: it must still respect that P
     rc = check_rho(ctx, M, ctx->P.data(), ctx->adj, ctx->alpha, rho, ctx->pull_weight);
@@ -1439,7 +1448,8 @@ int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const doub
   if (ctx->M >= kManyWorkers && link_speed_gbps && !prob && ctx->pull_weight <= 0.0 && rho <= 0.0) {
     rc = set_policy_from_links(ctx, link_speed_gbps);
     if (!rc && ctx->async_on) rc = need_host_tables(ctx);
-    return rc;
+    if (rc != NETMAX_OOM) return rc;
+    rc = NETMAX_OK;  // (no device memory to spare: piece by piece, as for few workers)
   }
   {
     struct Undo {  // leaves the policy in force untouched unless all of the new one is there
@@ -2140,16 +2150,11 @@ static int monitor_refresh(netmax_ctx* ctx) {
   }
   std::vector<double> P((size_t)M * M);
   double rho = 0.0;
-  int ndev = 0;
   const bool fixed = ctx->pull_weight > 0.0;  // constant pull weight: the extension section's form of Algorithm 3
-  const bool on_device = !fixed && M >= kManyWorkers && cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev;
   double floor_sel = 0.0;
   int rc = fixed ? netmax_policy_generate_fixed_weight(M, t.data(), ctx->adj.data(), ctx->pull_weight, ctx->policy_K, ctx->policy_R,
                                                        ctx->policy_rho_upper, P.data(), &floor_sel, nullptr)
-           : on_device ? netmax_policy_generate_device(M, t.data(), ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R,
-                                                     ctx->policy_rho_upper, ctx->device, ctx->stream, P.data(), &rho, nullptr)
-                     : netmax_policy_generate_ex(M, t.data(), ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R,
-                                                 ctx->policy_rho_upper, P.data(), &rho, nullptr);
+                 : generate_policy(ctx, t.data(), P.data(), &rho);
   if (rc == NETMAX_INFEASIBLE) return NETMAX_OK;
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
   ctx->P.swap(P);

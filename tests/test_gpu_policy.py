@@ -94,3 +94,46 @@ def test_device_policy_on_the_sampling_stress_config(nm):
     off = ~np.eye(w.M, dtype=bool)
     assert (Pd[off] >= 2 * w.lr * rhod * (1 - 1e-9)).all()                     # Eq. 11 floors
     assert dev_s < host_s
+
+
+def test_policy_change_without_device_memory_to_spare(nm):
+    """A program that has handed out all device memory: the matrices of Algorithm 3 have no room there, the policy is
+    generated on the host."""
+    import torch
+    M, d = 400, 64
+    rng = np.random.default_rng(8)
+    speeds = [np.triu(np.exp(rng.uniform(0.0, 4.0, (M, M))), 1) for _ in range(2)]
+    speeds = [s + s.T for s in speeds]
+    size = nm.Netmax.workspace_size(M, d)
+    kw = dict(M=M, d=d, lr=0.05, link_speed_gbps=speeds[0], policy_K=3, policy_R=3, seed=2)
+    memory = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+    g = nm.Netmax(workspace=(memory.data_ptr() + 255) // 256 * 256, workspace_bytes=size, **kw)
+    same = nm.Netmax(**kw)
+    for s in (g, same):        # (every kernel of a change of links has run before the memory is gone)
+        s.set_policy(link_speed_gbps=speeds[1])
+        s.set_policy(link_speed_gbps=speeds[0])
+        s.round(2)
+    same.set_policy(link_speed_gbps=speeds[1])
+    P, rho = same.get_policy()
+    cudart = torch.cuda.cudart()
+    held, step = [], 1 << 36
+    try:
+        while step >= 1 << 21:
+            try:
+                held.append(torch.cuda.caching_allocator_alloc(step))
+            except torch.cuda.OutOfMemoryError:
+                step >>= 1
+        assert cudart.cudaMemGetInfo(0)[0] < 8 << 20
+        g.set_policy(link_speed_gbps=speeds[1])
+    finally:
+        for p in held:
+            torch.cuda.caching_allocator_delete(p)
+        torch.cuda.empty_cache()
+    Pg, rhog = g.get_policy()
+    assert rhog == pytest.approx(rho, rel=1e-12)
+    np.testing.assert_allclose(Pg, P, atol=1e-10)
+    for s in (g, same):
+        s.round(3)
+    assert (g.peer_trace(2, 3) == same.peer_trace(2, 3)).mean() > 0.999
+    g.close()
+    same.close()
