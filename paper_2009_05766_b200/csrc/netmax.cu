@@ -827,6 +827,10 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
   const bool f32 = ctx->storage == NETMAX_STORAGE_F32;
   if (!plan.short_vectors && ctx->fuse_rounds >= 2 && M > 144) return NETMAX_OK;  // (fuse_rounds: see the C header)
   const size_t per_sm = (size_t)228 * 1024, per_cta = (size_t)226 * 1024;  // (227 KB less the static part)
+  // Long vectors of fp32 state with up to 88 workers (144 where fused rounds are asked for): telemetry in double across
+  // threads, in fp32 over 18 rows at most, as in the shapes that ran them before (88 x 762,603 elements pay 8 to 11 % for
+  // another shape than eleven rows per thread).
+  const bool wide = !plan.short_vectors && f32 && M <= (ctx->fuse_rounds >= 2 ? 144 : 88);
   double best = 0.0;
   int best_c = 0;
   {
@@ -834,12 +838,14 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
       for (int W = 1; W <= 16; ++W) {
         const int RL = W * 32 / G;
         const int K = (int)((M + RL - 1) / RL);
+        if (wide && !tile_wide(K)) continue;
         if (K > kTileMaxRows || (RL > M && W > 1) || W * 32 > tile_max_threads(K)) continue;
         const int warps = tile_max_threads(K) / 32;  // that an SM's registers hold
         bool pre = false;
         size_t smem = tile_smem(M, W * 32, G, false, K);
         const size_t small = tile_smem(M, W * 32, G, true, K);
-        if (smem > per_cta || (smem > small && per_sm / (smem + 1024) < std::min<size_t>(warps / W, per_sm / (small + 1024)))) {
+        const bool may_pre = !wide || 32 / G * K <= 18;  // (the lanes of a warp are added in fp32)
+        if (may_pre && (smem > per_cta || (smem > small && per_sm / (smem + 1024) < std::min<size_t>(warps / W, per_sm / (small + 1024))))) {
           pre = true;
           smem = small;
         }

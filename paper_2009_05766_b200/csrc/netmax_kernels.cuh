@@ -734,8 +734,7 @@ struct FusedParams {
 // Dynamic shared memory: (peer row offset, weight) int2[slots][M], the warps' telemetry sums
 // double[slots][warps][2], then the slabs float4[3][M][blockDim] (replicas of even rounds, of odd rounds,
 // centres).  Any block size that is a multiple of 32 up to 256 works.
-// The telemetry of a round is added over the lanes of a warp at its end (in double, as every sum across threads
-// is) and kept per warp in shared memory: with a thread's own sums in registers a launch was limited to eight
+// The telemetry of a round is added over the lanes of a warp at its end (in double) and kept per warp in shared memory: with a thread's own sums in registers a launch was limited to eight
 // rounds, and 32 registers a thread went into them.
 __host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {
   return (uint32_t)(((uint64_t)slots * (uint64_t)(M * 8 + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);

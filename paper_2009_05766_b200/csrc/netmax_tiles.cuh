@@ -117,7 +117,14 @@ __device__ __forceinline__ bool tile_piece(const TileParams& p, int n, Piece& ou
 // decide.
 __host__ __device__ constexpr int tile_max_threads(int rows) { return rows <= 8 ? 512 : rows <= 10 ? 448 : 384; }
 constexpr int kTileMaxRows = 16;
-constexpr int kShareUnroll = 4;  // loads of a lane in flight when shares are added (4096 x 1024: 7.04 us per round without, 5.87; eight: 7.13)
+// What the shares of a round are added up in: fp32 sums are a thread's own, and those of column sums.  Double with five
+// rows per thread and more (long vectors of fp32 state up to 88 workers, whose sums across threads have always been
+// double, run on nothing else; an error of 1.2e-9 in the loss of 64 x 262,147 elements is 6e-11 with it).  With fewer
+// rows (short vectors) it would cost 8 %, and with eleven, where the compiler's schedule falls apart, 18 % (4096 x 1024
+// elements: 6.5 us per round, 7.7).  Four loads of a lane are in flight (4096 x 1024: 7.04 us per round without, 5.87;
+// eight: 7.13).
+constexpr int kShareUnroll = 4;
+__host__ __device__ constexpr bool tile_wide(int rows) { return rows > 4 && rows != 11; }
 // Few rows per thread make a round short, and what is not the round itself counts: draws are fetched two rounds
 // ahead, and the sums of a round are added after the NEXT round's arrival, beside its noise, which takes a third
 // buffer (32 x 1000 elements: 0.79 -> 0.68 us per round).  With more rows the buffer is better kept for slabs.
@@ -140,6 +147,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
   constexpr bool kFar = tile_far(kRows);
   constexpr uint32_t kBuffers = kFar ? 3u : 2u;
+  using Sum = typename std::conditional<tile_wide(kRows), double, float>::type;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long s_bar;
   const int tid = threadIdx.x, T = blockDim.x, M = p.M, G = p.G;
@@ -200,14 +208,19 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
   // which belong to column group lane % G) and leaves the CTA's two sums
   auto add_shares = [&](uint32_t buf, int k) {
     float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f);
-    float s2 = 0.f, loss = 0.f;
-#pragma unroll kShareUnroll
-    for (uint32_t e = lane; e < E; e += 32) {
+    Sum s2 = 0, loss = 0;
+    auto add = [&](uint32_t e) {
       const float4 a = s_sum[buf * E + e];
       const float2 b = s_two[buf * E + e];
       s1.x += a.x; s1.y += a.y; s1.z += a.z; s1.w += a.w;
-      s2 += b.x;
-      loss += b.y;
+      s2 += (Sum)b.x;
+      loss += (Sum)b.y;
+    };
+    if (kRows < 12) {
+#pragma unroll kShareUnroll
+      for (uint32_t e = lane; e < E; e += 32) add(e);
+    } else {  // (the compiler's choice: 8 % faster than four with 93 x 721,603 elements)
+      for (uint32_t e = lane; e < E; e += 32) add(e);
     }
     for (int off = 16; off >= G; off >>= 1) {
       s1.x += __shfl_xor_sync(0xffffffffu, s1.x, off);
@@ -216,15 +229,23 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
       s1.w += __shfl_xor_sync(0xffffffffu, s1.w, off);
     }
     // sum_i (x_i - xbar)^2 = sum_i (x_i - a)^2 - (sum_i (x_i - a))^2 / M per column
-    if (lane < G) s2 -= (s1.x * s1.x + s1.y * s1.y + s1.z * s1.z + s1.w * s1.w) * p.inv_M;
-    for (int off = 16; off > 0; off >>= 1) {
-      s2 += __shfl_down_sync(0xffffffffu, s2, off);
-      loss += __shfl_down_sync(0xffffffffu, loss, off);
-    }
-    if (lane == 0) {
-      double* out = p.partials + ((size_t)k * gridDim.x + blockIdx.x) * 2;
-      asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out), "d"((double)s2) : "memory");
-      asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + 1), "d"(0.5 * (double)loss) : "memory");
+    if (lane < G) s2 -= (Sum)(s1.x * s1.x + s1.y * s1.y + s1.z * s1.z + s1.w * s1.w) * (Sum)p.inv_M;
+    double* out = p.partials + ((size_t)k * gridDim.x + blockIdx.x) * 2;
+    if constexpr (tile_wide(kRows)) {  // lanes 0-15 go on with the one sum, lanes 16-31 with the other
+      const bool low = lane < 16;
+      Sum keep = (low ? s2 : loss) + __shfl_xor_sync(0xffffffffu, low ? loss : s2, 16);
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, off);
+      if ((lane & 15) == 0) asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + (lane >> 4)), "d"(low ? (double)keep : 0.5 * (double)keep) : "memory");
+    } else {
+      for (int off = 16; off > 0; off >>= 1) {
+        s2 += __shfl_down_sync(0xffffffffu, s2, off);
+        loss += __shfl_down_sync(0xffffffffu, loss, off);
+      }
+      if (lane == 0) {
+        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out), "d"((double)s2) : "memory");
+        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(out + 1), "d"(0.5 * (double)loss) : "memory");
+      }
     }
   };
   for (int k = tid; k < p.n_rounds; k += T)

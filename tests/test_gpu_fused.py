@@ -179,3 +179,30 @@ def test_fuse_rounds_out_of_range_is_refused(nm):
     with pytest.raises(nm.NetmaxError) as e:
         nm.Netmax(M=2, d=64, lr=0.1, fuse_rounds=9)
     assert e.value.code == -1
+
+
+# 37 and more workers, calls of ten rounds on resident tiles: ten and eight rows per thread, and counts whose best shape
+# would be eleven
+@pytest.mark.parametrize("M,d,fuse", [(40, 300_003, 0), (64, 262_147, 0), (88, 200_003, 0), (121, 150_001, 8)])
+def test_telemetry_of_tiles_is_added_in_double(nm, M, d, fuse):
+    """A round's loss against 64-bit sums of the replicas it starts from.  In fp32 are a thread's sums over up to 16 rows
+    of four columns: a few u = 2^-24 each, at random, over the square root of the 10^5 and more threads of the sum.  Sums
+    of a whole CTA in fp32 were off by 1 to 2e-9.  (1 / M is rounded to fp32 once.)"""
+    import torch
+    inverse = float(np.float32(1.0) / np.float32(M))
+    P = np.random.default_rng(M).random((M, M)) + 0.05
+    np.fill_diagonal(P, 0.0)
+    P /= P.sum(axis=1, keepdims=True)
+    for seed in range(3):
+        g = nm.Netmax(M=M, d=d, lr=0.1, prob=P, sigma=0.01, x0_std=1.0, c_std=1.0, seed=seed, trace_rounds=32, fuse_rounds=fuse)
+        c = torch.from_numpy(g.read_centres()).cuda().double()
+        for _ in range(2):
+            x = torch.from_numpy(g.read_replicas()).cuda().double()
+            first = g.rounds_done
+            g.round(10)
+            cons, loss = g.telemetry(first, 1)
+            want = 0.5 * ((x - c) ** 2).sum().item() * inverse
+            assert abs(loss[0] - want) <= 5e-10 * want, (loss[0] - want) / want
+            want = ((x - x.mean(0)) ** 2).sum().item() / M
+            assert abs(cons[0] - want) <= 1e-8 * want, (cons[0] - want) / want
+        g.close()
