@@ -680,9 +680,16 @@ MultiRoundKernel pick_multi_kernel(int objective, int halves) {
 
 using FusedKernel = void (*)(const FusedParams);
 
-FusedKernel pick_fused_kernel(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true> : fused_rounds_kernel<0, true>;
-  return objective == 1 ? fused_rounds_kernel<1, false> : fused_rounds_kernel<0, false>;
+template <int kReg>
+FusedKernel pick_fused_kernel_r(int objective, int halves) {
+  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kReg> : fused_rounds_kernel<0, true, kReg>;
+  return objective == 1 ? fused_rounds_kernel<1, false, kReg> : fused_rounds_kernel<0, false, kReg>;
+}
+// The instance for launches of `rounds` rounds (all share one layout of the shared memory).
+FusedKernel pick_fused_kernel(int objective, int halves, int rounds) {
+  if (rounds <= 4) return pick_fused_kernel_r<4>(objective, halves);
+  if (rounds <= 8) return pick_fused_kernel_r<8>(objective, halves);
+  return pick_fused_kernel_r<0>(objective, halves);
 }
 
 using TileKernel = void (*)(const TileParams);
@@ -926,7 +933,9 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   if (ctx->M > NETMAX_FUSED_MAX_M) return NETMAX_OK;
 #endif
   const int64_t M = ctx->M;
-  const int want_rounds = ctx->fuse_rounds >= 2 ? std::min(ctx->fuse_rounds, kFusedMaxRounds) : kFusedMaxRounds;
+  // (two and three workers: a round is too short to hide its sums' shuffles, and launches of more than eight rounds lose
+  // 1.5 %; four workers: as fast)
+  const int want_rounds = ctx->fuse_rounds >= 2 ? std::min(ctx->fuse_rounds, kFusedMaxRounds) : M <= 3 ? 8 : kFusedMaxRounds;
   // 256 or 128 threads per CTA (a multiple of four warps keeps the SM's four schedulers evenly
   // loaded: 3 x 96 threads measured 587 us per cfg3 round against 508 for 2 x 128), whichever
   // puts more threads on an SM with at least two CTAs (one loads its tile while the other
@@ -937,8 +946,10 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   // faster than one launch per round (M x 4,000,002 elements, us per round, against rows over a cluster of CTAs:
   // M = 20: 132 against 144, 28: 182 against 214, 36: 227 against 287) -- no barrier, no pull that leaves
   // the CTA.  A single such CTA per SM (M = 37 ... 73) is slower (M = 40: 330 against 309), so the kernel is used down to 128 threads per SM.
-  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves);
-  NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
+  for (int rounds : {4, 8, kFusedMaxRounds})
+    NM_CUDA(ctx, cudaFuncSetAttribute(pick_fused_kernel(ctx->objective, ctx->L.halves, rounds), cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      (int)cudaSharedmemCarveoutMaxShared));
+  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves, 8);  // (the instance with the most registers)
   // The head of the shared memory (draws and telemetry sums) grows with the rounds of a launch: room for as
   // many as were asked for, unless fewer let more threads live on an SM (M = 36: the last kilobytes decide
   // between two CTAs and one).
@@ -1169,7 +1180,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
       fp.inv_M = p.inv_M;
       fp.q_offset = ctx->q_offset + (uint32_t)range.q0;
       fp.keys = p.keys;
-      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves);
+      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, chunk);
       NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
       fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
       ctx->launches += 1;

@@ -187,7 +187,7 @@ struct RoundParams {
   int32_t rows_per_group;  // ceil(M / rg)
   float4* colpart;       // rg > 1: per tile, per column group, per half: (sum, sum of squares) partials
   unsigned int* coltick; // rg > 1: arrivals per column tile (0 between launches)
-  float alpha, sigma;    // sigma: the noise scale sigma sqrt(2 ln 2) (see update_core_rnd)
+  float alpha, sigma;    // sigma: the noise scale sigma sqrt(2 ln 2) (see scaled_pair)
   float inv_M;
   uint32_t round_lo, ctr3;
   uint32_t q_offset;     // Philox block index (element / 4) of the context's first element in the global vector
@@ -238,14 +238,19 @@ __device__ __forceinline__ int live_lanes(bool ragged, int tail, int h) {
 // hold x = c = 0 and so stay at exactly +0).  ta, tb return x - c for the caller's loss statistic.
 // Operand counts matter here: a packed instruction with three distinct register pairs issues every 3.2
 // cycles, one with two every 2.2 -- hence subtractions instead of multiply-adds with -1, and the product
-// with alpha as two scalar multiply-adds that take alpha from the constant bank.
-template <int kObjective>
+// with alpha as scalar multiply-adds that take alpha from the constant bank, except where a kernel is faster with fewer
+// instructions (kPairs).
+template <int kObjective, int kForm>
 __device__ __forceinline__ ulonglong2 update_core(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm, float w,
                                                   pair_t& ta, pair_t& tb) {
   ta = sub2(xv.x, cv.x);
   tb = sub2(xv.y, cv.y);
   pair_t ha = xv.x, hb = xv.y;
-  if (kObjective == 1) {
+  if (kObjective == 1 && (kForm & kPairs)) {
+    const pair_t nalpha2 = pack2(-alpha, -alpha);
+    ha = fma2(nalpha2, add2(ta, n.x), xv.x);
+    hb = fma2(nalpha2, add2(tb, n.y), xv.y);
+  } else if (kObjective == 1) {
     float g0, g1, g2, g3, x0, x1, x2, x3;
     unpack2(add2(ta, n.x), g0, g1);
     unpack2(add2(tb, n.y), g2, g3);
@@ -259,16 +264,16 @@ __device__ __forceinline__ ulonglong2 update_core(float alpha, ulonglong2 n, ulo
 }
 
 // The noise of one column group of one worker, with its Philox block drawn on the spot.
-template <int kObjective>
+template <int kObjective, int kForm>
 __device__ __forceinline__ ulonglong2 draw_noise(float sigma_s, const PhiloxKeys& keys, uint32_t iter_lo, uint32_t ctr3, uint32_t q32,
                                                  uint32_t worker, int live) {
   if (kObjective != 1) return make_ulonglong2(0ull, 0ull);
-  const ulonglong2 n = scaled_normals4(philox4x32_10(q32, worker, iter_lo, ctr3, keys), sigma_s);
+  const ulonglong2 n = scaled_normals4<kForm>(philox4x32_10(q32, worker, iter_lo, ctr3, keys), sigma_s);
   return live < 4 ? mask_lanes(n, live) : n;
 }
 
 // update_core plus the telemetry sums of the round-start values.  kObjective == 2 measures only.
-template <int kObjective>
+template <int kObjective, int kForm>
 __device__ __forceinline__ ulonglong2 row_update(float alpha, ulonglong2 n, ulonglong2 xv, ulonglong2 cv, ulonglong2 xm,
                                                  ulonglong2 pivot, float w, ColAcc& acc, LossAcc& lacc) {
   pair_t ta, tb;
@@ -277,7 +282,7 @@ __device__ __forceinline__ ulonglong2 row_update(float alpha, ulonglong2 n, ulon
     ta = sub2(xv.x, cv.x);
     tb = sub2(xv.y, cv.y);
   } else {
-    o = update_core<kObjective>(alpha, n, xv, cv, xm, w, ta, tb);
+    o = update_core<kObjective, kForm>(alpha, n, xv, cv, xm, w, ta, tb);
   }
   const pair_t da = sub2(xv.x, pivot.x), db = sub2(xv.y, pivot.y);
   acc.s1a = add2(acc.s1a, da);
@@ -501,11 +506,15 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
             ulonglong2 o;
 #pragma unroll
             for (int h = 0; h < kHalves; ++h) {
-              const ulonglong2 noise = draw_noise<kObjective>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i,
-                                                              live_lanes(ragged, p.tail, h));
-              const ulonglong2 oh = row_update<kObjective>(p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
-                                                           group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h),
-                                                           __int_as_float(pw[u].y), acc[h], lacc);
+              // (scalar products, the mantissa by shift and or: 8 x 8,388,611 elements 154.2 us per round, with the funnel
+              // shift 159.9, on pairs 172.4; padding lanes cleared behind the update: a test between the noise and the
+              // update keeps their instructions apart, 157.0)
+              const ulonglong2 noise = draw_noise<kObjective, 0>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i, 4);
+              ulonglong2 oh = row_update<kObjective, 0>(p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
+                                                        group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h),
+                                                        __int_as_float(pw[u].y), acc[h], lacc);
+              const int live = live_lanes(ragged, p.tail, h);
+              if (live < 4) oh = mask_lanes(oh, live);
               if (kHalves == 1) o = oh;
               else if (h == 0) o.x = narrow_bf16x4(oh);
               else o.y = narrow_bf16x4(oh);
@@ -734,12 +743,14 @@ struct FusedParams {
 // Dynamic shared memory: (peer row offset, weight) int2[slots][M], the warps' telemetry sums
 // double[slots][warps][2], then the slabs float4[3][M][blockDim] (replicas of even rounds, of odd rounds,
 // centres).  Any block size that is a multiple of 32 up to 256 works.
-// The telemetry of a round is added over the lanes of a warp at its end (in double) and kept per warp in shared memory: with a thread's own sums in registers a launch was limited to eight
-// rounds, and 32 registers a thread went into them.
+// The telemetry of a round is added over the lanes of a warp at its end (in double) and kept per warp in shared memory,
+// for up to 32 rounds; launches of at most kReg rounds keep a thread's own sums in registers instead, which spares a
+// round's shuffles (us per call, sums in shared memory / in registers: 2 x 33,554,435 elements, 8 rounds 939 / 884, 4
+// rounds 504 / 479; 8 x 8,388,611: 685 / 667, 365 / 359; with eight rounds' registers four rounds of bfloat16 take 2 % longer).
 __host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {
   return (uint32_t)(((uint64_t)slots * (uint64_t)(M * 8 + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);
 }
-template <int kObjective, bool kBf16>
+template <int kObjective, bool kBf16, int kReg>
 __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -752,7 +763,11 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   const uint32_t plane = (uint32_t)M * stride;   // bytes of one [M][T] slab
   unsigned char* slab = smem_raw + head + (uint32_t)tid * 16u;  // this thread's column: slabs 0, 1 (replicas), 2 (centres)
 
-  for (int k = tid; k < p.n_rounds * nwarps * 2; k += T) s_tel[k] = 0.0;
+  double acc_cons[kReg > 0 ? kReg : 1], acc_loss[kReg > 0 ? kReg : 1];
+#pragma unroll
+  for (int k = 0; k < kReg; ++k) acc_cons[k] = acc_loss[k] = 0.0;
+  if (kReg == 0)
+    for (int k = tid; k < p.n_rounds * nwarps * 2; k += T) s_tel[k] = 0.0;
   for (int k = 0; k < p.n_rounds; ++k) {
     const int32_t* peers = p.trace + ((p.slot0 + k) % p.ring) * M;
     for (int i = tid; i < M; i += T) {
@@ -845,9 +860,9 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       uint64_t goff = 0;
       auto do_row = [&](int i, uint4 rnd) {
         const int2 d = pw[i];
-        ulonglong2 noise = kObjective == 1 ? scaled_normals4(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
+        ulonglong2 noise = kObjective == 1 ? scaled_normals4<kPairs>(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
         if (kRagged) noise = mask_lanes(noise, lanes);
-        const ulonglong2 o = row_update<kObjective>(
+        const ulonglong2 o = row_update<kObjective, kPairs>(
             p.alpha, noise, *reinterpret_cast<const ulonglong2*>(cur + off), *reinterpret_cast<const ulonglong2*>(cen + off),
             *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x), pivot, __int_as_float(d.y), acc, lacc);
         if (kLast) {
@@ -887,6 +902,16 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       const double cons = (double)((s2.x - s1.x * s1.x * p.inv_M) + (s2.y - s1.y * s1.y * p.inv_M) +
                                    (s2.z - s1.z * s1.z * p.inv_M) + (s2.w - s1.w * s1.w * p.inv_M));
       const double loss = (double)((l0 + l1) + (l2 + l3));
+      if constexpr (kReg > 0) {
+#pragma unroll
+        for (int kk = 0; kk < kReg; ++kk) {  // (k is known only at run time: predicated adds keep the sums in registers)
+          if (kk == k) {
+            acc_cons[kk] += cons;
+            acc_loss[kk] += loss;
+          }
+        }
+        return;
+      }
       // lanes 0-15 go on with the one sum, lanes 16-31 with the other
       const bool low = lane < 16;
       double keep = (low ? cons : loss) + __shfl_xor_sync(0xffffffffu, low ? loss : cons, 16);
@@ -908,6 +933,18 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   }
 
   // telemetry: per round, CTA partials; the last CTA to finish sums them
+#pragma unroll
+  for (int k = 0; k < kReg; ++k) {
+    double a = acc_cons[k], b = acc_loss[k];
+    for (int off = 16; off > 0; off >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, off);
+      b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+    if (lane == 0 && k < p.n_rounds) {
+      s_tel[(k * nwarps + warp) * 2] = a;
+      s_tel[(k * nwarps + warp) * 2 + 1] = b;
+    }
+  }
   __syncthreads();
   for (int e = tid; e < p.n_rounds * 2; e += T) {
     const int k = e >> 1;
@@ -1001,9 +1038,9 @@ __global__ void __launch_bounds__(256) step_kernel(const StepParams p) {
 #pragma unroll
     for (int h = 0; h < kHalves; ++h) {
       pair_t ta, tb;
-      const ulonglong2 noise = draw_noise<kObjective>(p.sigma, p.keys, e.iter_lo, e.ctr3, (uint32_t)q * kHalves + h + p.q_offset,
+      const ulonglong2 noise = draw_noise<kObjective, kFunnel>(p.sigma, p.keys, e.iter_lo, e.ctr3, (uint32_t)q * kHalves + h + p.q_offset,
                                                       (uint32_t)e.worker, live_lanes(ragged, p.tail, h));
-      const ulonglong2 oh = update_core<kObjective>(p.alpha, noise, group_half<kHalves>(xv, h), group_half<kHalves>(cv, h),
+      const ulonglong2 oh = update_core<kObjective, kFunnel>(p.alpha, noise, group_half<kHalves>(xv, h), group_half<kHalves>(cv, h),
                                                     group_half<kHalves>(xm, h), e.w, ta, tb);
       if (kHalves == 1) o = oh;
       else if (h == 0) o.x = narrow_bf16x4(oh);
@@ -1085,7 +1122,7 @@ __global__ void __launch_bounds__(256, 2) step_tiles_kernel(const __grid_constan
       ulonglong2 v = make_ulonglong2(0ull, 0ull);
       if (kObjective == 1) {
         const uint2 ctr = s_ctr[e];
-        v = scaled_normals4(philox4x32_10(q32, ctr.x, (uint32_t)s_ev[e].w, ctr.y, p.keys), p.sigma);
+        v = scaled_normals4<kFunnel>(philox4x32_10(q32, ctr.x, (uint32_t)s_ev[e].w, ctr.y, p.keys), p.sigma);
         if (live < 4) v = mask_lanes(v, live);
       }
       return v;
@@ -1093,7 +1130,7 @@ __global__ void __launch_bounds__(256, 2) step_tiles_kernel(const __grid_constan
     auto step = [&](int e, ulonglong2 noise) {
       const int4 d = s_ev[e];
       pair_t ta, tb;
-      const ulonglong2 o = update_core<kObjective>(p.alpha, noise, *reinterpret_cast<const ulonglong2*>(x + (uint32_t)d.x),
+      const ulonglong2 o = update_core<kObjective, kFunnel>(p.alpha, noise, *reinterpret_cast<const ulonglong2*>(x + (uint32_t)d.x),
                                                    *reinterpret_cast<const ulonglong2*>(cen + (uint32_t)d.x),
                                                    *reinterpret_cast<const ulonglong2*>(x + (uint32_t)d.y), __int_as_float(d.z), ta, tb);
       *reinterpret_cast<ulonglong2*>(x + (uint32_t)d.x) = kBf16 ? widen_bf16x4(narrow_bf16x4(o)) : o;

@@ -58,10 +58,17 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
   return make_uint4(c0, c1, c2, c3);
 }
 
+// How the same operations, with the same results, are issued.  Which form is faster is each kernel's own (its registers,
+// what else it issues), so every kernel names its form beside the figures.
+constexpr int kPairs = 1;   // the last products of the noise and the step along the gradient on fp32 pairs, not as scalars
+constexpr int kFunnel = 2;  // the radius's mantissa by one funnel shift instead of a shift and an or
+
 // u1 = (top23(a) + 1/2) / 2^23 in (0,1), exactly representable in fp32:
 // bits 0x3F800000 | top23 are the float 1 + top23 / 2^23; subtracting 1 - 2^-24 is exact.
+template <int kForm = 0>
 __device__ __forceinline__ float radius_uniform(uint32_t a) {
-  // (those bits are the funnel shift of 0x7F : a by 9, one instruction)
+  if (!(kForm & kFunnel)) return __uint_as_float(0x3F800000u | (a >> 9)) - 0.99999994039535522461f;
+  // (those bits are the funnel shift of 0x7F : a by 9)
   return __uint_as_float(__funnelshift_r(a, 0x7Fu, 9)) - 0.99999994039535522461f;
 }
 
@@ -128,19 +135,21 @@ __device__ __forceinline__ pair_t sub2(pair_t a, pair_t b) {
 // return +0 or a tiny positive value for u1 next to 1, hence |.| (an operand modifier, not an
 // instruction) instead of a negation under the square root.
 constexpr double kNormalScale = 1.17741002251547469101;  // sqrt(2 ln 2)
+template <int kForm>
 __device__ __forceinline__ pair_t scaled_pair(uint32_t a, uint32_t b, float sigma_s) {
-  const float u1 = radius_uniform(a);
+  const float u1 = radius_uniform<kForm>(a);
   const float ang = (float)((int32_t)b >> 8) * 3.74507028e-07f;  // 2 pi / 2^24
   float rad;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rad) : "f"(fabsf(log2_fast(u1))));
   rad *= sigma_s;
   float s, c;
   __sincosf(ang, &s, &c);
-  return pack2(rad * c, rad * s);
+  return (kForm & kPairs) ? mul2(pack2(rad, rad), pack2(c, s)) : pack2(rad * c, rad * s);
 }
 // sigma times the four normals of a Philox block.
+template <int kForm>
 __device__ __forceinline__ ulonglong2 scaled_normals4(uint4 r, float sigma_s) {
-  return make_ulonglong2(scaled_pair(r.x, r.y, sigma_s), scaled_pair(r.z, r.w, sigma_s));
+  return make_ulonglong2(scaled_pair<kForm>(r.x, r.y, sigma_s), scaled_pair<kForm>(r.z, r.w, sigma_s));
 }
 // Clears the lanes from `live` on (padding of a row's last, ragged group).
 __device__ __forceinline__ ulonglong2 mask_lanes(ulonglong2 v, int live) {
