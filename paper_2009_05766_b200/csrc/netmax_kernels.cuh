@@ -506,9 +506,8 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
             ulonglong2 o;
 #pragma unroll
             for (int h = 0; h < kHalves; ++h) {
-              // (scalar products, the mantissa by shift and or: 8 x 8,388,611 elements 154.2 us per round, with the funnel
-              // shift 159.9, on pairs 172.4; padding lanes cleared behind the update: a test between the noise and the
-              // update keeps their instructions apart, 157.0)
+              // (the mantissa by shift and or: 8 x 8,388,611 elements 154.2 us per round, with the funnel shift 159.9; padding
+              // lanes cleared behind the update: a test between the noise and the update keeps their instructions apart, 157.0)
               const ulonglong2 noise = draw_noise<kObjective, 0>(p.sigma, p.keys, round_lo, ctr3, q32 + h, (uint32_t)i, 4);
               ulonglong2 oh = row_update<kObjective, 0>(p.alpha, noise, group_half<kHalves>(xv[u], h), group_half<kHalves>(cv[u], h),
                                                         group_half<kHalves>(xm[u], h), group_half<kHalves>(pivot, h),
@@ -745,8 +744,8 @@ struct FusedParams {
 // centres).  Any block size that is a multiple of 32 up to 256 works.
 // The telemetry of a round is added over the lanes of a warp at its end (in double) and kept per warp in shared memory,
 // for up to 32 rounds; launches of at most kReg rounds keep a thread's own sums in registers instead, which spares a
-// round's shuffles (us per call, sums in shared memory / in registers: 2 x 33,554,435 elements, 8 rounds 939 / 884, 4
-// rounds 504 / 479; 8 x 8,388,611: 685 / 667, 365 / 359; with eight rounds' registers four rounds of bfloat16 take 2 % longer).
+// round's shuffles (us per call, sums in shared memory / in registers: 2 x 33,554,435 elements, 8 rounds 961 / 916, 4
+// rounds 515 / 492; 8 x 8,388,611: 702 / 690, 371 / 367).
 __host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {
   return (uint32_t)(((uint64_t)slots * (uint64_t)(M * 8 + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);
 }
@@ -787,6 +786,10 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   // bfloat16 state arrives as the 8 stored bytes in the low half of a 16-byte slot and is widened in
   // place when the tile starts.
   constexpr bool kPrefetch = NETMAX_FUSED_PREFETCH != 0;
+  // (us per call, scalar steps / steps on pairs: fp32, 36 x 1,864,138 elements, 4 rounds 462 / 475, 8 rounds 899 / 880;
+  // 8 x 8,388,611 367 / 371, 690 / 681, 20 rounds 1,707 / 1,680; bfloat16 state 387 / 381, 721 / 706; the radius's mantissa
+  // by a funnel shift: 1 to 2 % slower throughout)
+  constexpr int kForm = kBf16 || kReg != 4 ? kPairs : 0;
   uint32_t base = 0;
   bool fetched = false;  // has this tile been fetched by the previous one?
   for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
@@ -860,9 +863,9 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       uint64_t goff = 0;
       auto do_row = [&](int i, uint4 rnd) {
         const int2 d = pw[i];
-        ulonglong2 noise = kObjective == 1 ? scaled_normals4<kPairs>(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
+        ulonglong2 noise = kObjective == 1 ? scaled_normals4<kForm>(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
         if (kRagged) noise = mask_lanes(noise, lanes);
-        const ulonglong2 o = row_update<kObjective, kPairs>(
+        const ulonglong2 o = row_update<kObjective, kForm>(
             p.alpha, noise, *reinterpret_cast<const ulonglong2*>(cur + off), *reinterpret_cast<const ulonglong2*>(cen + off),
             *reinterpret_cast<const ulonglong2*>(cur + (uint32_t)d.x), pivot, __int_as_float(d.y), acc, lacc);
         if (kLast) {

@@ -60,7 +60,7 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 
 // How the same operations, with the same results, are issued.  Which form is faster is each kernel's own (its registers,
 // what else it issues), so every kernel names its form beside the figures.
-constexpr int kPairs = 1;   // the last products of the noise and the step along the gradient on fp32 pairs, not as scalars
+constexpr int kPairs = 1;   // the step along the gradient on fp32 pairs, not as scalars
 constexpr int kFunnel = 2;  // the radius's mantissa by one funnel shift instead of a shift and an or
 
 // u1 = (top23(a) + 1/2) / 2^23 in (0,1), exactly representable in fp32:
@@ -111,11 +111,6 @@ __device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-__device__ __forceinline__ pair_t mul2(pair_t a, pair_t b) {
-  pair_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 __device__ __forceinline__ pair_t add2(pair_t a, pair_t b) {
   pair_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -144,7 +139,7 @@ __device__ __forceinline__ pair_t scaled_pair(uint32_t a, uint32_t b, float sigm
   rad *= sigma_s;
   float s, c;
   __sincosf(ang, &s, &c);
-  return (kForm & kPairs) ? mul2(pack2(rad, rad), pack2(c, s)) : pack2(rad * c, rad * s);
+  return pack2(rad * c, rad * s);  // (not on pairs: the compiler contracts a packed product with the sum that follows, other bits)
 }
 // sigma times the four normals of a Philox block.
 template <int kForm>

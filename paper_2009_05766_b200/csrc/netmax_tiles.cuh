@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
       load_draws(draw);
     }
   };
-  // (scalar products and the funnel shift: without it 4096 x 1024 elements take 19 % longer, on pairs 23 %)
+  // (scalar steps and the funnel shift: without it 4096 x 1024 elements take 19 % longer)
   auto next_noise = [&](int64_t q, int k) {
     if (kObjective != 1) return;
     const uint64_t round = p.first_round + (uint64_t)k;
