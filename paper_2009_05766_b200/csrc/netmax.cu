@@ -231,8 +231,14 @@ struct netmax_ctx {
   float* wtab = nullptr;
   int32_t* trace = nullptr;
   int2* draws = nullptr;  // (peer, bits of the pull weight) of every draw in the trace ring
-  double* tel = nullptr;  // telemetry ring: in page-locked host memory (tel_on_host) or, when it is long, on the device
-  bool tel_on_host = false;
+  // A program that looks at telemetry or peers after every call finds them in page-locked host memory; the writes there
+  // cost the launches about 2 us (8 x 524,291 elements: 18.8 us per round, 20.8), so only the rounds of a call that
+  // follows such a look go there (and the first call's).  on_host says it for every slot of the rings.
+  double *tel_dev = nullptr, *tel_host = nullptr;  // telemetry rings; tel_host only where it is short enough
+  double* tel = nullptr;                           // the one of the two that the present call's rounds go to
+  bool tel_read = true, trace_read = true;         // looked at since the last call that ran rounds
+  bool trace_now = false;                          // the present call's peers go to trace_mirror as well
+  std::vector<uint8_t> on_host;                    // [trace_rounds]: 1 telemetry, 2 peers
   double* partials = nullptr;
   unsigned int* ticket = nullptr;
   float4* colpart = nullptr;
@@ -607,7 +613,7 @@ int launch_sampler(netmax_ctx* ctx, uint64_t first_round, int64_t n_rounds, int3
   p.last_nz = ctx->last_nz;
   p.out = out;
   p.draws = draws;
-  p.host_out = draws ? ctx->trace_mirror : nullptr;  // (draws into the context's own ring)
+  p.host_out = draws && ctx->trace_now ? ctx->trace_mirror : nullptr;  // (draws into the context's own ring)
   p.wtab = ctx->wtab;
   p.slot0 = slot0;
   p.ring = ring;
@@ -1350,7 +1356,7 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) try {
   ctx->wtab = (float*)(ctx->base + L.off_w);
   ctx->trace = (int32_t*)(ctx->base + L.off_trace);
   ctx->draws = (int2*)(ctx->base + L.off_draws);
-  ctx->tel = (double*)(ctx->base + L.off_tel);
+  ctx->tel_dev = (double*)(ctx->base + L.off_tel);
   ctx->partials = (double*)(ctx->base + L.off_partials);
   ctx->ticket = (unsigned int*)(ctx->base + L.off_ticket);
   ctx->colpart = (float4*)(ctx->base + L.off_colpart);
@@ -1359,17 +1365,17 @@ int netmax_create_ex(const netmax_config* cfg, netmax_ctx** out) try {
   ctx->dev_error = (volatile unsigned int*)ctx->pinned;
   ctx->measure_out = (double*)(ctx->pinned + 64);
   if ((size_t)ctx->trace_rounds * 16 <= kPinnedTrace - kPinnedTel) {
-    ctx->tel = (double*)(ctx->pinned + kPinnedTel);
-    ctx->tel_on_host = true;
+    ctx->tel_host = (double*)(ctx->pinned + kPinnedTel);
   }
   if ((size_t)ctx->trace_rounds * ctx->M * 4 <= kPinnedStaging - kPinnedTrace) ctx->trace_mirror = (int32_t*)(ctx->pinned + kPinnedTrace);
+  if (ctx->tel_host || ctx->trace_mirror) ctx->on_host.assign((size_t)ctx->trace_rounds, 0);
   ctx->coltick = (unsigned int*)(ctx->base + L.off_coltick);
   ctx->pipe_tel = (double*)(ctx->base + L.off_pipe_tel);
 
   if (!step(cudaMemsetAsync(ctx->ticket, 0, 256, ctx->stream), "cudaMemsetAsync(ticket)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->coltick, 0, (size_t)kMaxGrid * sizeof(unsigned int), ctx->stream), "cudaMemsetAsync(coltick)")) return bail(NETMAX_CUDA_ERROR);
   if (!step(cudaMemsetAsync(ctx->x[1], 0, L.plane, ctx->stream), "cudaMemsetAsync(x)")) return bail(NETMAX_CUDA_ERROR);
-  if (!ctx->tel_on_host && !step(cudaMemsetAsync(ctx->tel, 0, (size_t)ctx->trace_rounds * 2 * sizeof(double), ctx->stream), "cudaMemsetAsync(tel)")) return bail(NETMAX_CUDA_ERROR);
+  if (!step(cudaMemsetAsync(ctx->tel_dev, 0, (size_t)ctx->trace_rounds * 2 * sizeof(double), ctx->stream), "cudaMemsetAsync(tel)")) return bail(NETMAX_CUDA_ERROR);
   rc = upload_policy(ctx);
   if (rc) return bail(rc);
   rc = launch_init(ctx, ctx->x[0], cfg->x0_std, kTagX0);
@@ -1628,6 +1634,19 @@ int netmax_read_replicas(netmax_ctx* ctx, float* host_out) {
 }
 int netmax_read_centres(netmax_ctx* ctx, float* host_out) { return copy_out(ctx, ctx ? ctx->c : nullptr, host_out); }
 
+// Where the telemetry and the peers of the n rounds that follow go (see on_host).
+static void choose_rings(netmax_ctx* ctx, int64_t n) {
+  const bool tel = ctx->tel_host && ctx->tel_read;
+  ctx->trace_now = ctx->trace_mirror && ctx->trace_read;
+  ctx->tel = tel ? ctx->tel_host : ctx->tel_dev;
+  ctx->tel_read = ctx->trace_read = false;
+  if (ctx->on_host.empty()) return;
+  const uint8_t mark = (uint8_t)((tel ? 1 : 0) | (ctx->trace_now ? 2 : 0));
+  const int64_t ring = ctx->trace_rounds, count = std::min(n, ring), at = (ctx->rounds + n - count) % ring, first = std::min(count, ring - at);
+  std::memset(ctx->on_host.data() + at, mark, (size_t)first);
+  std::memset(ctx->on_host.data(), mark, (size_t)(count - first));
+}
+
 int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (n_rounds < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_rounds = %lld < 0", (long long)n_rounds);
@@ -1647,6 +1666,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   rc = plan_tiles(ctx, plan, fused, tiles);
   if (rc) return rc;
 
+  choose_rings(ctx, n_rounds);
   RoundParams p = make_round_params(ctx, plan);
 
   // A program that reads small replicas after every call gets them with the rounds: the last launch writes them to
@@ -1804,6 +1824,7 @@ int netmax_round_from_host(netmax_ctx* ctx, const float* host_x, const float* ho
   } while (0)
 
   const uint64_t first = (uint64_t)ctx->rounds;
+  choose_rings(ctx, n_rounds);
   ctx->host_writes = true;
   ctx->staged = false;
   rc = launch_sampler(ctx, first, n_rounds, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds, ctx->trace_rounds);
@@ -1970,7 +1991,10 @@ int netmax_peer_trace(netmax_ctx* ctx, int64_t first_round, int64_t n, int32_t* 
   if (n == 0) return NETMAX_OK;
   if (!host_out) return fail(ctx, NETMAX_INVALID_ARG, "host_out is NULL");
   DeviceGuard guard(ctx->device);
-  if (ctx->trace_mirror) {
+  ctx->trace_read = true;
+  bool mirrored = ctx->trace_mirror != nullptr;
+  for (int64_t r = first_round; mirrored && r < first_round + n; ++r) mirrored = (ctx->on_host[(size_t)(r % ctx->trace_rounds)] & 2) != 0;
+  if (mirrored) {
     rc = synchronise(ctx);
     if (rc) return rc;
   }
@@ -1980,7 +2004,7 @@ int netmax_peer_trace(netmax_ctx* ctx, int64_t first_round, int64_t n, int32_t* 
     const int64_t slot = r % ctx->trace_rounds;
     const int64_t piece = std::min<int64_t>(first_round + n - r, ctx->trace_rounds - slot);
     int32_t* out = host_out + (size_t)(r - first_round) * ctx->M;
-    if (ctx->trace_mirror) std::memcpy(out, ctx->trace_mirror + (size_t)slot * ctx->M, piece * row);
+    if (mirrored) std::memcpy(out, ctx->trace_mirror + (size_t)slot * ctx->M, piece * row);
     else if ((rc = read_back(ctx, out, ctx->trace + (size_t)slot * ctx->M, piece * row)) != NETMAX_OK) return rc;
     r += piece;
   }
@@ -1993,18 +2017,21 @@ int netmax_telemetry(netmax_ctx* ctx, int64_t first_round, int64_t n, double* ho
   if (rc) return rc;
   if (n == 0) return NETMAX_OK;
   DeviceGuard guard(ctx->device);
+  ctx->tel_read = true;
+  auto in_host = [&](int64_t slot) { return ctx->tel_host && (ctx->on_host[(size_t)slot] & 1); };
+  bool all = true;
+  for (int64_t k = 0; all && k < n; ++k) all = in_host((first_round + k) % ctx->trace_rounds);
   std::vector<double> copy;
-  const double* ring = ctx->tel;
-  if (ctx->tel_on_host) {
+  if (all) {
     rc = synchronise(ctx);
   } else {
     copy.resize((size_t)ctx->trace_rounds * 2);
-    rc = read_back(ctx, copy.data(), ctx->tel, copy.size() * sizeof(double));
-    ring = copy.data();
+    rc = read_back(ctx, copy.data(), ctx->tel_dev, copy.size() * sizeof(double));
   }
   if (rc) return rc;
   for (int64_t k = 0; k < n; ++k) {
     const int64_t slot = (first_round + k) % ctx->trace_rounds;
+    const double* ring = in_host(slot) ? ctx->tel_host : copy.data();
     if (host_consensus) host_consensus[k] = ring[2 * slot];
     if (host_loss) host_loss[k] = ring[2 * slot + 1];
   }

@@ -231,3 +231,28 @@ def test_replicas_changed_on_the_device_are_what_is_read(nm, when, own_workspace
         same.set_replicas(want)
     g.close()
     same.close()
+
+
+@pytest.mark.parametrize("M,d,ring", [(4, 1003, 16), (3, 400_003, 16), (70, 260, 7)])
+def test_telemetry_and_peers_do_not_depend_on_when_they_are_looked_at(nm, M, d, ring):
+    """Rounds of a call that follows a look leave telemetry and peers in host memory, others on the device: whatever the
+    order of looks, every round that is still in the ring reads the same."""
+    kw = dict(M=M, d=d, lr=0.05, prob=random_policy(M, np.random.default_rng(M)), sigma=0.1, x0_std=1.0, c_std=1.0, seed=9, trace_rounds=ring)
+    never, always, some = nm.Netmax(**kw), nm.Netmax(**kw), nm.Netmax(**kw)
+    for k, n in enumerate((2, 1, 5, 3, 2, 1, 4, 2 * ring + 3, 1, 6)):
+        for g in (never, always, some):
+            g.round(n)
+        first = max(0, never.rounds_done - ring)
+        if k % 3 == 2:
+            some.telemetry(first, 1)
+        if k % 4 == 1:
+            some.peer_trace(first, 1)
+        always.telemetry(first, 1)
+        always.peer_trace(first, 1)
+    want = never.telemetry(first, ring), never.peer_trace(first, ring)
+    for g in (always, some):
+        assert (g.peer_trace(first, ring) == want[1]).all()
+        for got, ref in zip(g.telemetry(first, ring), want[0]):
+            np.testing.assert_allclose(got, ref, rtol=1e-12)
+    for g in (never, always, some):
+        g.close()
