@@ -2321,8 +2321,14 @@ static StepTilePlan plan_step_tiles(const netmax_ctx* ctx) {
   const double items = (double)nq / 32.0 / (4.0 * ctx->sm_count), bytes = (double)ctx->d * ctx->L.elem;
   f.tile_us = std::max(1.0, items) * std::max(172.0, 480.0 / std::min(1.0 * std::max(1.0, best_warps / 4.0), std::max(1.0, items))) / 1965.0;
   if (best_warps < 4 && items > 1.0) f.tile_us *= 4.0 / (double)best_warps;  // (schedulers without a warp)
+  // Narrow CTAs, one or two to an SM (many workers): every lap is a thread's chain of steps, and its rows come in one after
+  // the other, four bfloat16 ones at a time (100 workers, 64 steps of 41,946 elements in two laps: 77 us in bfloat16 and 42
+  // in fp32 against 33 in launches of disjoint steps; 64 workers, 16 steps of 4,099: 20 against 13).
+  const double laps = std::ceil((double)((nq + f.threads - 1) / f.threads) / (double)(f.per_sm * ctx->sm_count));
+  f.tile_us = std::max(f.tile_us, laps * 480.0 / 1965.0 * (best_warps <= 4 ? 1.0 : 4.0 / (double)best_warps));
   f.step_us = std::max(0.5, 4.0 * bytes / 6.2e6);
-  f.load_us = 3.0 + 2.2 * (double)M * bytes / 6.2e6;  // (12 M bytes, a quarter of it beside the steps)
+  // (12 M bytes, a quarter of it beside the steps; or the rows' latencies)
+  f.load_us = 3.0 + std::max(2.2 * (double)M * bytes / 6.2e6, laps * (double)M * (ctx->L.halves == 2 ? 0.25 : 0.08));
   return f;
 }
 
