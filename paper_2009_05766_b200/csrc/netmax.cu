@@ -912,8 +912,10 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
     f.min_rounds = 2;
     f.max_rounds = std::min<int64_t>(f.max_rounds, ctx->fuse_rounds);
   } else {
-    // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the worker
-    // counts the header says so for; longer ones are where resident tiles gain most.
+    // fp32 state with more than 66 workers: calls of up to eight rounds keep to one launch per round at the worker counts
+    // the header names.  That line is older than this kernel: it was drawn where rows split over a cluster of CTAs were no
+    // faster.  This kernel is (nine rounds, 93 to 700 workers: 1.5 to 2 times; 64 workers, two to eight rounds: 1.2 to 1.5
+    // times), and such calls forgo that.
     static const unsigned char fused_short[22] = {0, 1, 1, 1, 0, 1, 1, 1, 1, 1, 1, 0, 0, 1, 0, 0, 0, 1, 1, 1, 1, 1};  // M = 67 ... 88
     const bool short_calls = M <= 66 || (M <= 88 && fused_short[M - 67]);
     // bfloat16 state: the tiles' narrow pieces are half as long, and the per-round kernel is nearer (one launch per round

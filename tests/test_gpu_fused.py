@@ -83,13 +83,13 @@ def test_fused_rounds_change_no_bit(nm, M, d, fuse, storage, objective):
 
 
 # more workers than the 128- and 256-thread CTAs hold: 64-thread CTAs of the same kernel up to M = 36 (19, 20, 24: three
-# per SM; 25, 33, 35: two), beyond that the rows of a tile are split over the CTAs of a cluster (M = 44 -> 4 CTAs;
-# 50 -> 5; 47, 57 -> 6; 56, 70 -> 7; 64, 100, 136 -> 8; ragged last CTAs, one with no row at all)
+# per SM; 25, 33, 35: two), beyond that the rows of a tile are shared out over
+# a CTA's threads
 @pytest.mark.parametrize("M,d,fuse", [(64, 80_003, 0), (20, 303_201, 0), (33, 152_002, 3), (100, 38_001, 4), (136, 40_001, 2),
                                       (19, 310_000, 4), (24, 303_203, 0), (25, 160_001, 0), (44, 160_002, 0), (50, 80_001, 2),
                                       (57, 80_003, 0), (35, 160_003, 0), (47, 160_001, 0), (56, 80_001, 0), (70, 80_002, 0)])
 @pytest.mark.parametrize("objective", [0, 1])
-def test_cluster_resident_rounds_change_no_bit(nm, M, d, fuse, objective):
+def test_rounds_on_shared_rows_change_no_bit(nm, M, d, fuse, objective):
     rng = np.random.default_rng(M * 7 + d)
     P = random_policy(M, rng, zeros=0.3)
     kw = dict(M=M, d=d, lr=0.05, prob=P, sigma=0.1, x0_std=1.0, c_std=1.0, objective=objective, seed=d + M, trace_rounds=64)
@@ -106,16 +106,15 @@ def test_cluster_resident_rounds_change_no_bit(nm, M, d, fuse, objective):
     assert (one.read_replicas().view(np.uint32) == many.read_replicas().view(np.uint32)).all()
     assert (one.peer_trace(0, rounds) == many.peer_trace(0, rounds)).all()
     (ca, la), (cb, lb) = one.telemetry(0, rounds), many.telemetry(0, rounds)
-    np.testing.assert_allclose(cb, ca, rtol=2e-6)      # the column sums are added CTA by CTA here: fp32 rounding of partial sums
+    np.testing.assert_allclose(cb, ca, rtol=2e-6)      # the column sums are added thread by thread here: fp32 rounding of partial sums
     np.testing.assert_allclose(lb, la, rtol=1e-6)
     one.close()
     many.close()
 
 
-def test_cluster_shape_is_taken_only_where_it_pays(nm):
-    """fuse_rounds = 0 fuses rounds for the worker counts where that was measured faster (in one CTA up to 36, over a
-    cluster for 37 ... 66 and most of 68 ... 88) and runs one launch per round elsewhere; fuse_rounds >= 2 fuses
-    wherever the rows fit (M <= 144)."""
+def test_calls_of_eight_rounds_keep_to_the_counts_the_header_names(nm):
+    """fuse_rounds = 0 fuses the eight rounds of a call up to 66 workers and at most counts up to 88, and runs one launch per
+    round elsewhere; fuse_rounds >= 2 fuses up to 144."""
     d = 400_001
     for M, fuse, fused in ((22, 0, True), (40, 0, True), (50, 0, True), (67, 0, False), (67, 4, True), (60, 0, True),
                            (81, 0, False), (81, 3, True), (100, 0, False), (150, 4, False)):
@@ -130,9 +129,9 @@ def test_cluster_shape_is_taken_only_where_it_pays(nm):
         g.close()
 
 
-# 64-thread CTAs of the single-CTA kernel (M = 28), clusters of 6, 7 and 8 CTAs
+# a column per thread in 64-thread CTAs (M = 28), rows shared out over the threads
 @pytest.mark.parametrize("M,d", [(64, 80_003), (28, 160_003), (48, 80_001), (56, 80_002)])
-def test_cluster_resident_rounds_match_the_oracle(nm, M, d):
+def test_rounds_on_shared_rows_match_the_oracle(nm, M, d):
     rng = np.random.default_rng(M + d)
     P = random_policy(M, rng, zeros=0.2)
     g = nm.Netmax(M=M, d=d, lr=0.05, prob=P, sigma=0.1, x0_std=1.0, c_std=1.0, objective=1, seed=7, trace_rounds=32)

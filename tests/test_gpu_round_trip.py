@@ -24,7 +24,7 @@ def random_policy(M, rng):
     return P / P.sum(axis=1, keepdims=True)
 
 
-# (M, d, fuse_rounds, storage, chunks): fused tiles, one launch per round, cluster-resident tiles, a ragged
+# (M, d, fuse_rounds, storage, chunks): fused tiles, one launch per round, tiles with shared rows, a ragged
 # tail, a chunk count that does not divide the vector, and the shapes that fall back to the plain sequence
 CASES = [(8, 400_003, 0, "f32", 0), (8, 400_003, 1, "f32", 5), (3, 310_001, 0, "f32", 32), (64, 90_002, 0, "f32", 3),
          (16, 330_000, 3, "f32", 7), (5, 4_099, 0, "f32", 4), (8, 700_003, 0, "bf16", 4)]
