@@ -2298,7 +2298,10 @@ struct StepTilePlan {
   int threads = 0;
   int64_t per_sm = 0;
   double tile_us = 0, step_us = 0, load_us = 0;
-  bool pays(int64_t steps) const { return threads > 0 && (double)steps * (step_us - tile_us) > load_us; }
+  bool pays(int64_t steps) const {  // (every launch brings the rows in)
+    const int64_t launches = (steps + kStepTileEvents - 1) / kStepTileEvents;
+    return threads > 0 && (double)steps * (step_us - tile_us) > (double)launches * load_us;
+  }
 };
 static StepTilePlan plan_step_tiles(const netmax_ctx* ctx) {
   StepTilePlan f;
@@ -2356,7 +2359,7 @@ static int enqueue_steps(netmax_ctx* ctx, std::vector<StepEvent>& events, const 
     const size_t slabs = (size_t)32 * ctx->M * threads;
     NM_CUDA(ctx, allow_smem((const void*)kernel, step_tile_head(kStepTileEvents, ctx->M) + slabs));
     const unsigned grid = (unsigned)std::min<int64_t>(p.n_tiles, plan.per_sm * ctx->sm_count);
-    while (plan.pays(n - done)) {
+    while (done < n) {
       const int64_t launches_left = (n - done + kStepTileEvents - 1) / kStepTileEvents;  // launches of even length
       p.n_events = (int32_t)((n - done + launches_left - 1) / launches_left);
       std::memcpy(p.ev, events.data() + done, p.n_events * sizeof(StepEvent));
