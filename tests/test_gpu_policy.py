@@ -100,7 +100,7 @@ def test_policy_change_without_device_memory_to_spare(nm):
     """A program that has handed out all device memory: the matrices of Algorithm 3 have no room there, the policy is
     generated on the host."""
     import torch
-    M, d = 400, 64
+    M, d = 1000, 64      # matrices of 8 MB, five of them
     rng = np.random.default_rng(8)
     speeds = [np.triu(np.exp(rng.uniform(0.0, 4.0, (M, M))), 1) for _ in range(2)]
     speeds = [s + s.T for s in speeds]
@@ -123,7 +123,7 @@ def test_policy_change_without_device_memory_to_spare(nm):
                 held.append(torch.cuda.caching_allocator_alloc(step))
             except torch.cuda.OutOfMemoryError:
                 step >>= 1
-        assert cudart.cudaMemGetInfo(0)[0] < 8 << 20
+        assert cudart.cudaMemGetInfo(0)[0] < 24 << 20     # (the allocator takes memory in pieces of 20 MB)
         g.set_policy(link_speed_gbps=speeds[1])
     finally:
         for p in held:
