@@ -57,24 +57,25 @@ KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh", "n
 NCU_HASH = "cf6c10a5122c6103"
 NCU_COUNTERS = {
     # (workload tag, kernel): dram bytes per element-launch, warp instructions per element-round, captured on
-    # (the per-round kernel's bytes on cfg2 are an earlier capture's; the latest one read 1,046,194,000)
-    ("cfg2_M8_resnet18", "round_kernel"): (1_041_843_000 / 89_391_696, 85_571_066 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_042_876_000 / 89_391_696, 670_157_455 / (89_391_696 * 8), "cfg2"),
-    ("cfg2_M8_resnet18/bf16", "round_kernel"): (507_162_000 / 89_391_696, 88_428_295 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (507_691_000 / 89_391_696, 722_424_204 / (89_391_696 * 8), "cfg2"),
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (1_502_230_000 / (16 * 8_000_002), 881_740_913 / (16 * 8_000_002 * 8), "cfg3 at d = 8,000,002"),
-    ("cfg3_M16_vgg19scale", "round_kernel"): (1_567_855_000 / (16 * 8_000_002), 111_945_198 / (16 * 8_000_002), "cfg3 at d = 8,000,002"),
-    ("cfg4_M64_resnet18", "tile_rounds_kernel"): (1_507_134_000 / (64 * 2_000_002), 1_239_779_448 / (64 * 2_000_002 * 10), "cfg4 at d = 2,000,002"),
-    ("cfg4_M64_resnet18", "round_kernel"): (1_557_018_000 / (64 * 2_000_002), 114_685_198 / (64 * 2_000_002), "cfg4 at d = 2,000,002"),
+    # (the per-round kernel's bytes on cfg2 are an earlier capture's; the latest one read 1,043,920,000)
+    ("cfg2_M8_resnet18", "round_kernel"): (1_041_843_000 / 89_391_696, 81_710_869 / 89_391_696, "cfg2"),
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_042_759_000 / 89_391_696, 1_560_426_213 / (89_391_696 * 20), "cfg2"),
+    ("cfg2_M8_resnet18/bf16", "round_kernel"): (508_386_000 / 89_391_696, 89_434_662 / 89_391_696, "cfg2"),
+    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (507_715_000 / 89_391_696, 681_139_124 / (89_391_696 * 8), "cfg2"),
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (1_503_016_000 / (16 * 8_000_002), 2_046_395_919 / (16 * 8_000_002 * 20), "cfg3 at d = 8,000,002"),
+    ("cfg3_M16_vgg19scale", "round_kernel"): (1_544_316_000 / (16 * 8_000_002), 107_175_885 / (16 * 8_000_002), "cfg3 at d = 8,000,002"),
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): (1_507_538_000 / (64 * 2_000_002), 1_245_561_983 / (64 * 2_000_002 * 10), "cfg4 at d = 2,000,002"),
+    ("cfg4_M64_resnet18", "round_kernel"): (1_536_297_000 / (64 * 2_000_002), 109_914_862 / (64 * 2_000_002), "cfg4 at d = 2,000,002"),
     ("cfg1_M4_d4096", "tile_rounds_kernel"): (None, 31_031_584 / (16_384 * 1000), "cfg1"),
-    ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_729_561_508 / (4_194_304 * 1000), "cfg5"),
+    ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_729_561_215 / (4_194_304 * 1000), "cfg5"),
 }
-# Busy fractions (of active SM cycles) of the issue slots and of the arithmetic pipes, from the same captures:
+# Issue slots used and instructions issued to the arithmetic pipes, as fractions of their peaks over active SM cycles, from the
+# same captures (wide multiplies hold the fmaheavy pipe for longer than they take to issue):
 # which unit a launch that is bound by instruction issue leans on hardest.
 NCU_PIPES = {
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.637, "fmaheavy": 0.643, "alu": 0.422, "captured_on": "cfg2"},
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.583, "fmaheavy": 0.620, "alu": 0.381, "captured_on": "cfg3 at d = 8,000,002"},
-    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.587, "fmaheavy": 0.628, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.617, "fmaheavy": 0.472, "alu": 0.400, "captured_on": "cfg2"},
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.563, "fmaheavy": 0.451, "alu": 0.360, "captured_on": "cfg3 at d = 8,000,002"},
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.586, "fmaheavy": 0.457, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
 }
 SM_COUNT, SCHEDULERS_PER_SM = 148, 4     # one warp instruction per scheduler and clock at most
 
