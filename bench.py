@@ -69,13 +69,13 @@ NCU_COUNTERS = {
     ("cfg1_M4_d4096", "tile_rounds_kernel"): (None, 31_031_584 / (16_384 * 1000), "cfg1"),
     ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_729_561_215 / (4_194_304 * 1000), "cfg5"),
 }
-# Issue slots used and instructions issued to the arithmetic pipes, as fractions of their peaks over active SM cycles, from the
-# same captures (wide multiplies hold the fmaheavy pipe for longer than they take to issue):
-# which unit a launch that is bound by instruction issue leans on hardest.
+# Busy fractions (of active SM cycles) of the issue slots and of the arithmetic pipes: which unit a launch that is bound by
+# instruction issue leans on hardest.  Issue slots and alu from the same captures; fmaheavy, the cycles that wide multiplies
+# hold it for, from an earlier one with the same multiplies per element.
 NCU_PIPES = {
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.617, "fmaheavy": 0.472, "alu": 0.400, "captured_on": "cfg2"},
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.563, "fmaheavy": 0.451, "alu": 0.360, "captured_on": "cfg3 at d = 8,000,002"},
-    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.586, "fmaheavy": 0.457, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.617, "fmaheavy": 0.643, "alu": 0.400, "captured_on": "cfg2"},
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.563, "fmaheavy": 0.620, "alu": 0.360, "captured_on": "cfg3 at d = 8,000,002"},
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.586, "fmaheavy": 0.628, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
 }
 SM_COUNT, SCHEDULERS_PER_SM = 148, 4     # one warp instruction per scheduler and clock at most
 
