@@ -672,6 +672,9 @@ template <int kHalves>
 RoundKernel pick_kernel_h(int objective, bool short_vectors) {
   if (objective == 2) return short_vectors ? round_kernel<2, 4, kHalves> : round_kernel<2, 1, kHalves>;
   if (short_vectors) return objective == 1 ? round_kernel<1, 4, kHalves> : round_kernel<0, 4, kHalves>;
+#ifdef NETMAX_BF16_LONG_RIF
+  if (kHalves == 2) return objective == 1 ? round_kernel<1, NETMAX_BF16_LONG_RIF, kHalves> : round_kernel<0, NETMAX_BF16_LONG_RIF, kHalves>;
+#endif
   return objective == 1 ? round_kernel<1, 1, kHalves> : round_kernel<0, 1, kHalves>;
 }
 RoundKernel pick_kernel(int objective, bool short_vectors, int halves) {
@@ -938,6 +941,9 @@ int plan_tiles(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, T
 int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   f = FusedPlan();
   if (ctx->fuse_rounds == 1 || plan.short_vectors) return NETMAX_OK;
+#ifdef NETMAX_FUSED_MAX_M
+  if (ctx->M > NETMAX_FUSED_MAX_M) return NETMAX_OK;
+#endif
   const int64_t M = ctx->M;
   // (two and three workers: a round is too short to hide its sums' shuffles, and launches of more than eight rounds lose
   // 1.5 %; four workers: as fast)

@@ -410,8 +410,12 @@ __device__ __forceinline__ void finalize_rounds(const double* partials, int n_ro
 // c and on the output measured slower.
 // Dynamic shared memory: (peer, weight) int2[M], then (rl > 1) 2 * kHalves * blockDim float4 of
 // column-sum scratch, then 64 doubles for the block reduction.
-constexpr int kRoundMinCtas = 4;  // CTAs per SM the register allocation leaves room for
-constexpr int kRoundMinCtasBf16 = 2;  // bfloat16 state: eight elements per thread; measured 152 us (2), 161 (3), 157 (4) per cfg2 round
+#ifndef NETMAX_ROUND_MIN_CTAS
+#define NETMAX_ROUND_MIN_CTAS 4  // CTAs per SM the register allocation leaves room for
+#endif
+#ifndef NETMAX_ROUND_MIN_CTAS_BF16
+#define NETMAX_ROUND_MIN_CTAS_BF16 2  // bfloat16 state: eight elements per thread; measured 152 us (2), 161 (3), 157 (4) per cfg2 round
+#endif
 
 // kRowsInFlight = 1 (64 registers, 4 CTAs/SM) is the streaming shape for long vectors, where
 // occupancy hides the HBM latency; kRowsInFlight = 4 (2 CTAs/SM) serves short, L2-resident
@@ -600,7 +604,7 @@ __device__ __forceinline__ void round_tiles(const RoundParams& p, const float4* 
 // occupancy hides the HBM latency; kRowsInFlight = 4 (2 CTAs/SM) serves short, L2-resident
 // problems, where a thread's chain of dependent row loads is what takes the time.
 template <int kObjective, int kRowsInFlight, int kHalves>
-__global__ void __launch_bounds__(256, kRowsInFlight != 1 ? 2 : kHalves == 1 ? kRoundMinCtas : kRoundMinCtasBf16)
+__global__ void __launch_bounds__(256, kRowsInFlight != 1 ? 2 : kHalves == 1 ? NETMAX_ROUND_MIN_CTAS : NETMAX_ROUND_MIN_CTAS_BF16)
     round_kernel(const RoundParams p) {
   if (kRowsInFlight != 1) wait_for_previous();
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -705,8 +709,14 @@ __global__ void __launch_bounds__(256, 2) multi_round_kernel(const MultiRoundPar
 // thread's column group is four bfloat16 values (8 bytes of global memory), widened on the way
 // in, and every round's result is rounded to bfloat16 before it is written to the slab, exactly
 // as a store to and a load from the bfloat16 state would.
+#ifndef NETMAX_FUSED_UNROLL
+#define NETMAX_FUSED_UNROLL 2
+#endif
+#ifndef NETMAX_FUSED_PREFETCH
+#define NETMAX_FUSED_PREFETCH 1  // fetch the next tile under the last round of the current one (fp32 state)
+#endif
 constexpr int kFusedMaxRounds = 32;  // rounds per launch of fused_rounds_kernel, at most
-constexpr int kFusedUnroll = 2;  // rows of a round in flight per thread
+constexpr int kFusedUnroll = NETMAX_FUSED_UNROLL;  // rows of a round in flight per thread
 
 struct FusedParams {
   const float4* x_cur;   // [M][ldq] replicas at the start of the first round
@@ -775,6 +785,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   // read and written by its own thread only, so cp.async.wait_all is all the synchronisation needed.
   // bfloat16 state arrives as the 8 stored bytes in the low half of a 16-byte slot and is widened in
   // place when the tile starts.
+  constexpr bool kPrefetch = NETMAX_FUSED_PREFETCH != 0;
   // (us per call, scalar steps / steps on pairs: fp32, 36 x 1,864,138 elements, 4 rounds 462 / 475, 8 rounds 899 / 880;
   // 8 x 8,388,611 367 / 371, 690 / 681, 20 rounds 1,707 / 1,680; bfloat16 state 387 / 381, 721 / 706; the radius's mantissa
   // by a funnel shift: 1 to 2 % slower throughout)
@@ -787,7 +798,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     const int lanes = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
     const uint32_t q32 = (uint32_t)q + p.q_offset;
     const int64_t q_next = q + (int64_t)gridDim.x * T;
-    const bool have_next = tile + gridDim.x < p.n_tiles && q_next < p.nq;
+    const bool have_next = kPrefetch && tile + gridDim.x < p.n_tiles && q_next < p.nq;
     if (fetched) {
       cp_async_wait_all();
       if (kBf16) {

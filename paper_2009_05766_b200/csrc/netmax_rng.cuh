@@ -75,9 +75,13 @@ __device__ __forceinline__ float radius_uniform(uint32_t a) {
 // Hardware log2 of a normal number (u1 >= 2^-24 here, so flushing subnormals changes nothing
 // and saves the subnormal-input handling around the instruction).
 __device__ __forceinline__ float log2_fast(float v) {
+#ifdef NETMAX_LG2_NO_FTZ
+  return __log2f(v);
+#else
   float r;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
   return r;
+#endif
 }
 
 // Accurate pair (library logf / sincospif / sqrtf): used where speed does not matter.
