@@ -169,6 +169,9 @@ int netmax_set_centres(netmax_ctx* ctx, const float* host_c);
  * shared-memory-resident columns: CTAs own disjoint columns and never exchange anything.  A call
  * has to run enough rounds to repay bringing the columns on chip (2 for up to a million elements,
  * up to 16 for the largest problems); shorter calls take the per-round kernels.
+ * Small problems of up to 100 workers (the rows of a column group or more in one warp's registers; up to about ten warps'
+ * worth per SM) run calls of four rounds and more (eight from 65 workers on) in a form of this in which other warps draw the
+ * noise and add up the telemetry.
  * Other short-vector shapes (and fuse_rounds = 1) run all rounds of a call in one cooperative
  * launch with a grid-wide barrier per round; its waits are bounded, and one that runs out is
  * reported by the next synchronising call as NETMAX_CUDA_ERROR (the replicas are then not

@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnetmax.so")
 SOURCES = ["netmax.cu", "netmax_policy.cpp", "netmax_policy_gpu.cu"]
-DEPS = SOURCES + ["netmax_policy_gpu_host.inc", "netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh", "netmax_search.h", "netmax_policy.h", "netmax_bulk.h", os.path.join("..", "..", "include", "netmax.h")]
+DEPS = SOURCES + ["netmax_policy_gpu_host.inc", "netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_search.h", "netmax_policy.h", "netmax_bulk.h", os.path.join("..", "..", "include", "netmax.h")]
 
 
 def _nvcc() -> str:

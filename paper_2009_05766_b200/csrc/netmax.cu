@@ -23,6 +23,7 @@
 
 #include "netmax_kernels.cuh"
 #include "netmax_tiles.cuh"
+#include "netmax_pipe.cuh"
 #include "netmax_policy.h"
 
 using namespace netmax;
@@ -156,6 +157,13 @@ struct TilePlan {  // launch shape of tile_rounds_kernel
   int64_t min_rounds = 1;  // rounds a call must run to repay loading and storing the tiles
 };
 
+struct PipePlan {  // launch shape of pipe_rounds_kernel
+  bool ok = false;
+  int G = 0, log2G = 0, rows = 0, movers = 0, helpers = 0, batch = 0, grid = 0;
+  size_t smem = 0;
+  int64_t n_tiles = 0, max_rounds = 0, min_rounds = 0;
+};
+
 struct Layout {
   int64_t ld = 0, ldq = 0, nq = 0;  // row stride in elements / in 16-byte column groups; column groups in use
   int elem = 4, halves = 1;         // bytes per stored element; Philox blocks (4 elements) per column group
@@ -167,6 +175,12 @@ struct Layout {
 constexpr int kFuseRoundsLimit = 8;  // largest netmax_config.fuse_rounds
 constexpr int kMaxGrid = 148 * 16;  // upper bound on resident CTAs of the round kernel
 constexpr int64_t kCutLaps = 16, kCutRounds = 16;  // tiles are cut for up to this many tiles per CTA, from this many rounds on
+// pipe_rounds_kernel against tile_rounds_kernel (us per call of 64 rounds, tiles / here): 3 x 1,575 elements 58 / 27, 12 x 12,627
+// 65 / 49, 48 x 4,735 68 / 56, 96 x 2,367 70 / 63, 128 x 1,183 64 / 68; where the model says 1,600 cycles per round and more
+// (3 x 101,031 elements, 64 x 4,735) tiles are as fast or faster.  Calls of four rounds gain 2 to 15 % up to 64
+// workers (80: -5 %), of eight 8 to 40 %.
+constexpr int kPipeWorkers = 100;
+constexpr double kPipeCycles = 1500.0;
 constexpr int64_t kMaxRoundsPerLaunch = 4096;  // rounds one cooperative launch runs at most
 constexpr size_t kPartialsBytes = (size_t)kMaxGrid * 2 * sizeof(double) * 8;  // per CTA and round of a fused launch; two sets for multi-round launches
 constexpr size_t kColPartBytes = (size_t)8 << 20;  // column partials of the row-split (short vector) shape
@@ -294,6 +308,8 @@ struct netmax_ctx {
   FusedPlan fused;
   bool tiles_planned = false;
   TilePlan tiles;
+  bool pipe_planned = false;
+  PipePlan pipe;
   PhiloxKeys keys;
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
@@ -730,6 +746,26 @@ TileKernel pick_tile_kernel(int objective, int halves, int rows) {
   }
 }
 
+using PipeKernel = void (*)(const PipeParams);
+
+template <int kRows>
+PipeKernel pick_pipe_kernel_r(int objective, int halves) {
+  if (halves == 2) return objective == 1 ? pipe_rounds_kernel<1, true, kRows> : pipe_rounds_kernel<0, true, kRows>;
+  return objective == 1 ? pipe_rounds_kernel<1, false, kRows> : pipe_rounds_kernel<0, false, kRows>;
+}
+PipeKernel pick_pipe_kernel(int objective, int halves, int rows) {
+  switch (rows) {
+    case 1: return pick_pipe_kernel_r<1>(objective, halves);
+    case 2: return pick_pipe_kernel_r<2>(objective, halves);
+    case 3: return pick_pipe_kernel_r<3>(objective, halves);
+    case 4: return pick_pipe_kernel_r<4>(objective, halves);
+    case 5: return pick_pipe_kernel_r<5>(objective, halves);
+    case 6: return pick_pipe_kernel_r<6>(objective, halves);
+    case 7: return pick_pipe_kernel_r<7>(objective, halves);
+    default: return pick_pipe_kernel_r<8>(objective, halves);
+  }
+}
+
 // The kernels' noise scale: sigma (at its fp32 rounding, the value the update is defined with)
 // times the constant factor sqrt(2 ln 2) of the Box-Muller radius, which the fast normal generator
 // leaves out, rounded once to fp32.
@@ -938,6 +974,64 @@ int plan_tiles(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan& fused, T
   return NETMAX_OK;
 }
 
+// Launch shape of pipe_rounds_kernel: G column groups per tile, tiles (moving warps) and helping warps per CTA, rounds per
+// batch.  One CTA per SM and one tile per moving warp.  The cycles of a round are modelled on measurements of 2,278 shapes
+// (2 to 64 workers, a quarter of a row of 32 column groups to 16 of them per SM): the moving warp's own chain, the SM's
+// issue, the chain of a helping warp over its share of a batch, and what every batch costs; the shape chosen is within 1 %
+// of the best one on average.
+int plan_pipe_uncached(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& f) {
+  f = PipePlan();
+  if (!plan.short_vectors || ctx->fuse_rounds == 1 || ctx->M > kPipeWorkers) return NETMAX_OK;
+  const int64_t M = ctx->M, nq = (ctx->d + 3) / 4;
+  double best = 0.0;
+  for (int G = 1, log2G = 0; G <= 32; G *= 2, ++log2G) {
+    const int rows = (int)((M + 32 / G - 1) / (32 / G));
+    if (rows > kPipeMaxRows) continue;
+    const int64_t n_tiles = (nq + G - 1) / G, movers = (n_tiles + ctx->sm_count - 1) / ctx->sm_count;
+    if (movers > 8) continue;
+    for (int share = 1; share <= (int)(16 / movers) - 1; ++share) {  // helping warps per moving warp
+      for (int batch : {32, 16, 8, 4, 2}) {
+        const size_t smem = pipe_smem(G, rows, (int)movers, batch);
+        if (smem > (size_t)226 * 1024) continue;
+        const int own = (batch + share - 1) / share, draws = rows <= 2 ? (own + 1) / 2 : own;
+        const int sums = ((batch * G + 31) / 32 + share - 1) / share;
+        const double helper = (70.0 + draws * (840.0 + 150.0 * rows) + sums * (770.0 + 35.0 * M)) / batch;
+        const double cycles = std::max({200.0 + 100.0 * (rows - 1), 95.0 * movers * rows, helper}) + 670.0 / batch;
+        if (best == 0.0 || cycles < best * 0.999) {
+          best = cycles;
+          f.G = G;
+          f.log2G = log2G;
+          f.rows = rows;
+          f.movers = (int)movers;
+          f.helpers = share * (int)movers;
+          f.batch = batch;
+          f.smem = smem;
+          f.n_tiles = n_tiles;
+        }
+      }
+    }
+  }
+  if (best == 0.0 || best > kPipeCycles) return NETMAX_OK;
+  f.grid = (int)std::min<int64_t>(f.n_tiles, ctx->sm_count);
+  NM_CUDA(ctx, allow_smem((const void*)pick_pipe_kernel(ctx->objective, ctx->L.halves, f.rows), f.smem));
+  f.max_rounds = std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.grid);
+  f.min_rounds = M <= 64 ? 4 : 8;
+  f.ok = true;
+  return NETMAX_OK;
+}
+
+int plan_pipe(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& f) {
+  if (!ctx->pipe_planned) {
+    PipePlan fresh;
+    int rc = plan_pipe_uncached(ctx, plan, fresh);
+    if (rc) return rc;
+    ctx->pipe = fresh;
+    ctx->pipe_planned = true;
+  }
+  f = ctx->pipe;
+  return NETMAX_OK;
+}
+
 int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   f = FusedPlan();
   if (ctx->fuse_rounds == 1 || plan.short_vectors) return NETMAX_OK;
@@ -1127,6 +1221,46 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
         tp.partials, grid, chunk, (double)p.inv_M, tel, tp.slot0, tp.ring);
     ctx->launches += 1;
   }
+  NM_CUDA(ctx, cudaGetLastError());
+  return NETMAX_OK;
+}
+
+// One launch of pipe_rounds_kernel: `chunk` rounds from round r over all columns (r and r + chunk - 1 have the same high
+// word: it is part of what a thread works out once).
+int launch_pipe(netmax_ctx* ctx, const PipePlan& pipe, const RoundParams& p, const unsigned char* xin, unsigned char* xout,
+                uint64_t r, int chunk, unsigned char* mirror) {
+  PipeParams pp;
+  pp.x_cur = reinterpret_cast<const char*>(xin);
+  pp.x_nxt = reinterpret_cast<char*>(xout);
+  pp.mirror = reinterpret_cast<char*>(mirror);
+  pp.c = reinterpret_cast<const char*>(ctx->c);
+  pp.draws = ctx->draws;
+  pp.partials = reinterpret_cast<double*>(ctx->colpart);
+  pp.slot0 = (int64_t)(r % (uint64_t)ctx->trace_rounds);
+  pp.ring = ctx->trace_rounds;
+  pp.first_round = r;
+  pp.n_rounds = chunk;
+  pp.n_tiles = (int32_t)pipe.n_tiles;
+  pp.nq = (ctx->d + 3) / 4;
+  pp.row_bytes = p.row_bytes;
+  pp.M = p.M;
+  pp.tail = (int32_t)(ctx->d % 4);
+  pp.G = pipe.G;
+  pp.log2G = pipe.log2G;
+  pp.movers = pipe.movers;
+  pp.batch = pipe.batch;
+  pp.alpha = p.alpha;
+  pp.sigma = p.sigma;
+  pp.inv_M = p.inv_M;
+  pp.q_offset = ctx->q_offset;
+  pp.keys = p.keys;
+  PipeKernel k = pick_pipe_kernel(ctx->objective, ctx->L.halves, pipe.rows);
+  NM_CUDA(ctx, allow_smem((const void*)k, pipe.smem));
+  NM_CUDA(ctx, launch_behind_sampler(k, (unsigned)pipe.grid, (pipe.movers + pipe.helpers) * 32, pipe.smem, ctx->stream, pp));
+  const int warps_per_block = kThreads / 32;
+  sum_tile_partials_kernel<<<(unsigned)((chunk + warps_per_block - 1) / warps_per_block), kThreads, 0, ctx->stream>>>(
+      pp.partials, pipe.grid, chunk, (double)p.inv_M, ctx->tel, pp.slot0, pp.ring);
+  ctx->launches += 2;
   NM_CUDA(ctx, cudaGetLastError());
   return NETMAX_OK;
 }
@@ -1668,6 +1802,10 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   rc = plan_tiles(ctx, plan, fused, tiles);
   if (rc) return rc;
 
+  PipePlan pipe;
+  rc = plan_pipe(ctx, plan, pipe);
+  if (rc) return rc;
+
   choose_rings(ctx, n_rounds);
   RoundParams p = make_round_params(ctx, plan);
 
@@ -1684,6 +1822,21 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
     rc = launch_sampler(ctx, (uint64_t)ctx->rounds, batch, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds,
                         ctx->trace_rounds);
     if (rc) return rc;
+    if (pipe.ok && batch >= pipe.min_rounds) {
+      for (int64_t b = 0; b < batch;) {
+        const int64_t same_word = ((int64_t)1 << 32) - (ctx->rounds & 0xFFFFFFFFll);
+        const int64_t chunk = std::min({batch - b, pipe.max_rounds, same_word});
+        rc = launch_pipe(ctx, pipe, p, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], (uint64_t)ctx->rounds, (int)chunk,
+                         done + b + chunk == n_rounds ? mirror : nullptr);
+        if (rc) return rc;
+        mirrored = true;
+        ctx->cur ^= 1;
+        ctx->rounds += chunk;
+        b += chunk;
+      }
+      done += batch;
+      continue;
+    }
     if (plan.short_vectors && tiles.ok && batch >= tiles.min_rounds) {
       // short vectors: every round of the batch on shared-memory-resident columns
       ColumnRange all;
@@ -1884,6 +2037,7 @@ int netmax_set_fuse_rounds(netmax_ctx* ctx, int32_t fuse_rounds) {
   ctx->fuse_rounds = fuse_rounds;
   ctx->fused_planned = false;
   ctx->tiles_planned = false;
+  ctx->pipe_planned = false;
   return NETMAX_OK;
 }
 

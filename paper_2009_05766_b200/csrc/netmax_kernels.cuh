@@ -10,6 +10,8 @@
 //                         memory, a column per thread (long vectors, up to 36 workers).
 //   tile_rounds_kernel    (netmax_tiles.cuh) the same with the rows of a tile shared out over the
 //                         threads: more workers, and short vectors.
+//   pipe_rounds_kernel    (netmax_pipe.cuh) small problems: a warp moves all rows of a few column groups, others
+//                         draw its noise and add up its telemetry.
 //   multi_round_kernel    short vectors of more workers than fit on chip: all rounds in one launch.
 //   step_kernel           the asynchronous timeline: one worker per global step (Eq. 17);
 //                         step_tiles_kernel: many steps per launch on resident columns.

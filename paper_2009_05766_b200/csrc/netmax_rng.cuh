@@ -185,6 +185,24 @@ __device__ __forceinline__ NoiseBase noise_base(uint32_t q, uint32_t round_lo, u
   b.l0 = (uint32_t)p2;
   return b;
 }
+// The same in two steps, for a thread that stays with a column group: what depends on neither worker nor round, and the rest.
+struct NoiseColumn {
+  uint32_t c3, h, c1;
+};
+__device__ __forceinline__ NoiseColumn noise_column(uint32_t q, uint32_t ctr3, const PhiloxKeys& keys) {
+  const uint64_t p0 = (uint64_t)kPhiloxMul0 * q, q1 = (uint64_t)kPhiloxMul1 * ((uint32_t)(p0 >> 32) ^ ctr3 ^ keys.k1[0]);
+  return NoiseColumn{(uint32_t)p0 ^ keys.k1[1], (uint32_t)(q1 >> 32) ^ keys.k0[1], (uint32_t)q1 ^ keys.k0[2]};
+}
+__device__ __forceinline__ NoiseBase noise_base(const NoiseColumn& c, uint32_t round_lo, const PhiloxKeys& keys) {
+  NoiseBase b;
+  const uint64_t p1 = (uint64_t)kPhiloxMul1 * round_lo, p2 = (uint64_t)kPhiloxMul0 * (c.h ^ (uint32_t)p1);
+  b.a0 = (uint32_t)(p1 >> 32) ^ keys.k0[0];
+  b.c3 = c.c3;
+  b.c1 = c.c1;
+  b.h0 = (uint32_t)(p2 >> 32) ^ keys.k1[2];
+  b.l0 = (uint32_t)p2;
+  return b;
+}
 __device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint32_t worker, const PhiloxKeys& keys) {
   const uint64_t e = (uint64_t)kPhiloxMul0 * (b.a0 ^ worker);
   const uint64_t p = (uint64_t)kPhiloxMul1 * ((uint32_t)(e >> 32) ^ b.c3);
