@@ -132,6 +132,24 @@ cudaError_t allow_smem(const void* kernel, size_t bytes) {
   return e;
 }
 
+// Doubles that are not cleared when the vector grows (that would touch every page on one thread).
+template <typename T>
+struct Uncleared : std::allocator<T> {
+  template <typename U>
+  struct rebind {
+    typedef Uncleared<U> other;
+  };
+  template <typename U>
+  void construct(U* p) {
+    ::new ((void*)p) U;
+  }
+  template <typename U, typename... Args>
+  void construct(U* p, Args&&... args) {
+    ::new ((void*)p) U(std::forward<Args>(args)...);
+  }
+};
+typedef std::vector<double, Uncleared<double>> HostMatrix;
+
 struct RoundPlan {  // launch shape of round_kernel and multi_round_kernel
   int cg = kThreads, rl = 1, rg = 1, rows_per_group = 0;
   bool short_vectors = false;  // fewer than two streaming tiles per SM: the L2-resident shape
@@ -266,7 +284,8 @@ struct netmax_ctx {
   std::vector<uint32_t> h_thr;
   std::vector<int32_t> h_last;
   std::vector<float> h_w;
-  std::vector<double> t_iter;  // iteration times derived from the link speeds in force
+  HostMatrix t_iter;           // iteration times derived from the link speeds in force
+  HostMatrix t_spare;          // many workers: where those of new link speeds are worked out while the policy is searched
   // asynchronous timeline (one worker per global step)
   bool async_on = false;
   double beta = 0.0;
@@ -311,6 +330,7 @@ struct netmax_ctx {
   bool pipe_planned = false;
   PipePlan pipe;
   PhiloxKeys keys;
+  DeviceArena arena;          // work on policies (many workers)
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
   int sm_count = 148;
@@ -340,9 +360,10 @@ int fail(netmax_ctx* ctx, int code, const char* fmt, ...) {
                   #call, cudaGetErrorString(e_));                                                  \
   } while (0)
 
-// From here on whole M x M matrices are worked on by threads or on the device (256 workers: 5.4 ms for a policy on
-// the host, 4.7 on the device; 512: 22 and 7).
+// From here on whole M x M matrices are worked on by threads, and Algorithm 3 on the device (ms for a change of links, host / device,
+// K = R = 8: 128 workers 2.1 / 2.2, 160: 2.9 / 2.3, 260: 7.3 / 2.4; K = R = 20: 100 workers 3.1 / 6.6, 200: 9.3 / 7.3).
 constexpr int32_t kManyWorkers = 320;
+constexpr int32_t kDevicePolicy = 180;
 
 // Link graph from speeds: d_im = 1 iff i != m and the speed is positive (symmetrised).
 int build_adjacency(netmax_ctx* ctx, int32_t M, const double* speed, std::vector<uint8_t>& adj) {
@@ -503,10 +524,10 @@ constexpr int32_t kDeviceTables = 600;
 int upload_policy(netmax_ctx* ctx) {
   if (ctx->M >= kDeviceTables) {
     const size_t MM = (size_t)ctx->M * ctx->M;
-    DeviceBuffers buf;
-    double* d_P = nullptr;
-    uint8_t* d_adj = nullptr;
-    if (buf.get(&d_P, MM) && buf.get(&d_adj, MM)) {
+    ArenaUse use(ctx->arena);
+    if (ctx->arena.begin(DeviceArena::room(MM * sizeof(double)) + MM)) {
+      double* d_P = ctx->arena.take<double>(MM);
+      uint8_t* d_adj = ctx->arena.take<uint8_t>(MM);
       NM_CUDA(ctx, BulkPool::get().to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
       NM_CUDA(ctx, BulkPool::get().to_device(d_adj, ctx->adj.data(), MM, ctx->device, ctx->stream));
       return device_tables(ctx, d_P, d_adj);
@@ -545,10 +566,12 @@ int refresh_iteration_times(netmax_ctx* ctx, const double* speed) {
 // to spare beside the caller's workspace.
 int generate_policy(netmax_ctx* ctx, const double* t_iter, double* P, double* rho) {
   int ndev = 0;
-  if (ctx->M >= kManyWorkers) {
+  if (ctx->M >= kDevicePolicy) {
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev) {
-      const int rc = netmax_policy_generate_device(ctx->M, t_iter, ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R,
-                                                   ctx->policy_rho_upper, ctx->device, ctx->stream, P, rho, nullptr);
+      DeviceGuard guard(ctx->device);
+      ArenaUse use(ctx->arena);
+      const int rc = policy_generate_device(ctx->M, t_iter, ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
+                                            ctx->stream, ctx->arena, P, rho, nullptr);
       if (rc != NETMAX_OOM) return rc;
     }
     cudaGetLastError();
@@ -1576,30 +1599,31 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   // the work is done at get())
   constexpr auto kBeside = std::launch::async | std::launch::deferred;
   std::future<int> graph = std::async(kBeside, [&] {
-    const int rc = build_adjacency(nullptr, M, speed, adj);  // (its message goes to this thread's g_error)
+    int rc = build_adjacency(nullptr, M, speed, adj);  // (its message goes to this thread's g_error)
+    if (!rc) {
+      ctx->t_spare.resize((size_t)M * M);
+      rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_spare.data(), adj.data());  // (the same graph)
+    }
     if (rc) graph_error = g_error;
     return rc;
   });
-  DeviceBuffers buf;
+  ArenaUse use(ctx->arena);
   double* d_P = nullptr;
   uint8_t* d_adj = nullptr;
   double rho = 0.0;
   const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
-                                          ctx->device, ctx->stream, buf, &d_P, &d_adj, &rho);
+                                          ctx->device, ctx->stream, ctx->arena, &d_P, &d_adj, &rho);
   const int graph_rc = graph.get();
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
-  ctx->t_iter.resize((size_t)M * M);
-  std::future<int> times = std::async(kBeside, [&] { return netmax_iteration_times(M, ctx->d, speed, ctx->t_iter.data(), adj.data()); });
   ctx->rho = rho;
+  ctx->t_iter.swap(ctx->t_spare);
   int done = device_tables(ctx, d_P, d_adj);
   if (!done) {
     const cudaError_t e = BulkPool::get().to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
     if (e != cudaSuccess) done = fail(ctx, NETMAX_CUDA_ERROR, "reading P back: %s", cudaGetErrorString(e));
   }
-  const int times_rc = times.get();
   ctx->adj.swap(adj);
-  if (!done && times_rc) done = fail(ctx, times_rc, "iteration times of the new speeds");
   return done;
 }
 
@@ -1608,7 +1632,7 @@ int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const doub
   if (!std::isfinite(rho)) return fail(ctx, NETMAX_INVALID_ARG, "rho is not finite");
   DeviceGuard guard(ctx->device);
   int rc = NETMAX_OK;
-  if (ctx->M >= kManyWorkers && link_speed_gbps && !prob && ctx->pull_weight <= 0.0 && rho <= 0.0) {
+  if (ctx->M >= kDevicePolicy && link_speed_gbps && !prob && ctx->pull_weight <= 0.0 && rho <= 0.0) {
     rc = set_policy_from_links(ctx, link_speed_gbps);
     if (!rc && ctx->async_on) rc = need_host_tables(ctx);
     if (rc != NETMAX_OOM) return rc;
@@ -1619,7 +1643,8 @@ int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const doub
       netmax_ctx* ctx;
       bool links, generated;  // what is replaced: link graph and times; P (a caller's P is checked before it replaces the one in force)
       std::vector<uint8_t> adj;
-      std::vector<double> P, t;
+      std::vector<double> P;
+      HostMatrix t;
       double rho;
       bool done = false;
       ~Undo() {
@@ -1632,7 +1657,8 @@ int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const doub
         ctx->rho = rho;
       }
     };
-    std::vector<double> old_P, old_t;
+    std::vector<double> old_P;
+    HostMatrix old_t;
     if (!prob) old_P = ctx->P;
     if (link_speed_gbps) old_t = ctx->t_iter;
     Undo undo{ctx, link_speed_gbps != nullptr, prob == nullptr, {}, std::move(old_P), std::move(old_t), ctx->rho};

@@ -126,135 +126,285 @@ __global__ void __launch_bounds__(kRowThreads) row_info_kernel(int M, const doub
   }
 }
 
-// Sums of three values over the CTA, returned to every thread.  s_buf: 99 doubles.
-__device__ void block_sum3(double& a, double& b, double& c, double* s_buf) {
+// Sums of three or four values over the CTA, returned to every thread.  s_buf: 33 doubles for each.
+template <int kValues>
+__device__ void block_sums(double (&v)[kValues], double* s_buf) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  a = warp_sum(a);
-  b = warp_sum(b);
-  c = warp_sum(c);
+#pragma unroll
+  for (int k = 0; k < kValues; ++k) v[k] = warp_sum(v[k]);
   __syncthreads();
   if (lane == 0) {
-    s_buf[warp] = a;
-    s_buf[33 + warp] = b;
-    s_buf[66 + warp] = c;
+#pragma unroll
+    for (int k = 0; k < kValues; ++k) s_buf[33 * k + warp] = v[k];
   }
   __syncthreads();
-  if (warp < 3) {
+  if (warp < kValues) {
     double t = lane < nw ? s_buf[33 * warp + lane] : 0.0;
     t = warp_sum(t);
     if (lane == 0) s_buf[33 * warp + 32] = t;
   }
   __syncthreads();
-  a = s_buf[32];
-  b = s_buf[65];
-  c = s_buf[98];
+#pragma unroll
+  for (int k = 0; k < kValues; ++k) v[k] = s_buf[33 * k + 32];
+}
+__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, double* s_buf) {
+  double v[3] = {a, b, c};
+  block_sums(v, s_buf);
+  a = v[0];
+  b = v[1];
+  c = v[2];
+}
+__device__ __forceinline__ void block_sum4(double& a, double& b, double& c, double& d, double* s_buf) {
+  double v[4] = {a, b, c, d};
+  block_sums(v, s_buf);
+  a = v[0];
+  b = v[1];
+  c = v[2];
+  d = v[3];
 }
 
-// What the host looks at after every grid point.
-struct PointResult {
-  double rq;        // Rayleigh quotient of the probe vector
-  int infeasible;   // some row of the LP has no solution
+// exp(x) for |x| <= 600 by a table of powers of two (Tang, "Table-driven implementation of the exponential function"): x =
+// (16 e + j) ln 2 / 16 + r with the multiple taken off in two parts, exp(r) by its Taylor polynomial of degree 7 (|r| <= ln 2 / 32:
+// remainder below 2e-18), times 2^(j/16) out of shared memory, with e added to the exponent.  Sixteen doubles fill the 32 banks once,
+// so no access conflicts.  Twelve operations of the fp64 pipe, which is what bounds the row kernels (see row_solve_kernel).
+constexpr int kExpTable = 16;
+__device__ __forceinline__ void exp_table(double* s_table) {  // (before a __syncthreads)
+  if (threadIdx.x < kExpTable) s_table[threadIdx.x] = exp2((double)threadIdx.x / kExpTable);
+}
+__device__ __forceinline__ double table_exp(double x, const double* s_table) {
+  const double shift = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer in the low mantissa bits
+  const double t = fma(x, 23.083120654223414, shift), k = t - shift;  // 16 / ln 2
+  const int n = __double2loint(t);
+  double r = fma(k, -0x1.62e42fefp-5, x);          // ln 2 / 16: its leading 32 bits (k has 14), and the rest
+  r = fma(k, -0x1.473de6af278edp-38, r);
+  double q = fma(r, 1.0 / 5040.0, 1.0 / 720.0);
+  q = fma(q, r, 1.0 / 120.0);
+  q = fma(q, r, 1.0 / 24.0);
+  q = fma(q, r, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  q = fma(q, r, 1.0) * r;
+  const double p = s_table[n & (kExpTable - 1)];
+  const double v = fma(p, q, p);
+  return __hiloint2double(__double2hiint(v) + ((n >> 4) << 20), __double2loint(v));
+}
+
+// Grid points t_bar_r, r = first + 1 ... first + n, of one rho: alpha rho and the inner grid.
+struct PointGrid {
+  double ar, U, delta;
+  int R, first, n;
+  // T = M t_bar_r, t_bar_r = U - (R - r) delta, one rounding per operation as on the host
+  __device__ __forceinline__ double time(int M, int k) const { return __dmul_rn((double)M, __dsub_rn(U, __dmul_rn((double)(R - 1 - first - k), delta))); }
+};
+// A row of the LP at one grid point: p_im = alpha rho (d_im + d_mi) + share exp(-eta s_m), or, with p_ii > 0 or equal
+// times (eta unused), the share on the fastest links or on all.
+enum RowKind : int { kNoRow = 0, kTilted, kEven, kFastest };
+struct RowPoint {
+  double eta, share, pii;
+  int kind;
+};
+// Where a row's search stands: eta of the last point solved, and mean, variance and third central moment of s under its
+// weights (var = 0: none yet).
+struct RowState {
+  double eta, mean, var, third;
 };
 
-// One row of the LP at (alpha rho, T = M t_bar); an infeasible row raises out->infeasible.
-// Bound by fp64 exponentials: the row's times, mapped to [0, 1], stay in shared memory (-1: no link) for
-// all Newton steps, which start from the previous grid point's solution (eta[i]) and so are two or three.
+// One row of the LP at the points of a grid; a row without a solution is kNoRow and raises infeasible[point].  Bound by fp64
+// exponentials: the row's times, mapped to [0, 1], stay in shared memory (-1: no link) for all points and steps.  The steps are
+// Halley's: the mean's first two derivatives are moments that come with it (d mean / d eta = -var, d var / d eta = -third).
+// They start from the previous point's solution, whose moments are known, so that the first step costs nothing; two or three
+// passes over the row follow.  4,096 workers, eight grid points per launch: 1,085 us with Newton's steps from a pass at the old
+// solution on and the library's exp, 725 so; with a launch per grid point, which reads the times every time and stores P, 171 us
+// per point.
 __global__ void __launch_bounds__(kRowThreads) row_solve_kernel(int M, const double* t, const uint8_t* adj, const RowInfo* info,
-                                                                double ar, double T, double* P, double* eta_io, PointResult* out) {
+                                                                const PointGrid grid, RowState* state, RowPoint* points, int* infeasible) {
   extern __shared__ double s_time[];
-  __shared__ double s_buf[99];
+  __shared__ double s_buf[132], s_table[kExpTable];
   const int i = blockIdx.x;
   const RowInfo r = info[i];
   const double* ti = t + (size_t)i * M;
   const uint8_t* ai = adj + (size_t)i * M;
-  double* pi = P + (size_t)i * M;
-  const double F = ar * r.sum_f1;
-  const double free_mass = 1.0 - F, A = ar * r.sum_f1t;
+  const double F = grid.ar * r.sum_f1;
+  const double free_mass = 1.0 - F, A = grid.ar * r.sum_f1t;
   const double lo = A + free_mass * r.tmin, hi = A + free_mass * r.tmax;
-  if (F > 1.0 || T > hi * (1.0 + kTie)) {
-    if (threadIdx.x == 0) out->infeasible = 1;
-    return;
+  const double scale = r.tmax - r.tmin;
+  const bool flat = !(scale > kTie * r.tmax) || free_mass <= 0.0;
+  if (!flat) {
+    const double inv_scale = 1.0 / scale;
+    for (int m = threadIdx.x; m < M; m += blockDim.x) s_time[m] = (m != i && ai[m]) ? (ti[m] - r.tmin) * inv_scale : -1.0;
   }
-  auto f1_of = [&](int m) { return r.both ? 2.0 : (double)ai[m] + (double)adj[(size_t)m * M + i]; };
-  if (T >= lo * (1.0 - kTie)) {
-    const double scale = r.tmax - r.tmin;
-    const bool flat = !(scale > kTie * r.tmax) || free_mass <= 0.0;
-    double eta = 0.0, z = (double)r.n_nb;
-    if (!flat) {
-      const double target = fmin(fmax((T - A) / free_mass, r.tmin), r.tmax);
-      const double sig = (target - r.tmin) / scale, inv_scale = 1.0 / scale;
-      for (int m = threadIdx.x; m < M; m += blockDim.x) s_time[m] = (m != i && ai[m]) ? (ti[m] - r.tmin) * inv_scale : -1.0;
-      // mean and variance of s under q ~ exp(-eta s)  (every thread reads back only what it wrote)
-      double mean, var;
-      auto stats = [&](double e) {
-        double a0 = 0, a1 = 0, a2 = 0;
-        for (int m = threadIdx.x; m < M; m += blockDim.x) {
-          const double s = s_time[m];
-          if (s < 0.0) continue;
-          const double w = exp(-e * s);
-          a0 += w;
-          a1 += w * s;
-          a2 += w * s * s;
-        }
-        block_sum3(a0, a1, a2, s_buf);
-        z = a0;
-        mean = a1 / a0;
-        var = a2 / a0 - mean * mean;
-      };
-      double elo = -kEtaCap, ehi = kEtaCap;
-      if (sig >= r.mean_lo) {
-        stats(eta = elo);
-      } else if (sig <= r.mean_hi) {
-        stats(eta = ehi);
+  exp_table(s_table);
+  __syncthreads();
+  RowState at = state[i];  // (every thread reads back only what it wrote in s_time)
+  for (int k = 0; k < grid.n; ++k) {
+    const double T = grid.time(M, k);
+    RowPoint out = {0.0, 0.0, 0.0, kNoRow};
+    bool ok = !(F > 1.0 || T > hi * (1.0 + kTie));
+    if (ok && T >= lo * (1.0 - kTie)) {
+      if (flat) {
+        out.kind = kEven;
+        out.share = free_mass > 0.0 ? free_mass / (double)r.n_nb : 0.0;
       } else {
-        eta = eta_io[i];
-        stats(eta);
-        for (int it = 0; it < 200; ++it) {  // Newton steps kept inside a shrinking bracket
-          const double gap = mean - sig;
-          if (fabs(gap) <= 1e-15) break;
-          if (gap > 0) elo = eta; else ehi = eta;
-          double next = (var > 1e-300) ? eta + gap / var : 0.5 * (elo + ehi);
-          if (!(next > elo && next < ehi)) next = 0.5 * (elo + ehi);
-          if (next == eta || ehi - elo <= 1e-15 * (1.0 + fabs(eta))) break;
-          // a Newton step this short leaves an error of its square: below the rounding of the sums
-          const bool last = fabs(next - eta) <= 1e-9 * (1.0 + fabs(eta)) && fabs(gap) <= 1e-9;
-          eta = next;
-          stats(eta);
-          if (last) break;
+        const double target = fmin(fmax((T - A) / free_mass, r.tmin), r.tmax);
+        const double sig = (target - r.tmin) / scale;
+        double z = 1.0;
+        RowState now = at;
+        // moments of s under q ~ exp(-eta s)
+        auto stats = [&](double e) {
+          double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+          for (int m = threadIdx.x; m < M; m += blockDim.x) {
+            const double s = s_time[m];
+            if (s < 0.0) continue;
+            const double w = table_exp(-e * s, s_table), ws = w * s, wss = ws * s;
+            a0 += w;
+            a1 += ws;
+            a2 += wss;
+            a3 += wss * s;
+          }
+          block_sum4(a0, a1, a2, a3, s_buf);
+          z = a0;
+          now.eta = e;
+          now.mean = a1 / a0;
+          now.var = a2 / a0 - now.mean * now.mean;
+          now.third = a3 / a0 - now.mean * (3.0 * now.var + now.mean * now.mean);
+        };
+        double elo = -kEtaCap, ehi = kEtaCap;
+        if (sig >= r.mean_lo) {
+          stats(elo);
+        } else if (sig <= r.mean_hi) {
+          stats(ehi);
+        } else {
+          bool fresh = false;  // have the weights of this eta been added up?
+          if (!(now.var > 0.0)) {
+            stats(0.0);
+            fresh = true;
+          }
+          for (int it = 0; it < 200; ++it) {  // steps kept inside a shrinking bracket
+            const double gap = now.mean - sig;
+            if (fresh && fabs(gap) <= 1e-15) break;
+            if (gap > 0) elo = now.eta; else ehi = now.eta;
+            const double slope = now.var * now.var - 0.5 * gap * now.third;
+            double next = (now.var > 1e-300) ? now.eta + (slope > 0.5 * now.var * now.var ? gap * now.var / slope : gap / now.var) : 0.5 * (elo + ehi);
+            if (!(next > elo && next < ehi)) next = 0.5 * (elo + ehi);
+            if (fresh && (next == now.eta || ehi - elo <= 1e-15 * (1.0 + fabs(now.eta)))) break;
+            // a step this short leaves an error of its square or less: below the rounding of the sums
+            const bool last = fabs(next - now.eta) <= 1e-9 * (1.0 + fabs(now.eta)) && fabs(gap) <= 1e-9;
+            stats(next);
+            fresh = true;
+            if (last) break;
+          }
+          at = now;
         }
-        __syncthreads();  // (every thread has read eta_io[i])
-        if (threadIdx.x == 0) eta_io[i] = eta;
+        const double mean = now.mean, eta = now.eta;
+        ok = fabs(mean - sig) <= 1e-9;
+        out.kind = kTilted;
+        out.eta = eta;
+        out.share = free_mass / z;
       }
-      if (threadIdx.x == 0 && !(fabs(mean - sig) <= 1e-9)) out->infeasible = 1;
+    } else if (ok) {
+      const double pii = (lo - T) / (r.tmin - r.C);
+      ok = !(pii > free_mass * (1.0 + kTie));
+      out.kind = kFastest;
+      out.pii = fmin(pii, free_mass);
+      out.share = (free_mass - out.pii) / r.n_fast;
     }
-    const double share = flat ? (free_mass > 0.0 ? free_mass / (double)r.n_nb : 0.0) : free_mass / z;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-      double p = 0.0;
-      if (m != i && ai[m]) p = ar * f1_of(m) + (flat ? share : share * exp(-eta * s_time[m]));
-      pi[m] = p;
+    if (threadIdx.x == 0) {
+      if (!ok) {
+        out.kind = kNoRow;
+        infeasible[k] = 1;
+      }
+      points[(size_t)k * M + i] = out;
     }
-    return;
   }
-  double pii = (lo - T) / (r.tmin - r.C);
-  if (pii > free_mass * (1.0 + kTie)) {
-    if (threadIdx.x == 0) out->infeasible = 1;
-    return;
-  }
-  pii = fmin(pii, free_mass);
+  if (threadIdx.x == 0) state[i] = at;
+}
+
+// p_im of a link (i, m): f1 = d_im + d_mi.
+__device__ __forceinline__ double row_entry(const RowInfo& r, const RowPoint& p, double ar, double f1, double t, double inv_scale, const double* s_table) {
+  double p_im = ar * f1;
+  if (p.kind == kTilted) p_im += p.share * table_exp(-p.eta * ((t - r.tmin) * inv_scale), s_table);
+  else if (p.kind == kEven || t <= r.tmin * (1.0 + kTie)) p_im += p.share;
+  return p_im;
+}
+
+// P at one grid point.
+__global__ void __launch_bounds__(kRowThreads) store_rows_kernel(int M, const double* t, const uint8_t* adj, const RowInfo* info, double ar,
+                                                                 const RowPoint* points, double* P) {
+  __shared__ double s_table[kExpTable];
+  exp_table(s_table);
+  __syncthreads();
+  const int i = blockIdx.x;
+  const RowInfo r = info[i];
+  const RowPoint p = points[i];
+  const double inv_scale = 1.0 / (r.tmax - r.tmin);
   for (int m = threadIdx.x; m < M; m += blockDim.x) {
-    double p = 0.0;
-    if (m == i) p = pii;
-    else if (ai[m]) p = ar * f1_of(m) + (ti[m] <= r.tmin * (1.0 + kTie) ? (free_mass - pii) / r.n_fast : 0.0);
-    pi[m] = p;
+    const size_t at = (size_t)i * M + m;
+    double v = m == i ? p.pii : 0.0;
+    if (m != i && adj[at]) v = row_entry(r, p, ar, r.both ? 2.0 : (double)adj[at] + (double)adj[(size_t)m * M + i], t[at], inv_scale, s_table);
+    P[at] = v;
   }
 }
 
-// Off-diagonal entries of Y_P (Eq. 22) with p_i = 1/M: p_im gamma_im = (d_im+d_mi)/2,
-// p_im gamma_im^2 = (d_im+d_mi)^2/(4 p_im).  y_im = y_mi needs p_im and p_mi: a CTA takes the tile (bi, bj)
-// of the upper triangle and its mirror image, so that P is read once and coalesced.
-//   kStore  writes both tiles of Y, with a zero diagonal (the products with Y below never use it);
-//   else    sums y_im (v_i - v_m)^2 over the tile: 1 minus the sum over all tiles is the Rayleigh quotient
-//           v^T Y v of a unit vector.  The last CTA adds the tiles in order and leaves the result in out->rq.
+// 1 / x for x well inside the range of normal numbers: Newton's iteration on the hardware's approximation (about 20 bits, then
+// 40, then rounding).
+__device__ __forceinline__ double fast_reciprocal(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
+// How far the Rayleigh quotient v^T Y_P v of a unit vector (sum v_m = 0) lies below 1 at the points of a grid:
+//   sum_{i < m} y_im (v_i - v_m)^2,  y_im (Eq. 22 with p_i = 1/M) = alpha rho/M [h(p_im) + h(p_mi)],
+//   h(p) = (d_im+d_mi)/2 - alpha rho (d_im+d_mi)^2/(4p)  for p > 0,
+// so every row adds up its own p_im and neither P nor Y need be stored (a pass over a stored P took 98 us per grid point of 4,096
+// workers; this 27, bound by the fp64 pipe).  parts[k][i]: row i's share.
+__global__ void __launch_bounds__(kRowThreads) row_quotient_kernel(int M, const double* t, const uint8_t* adj, const RowInfo* info,
+                                                                   const PointGrid grid, const RowPoint* points, const double* v, double* parts) {
+  extern __shared__ double s_time[];
+  __shared__ double s_buf[33], s_table[kExpTable];
+  exp_table(s_table);
+  const int i = blockIdx.x;
+  const RowInfo r = info[i];
+  const double inv_scale = 1.0 / (r.tmax - r.tmin), vi = v[i], ar = grid.ar;
+  for (int m = threadIdx.x; m < M; m += blockDim.x)
+    s_time[m] = (m != i && adj[(size_t)i * M + m]) ? t[(size_t)i * M + m] : -1.0;  // (every thread reads back only what it wrote)
+  __syncthreads();
+  for (int k = 0; k < grid.n; ++k) {
+    const RowPoint p = points[(size_t)k * M + i];
+    double acc = 0.0;
+    if (p.kind == kTilted && r.both) {  // the common form, its constants taken out: h(p) = 1 - ar / p, p = 2 ar + share exp(...)
+      const double scaled = -p.eta * inv_scale, floor_im = 2.0 * ar;
+      for (int m = threadIdx.x; m < M; m += blockDim.x) {
+        const double tm = s_time[m];
+        if (tm < 0.0) continue;
+        const double d = vi - v[m];
+        acc += fma(-ar, fast_reciprocal(fma(p.share, table_exp(scaled * (tm - r.tmin), s_table), floor_im)), 1.0) * (d * d);
+      }
+    } else if (p.kind != kNoRow) {
+      for (int m = threadIdx.x; m < M; m += blockDim.x) {
+        const double tm = s_time[m];
+        if (tm < 0.0) continue;
+        const double f1 = r.both ? 2.0 : 1.0 + (double)adj[(size_t)m * M + i];
+        const double p_im = row_entry(r, p, ar, f1, tm, inv_scale, s_table), d = vi - v[m];
+        if (p_im > 0.0) acc += (0.5 * f1 - ar * 0.25 * f1 * f1 * fast_reciprocal(p_im)) * d * d;
+      }
+    }
+    acc = block_sum(acc, s_buf);
+    if (threadIdx.x == 0) parts[(size_t)k * M + i] = ar / M * acc;
+  }
+}
+// quotient[k] = 1 - sum of parts[k][.], in a fixed order.
+__global__ void __launch_bounds__(256) quotient_sums_kernel(int M, const double* parts, double* quotient) {
+  __shared__ double s_buf[33];
+  double a = 0.0;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) a += parts[(size_t)blockIdx.x * M + i];
+  a = block_sum(a, s_buf);
+  if (threadIdx.x == 0) quotient[blockIdx.x] = 1.0 - a;
+}
+
+// Off-diagonal entries of Y_P (Eq. 22) with p_i = 1/M in the place of P: p_im gamma_im = (d_im+d_mi)/2,
+// p_im gamma_im^2 = (d_im+d_mi)^2/(4 p_im).  y_im = y_mi needs p_im and p_mi: a CTA takes the tile (bi, bj) of the upper
+// triangle and its mirror image, which nobody else looks at.  The diagonal is zero (the products with Y below never use it).
 constexpr int kTile = 32;
 struct TileIndex {
   int bi, bj;
@@ -269,12 +419,9 @@ __device__ __forceinline__ TileIndex triangle_tile(long long idx, int nb) {
   while (bi + 1 < nb && start(bi + 1) <= idx) ++bi;
   return {bi, bi + (int)(idx - start(bi))};
 }
-template <bool kStore>
-__global__ void __launch_bounds__(256) y_tiles_kernel(int M, const double* P, const uint8_t* adj, double ar, double* Y, const double* v,
-                                                      double* partial, unsigned int* ticket, PointResult* out) {
+__global__ void __launch_bounds__(256) y_tiles_kernel(int M, double* P, const uint8_t* adj, double ar) {
   __shared__ double s_mirror[kTile][kTile + 1];
   __shared__ uint8_t s_adj[kTile][kTile + 4];
-  __shared__ double s_buf[33];
   const int nb = (M + kTile - 1) / kTile;
   const TileIndex at = triangle_tile((long long)blockIdx.x, nb);
   const int bi = at.bi, bj = at.bj;
@@ -287,7 +434,6 @@ __global__ void __launch_bounds__(256) y_tiles_kernel(int M, const double* P, co
     s_adj[r][c] = in ? adj[(size_t)row * M + col] : 0;
   }
   __syncthreads();
-  double acc = 0.0;
   double y[kTile * kTile / 256];
 #pragma unroll
   for (int k = 0; k < kTile * kTile / 256; ++k) {
@@ -300,45 +446,21 @@ __global__ void __launch_bounds__(256) y_tiles_kernel(int M, const double* P, co
       if (pim > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pim); }
       if (pmi > 0.0) { lin += 0.5 * ds; quad += ds * ds / (4.0 * pmi); }
       y[k] = (ar * lin - ar * ar * quad) / M;
-      if (!kStore && i < m) {
-        const double d = v[i] - v[m];
-        acc += y[k] * d * d;
-      }
     }
-  }
-  if (kStore) {
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kTile * kTile / 256; ++k) {
-      const int r = r0 + k * (256 / kTile), i = i0 + r, m = j0 + c;
-      if (i < M && m < M) Y[(size_t)i * M + m] = y[k];
-      s_mirror[c][r] = y[k];
-    }
-    __syncthreads();
-    if (bi != bj)
-      for (int r = r0; r < kTile; r += 256 / kTile) {
-        const int row = j0 + r, col = i0 + c;
-        if (row < M && col < M) Y[(size_t)row * M + col] = s_mirror[r][c];
-      }
-    return;
-  }
-  acc = block_sum(acc, s_buf);
-  __shared__ bool s_last;
-  if (threadIdx.x == 0) {
-    partial[blockIdx.x] = acc;
-    __threadfence();
-    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  double sum = 0.0;
-  for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) sum += __ldcg(partial + k);
-  sum = block_sum(sum, s_buf);
-  if (threadIdx.x == 0) {
-    out->rq = 1.0 - sum;
-    *ticket = 0u;
+#pragma unroll
+  for (int k = 0; k < kTile * kTile / 256; ++k) {
+    const int r = r0 + k * (256 / kTile), i = i0 + r, m = j0 + c;
+    if (i < M && m < M) P[(size_t)i * M + m] = y[k];
+    s_mirror[c][r] = y[k];
   }
+  __syncthreads();
+  if (bi != bj)
+    for (int r = r0; r < kTile; r += 256 / kTile) {
+      const int row = j0 + r, col = i0 + c;
+      if (row < M && col < M) P[(size_t)row * M + col] = s_mirror[r][c];
+    }
 }
 
 // ---- Lanczos on the complement of the all-ones vector (fp64) -----------------------------------------
@@ -350,10 +472,11 @@ __global__ void __launch_bounds__(256) y_tiles_kernel(int M, const double* P, co
 // has the size of the spectrum's spread (Y itself is close to I for many workers, and the rounding of
 // numbers near 1 would swamp a beta of 1e-4 within a few steps).  No reorthogonalisation: the top of the
 // spectrum converges all the same, copies of a converged value do not move it, and the component along
-// the all-ones vector is taken out of every u.  Bound by reading Y (134 MB at M = 4096).
+// the all-ones vector is taken out of every u.  Bound by reading Y (134 MB at M = 4096: 41 us per step with three CTAs per SM
+// and 16-byte loads, 57 with one and 8-byte loads).
 struct LanczosParams {
   int M, k;
-  const double* Y;
+  const double* Y;  // row-major; its block starts on 256 bytes
   double* V;        // [steps + 1][M]; row 0 is the start vector
   const double* w_in;
   double* w_out;
@@ -364,7 +487,7 @@ struct LanczosParams {
 };
 constexpr int kLanczosThreads = 512;
 __global__ void __launch_bounds__(kLanczosThreads) lanczos_step_kernel(const LanczosParams p) {
-  extern __shared__ double s_v[];
+  extern __shared__ __align__(16) double s_v[];
   __shared__ double s_buf[99];
   const int M = p.M, tid = threadIdx.x, T = blockDim.x;
   double beta_prev = 0.0;
@@ -406,14 +529,32 @@ __global__ void __launch_bounds__(kLanczosThreads) lanczos_step_kernel(const Lan
     const double vi = s_v[row];
     double acc = 0.0;
     int j = lane;
-    for (; j + 96 < M; j += 128) {  // four loads in flight
-      const double y0 = y[j], y1 = y[j + 32], y2 = y[j + 64], y3 = y[j + 96];
-      acc += y0 * (s_v[j] - vi);
-      acc += y1 * (s_v[j + 32] - vi);
-      acc += y2 * (s_v[j + 64] - vi);
-      acc += y3 * (s_v[j + 96] - vi);
+    if ((M & 1) == 0) {  // pairs of columns (rows start on 16 bytes), eight loads in flight
+      const double2* y2 = reinterpret_cast<const double2*>(y);
+      const double2* v2 = reinterpret_cast<const double2*>(s_v);
+      double other = 0.0;
+      for (; 2 * (j + 224) < M; j += 256) {
+        double2 in[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a)  // (volatile: issued one behind the other; left to itself the compiler keeps two in flight)
+          asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(in[a].x), "=d"(in[a].y) : "l"(y2 + j + 32 * a));
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+          const double2 v = v2[j + 32 * a];
+          acc += in[a].x * (v.x - vi);
+          other += in[a].y * (v.y - vi);
+        }
+      }
+      for (; 2 * j < M; j += 32) {
+        const double2 in = __ldg(y2 + j), v = v2[j];
+        acc += in.x * (v.x - vi);
+        other += in.y * (v.y - vi);
+      }
+      acc += other;
+    } else {
+#pragma unroll 8
+      for (; j < M; j += 32) acc += y[j] * (s_v[j] - vi);
     }
-    for (; j < M; j += 32) acc += y[j] * (s_v[j] - vi);
     acc = warp_sum(acc);
     if (lane == 0) {
       const double w = acc - (p.k > 0 ? beta_prev * v_prev[row] : 0.0);
@@ -507,13 +648,14 @@ __global__ void __launch_bounds__(256) iteration_times_kernel(int M, double* t, 
 
 // T_j = floor(cum_j 2^32 + 1/2) over the left-to-right prefix sums of a row of P (in this order: the draws
 // are exact against these integers), non-decreasing, saturated, pinned to the top from the last positive
-// entry on; and the pull weights.  A CTA takes 32 rows, 64 columns at a time: one warp runs along its 32
-// rows' sums, one row per lane, out of shared memory while the others convert the weights.
-constexpr int kTableRows = 32, kTableCols = 64, kTableThreads = 256;
+// entry on; and the pull weights.  A CTA takes eight rows, 128 columns at a time: a warp runs along its
+// rows' sums, one row per lane, out of shared memory while the others convert the weights; all of them then turn sums into
+// thresholds (with that in the chain 4,096 workers took 413 us).
+constexpr int kTableRows = 8, kTableCols = 128, kTableThreads = 256;
 __global__ void __launch_bounds__(kTableThreads) tables_kernel(int M, const double* P, const uint8_t* adj, double alpha_rho,
                                                                double pull_weight, uint32_t* thr, int32_t* last_nz, float* w) {
   __shared__ double s_p[kTableRows][kTableCols + 1];
-  __shared__ uint32_t s_t[kTableRows][kTableCols + 1];
+  __shared__ double s_cum[kTableRows][kTableCols + 1];
   __shared__ int s_last[kTableRows];
   const int i0 = blockIdx.x * kTableRows, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int r = warp; r < kTableRows; r += kTableThreads / 32) {  // last positive entry, from the end
@@ -533,7 +675,6 @@ __global__ void __launch_bounds__(kTableThreads) tables_kernel(int M, const doub
     if (lane == 0) s_last[r] = last;
   }
   double cum = 0.0;
-  unsigned long long prev = 0;
   for (int j0 = 0; j0 < M; j0 += kTableCols) {
     __syncthreads();
     for (int k = tid; k < kTableRows * kTableCols; k += kTableThreads) {
@@ -542,14 +683,12 @@ __global__ void __launch_bounds__(kTableThreads) tables_kernel(int M, const doub
     }
     __syncthreads();
     if (warp == 0) {
-      const int last = s_last[lane];
-      for (int c = 0; c < kTableCols; ++c) {
-        cum += s_p[lane][c];
-        unsigned long long t = (unsigned long long)floor(cum * 4294967296.0 + 0.5);
-        t = t > prev ? t : prev;
-        if (t > 0xFFFFFFFFull || j0 + c >= last) t = 0xFFFFFFFFull;
-        s_t[lane][c] = (uint32_t)t;
-        prev = t;
+      if (lane < kTableRows) {
+#pragma unroll 16
+        for (int c = 0; c < kTableCols; ++c) {
+          cum += s_p[lane][c];
+          s_cum[lane][c] = cum;
+        }
       }
     } else {
       for (int k = tid - 32; k < kTableRows * kTableCols; k += kTableThreads - 32) {
@@ -567,7 +706,9 @@ __global__ void __launch_bounds__(kTableThreads) tables_kernel(int M, const doub
     __syncthreads();
     for (int k = tid; k < kTableRows * kTableCols; k += kTableThreads) {
       const int r = k / kTableCols, c = k % kTableCols, i = i0 + r, j = j0 + c;
-      if (i < M && j < M) thr[(size_t)i * M + j] = s_t[r][c];
+      if (i >= M || j >= M) continue;
+      const double t = floor(s_cum[r][c] * 4294967296.0 + 0.5);  // (sums of entries >= 0 never decrease, nor do their roundings)
+      thr[(size_t)i * M + j] = t > 4294967295.0 || j >= s_last[r] ? 0xFFFFFFFFu : (uint32_t)t;
     }
   }
 }
