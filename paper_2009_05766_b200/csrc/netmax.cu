@@ -729,16 +729,17 @@ MultiRoundKernel pick_multi_kernel(int objective, int halves) {
 
 using FusedKernel = void (*)(const FusedParams);
 
-template <int kReg>
+template <int kReg, bool kStart>
 FusedKernel pick_fused_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kReg> : fused_rounds_kernel<0, true, kReg>;
-  return objective == 1 ? fused_rounds_kernel<1, false, kReg> : fused_rounds_kernel<0, false, kReg>;
+  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kReg, kStart> : fused_rounds_kernel<0, true, kReg, kStart>;
+  return objective == 1 ? fused_rounds_kernel<1, false, kReg, kStart> : fused_rounds_kernel<0, false, kReg, kStart>;
 }
-// The instance for launches of `rounds` rounds (all share one layout of the shared memory).
-FusedKernel pick_fused_kernel(int objective, int halves, int rounds) {
-  if (rounds <= 4) return pick_fused_kernel_r<4>(objective, halves);
-  if (rounds <= 8) return pick_fused_kernel_r<8>(objective, halves);
-  return pick_fused_kernel_r<0>(objective, halves);
+// The instance for M workers and launches of `rounds` rounds (all of one M share one layout of the shared memory).
+FusedKernel pick_fused_kernel(int objective, int halves, int32_t M, int rounds) {
+  const bool start = M <= kStartWorkers;
+  if (rounds <= 4) return start ? pick_fused_kernel_r<4, true>(objective, halves) : pick_fused_kernel_r<4, false>(objective, halves);
+  if (rounds <= 8) return start ? pick_fused_kernel_r<8, true>(objective, halves) : pick_fused_kernel_r<8, false>(objective, halves);
+  return start ? pick_fused_kernel_r<0, true>(objective, halves) : pick_fused_kernel_r<0, false>(objective, halves);
 }
 
 using TileKernel = void (*)(const TileParams);
@@ -1076,9 +1077,9 @@ int plan_fused_uncached(netmax_ctx* ctx, const RoundPlan& plan, FusedPlan& f) {
   // M = 20: 132 against 144, 28: 182 against 214, 36: 227 against 287) -- no barrier, no pull that leaves
   // the CTA.  A single such CTA per SM (M = 37 ... 73) is slower (M = 40: 330 against 309), so the kernel is used down to 128 threads per SM.
   for (int rounds : {4, 8, kFusedMaxRounds})
-    NM_CUDA(ctx, cudaFuncSetAttribute(pick_fused_kernel(ctx->objective, ctx->L.halves, rounds), cudaFuncAttributePreferredSharedMemoryCarveout,
+    NM_CUDA(ctx, cudaFuncSetAttribute(pick_fused_kernel(ctx->objective, ctx->L.halves, ctx->M, rounds), cudaFuncAttributePreferredSharedMemoryCarveout,
                                       (int)cudaSharedmemCarveoutMaxShared));
-  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves, 8);  // (the instance with the most registers)
+  FusedKernel k = pick_fused_kernel(ctx->objective, ctx->L.halves, ctx->M, 8);  // (the instance with the most registers)
   // The head of the shared memory (draws and telemetry sums) grows with the rounds of a launch: room for as
   // many as were asked for, unless fewer let more threads live on an SM (M = 36: the last kilobytes decide
   // between two CTAs and one).
@@ -1324,7 +1325,8 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
     if (fused.ok && n - b >= 2) {  // the next rounds in one launch over resident tiles
       // launches of even length (20 rounds at 8 per launch: 7 + 7 + 6, not 8 + 8 + 4)
       const int64_t launches_left = (n - b + fused.max_rounds - 1) / fused.max_rounds;
-      const int chunk = (int)((n - b + launches_left - 1) / launches_left);
+      const int64_t same_word = ((int64_t)1 << 32) - (int64_t)(r & 0xFFFFFFFFull);  // rounds of a launch share their number's high word
+      const int chunk = (int)std::min((n - b + launches_left - 1) / launches_left, same_word);
       FusedParams fp;
       fp.x_cur = reinterpret_cast<const float4*>(xin);
       fp.x_nxt = reinterpret_cast<float4*>(xout);
@@ -1349,7 +1351,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
       fp.inv_M = p.inv_M;
       fp.q_offset = ctx->q_offset + (uint32_t)range.q0;
       fp.keys = p.keys;
-      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, chunk);
+      FusedKernel fk = pick_fused_kernel(ctx->objective, ctx->L.halves, ctx->M, chunk);
       NM_CUDA(ctx, allow_smem((const void*)fk, fused.smem));
       fk<<<(unsigned)std::min<int64_t>(fused.grid, fp.n_tiles), fused.threads, fused.smem, stream>>>(fp);
       ctx->launches += 1;
@@ -2542,6 +2544,8 @@ static int enqueue_steps(netmax_ctx* ctx, std::vector<StepEvent>& events, const 
     while (done < n) {
       const int64_t launches_left = (n - done + kStepTileEvents - 1) / kStepTileEvents;  // launches of even length
       p.n_events = (int32_t)((n - done + launches_left - 1) / launches_left);
+      for (int e = 1; e < p.n_events; ++e)  // one high word of the iteration per launch
+        if (events[done + e].ctr3 != events[done].ctr3) p.n_events = e;
       std::memcpy(p.ev, events.data() + done, p.n_events * sizeof(StepEvent));
       kernel<<<grid, threads, step_tile_head(p.n_events, ctx->M) + slabs, ctx->stream>>>(p);
       ctx->launches += 1;

@@ -711,14 +711,10 @@ __global__ void __launch_bounds__(256, 2) multi_round_kernel(const MultiRoundPar
 // thread's column group is four bfloat16 values (8 bytes of global memory), widened on the way
 // in, and every round's result is rounded to bfloat16 before it is written to the slab, exactly
 // as a store to and a load from the bfloat16 state would.
-#ifndef NETMAX_FUSED_UNROLL
-#define NETMAX_FUSED_UNROLL 2
-#endif
 #ifndef NETMAX_FUSED_PREFETCH
 #define NETMAX_FUSED_PREFETCH 1  // fetch the next tile under the last round of the current one (fp32 state)
 #endif
 constexpr int kFusedMaxRounds = 32;  // rounds per launch of fused_rounds_kernel, at most
-constexpr int kFusedUnroll = NETMAX_FUSED_UNROLL;  // rows of a round in flight per thread
 
 struct FusedParams {
   const float4* x_cur;   // [M][ldq] replicas at the start of the first round
@@ -730,7 +726,7 @@ struct FusedParams {
   double* partials;      // [n_rounds][gridDim.x][2]
   unsigned int* ticket;  // last-CTA-done counter (0 between launches)
   int64_t slot0, ring;   // ring slot of the first round
-  uint64_t first_round;
+  uint64_t first_round;  // (its high word is that of all rounds of the launch)
   int32_t n_rounds;      // 1 .. slots
   int32_t slots;         // rounds the table of draws at the head of the shared memory has room for (<= kFusedMaxRounds)
   int64_t nq, n_tiles;   // column groups of FOUR elements per row (whatever the storage), tiles of blockDim of them
@@ -741,24 +737,34 @@ struct FusedParams {
   PhiloxKeys keys;
 };
 
-// Dynamic shared memory: (peer row offset, weight) int2[slots][M], the warps' telemetry sums
-// double[slots][warps][2], then the slabs float4[3][M][blockDim] (replicas of even rounds, of odd rounds,
+// Dynamic shared memory: (peer row offset, weight) int2[slots][M] -- with kStart (peer row offset, weight, noise_start of the
+// row) int4[slots][M] --, the warps' telemetry sums double[slots][warps][2], then the slabs float4[3][M][blockDim] (replicas of even rounds, of odd rounds,
 // centres).  Any block size that is a multiple of 32 up to 256 works.
 // The telemetry of a round is added over the lanes of a warp at its end (in double) and kept per warp in shared memory,
 // for up to 32 rounds; launches of at most kReg rounds keep a thread's own sums in registers instead, which spares a
 // round's shuffles (us per call, sums in shared memory / in registers: 2 x 33,554,435 elements, 8 rounds 961 / 916, 4
 // rounds 515 / 492; 8 x 8,388,611: 702 / 690, 371 / 367).
+// kStart: the first product of a row's noise depends on the worker and the round alone, so a table holds it for all threads;
+// column and round parts of the others are worked out once per tile and once per round (noise_column, noise_base).  us per
+// launch of 20 rounds, without / with all three: 8 x 11,173,962 elements 2,204 / 2,060, bfloat16 state 2,336 / 2,130, 16 x
+// 8,000,002 3,168 / 3,050, 4 x 8,000,002 912 / 843; eight rounds of 2 x 33,554,435 899 / 802.  Above kStartWorkers the wider
+// table costs rounds per launch, and the one warp per scheduler gains nothing from it (28 x 2,000,002, 8 rounds: 769 before, 765
+// with it, 745 without).
+constexpr int kStartWorkers = 17;
+__host__ __device__ inline uint32_t fused_draw_bytes(int64_t M) { return M <= kStartWorkers ? 16u : 8u; }
 __host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {
-  return (uint32_t)(((uint64_t)slots * (uint64_t)(M * 8 + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);
+  return (uint32_t)(((uint64_t)slots * (uint64_t)(M * fused_draw_bytes(M) + (threads >> 5) * 16) + 127u) & ~(uint64_t)127u);
 }
-template <int kObjective, bool kBf16, int kReg>
+template <int kObjective, bool kBf16, int kReg, bool kStart>
 __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
+  constexpr int kUnroll = kStart ? 2 : 4;             // rows of a round in flight per thread
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int tid = threadIdx.x, T = blockDim.x, M = p.M;
-  int2* s_pw = reinterpret_cast<int2*>(smem_raw);  // (byte offset of the peer's row in a slab, pull weight)
+  using Draw = typename std::conditional<kStart, int4, int2>::type;
+  Draw* s_pw = reinterpret_cast<Draw*>(smem_raw);  // (byte offset of the peer's row in a slab, pull weight, start of the noise)
   const uint32_t head = fused_head(p.slots, M, T);
-  double* s_tel = reinterpret_cast<double*>(smem_raw + (size_t)p.slots * M * 8);
+  double* s_tel = reinterpret_cast<double*>(smem_raw + (size_t)p.slots * M * sizeof(Draw));
   const int lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
   const uint32_t stride = (uint32_t)T * 16u;     // bytes between consecutive rows of a slab
   const uint32_t plane = (uint32_t)M * stride;   // bytes of one [M][T] slab
@@ -773,7 +779,15 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     const int32_t* peers = p.trace + ((p.slot0 + k) % p.ring) * M;
     for (int i = tid; i < M; i += T) {
       const int32_t m = __ldg(peers + i);
-      s_pw[k * M + i] = make_int2((int)((uint32_t)m * stride), __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * M + m)));
+      Draw d;
+      d.x = (int)((uint32_t)m * stride);
+      d.y = __float_as_int((m == i) ? 0.0f : __ldg(p.wtab + (size_t)i * M + m));
+      if constexpr (kStart) {
+        const uint64_t start = noise_start((uint32_t)i, (uint32_t)(p.first_round + (uint64_t)k), p.keys);
+        d.z = (int)(uint32_t)start;
+        d.w = (int)(uint32_t)(start >> 32);
+      }
+      s_pw[k * M + i] = d;
     }
   }
   __syncthreads();
@@ -797,8 +811,8 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
   for (int64_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
     const int64_t q = tile * T + tid;
     const bool live = q < p.nq;  // (no barrier below: warps are independent)
-    const int lanes = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
-    const uint32_t q32 = (uint32_t)q + p.q_offset;
+    const int lanes = live ? live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0) : 0;
+    const NoiseColumn column = noise_column((uint32_t)q + p.q_offset, philox_ctr3(kTagNoise, p.first_round), p.keys);
     const int64_t q_next = q + (int64_t)gridDim.x * T;
     const bool have_next = kPrefetch && tile + gridDim.x < p.n_tiles && q_next < p.nq;
     if (fetched) {
@@ -842,8 +856,6 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
     auto run_round = [&](int k, auto last_tag, auto ragged_tag) {
       constexpr bool kLast = decltype(last_tag)::value;
       constexpr bool kRagged = decltype(ragged_tag)::value;
-      const uint64_t round = p.first_round + (uint64_t)k;
-      const uint32_t round_lo = (uint32_t)round, ctr3 = philox_ctr3(kTagNoise, round);
       const unsigned char* cur = slab + ((base + (uint32_t)k) & 1u) * plane;
       unsigned char* nxt = slab + ((base + (uint32_t)k + 1u) & 1u) * plane;
       if (kLast && have_next) {
@@ -857,14 +869,14 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
           sx += stride;
         }
       }
-      const int2* pw = s_pw + k * M;
+      const Draw* pw = s_pw + k * M;
       const ulonglong2 pivot = *reinterpret_cast<const ulonglong2*>(cur);
       ColAcc acc;
       LossAcc lacc;
       uint32_t off = 0;
       uint64_t goff = 0;
-      auto do_row = [&](int i, uint4 rnd) {
-        const int2 d = pw[i];
+      auto do_row = [&](Draw d, uint4 rnd) {
+        if (kRagged && !live) return;
         ulonglong2 noise = kObjective == 1 ? scaled_normals4<kForm>(rnd, p.sigma) : make_ulonglong2(0ull, 0ull);
         if (kRagged) noise = mask_lanes(noise, lanes);
         const ulonglong2 o = row_update<kObjective, kForm>(
@@ -885,17 +897,22 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       };
       // the Philox block of row i + 1 is drawn while row i goes through Box-Muller and Eq. 15-16:
       // the two are independent, so the integer multiplies of the one fill the latencies of the other
-      if (live) {
-      const NoiseBase nb = noise_base(q32, round_lo, ctr3, p.keys);
-      uint4 rnd = noise_words(nb, 0u, p.keys);
-#pragma unroll kFusedUnroll
+      const NoiseBase nb = noise_base(column, (uint32_t)(p.first_round + (uint64_t)k), p.keys);
+      auto words = [&](int i, Draw d) {
+        if constexpr (kStart) return noise_words(nb, (uint32_t)d.z | (uint64_t)(uint32_t)d.w << 32, p.keys);
+        else return noise_words(nb, (uint32_t)i, p.keys);
+      };
+      Draw next = pw[0];
+      uint4 rnd = words(0, next);
+#pragma unroll kUnroll
       for (int i = 0; i + 1 < M; ++i) {
-        const uint4 rnd_next = noise_words(nb, (uint32_t)(i + 1), p.keys);
-        do_row(i, rnd);
+        const Draw d = next;
+        next = pw[i + 1];
+        const uint4 rnd_next = words(i + 1, next);
+        do_row(d, rnd);
         rnd = rnd_next;
       }
-      do_row(M - 1, rnd);
-      }
+      do_row(next, rnd);
       float4 s1, s2;
       unpack2(acc.s1a, s1.x, s1.y);
       unpack2(acc.s1b, s1.z, s1.w);
@@ -925,7 +942,7 @@ __global__ void __launch_bounds__(256, 2) fused_rounds_kernel(const FusedParams 
       if ((lane & 15) == 0) s_tel[(k * nwarps + warp) * 2 + (lane >> 4)] += keep;
     };
     // (a test for padding lanes in every row would keep the rows' instructions apart: the one warp that has
-    // any runs its own instance of the round)
+    // any, or columns behind the last, runs its own instance of the round)
     if (__all_sync(0xffffffffu, lanes == 4)) {
       for (int k = 0; k + 1 < p.n_rounds; ++k) run_round(k, std::false_type(), std::false_type());
       run_round(p.n_rounds - 1, std::true_type(), std::false_type());
@@ -1072,10 +1089,12 @@ struct StepTileParams {
   uint32_t q_offset;
   int32_t n_events;
   PhiloxKeys keys;
-  StepEvent ev[kStepTileEvents];
+  StepEvent ev[kStepTileEvents];  // (all of one high word of the iteration: the same ctr3)
 };
-// Dynamic shared memory: events (offset of the worker's row, of the peer's, weight, iteration) int4[n] and (worker,
-// fourth counter word) uint2[n], what happens to each row (1: written, 2: read), slabs float4[2][M][blockDim].
+// Noise: column and event parts of its first products are worked out once per column and once per event (noise_column,
+// noise_start); 16 of 20 wide multiplies are left (8 x 11,173,962 elements, 128 steps: 1,603 us, 1,493 so).
+// Dynamic shared memory: events (offset of the worker's row, of the peer's, weight, low word of the iteration's product) int4[n]
+// and noise_start uint2[n], what happens to each row (1: written, 2: read), slabs float4[2][M][blockDim].
 __host__ __device__ inline uint32_t step_tile_head(int events, int64_t M) { return (uint32_t)((events * 24 + M + 127) & ~(int64_t)127); }
 
 template <int kObjective, bool kBf16>
@@ -1086,15 +1105,16 @@ __global__ void __launch_bounds__(256, 2) step_tiles_kernel(const __grid_constan
   const int tid = threadIdx.x, T = blockDim.x, M = p.M, n = p.n_events;
   const uint32_t stride = (uint32_t)T * 16u, plane = (uint32_t)M * stride;
   int4* s_ev = reinterpret_cast<int4*>(smem_raw);
-  uint2* s_ctr = reinterpret_cast<uint2*>(s_ev + n);
+  uint2* s_start = reinterpret_cast<uint2*>(s_ev + n);
   unsigned char* s_use = smem_raw + (size_t)n * 24;
   unsigned char* const x = smem_raw + step_tile_head(n, M) + (uint32_t)tid * 16u;  // this thread's column, row i at i * stride
   unsigned char* const cen = x + plane;
   for (int i = tid; i < M; i += T) s_use[i] = 0;
   for (int e = tid; e < n; e += T) {
     const StepEvent& ev = p.ev[e];
-    s_ev[e] = make_int4((int)((uint32_t)ev.worker * stride), (int)((uint32_t)ev.peer * stride), __float_as_int(ev.w), (int)ev.iter_lo);
-    s_ctr[e] = make_uint2((uint32_t)ev.worker, ev.ctr3);
+    s_ev[e] = make_int4((int)((uint32_t)ev.worker * stride), (int)((uint32_t)ev.peer * stride), __float_as_int(ev.w), (int)(kPhiloxMul1 * ev.iter_lo));
+    const uint64_t start = noise_start((uint32_t)ev.worker, ev.iter_lo, p.keys);
+    s_start[e] = make_uint2((uint32_t)start, (uint32_t)(start >> 32));
   }
   __syncthreads();
   for (int e = tid; e < n; e += T) s_use[p.ev[e].peer] = 2;
@@ -1121,13 +1141,13 @@ __global__ void __launch_bounds__(256, 2) step_tiles_kernel(const __grid_constan
       }
     }
     cp_async_wait_all();
-    const uint32_t q32 = (uint32_t)q + p.q_offset;
+    const NoiseColumn column = noise_column((uint32_t)q + p.q_offset, p.ev[0].ctr3, p.keys);
     const int live = live_lanes((p.tail != 0) && (q == p.nq - 1), p.tail, 0);
     auto draw = [&](int e) {  // event e's noise
       ulonglong2 v = make_ulonglong2(0ull, 0ull);
       if (kObjective == 1) {
-        const uint2 ctr = s_ctr[e];
-        v = scaled_normals4<kFunnel>(philox4x32_10(q32, ctr.x, (uint32_t)s_ev[e].w, ctr.y, p.keys), p.sigma);
+        const uint2 start = s_start[e];
+        v = scaled_normals4<kFunnel>(noise_words(noise_base_of_product(column, (uint32_t)s_ev[e].w, p.keys), start.x | (uint64_t)start.y << 32, p.keys), p.sigma);
         if (live < 4) v = mask_lanes(v, live);
       }
       return v;

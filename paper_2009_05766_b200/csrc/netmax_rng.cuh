@@ -203,8 +203,16 @@ __device__ __forceinline__ NoiseBase noise_base(const NoiseColumn& c, uint32_t r
   b.l0 = (uint32_t)p2;
   return b;
 }
-__device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint32_t worker, const PhiloxKeys& keys) {
-  const uint64_t e = (uint64_t)kPhiloxMul0 * (b.a0 ^ worker);
+// The one product that depends on worker and round alone.
+__device__ __forceinline__ uint64_t noise_start(uint32_t worker, uint32_t round_lo, const PhiloxKeys& keys) {
+  return (uint64_t)kPhiloxMul0 * (__umulhi(kPhiloxMul1, round_lo) ^ keys.k0[0] ^ worker);
+}
+// What noise_words takes when that product is given, from the low word of the round's product alone.
+__device__ __forceinline__ NoiseBase noise_base_of_product(const NoiseColumn& c, uint32_t round_product, const PhiloxKeys& keys) {
+  const uint64_t p2 = (uint64_t)kPhiloxMul0 * (c.h ^ round_product);
+  return NoiseBase{0u, c.c3, c.c1, (uint32_t)(p2 >> 32) ^ keys.k1[2], (uint32_t)p2};
+}
+__device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint64_t e, const PhiloxKeys& keys) {
   const uint64_t p = (uint64_t)kPhiloxMul1 * ((uint32_t)(e >> 32) ^ b.c3);
   uint32_t c0 = (uint32_t)(p >> 32) ^ b.c1, c1 = (uint32_t)p, c2 = b.h0 ^ (uint32_t)e, c3 = b.l0;
 #pragma unroll
@@ -217,6 +225,9 @@ __device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint32_t worker
     c3 = (uint32_t)p0;
   }
   return make_uint4(c0, c1, c2, c3);
+}
+__device__ __forceinline__ uint4 noise_words(const NoiseBase& b, uint32_t worker, const PhiloxKeys& keys) {
+  return noise_words(b, (uint64_t)kPhiloxMul0 * (b.a0 ^ worker), keys);
 }
 
 }  // namespace netmax
