@@ -795,6 +795,10 @@ PipeKernel pick_pipe_kernel(int objective, int halves, int rows) {
 // leaves out, rounded once to fp32.
 float noise_scale(const netmax_ctx* ctx) { return (float)((double)(float)ctx->sigma * kNormalScale); }
 
+// Rounds from r on whose numbers have the same high word: a launch of many rounds works that part of the noise's counters out
+// once.
+int64_t same_high_word(uint64_t r) { return ((int64_t)1 << 32) - (int64_t)(r & 0xFFFFFFFFull); }
+
 int floor_pow2(int64_t v) {
   int r = 1;
   while ((int64_t)r * 2 <= v) r *= 2;
@@ -1249,8 +1253,7 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
   return NETMAX_OK;
 }
 
-// One launch of pipe_rounds_kernel: `chunk` rounds from round r over all columns (r and r + chunk - 1 have the same high
-// word: it is part of what a thread works out once).
+// One launch of pipe_rounds_kernel: `chunk` rounds from round r over all columns (see same_high_word).
 int launch_pipe(netmax_ctx* ctx, const PipePlan& pipe, const RoundParams& p, const unsigned char* xin, unsigned char* xout,
                 uint64_t r, int chunk, unsigned char* mirror) {
   PipeParams pp;
@@ -1314,7 +1317,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
     unsigned char* xout = ctx->x[cur ^ 1] + shift;
     if (tiles.ok && n >= tiles.min_rounds && n - b >= 2) {
       const int64_t launches_left = (n - b + tiles.max_rounds - 1) / tiles.max_rounds;
-      const int64_t chunk = (n - b + launches_left - 1) / launches_left;
+      const int64_t chunk = std::min((n - b + launches_left - 1) / launches_left, same_high_word(r));
       int rc = launch_tiles(ctx, stream, tiles, p, range, xin, xout, cbase, tel, r, (int)chunk, true, nullptr);
       if (rc) return rc;
       cur ^= 1;
@@ -1325,8 +1328,7 @@ int launch_long_rounds(netmax_ctx* ctx, cudaStream_t stream, const RoundPlan& pl
     if (fused.ok && n - b >= 2) {  // the next rounds in one launch over resident tiles
       // launches of even length (20 rounds at 8 per launch: 7 + 7 + 6, not 8 + 8 + 4)
       const int64_t launches_left = (n - b + fused.max_rounds - 1) / fused.max_rounds;
-      const int64_t same_word = ((int64_t)1 << 32) - (int64_t)(r & 0xFFFFFFFFull);  // rounds of a launch share their number's high word
-      const int chunk = (int)std::min((n - b + launches_left - 1) / launches_left, same_word);
+      const int chunk = (int)std::min((n - b + launches_left - 1) / launches_left, same_high_word(r));
       FusedParams fp;
       fp.x_cur = reinterpret_cast<const float4*>(xin);
       fp.x_nxt = reinterpret_cast<float4*>(xout);
@@ -1852,8 +1854,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
     if (rc) return rc;
     if (pipe.ok && batch >= pipe.min_rounds) {
       for (int64_t b = 0; b < batch;) {
-        const int64_t same_word = ((int64_t)1 << 32) - (ctx->rounds & 0xFFFFFFFFll);
-        const int64_t chunk = std::min({batch - b, pipe.max_rounds, same_word});
+        const int64_t chunk = std::min({batch - b, pipe.max_rounds, same_high_word((uint64_t)ctx->rounds)});
         rc = launch_pipe(ctx, pipe, p, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], (uint64_t)ctx->rounds, (int)chunk,
                          done + b + chunk == n_rounds ? mirror : nullptr);
         if (rc) return rc;
@@ -1871,7 +1872,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
       all.nq4 = (ctx->d + 3) / 4;
       all.tail4 = (int32_t)(ctx->d % 4);
       for (int64_t b = 0; b < batch;) {
-        const int64_t chunk = std::min<int64_t>(batch - b, tiles.max_rounds);
+        const int64_t chunk = std::min({batch - b, tiles.max_rounds, same_high_word((uint64_t)ctx->rounds)});
         rc = launch_tiles(ctx, ctx->stream, tiles, p, all, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], ctx->c, ctx->tel,
                           (uint64_t)ctx->rounds, (int)chunk, false, done + b + chunk == n_rounds ? mirror : nullptr);
         if (rc) return rc;

@@ -12,7 +12,9 @@
 // carries it over in registers (4 per row; at most kRows rows per thread).  The barrier, the slowest warp
 // and the telemetry sums then hide behind work that has to be done anyway.  On 64 x 11.2 M elements the
 // same tile with noise drawn inside the round and a CTA barrier measured 1,685 us per round, rows over a
-// cluster of eight CTAs 1,380.
+// cluster of eight CTAs 1,380.  What of the noise's first products depends on the column alone is worked out once per tile, and a
+// thread's rows lie a constant distance apart: per row of a column group and scheduler 214 -> 207 cycles with 64 workers (bfloat16
+// state 224 -> 216), 93 in bfloat16 247 -> 236, 1,000 workers 205 -> 196, 4,096 200 -> 193.
 #pragma once
 #include "netmax_kernels.cuh"
 
@@ -53,7 +55,7 @@ struct TileParams {
   unsigned int* ticket;   // last-CTA-done counter (0 between launches)
   unsigned int* error;
   int64_t slot0, ring;
-  uint64_t first_round;
+  uint64_t first_round;   // (its high word is that of all rounds of the launch)
   int32_t n_rounds;
   int64_t nq, n_tiles;    // column groups of four elements per row; tiles of G of them
   uint32_t row_bytes;
@@ -155,11 +157,11 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
   const int g = tid & (G - 1), r = tid >> p.log2G, RL = T >> p.log2G;
   const uint32_t stride = (uint32_t)G * 16u;    // bytes between consecutive rows of a slab
   const uint32_t plane = (uint32_t)M * stride;
-  const uint32_t step = (uint32_t)RL * stride;  // bytes between consecutive rows of a thread
+  const uint32_t step = (uint32_t)T * 16u;      // bytes between consecutive rows of a thread: RL rows on
   const bool full = r + (kRows - 1) * RL < M;   // has this thread a last row?
   const uint64_t row_step = (uint64_t)(uint32_t)RL * p.row_bytes, row_first = (uint64_t)(uint32_t)r * p.row_bytes;
   unsigned char* const col = smem_raw + (uint32_t)g * 16u;
-  unsigned char* const own = col + (uint32_t)r * stride;
+  unsigned char* const own = smem_raw + (uint32_t)tid * 16u;  // row r of group g
   const uint32_t E = tile_share_entries(T, G, p.pre_reduce != 0);
   float4* const s_sum = reinterpret_cast<float4*>(smem_raw + 3u * plane);     // [kBuffers][E]
   float2* const s_two = reinterpret_cast<float2*>(s_sum + kBuffers * E);      // [kBuffers][E]
@@ -197,10 +199,11 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
     }
   };
   // (scalar steps and the funnel shift: without it 4096 x 1024 elements take 19 % longer)
+  NoiseColumn column;  // of the group whose noise is drawn
+  auto enter_column = [&](int64_t q) { column = noise_column((uint32_t)q + p.q_offset, philox_ctr3(kTagNoise, p.first_round), p.keys); };
   auto next_noise = [&](int64_t q, int k) {
     if (kObjective != 1) return;
-    const uint64_t round = p.first_round + (uint64_t)k;
-    const NoiseBase nb = noise_base((uint32_t)q + p.q_offset, (uint32_t)round, philox_ctr3(kTagNoise, round), p.keys);
+    const NoiseBase nb = noise_base(column, (uint32_t)(p.first_round + (uint64_t)k), p.keys);
     rows([&](int j) { noise[j] = scaled_normals4<kFunnel>(noise_words(nb, (uint32_t)(r + j * RL), p.keys), p.sigma); });
     if (p.tail != 0 && q == p.nq - 1)
       rows([&](int j) { noise[j] = mask_lanes(noise[j], p.tail); });
@@ -282,6 +285,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
       });
     }
     first_draws(pc.k0);
+    enter_column(q);
     next_noise(q, pc.k0);
     cp_async_wait_all();
     __syncwarp();
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
         next_noise(q, k + 1);
       } else if (ahead) {
         first_draws(0);
+        enter_column(q_next);
         next_noise(q_next, 0);
       }
       if (kFar && last_k >= 0 && warp == turn) add_shares(buf == 0 ? 2u : buf - 1u, last_k);  // (not written again before two more barriers)
