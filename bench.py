@@ -47,35 +47,34 @@ UNIQUE_FRACTION = 0.75          # x_peer is a row the same tile reads anyway (a 
                                 # bytes (6 of 8) have to cross the DRAM pins, and the HBM roofline is taken against those
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0
-KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_rng.cuh", "netmax_search.h")
+KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_search.h")
 # Counters of one launch, from ncu captures of this file's own commands (see profiles/): DRAM bytes
 # (dram__bytes_read.sum + dram__bytes_write.sum) per element of the launch and warp instructions
 # (smsp__inst_executed.sum) per element and round.  Captured on the workload itself where that is small
 # enough to profile, else on the same M and tile shape with a shorter vector (`captured_on`); bytes and
 # instructions per element are what carries over.  Only reported while the kernel sources still hash to
 # the value the capture was taken at.
-NCU_HASH = "cf6c10a5122c6103"
+NCU_HASH = "495f709bd182561f"
 NCU_COUNTERS = {
     # (workload tag, kernel): dram bytes per element-launch, warp instructions per element-round, captured on
     # (the per-round kernel's bytes on cfg2 are an earlier capture's; the latest one read 1,043,920,000)
     ("cfg2_M8_resnet18", "round_kernel"): (1_041_843_000 / 89_391_696, 81_710_869 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_042_759_000 / 89_391_696, 1_560_426_213 / (89_391_696 * 20), "cfg2"),
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): (1_044_720_000 / 89_391_696, 1_506_929_913 / (89_391_696 * 20), "cfg2"),
     ("cfg2_M8_resnet18/bf16", "round_kernel"): (508_386_000 / 89_391_696, 89_434_662 / 89_391_696, "cfg2"),
-    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (507_715_000 / 89_391_696, 681_139_124 / (89_391_696 * 8), "cfg2"),
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (1_503_016_000 / (16 * 8_000_002), 2_046_395_919 / (16 * 8_000_002 * 20), "cfg3 at d = 8,000,002"),
+    ("cfg2_M8_resnet18/bf16", "fused_rounds_kernel"): (507_694_000 / 89_391_696, 647_673_211 / (89_391_696 * 8), "cfg2"),
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): (1_503_282_000 / (16 * 8_000_002), 2_015_384_967 / (16 * 8_000_002 * 20), "cfg3 at d = 8,000,002"),
     ("cfg3_M16_vgg19scale", "round_kernel"): (1_544_316_000 / (16 * 8_000_002), 107_175_885 / (16 * 8_000_002), "cfg3 at d = 8,000,002"),
-    ("cfg4_M64_resnet18", "tile_rounds_kernel"): (1_507_538_000 / (64 * 2_000_002), 1_245_561_983 / (64 * 2_000_002 * 10), "cfg4 at d = 2,000,002"),
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): (1_506_737_000 / (64 * 2_000_002), 1_218_109_733 / (64 * 2_000_002 * 10), "cfg4 at d = 2,000,002"),
     ("cfg4_M64_resnet18", "round_kernel"): (1_536_297_000 / (64 * 2_000_002), 109_914_862 / (64 * 2_000_002), "cfg4 at d = 2,000,002"),
-    ("cfg1_M4_d4096", "tile_rounds_kernel"): (None, 31_031_584 / (16_384 * 1000), "cfg1"),
-    ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_729_561_215 / (4_194_304 * 1000), "cfg5"),
+    ("cfg1_M4_d4096", "pipe_rounds_kernel"): (None, 42_608_032 / (16_384 * 1000), "cfg1"),
+    ("cfg5_M4096_sampling", "tile_rounds_kernel"): (None, 3_628_333_875 / (4_194_304 * 1000), "cfg5"),
 }
 # Busy fractions (of active SM cycles) of the issue slots and of the arithmetic pipes: which unit a launch that is bound by
-# instruction issue leans on hardest.  Issue slots and alu from the same captures; fmaheavy, the cycles that wide multiplies
-# hold it for, from an earlier one with the same multiplies per element.
+# instruction issue leans on hardest.  From the same captures.
 NCU_PIPES = {
-    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.617, "fmaheavy": 0.643, "alu": 0.400, "captured_on": "cfg2"},
-    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.563, "fmaheavy": 0.620, "alu": 0.360, "captured_on": "cfg3 at d = 8,000,002"},
-    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.586, "fmaheavy": 0.628, "alu": 0.384, "captured_on": "cfg4 at d = 2,000,002"},
+    ("cfg2_M8_resnet18", "fused_rounds_kernel"): {"issue": 0.637, "fmaheavy": 0.674, "alu": 0.406, "captured_on": "cfg2"},
+    ("cfg3_M16_vgg19scale", "fused_rounds_kernel"): {"issue": 0.575, "fmaheavy": 0.637, "alu": 0.368, "captured_on": "cfg3 at d = 8,000,002"},
+    ("cfg4_M64_resnet18", "tile_rounds_kernel"): {"issue": 0.592, "fmaheavy": 0.640, "alu": 0.373, "captured_on": "cfg4 at d = 2,000,002"},
 }
 SM_COUNT, SCHEDULERS_PER_SM = 148, 4     # one warp instruction per scheduler and clock at most
 
@@ -333,6 +332,8 @@ def launch_shape(g, rounds, ring):
     g.round(rounds)
     per = rounds / max(1, g.kernel_launches - before - (rounds + ring - 1) // ring)      # sampler launches excluded
     if per > 1.5:
+        if g.M <= 100 and g.M * g.d <= 1 << 17:
+            return "%d rounds per launch, a warp per tile, noise and telemetry on others" % round(per), "pipe_rounds_kernel", per
         if g.M * g.d < (1 << 23) or g.M > 36 or per > 32.5:     # rows shared out over a CTA's threads
             return "%d rounds per launch over tiles with the rows shared out over the threads" % round(per), "tile_rounds_kernel", per
         return "%d rounds per launch over resident tiles" % round(per), "fused_rounds_kernel", per
@@ -533,7 +534,8 @@ def run_ours(args, w):
     sm_max_mhz = clocks.summary()["sm_max_mhz"]
     if fused or resident:
         kernel = (("tile_rounds_kernel" if w.M > 36 else "fused_rounds_kernel") if fused else
-                  ("multi_round_kernel" if args.fuse_rounds == 1 else "tile_rounds_kernel"))
+                  ("multi_round_kernel" if args.fuse_rounds == 1 else
+                   "pipe_rounds_kernel" if w.M <= 100 and w.M * w.d <= 1 << 17 else "tile_rounds_kernel"))
         roofline = issue_roofline(tag, kernel, per_round_ms, elements, bytes_per_element, rounds_per_launch, sm_max_mhz,
                                   peak, peak_kind)
     else:
