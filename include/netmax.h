@@ -145,7 +145,9 @@ void netmax_destroy(netmax_ctx* ctx);
 /*
  * Replaces P, the link graph and rho between rounds (Algorithm 2: "if received new policy").
  * Arguments as in netmax_config; prob == NULL reruns Algorithm 3; link_speed_gbps == NULL
- * keeps the current graph.  Takes effect from the next round.
+ * keeps the current graph.  Takes effect from the next round.  With 180 workers and more the work is done on the
+ * device, in memory beside the context's own (about 17 M*M bytes, one block), which the context keeps for the next
+ * change if it is no more than 512 MB and frees in netmax_destroy; without that memory it is done on the host.
  */
 int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const double* prob, double rho);
 
@@ -405,7 +407,7 @@ int netmax_policy_fixed_weight_at(int32_t M, const double* t_iter, const uint8_t
  * grids, the same row-wise LP optimum and the same selection as netmax_policy_generate, with
  * one CTA per row of P, Y_P (Eq. 22) kept in device memory and lambda_2 by Lanczos on the
  * device.  Host arrays in and out as for netmax_policy_generate; allocates its own device
- * buffers (about 4 M*M doubles) on `device` and works on `stream` (a cudaStream_t, may be
+ * buffers (about 2 M*M doubles) on `device` and works on `stream` (a cudaStream_t, may be
  * NULL); synchronises before returning.  Results agree with the host generator to rounding.
  */
 int netmax_policy_generate_device(int32_t M, const double* t_iter, const uint8_t* adj, double lr, int32_t K, int32_t R,

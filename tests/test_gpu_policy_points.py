@@ -65,3 +65,38 @@ def test_changes_of_links_in_several_contexts(nm):
             sim.round(2)
     for sim in sims:
         sim.close()
+
+
+def test_first_change_without_device_memory_to_spare(nm):
+    """A context that has kept no block yet (590 workers: tables come from the host at creation), in a program that has handed
+    out all device memory: the policy is searched on the host."""
+    import torch
+    M, d = 590, 64     # a block of 7 MB
+    kw = dict(M=M, d=d, lr=0.05, prob=np.full((M, M), 1.0 / M), link_speed_gbps=_speeds(M, 1), policy_K=3, policy_R=3, seed=2)
+    with_block, without = nm.Netmax(**kw), nm.Netmax(**kw)
+    with_block.set_policy(link_speed_gbps=_speeds(M, 3))      # (every kernel has run before the memory is gone)
+    for sim in (with_block, without):
+        sim.round(2)
+        sim.peer_trace(0, 2)
+    held, step = [], 1 << 36
+    try:
+        while step >= 1 << 18:
+            try:
+                held.append(torch.cuda.caching_allocator_alloc(step))
+            except torch.cuda.OutOfMemoryError:
+                step >>= 1
+        assert torch.cuda.cudart().cudaMemGetInfo(0)[0] < 7 << 20
+        without.set_policy(link_speed_gbps=_speeds(M, 3))
+    finally:
+        for p in held:
+            torch.cuda.caching_allocator_delete(p)
+        torch.cuda.empty_cache()
+    P, rho = with_block.get_policy()
+    Pw, rhow = without.get_policy()
+    assert rhow == pytest.approx(rho, rel=1e-12)
+    np.testing.assert_allclose(Pw, P, atol=1e-10)
+    for sim in (with_block, without):
+        sim.round(3)
+    assert (with_block.peer_trace(2, 3) == without.peer_trace(2, 3)).mean() > 0.999
+    with_block.close()
+    without.close()
