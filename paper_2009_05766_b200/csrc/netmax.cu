@@ -749,7 +749,24 @@ TileKernel pick_tile_kernel_r(int objective, int halves) {
   if (halves == 2) return objective == 1 ? tile_rounds_kernel<1, true, kRows> : tile_rounds_kernel<0, true, kRows>;
   return objective == 1 ? tile_rounds_kernel<1, false, kRows> : tile_rounds_kernel<0, false, kRows>;
 }
-TileKernel pick_tile_kernel(int objective, int halves, int rows) {
+// Instances for one shape (see tile_shape_of_its_own); with zero gradients any shape's is taken.
+template <int kRows, int kG, int kWarps>
+TileKernel own_tile_kernel(int halves) {
+  static_assert(tile_shape_of_its_own(kRows, kG, kWarps), "no such shape");
+  return halves == 2 ? tile_rounds_kernel<1, true, kRows, kG, kWarps> : tile_rounds_kernel<1, false, kRows, kG, kWarps>;
+}
+TileKernel pick_tile_kernel(int objective, int halves, int rows, int G, int warps) {
+  if (objective == 1 && tile_shape_of_its_own(rows, G, warps)) {
+    if (warps == 8) return rows == 7 ? own_tile_kernel<7, 32, 8>(halves) : own_tile_kernel<8, 32, 8>(halves);
+    switch (G) {
+      case 1: return own_tile_kernel<10, 1, 4>(halves);
+      case 2: return own_tile_kernel<10, 2, 4>(halves);
+      case 4: return own_tile_kernel<10, 4, 4>(halves);
+      case 8: return own_tile_kernel<10, 8, 4>(halves);
+      case 16: return own_tile_kernel<10, 16, 4>(halves);
+      default: return own_tile_kernel<10, 32, 4>(halves);
+    }
+  }
   switch (rows) {
     case 1: return pick_tile_kernel_r<1>(objective, halves);
     case 2: return pick_tile_kernel_r<2>(objective, halves);
@@ -954,7 +971,7 @@ int plan_tiles_uncached(netmax_ctx* ctx, const RoundPlan& plan, const FusedPlan&
     }
   }
   if (best == 0.0) return NETMAX_OK;
-  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, f.rows);
+  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, f.rows, f.G, f.threads / 32);
   NM_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   NM_CUDA(ctx, allow_smem((const void*)k, f.smem));
   int fit = 0;
@@ -1225,7 +1242,7 @@ int launch_tiles(netmax_ctx* ctx, cudaStream_t stream, const TilePlan& tiles, co
   tp.inv_M = p.inv_M;
   tp.q_offset = ctx->q_offset + (uint32_t)range.q0;
   tp.keys = p.keys;
-  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, tiles.rows);
+  TileKernel k = pick_tile_kernel(ctx->objective, ctx->L.halves, tiles.rows, tiles.G, tiles.threads / 32);
   NM_CUDA(ctx, allow_smem((const void*)k, tiles.smem));
   const int64_t grid = std::min<int64_t>(tiles.grid, tp.n_tiles);
   // Few tiles per CTA and enough rounds: equal lengths of cut tiles instead of whole ones, where the last lap

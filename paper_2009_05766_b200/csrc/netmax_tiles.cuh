@@ -119,6 +119,7 @@ __device__ __forceinline__ bool tile_piece(const TileParams& p, int n, Piece& ou
 // decide.
 __host__ __device__ constexpr int tile_max_threads(int rows) { return rows <= 8 ? 512 : rows <= 10 ? 448 : 384; }
 constexpr int kTileMaxRows = 16;
+__host__ __device__ constexpr int log2_of(int g) { return g <= 1 ? 0 : 1 + log2_of(g >> 1); }
 // What the shares of a round are added up in: fp32 sums are a thread's own, and those of column sums.  Double with five
 // rows per thread and more (long vectors of fp32 state up to 88 workers, whose sums across threads have always been
 // double, run on nothing else; an error of 1.2e-9 in the loss of 64 x 262,147 elements is 6e-11 with it).  With fewer
@@ -144,7 +145,15 @@ __host__ __device__ inline size_t tile_smem(int64_t M, int threads, int G, bool 
 // kRows: rows per thread, ceil(M / RL).  Exact, so that only a thread's LAST row can be missing: rows before it
 // run without a test between them and the scheduler can mix their instructions (with a test per row the same
 // rows took 282 cycles each instead of 195).
-template <int kObjective, bool kBf16, int kRows>
+// kG, kWarps: column groups per tile and warps per CTA where the instance is made for one shape (0: any).  A thread's addresses are
+// then one register and constants: per row of a column group and scheduler, any shape / its own, 40 workers (32 groups, 4 warps)
+// 214 / 195 cycles, 54 (32, 8) 221 / 208, 64 (32, 8) 207 / 201 (bfloat16 state 216 / 212), 150 (8, 4) 223 / 203, 300 (4, 4) 225 /
+// 208.  The shapes that the plan chooses most have such instances (tile_shape_of_its_own); twelve warps gained 0 to 2 %, six rows per
+// thread lost 2 %.
+__host__ __device__ constexpr bool tile_shape_of_its_own(int rows, int G, int warps) {
+  return (warps == 4 && rows == 10) || (warps == 8 && G == 32 && (rows == 7 || rows == 8));
+}
+template <int kObjective, bool kBf16, int kRows, int kG = 0, int kWarps = 0>
 __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel(const TileParams p) {
   constexpr uint32_t kGroupBytes = kBf16 ? 8u : 16u;  // four elements in global memory
   constexpr bool kFar = tile_far(kRows);
@@ -152,9 +161,10 @@ __global__ void __launch_bounds__(tile_max_threads(kRows), 1) tile_rounds_kernel
   using Sum = typename std::conditional<tile_wide(kRows), double, float>::type;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long s_bar;
-  const int tid = threadIdx.x, T = blockDim.x, M = p.M, G = p.G;
+  const int tid = threadIdx.x, T = kWarps ? kWarps * 32 : blockDim.x, M = p.M, G = kG ? kG : p.G;
+  const int log2G = kG ? log2_of(kG) : p.log2G;
   const int lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
-  const int g = tid & (G - 1), r = tid >> p.log2G, RL = T >> p.log2G;
+  const int g = tid & (G - 1), r = tid >> log2G, RL = T >> log2G;
   const uint32_t stride = (uint32_t)G * 16u;    // bytes between consecutive rows of a slab
   const uint32_t plane = (uint32_t)M * stride;
   const uint32_t step = (uint32_t)T * 16u;      // bytes between consecutive rows of a thread: RL rows on
