@@ -285,7 +285,6 @@ struct netmax_ctx {
   std::vector<int32_t> h_last;
   std::vector<float> h_w;
   HostMatrix t_iter;           // iteration times derived from the link speeds in force
-  HostMatrix t_spare;          // many workers: where those of new link speeds are worked out while the policy is searched
   // asynchronous timeline (one worker per global step)
   bool async_on = false;
   double beta = 0.0;
@@ -330,7 +329,6 @@ struct netmax_ctx {
   bool pipe_planned = false;
   PipePlan pipe;
   PhiloxKeys keys;
-  DeviceArena arena;          // work on policies (many workers)
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
   int sm_count = 148;
@@ -524,10 +522,10 @@ constexpr int32_t kDeviceTables = 600;
 int upload_policy(netmax_ctx* ctx) {
   if (ctx->M >= kDeviceTables) {
     const size_t MM = (size_t)ctx->M * ctx->M;
-    ArenaUse use(ctx->arena);
-    if (ctx->arena.begin(DeviceArena::room(MM * sizeof(double)) + MM)) {
-      double* d_P = ctx->arena.take<double>(MM);
-      uint8_t* d_adj = ctx->arena.take<uint8_t>(MM);
+    DeviceArena arena;
+    if (arena.allocate(DeviceArena::room(MM * sizeof(double)) + MM)) {
+      double* d_P = arena.take<double>(MM);
+      uint8_t* d_adj = arena.take<uint8_t>(MM);
       NM_CUDA(ctx, BulkPool::get().to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
       NM_CUDA(ctx, BulkPool::get().to_device(d_adj, ctx->adj.data(), MM, ctx->device, ctx->stream));
       return device_tables(ctx, d_P, d_adj);
@@ -569,9 +567,9 @@ int generate_policy(netmax_ctx* ctx, const double* t_iter, double* P, double* rh
   if (ctx->M >= kDevicePolicy) {
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ctx->device < ndev) {
       DeviceGuard guard(ctx->device);
-      ArenaUse use(ctx->arena);
+      DeviceArena arena;
       const int rc = policy_generate_device(ctx->M, t_iter, ctx->adj.data(), ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
-                                            ctx->stream, ctx->arena, P, rho, nullptr);
+                                            ctx->stream, arena, P, rho, nullptr);
       if (rc != NETMAX_OOM) return rc;
     }
     cudaGetLastError();
@@ -1615,6 +1613,7 @@ void netmax_destroy(netmax_ctx* ctx) {
 static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   const int32_t M = ctx->M;
   std::vector<uint8_t> adj;
+  HostMatrix times;
   std::string graph_error;
   // (a future's destructor waits for its thread, whichever way this function is left; without a thread to be had
   // the work is done at get())
@@ -1622,23 +1621,23 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   std::future<int> graph = std::async(kBeside, [&] {
     int rc = build_adjacency(nullptr, M, speed, adj);  // (its message goes to this thread's g_error)
     if (!rc) {
-      ctx->t_spare.resize((size_t)M * M);
-      rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_spare.data(), adj.data());  // (the same graph)
+      times.resize((size_t)M * M);
+      rc = netmax_iteration_times(M, ctx->d, speed, times.data(), adj.data());  // (the same graph)
     }
     if (rc) graph_error = g_error;
     return rc;
   });
-  ArenaUse use(ctx->arena);
+  DeviceArena arena;
   double* d_P = nullptr;
   uint8_t* d_adj = nullptr;
   double rho = 0.0;
   const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
-                                          ctx->device, ctx->stream, ctx->arena, &d_P, &d_adj, &rho);
+                                          ctx->device, ctx->stream, arena, &d_P, &d_adj, &rho);
   const int graph_rc = graph.get();
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
   ctx->rho = rho;
-  ctx->t_iter.swap(ctx->t_spare);
+  ctx->t_iter.swap(times);
   int done = device_tables(ctx, d_P, d_adj);
   if (!done) {
     const cudaError_t e = BulkPool::get().to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);

@@ -47,7 +47,7 @@ def test_device_generator_matches_host_generator(nm, M, K, R, missing, spread):
 
 
 def test_changes_of_links_in_several_contexts(nm):
-    """The block of device memory that a context keeps for the next change serves changes of either kind, in turn."""
+    """Changes of either kind in several contexts, in turn, with the searches' device memory borrowed and given back each time."""
     sizes = (190, 400, 613)
     sims = [nm.Netmax(M=M, d=64, lr=0.05, prob=np.full((M, M), 1.0 / M), link_speed_gbps=_speeds(M, 1), policy_K=3, policy_R=3, seed=M)
             for M in sizes]
@@ -68,10 +68,10 @@ def test_changes_of_links_in_several_contexts(nm):
 
 
 def test_first_change_without_device_memory_to_spare(nm):
-    """A context that has kept no block yet (590 workers: tables come from the host at creation), in a program that has handed
-    out all device memory: the policy is searched on the host."""
+    """In a program that has handed out all device memory the policy is searched on the host (590 workers: tables come from the host
+    at creation)."""
     import torch
-    M, d = 590, 64     # a block of 7 MB
+    M, d = 590, 64     # the search wants 7 MB
     kw = dict(M=M, d=d, lr=0.05, prob=np.full((M, M), 1.0 / M), link_speed_gbps=_speeds(M, 1), policy_K=3, policy_R=3, seed=2)
     with_block, without = nm.Netmax(**kw), nm.Netmax(**kw)
     with_block.set_policy(link_speed_gbps=_speeds(M, 3))      # (every kernel has run before the memory is gone)
