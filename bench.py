@@ -47,7 +47,7 @@ UNIQUE_FRACTION = 0.75          # x_peer is a row the same tile reads anyway (a 
                                 # bytes (6 of 8) have to cross the DRAM pins, and the HBM roofline is taken against those
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0
-KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_tiles.cuh", "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_search.h")
+KERNEL_SOURCES = ("netmax_kernels.cuh", "netmax_plain.cuh", "netmax_tiles.cuh", "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_search.h")
 # Counters of one launch, from ncu captures of this file's own commands (see profiles/): DRAM bytes
 # (dram__bytes_read.sum + dram__bytes_write.sum) per element of the launch and warp instructions
 # (smsp__inst_executed.sum) per element and round.  Captured on the workload itself where that is small

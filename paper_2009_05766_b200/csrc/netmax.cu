@@ -21,9 +21,8 @@
 
 #include <cuda_runtime.h>
 
-#include "netmax_kernels.cuh"
-#include "netmax_tiles.cuh"
-#include "netmax_pipe.cuh"
+#include "netmax_plain.cuh"
+#include "netmax_instances.h"
 #include "netmax_policy.h"
 
 using namespace netmax;
@@ -198,6 +197,7 @@ constexpr int64_t kCutLaps = 16, kCutRounds = 16;  // tiles are cut for up to th
 // (3 x 101,031 elements, 64 x 4,735) tiles are as fast or faster.  Calls of four rounds gain 2 to 15 % up to 64
 // workers (80: -5 %), of eight 8 to 40 %.
 constexpr int kPipeWorkers = 100;
+constexpr int64_t kPipeMinRounds = 4;
 constexpr double kPipeCycles = 1500.0;
 constexpr int64_t kMaxRoundsPerLaunch = 4096;  // rounds one cooperative launch runs at most
 constexpr size_t kPartialsBytes = (size_t)kMaxGrid * 2 * sizeof(double) * 8;  // per CTA and round of a fused launch; two sets for multi-round launches
@@ -725,86 +725,6 @@ MultiRoundKernel pick_multi_kernel(int objective, int halves) {
   return objective == 1 ? multi_round_kernel<1, 1> : multi_round_kernel<0, 1>;
 }
 
-using FusedKernel = void (*)(const FusedParams);
-
-template <int kReg, bool kStart>
-FusedKernel pick_fused_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? fused_rounds_kernel<1, true, kReg, kStart> : fused_rounds_kernel<0, true, kReg, kStart>;
-  return objective == 1 ? fused_rounds_kernel<1, false, kReg, kStart> : fused_rounds_kernel<0, false, kReg, kStart>;
-}
-// The instance for M workers and launches of `rounds` rounds (all of one M share one layout of the shared memory).
-FusedKernel pick_fused_kernel(int objective, int halves, int32_t M, int rounds) {
-  const bool start = M <= kStartWorkers;
-  if (rounds <= 4) return start ? pick_fused_kernel_r<4, true>(objective, halves) : pick_fused_kernel_r<4, false>(objective, halves);
-  if (rounds <= 8) return start ? pick_fused_kernel_r<8, true>(objective, halves) : pick_fused_kernel_r<8, false>(objective, halves);
-  return start ? pick_fused_kernel_r<0, true>(objective, halves) : pick_fused_kernel_r<0, false>(objective, halves);
-}
-
-using TileKernel = void (*)(const TileParams);
-
-template <int kRows>
-TileKernel pick_tile_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? tile_rounds_kernel<1, true, kRows> : tile_rounds_kernel<0, true, kRows>;
-  return objective == 1 ? tile_rounds_kernel<1, false, kRows> : tile_rounds_kernel<0, false, kRows>;
-}
-// Instances for one shape (see tile_shape_of_its_own); with zero gradients any shape's is taken.
-template <int kRows, int kG, int kWarps>
-TileKernel own_tile_kernel(int halves) {
-  static_assert(tile_shape_of_its_own(kRows, kG, kWarps), "no such shape");
-  return halves == 2 ? tile_rounds_kernel<1, true, kRows, kG, kWarps> : tile_rounds_kernel<1, false, kRows, kG, kWarps>;
-}
-TileKernel pick_tile_kernel(int objective, int halves, int rows, int G, int warps) {
-  if (objective == 1 && tile_shape_of_its_own(rows, G, warps)) {
-    if (warps == 8) return rows == 7 ? own_tile_kernel<7, 32, 8>(halves) : own_tile_kernel<8, 32, 8>(halves);
-    switch (G) {
-      case 1: return own_tile_kernel<10, 1, 4>(halves);
-      case 2: return own_tile_kernel<10, 2, 4>(halves);
-      case 4: return own_tile_kernel<10, 4, 4>(halves);
-      case 8: return own_tile_kernel<10, 8, 4>(halves);
-      case 16: return own_tile_kernel<10, 16, 4>(halves);
-      default: return own_tile_kernel<10, 32, 4>(halves);
-    }
-  }
-  switch (rows) {
-    case 1: return pick_tile_kernel_r<1>(objective, halves);
-    case 2: return pick_tile_kernel_r<2>(objective, halves);
-    case 3: return pick_tile_kernel_r<3>(objective, halves);
-    case 4: return pick_tile_kernel_r<4>(objective, halves);
-    case 5: return pick_tile_kernel_r<5>(objective, halves);
-    case 6: return pick_tile_kernel_r<6>(objective, halves);
-    case 7: return pick_tile_kernel_r<7>(objective, halves);
-    case 8: return pick_tile_kernel_r<8>(objective, halves);
-    case 9: return pick_tile_kernel_r<9>(objective, halves);
-    case 10: return pick_tile_kernel_r<10>(objective, halves);
-    case 11: return pick_tile_kernel_r<11>(objective, halves);
-    case 12: return pick_tile_kernel_r<12>(objective, halves);
-    case 13: return pick_tile_kernel_r<13>(objective, halves);
-    case 14: return pick_tile_kernel_r<14>(objective, halves);
-    case 15: return pick_tile_kernel_r<15>(objective, halves);
-    default: return pick_tile_kernel_r<16>(objective, halves);
-  }
-}
-
-using PipeKernel = void (*)(const PipeParams);
-
-template <int kRows>
-PipeKernel pick_pipe_kernel_r(int objective, int halves) {
-  if (halves == 2) return objective == 1 ? pipe_rounds_kernel<1, true, kRows> : pipe_rounds_kernel<0, true, kRows>;
-  return objective == 1 ? pipe_rounds_kernel<1, false, kRows> : pipe_rounds_kernel<0, false, kRows>;
-}
-PipeKernel pick_pipe_kernel(int objective, int halves, int rows) {
-  switch (rows) {
-    case 1: return pick_pipe_kernel_r<1>(objective, halves);
-    case 2: return pick_pipe_kernel_r<2>(objective, halves);
-    case 3: return pick_pipe_kernel_r<3>(objective, halves);
-    case 4: return pick_pipe_kernel_r<4>(objective, halves);
-    case 5: return pick_pipe_kernel_r<5>(objective, halves);
-    case 6: return pick_pipe_kernel_r<6>(objective, halves);
-    case 7: return pick_pipe_kernel_r<7>(objective, halves);
-    default: return pick_pipe_kernel_r<8>(objective, halves);
-  }
-}
-
 // The kernels' noise scale: sigma (at its fp32 rounding, the value the update is defined with)
 // times the constant factor sqrt(2 ln 2) of the Box-Muller radius, which the fast normal generator
 // leaves out, rounded once to fp32.
@@ -1058,7 +978,7 @@ int plan_pipe_uncached(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& f) {
   f.grid = (int)std::min<int64_t>(f.n_tiles, ctx->sm_count);
   NM_CUDA(ctx, allow_smem((const void*)pick_pipe_kernel(ctx->objective, ctx->L.halves, f.rows), f.smem));
   f.max_rounds = std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.grid);
-  f.min_rounds = M <= 64 ? 4 : 8;
+  f.min_rounds = M <= 64 ? kPipeMinRounds : 8;
   f.ok = true;
   return NETMAX_OK;
 }
@@ -1841,15 +1761,18 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   if (rc) return rc;
   ctx->host_writes = true;
   ctx->staged = false;
-  FusedPlan fused;
-  rc = plan_fused(ctx, plan, fused);
-  if (rc) return rc;
-  TilePlan tiles;
-  rc = plan_tiles(ctx, plan, fused, tiles);
-  if (rc) return rc;
-
+  // Plans ask for their kernels, and with the first one of a family its module is loaded: only what a batch may take is planned.
+  const int64_t rest = n_rounds % ctx->trace_rounds, most = std::min(n_rounds, ctx->trace_rounds);
+  const int64_t least = n_rounds < ctx->trace_rounds || rest == 0 ? most : rest;  // rounds of the longest and the shortest batch
   PipePlan pipe;
-  rc = plan_pipe(ctx, plan, pipe);
+  if (most >= kPipeMinRounds) rc = plan_pipe(ctx, plan, pipe);
+  if (rc) return rc;
+  FusedPlan fused;
+  TilePlan tiles;
+  if (most >= 2 && !(pipe.ok && least >= pipe.min_rounds)) {
+    rc = plan_fused(ctx, plan, fused);
+    if (!rc) rc = plan_tiles(ctx, plan, fused, tiles);
+  }
   if (rc) return rc;
 
   choose_rings(ctx, n_rounds);
