@@ -10,7 +10,7 @@
 //   moving warps    one tile each; in registers the tile's own rows and centres, in shared memory a ring of states
 //   helping warps   while batch b of rounds runs: the noise and draws of batch b + 1, the telemetry of batch b - 1
 //
-// All warps meet (__syncthreads) once per batch of rounds, not once per round.
+// All warps meet (meet_at_batch) once per batch of rounds, not once per round.
 //
 // Bound by latency: a round takes the moving warp about 125 cycles with one row per lane (the peer's value by a shuffle,
 // the noise and draws of the next round read under it), a batch about 670 besides.  4 x 4,096 elements, 500 rounds: 281 us
@@ -59,6 +59,10 @@ constexpr int kPipeSumRows = 8;
 __host__ __device__ inline size_t pipe_smem(int G, int per_lane, int movers, int batch) {
   return (size_t)movers * per_lane * 512 * (4 * batch + 2) + (size_t)2 * batch * (32 / G * per_lane) * 8 + (size_t)2 * batch * movers * 16;
 }
+
+// The warps of a CTA meet from two places of the program, the moving ones' loop and the helping ones': a barrier by name and number of
+// threads, which says so (__syncthreads is only defined where the whole CTA takes the same branch).
+__device__ __forceinline__ void meet_at_batch() { asm volatile("barrier.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
 
 // kRows: rows per lane, ceil(M G / 32).
 template <int kObjective, bool kBf16, int kRows>
@@ -111,7 +115,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) pipe_rounds_kernel(const __gr
     unsigned char *cur = mine + (uint32_t)g * 16u, *const last = cur + (size_t)(R - 1) * state;  // the present state, this lane's group
     const uint32_t row_at = lane_at - (uint32_t)g * 16u;
     for (int ph = 0; ph < batches + 3; ++ph) {
-      __syncthreads();  // the noise and draws of batch ph are there
+      meet_at_batch();  // the noise and draws of batch ph are there
       if (ph >= batches || tile >= p.n_tiles) continue;
       const int len = min(B, n - ph * B);
       const unsigned char* nz = s_noise + (size_t)(ph & 1) * B * state + lane_at;
@@ -303,7 +307,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) pipe_rounds_kernel(const __gr
         }
       }
       cp_async_wait_all();
-      __syncthreads();
+      meet_at_batch();
     }
   }
 }
