@@ -147,7 +147,7 @@ void netmax_destroy(netmax_ctx* ctx);
 /*
  * Replaces P, the link graph and rho between rounds (Algorithm 2: "if received new policy").
  * Arguments as in netmax_config; prob == NULL reruns Algorithm 3; link_speed_gbps == NULL
- * keeps the current graph.  Takes effect from the next round.  With 180 workers and more the work is done on the
+ * keeps the current graph.  Takes effect from the next round.  With 288 workers and more the work is done on the
  * device, in memory beside the context's own (about 17 M*M bytes, one block) that is given back before the call
  * returns; without that memory it is done on the host.  Creation with 600 workers and more borrows about 9 M*M bytes so.
  */

@@ -358,10 +358,13 @@ int fail(netmax_ctx* ctx, int code, const char* fmt, ...) {
                   #call, cudaGetErrorString(e_));                                                  \
   } while (0)
 
-// From here on whole M x M matrices are worked on by threads, and Algorithm 3 on the device (ms for a change of links, host / device,
-// K = R = 8: 128 workers 2.1 / 2.2, 160: 2.9 / 2.3, 260: 7.3 / 2.4; K = R = 20: 100 workers 3.1 / 6.6, 200: 9.3 / 7.3).
+// From here on whole M x M matrices are worked on by threads.
 constexpr int32_t kManyWorkers = 320;
-constexpr int32_t kDevicePolicy = 180;
+// From here on Algorithm 3 runs on the device.  ms for a change of links, host / device, K = R = 8: 200 workers 3.9 / 2.4, 256: 5.9 / 2.3,
+// 288: 7.3 / 2.2; K = R = 20: 200 workers 7.0 / 7.0 (half the links: 7.0-9.7 / 8.3-9.3), 256: 11.3 / 6.9, 288: 13.9 / 6.2.  A process's
+// first change loads the device's kernels, about 6 ms (K = R = 8: 200 workers 5.8 / 9.3, 256: 8 / 10, 288: 10.3 / 9.3): the line lies
+// where that one is no slower either.
+constexpr int32_t kDevicePolicy = 288;
 
 // Link graph from speeds: d_im = 1 iff i != m and the speed is positive (symmetrised).
 int build_adjacency(netmax_ctx* ctx, int32_t M, const double* speed, std::vector<uint8_t>& adj) {
