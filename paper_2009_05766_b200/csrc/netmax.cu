@@ -198,7 +198,11 @@ constexpr int64_t kCutLaps = 16, kCutRounds = 16;  // tiles are cut for up to th
 // workers (80: -5 %), of eight 8 to 40 %.
 constexpr int kPipeWorkers = 100;
 constexpr int64_t kPipeMinRounds = 4;
-constexpr double kPipeCycles = 1500.0;
+// With more than 36 workers the model knows too little of the telemetry's share from 1,300 cycles on (us per call of 6 and 64 rounds, tiles /
+// here, at 1,498: 57 x 3,783 elements 23.3 / 25.1 and 73.7 / 77.1, 56 x 4,719 23.7 / 25.1 and 73.2 / 68.1; 7 x 30,291 24.4 / 22.7 and
+// 73.4 / 56.3; at 1,224: 98 x 1,538 23.4 / 23.4 and 74.5 / 60.2).
+constexpr double kPipeCycles = 1500.0, kPipeCyclesMany = 1300.0;
+constexpr int kPipeMany = 36;
 constexpr int64_t kMaxRoundsPerLaunch = 4096;  // rounds one cooperative launch runs at most
 constexpr size_t kPartialsBytes = (size_t)kMaxGrid * 2 * sizeof(double) * 8;  // per CTA and round of a fused launch; two sets for multi-round launches
 constexpr size_t kColPartBytes = (size_t)8 << 20;  // column partials of the row-split (short vector) shape
@@ -977,7 +981,7 @@ int plan_pipe_uncached(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& f) {
       }
     }
   }
-  if (best == 0.0 || best > kPipeCycles) return NETMAX_OK;
+  if (best == 0.0 || best > (M > kPipeMany ? kPipeCyclesMany : kPipeCycles)) return NETMAX_OK;
   f.grid = (int)std::min<int64_t>(f.n_tiles, ctx->sm_count);
   NM_CUDA(ctx, allow_smem((const void*)pick_pipe_kernel(ctx->objective, ctx->L.halves, f.rows), f.smem));
   f.max_rounds = std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.grid);
