@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnetmax.so")
 SOURCES = ["netmax.cu", "netmax_fused.cu", "netmax_tiles_f32.cu", "netmax_tiles_bf16.cu", "netmax_pipe.cu", "netmax_policy.cpp", "netmax_policy_gpu.cu"]
 HEADERS = ["netmax_policy_gpu_host.inc", "netmax_tile_instances.inc", "netmax_instances.h", "netmax_kernels.cuh", "netmax_plain.cuh", "netmax_tiles.cuh",
-           "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_search.h", "netmax_policy.h", "netmax_bulk.h", os.path.join("..", "..", "include", "netmax.h")]
+           "netmax_pipe.cuh", "netmax_rng.cuh", "netmax_fp64.cuh", "netmax_search.h", "netmax_policy.h", "netmax_bulk.h", os.path.join("..", "..", "include", "netmax.h")]
 DEPS = SOURCES + HEADERS
 
 

@@ -16,9 +16,15 @@
 
 #include <cuda_runtime.h>
 
+#include "netmax_fp64.cuh"
 #include "netmax_policy.h"
 
 namespace {
+
+using netmax::exp_table;
+using netmax::fast_reciprocal;
+using netmax::kExpTable;
+using netmax::table_exp;
 
 constexpr int kRowThreads = 256;
 constexpr double kEtaCap = 600.0;
@@ -161,31 +167,6 @@ __device__ __forceinline__ void block_sum4(double& a, double& b, double& c, doub
   b = v[1];
   c = v[2];
   d = v[3];
-}
-
-// exp(x) for |x| <= 600 by a table of powers of two (Tang, "Table-driven implementation of the exponential function"): x =
-// (16 e + j) ln 2 / 16 + r with the multiple taken off in two parts, exp(r) by its Taylor polynomial of degree 7 (|r| <= ln 2 / 32:
-// remainder below 2e-18), times 2^(j/16) out of shared memory, with e added to the exponent.  Sixteen doubles fill the 32 banks once,
-// so no access conflicts.  Twelve operations of the fp64 pipe, which is what bounds the row kernels (see row_solve_kernel).
-constexpr int kExpTable = 16;
-__device__ __forceinline__ void exp_table(double* s_table) {  // (before a __syncthreads)
-  if (threadIdx.x < kExpTable) s_table[threadIdx.x] = exp2((double)threadIdx.x / kExpTable);
-}
-__device__ __forceinline__ double table_exp(double x, const double* s_table) {
-  const double shift = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer in the low mantissa bits
-  const double t = fma(x, 23.083120654223414, shift), k = t - shift;  // 16 / ln 2
-  const int n = __double2loint(t);
-  double r = fma(k, -0x1.62e42fefp-5, x);          // ln 2 / 16: its leading 32 bits (k has 14), and the rest
-  r = fma(k, -0x1.473de6af278edp-38, r);
-  double q = fma(r, 1.0 / 5040.0, 1.0 / 720.0);
-  q = fma(q, r, 1.0 / 120.0);
-  q = fma(q, r, 1.0 / 24.0);
-  q = fma(q, r, 1.0 / 6.0);
-  q = fma(q, r, 0.5);
-  q = fma(q, r, 1.0) * r;
-  const double p = s_table[n & (kExpTable - 1)];
-  const double v = fma(p, q, p);
-  return __hiloint2double(__double2hiint(v) + ((n >> 4) << 20), __double2loint(v));
 }
 
 // Grid points t_bar_r, r = first + 1 ... first + n, of one rho: alpha rho and the inner grid.
@@ -344,15 +325,6 @@ __global__ void __launch_bounds__(kRowThreads) store_rows_kernel(int M, const do
   }
 }
 
-// 1 / x for x well inside the range of normal numbers: Newton's iteration on the hardware's approximation (about 20 bits, then
-// 40, then rounding).
-__device__ __forceinline__ double fast_reciprocal(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-
 // How far the Rayleigh quotient v^T Y_P v of a unit vector (sum v_m = 0) lies below 1 at the points of a grid:
 //   sum_{i < m} y_im (v_i - v_m)^2,  y_im (Eq. 22 with p_i = 1/M) = alpha rho/M [h(p_im) + h(p_mi)],
 //   h(p) = (d_im+d_mi)/2 - alpha rho (d_im+d_mi)^2/(4p)  for p > 0,
@@ -472,8 +444,8 @@ __global__ void __launch_bounds__(256) y_tiles_kernel(int M, double* P, const ui
 // has the size of the spectrum's spread (Y itself is close to I for many workers, and the rounding of
 // numbers near 1 would swamp a beta of 1e-4 within a few steps).  No reorthogonalisation: the top of the
 // spectrum converges all the same, copies of a converged value do not move it, and the component along
-// the all-ones vector is taken out of every u.  Bound by reading Y (134 MB at M = 4096: 41 us per step with three CTAs per SM
-// and 16-byte loads, 57 with one and 8-byte loads).
+// the all-ones vector is taken out of every u.  Bound by reading Y (134 MB at M = 4096: 41 us per step with a CTA for every 16 rows, 256 of them,
+// and 16-byte loads, 57 with one CTA per SM and 8-byte loads).
 struct LanczosParams {
   int M, k;
   const double* Y;  // row-major; its block starts on 256 bytes
