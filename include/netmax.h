@@ -425,6 +425,20 @@ int netmax_policy_generate_device(int32_t M, const double* t_iter, const uint8_t
  */
 int netmax_debug_absent_ctas(netmax_ctx* ctx, int32_t n);
 
+/*
+ * The launch shape that netmax_round(n_rounds) takes for its (first, longest) batch of rounds: for tests that a case runs on the
+ * kernel it is meant for.  Changes nothing.
+ */
+enum { NETMAX_KERNEL_ROUND = 0, NETMAX_KERNEL_MULTI_ROUND = 1, NETMAX_KERNEL_FUSED = 2, NETMAX_KERNEL_TILES = 3, NETMAX_KERNEL_PIPE = 4 };
+typedef struct netmax_shape {
+  int32_t kernel;        /* NETMAX_KERNEL_*                                                            */
+  int32_t groups;        /* column groups per tile (fp32: of four elements)                            */
+  int32_t rows;          /* rows of a column group per thread                                          */
+  int32_t warps;         /* per CTA                                                                    */
+  int32_t own_instance;  /* 1: an instance compiled for this shape                                     */
+} netmax_shape;
+int netmax_launch_shape(netmax_ctx* ctx, int64_t n_rounds, netmax_shape* out);
+
 /* Counters for benchmarks: kernels launched by this context so far. */
 int64_t netmax_kernel_launches(const netmax_ctx* ctx);
 

@@ -27,7 +27,7 @@ EXPORTS = [
     "netmax_peer_trace", "netmax_telemetry", "netmax_replicas_device", "netmax_sample_peers",
     "netmax_measure", "netmax_async_begin", "netmax_async_set_times", "netmax_async_steps", "netmax_async_time",
     "netmax_async_trace", "netmax_async_ema", "netmax_async_monitor", "netmax_async_monitor_refreshes",
-    "netmax_iteration_times", "netmax_policy_generate", "netmax_policy_generate_ex", "netmax_policy_generate_device", "netmax_policy_generate_fixed_weight", "netmax_policy_fixed_weight_at", "netmax_debug_absent_ctas", "netmax_kernel_launches", "netmax_last_error",
+    "netmax_iteration_times", "netmax_policy_generate", "netmax_policy_generate_ex", "netmax_policy_generate_device", "netmax_policy_generate_fixed_weight", "netmax_policy_fixed_weight_at", "netmax_debug_absent_ctas", "netmax_launch_shape", "netmax_kernel_launches", "netmax_last_error",
 ]
 
 
@@ -47,6 +47,11 @@ class Config(C.Structure):
         ("fuse_rounds", C.c_int32), ("first_round", C.c_int64),
     ]
 
+class Shape(C.Structure):
+    _fields_ = [("kernel", C.c_int32), ("groups", C.c_int32), ("rows", C.c_int32), ("warps", C.c_int32), ("own_instance", C.c_int32)]
+
+
+KERNELS = ("round", "multi_round", "fused", "tiles", "pipe")
 STORAGE = {"f32": 0, "bf16": 1}
 
 
@@ -104,6 +109,7 @@ def lib():
             "netmax_policy_generate_fixed_weight": ([i32, vp, vp, dbl, i32, i32, dbl, vp, vp, vp], C.c_int),
             "netmax_policy_fixed_weight_at": ([i32, vp, vp, dbl, dbl, vp], C.c_int),
             "netmax_debug_absent_ctas": ([vp, i32], C.c_int),
+            "netmax_launch_shape": ([vp, i64, vp], C.c_int),
             "netmax_kernel_launches": ([vp], i64),
             "netmax_last_error": ([vp], C.c_char_p),
         }
@@ -407,6 +413,12 @@ class Netmax:
         count = np.empty((self.M, self.M), dtype=np.int64)
         _check(lib().netmax_async_ema(self._h, _p(ema), _p(count)), self._h)
         return ema, count
+
+    def launch_shape(self, n_rounds: int):
+        """(kernel, column groups per tile, rows per thread, warps per CTA, instance of its own) of netmax_round(n_rounds)."""
+        out = Shape()
+        _check(lib().netmax_launch_shape(self._h, int(n_rounds), C.addressof(out)), self._h)
+        return KERNELS[out.kernel], out.groups, out.rows, out.warps, bool(out.own_instance)
 
     def debug_absent_ctas(self, n: int):
         _check(lib().netmax_debug_absent_ctas(self._h, int(n)), self._h)

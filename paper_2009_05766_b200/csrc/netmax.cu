@@ -1756,6 +1756,30 @@ static void choose_rings(netmax_ctx* ctx, int64_t n) {
   std::memset(ctx->on_host.data(), mark, (size_t)(count - first));
 }
 
+// The plans of a call of n_rounds.  Plans ask for their kernels, and with the first one of a family its module is loaded: only what a batch
+// may take is planned.
+static int plan_call(netmax_ctx* ctx, const RoundPlan& plan, int64_t n_rounds, PipePlan& pipe, FusedPlan& fused, TilePlan& tiles) {
+  int rc = NETMAX_OK;
+  const int64_t rest = n_rounds % ctx->trace_rounds, most = std::min(n_rounds, ctx->trace_rounds);
+  const int64_t least = n_rounds < ctx->trace_rounds || rest == 0 ? most : rest;  // rounds of the longest and the shortest batch
+  if (most >= kPipeMinRounds) rc = plan_pipe(ctx, plan, pipe);
+  if (rc) return rc;
+  if (most >= 2 && !(pipe.ok && least >= pipe.min_rounds)) {
+    rc = plan_fused(ctx, plan, fused);
+    if (!rc) rc = plan_tiles(ctx, plan, fused, tiles);
+  }
+  return rc;
+}
+
+// Which kernel a batch of rounds takes.
+static int batch_kernel(const netmax_ctx* ctx, const RoundPlan& plan, const PipePlan& pipe, const FusedPlan& fused, const TilePlan& tiles, int64_t batch) {
+  if (pipe.ok && batch >= pipe.min_rounds) return NETMAX_KERNEL_PIPE;
+  if (tiles.ok && batch >= tiles.min_rounds) return NETMAX_KERNEL_TILES;
+  if (plan.short_vectors && ctx->cooperative && batch >= 2) return NETMAX_KERNEL_MULTI_ROUND;
+  if (fused.ok && batch >= 2) return NETMAX_KERNEL_FUSED;
+  return NETMAX_KERNEL_ROUND;
+}
+
 int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
   if (n_rounds < 0) return fail(ctx, NETMAX_INVALID_ARG, "n_rounds = %lld < 0", (long long)n_rounds);
@@ -1768,18 +1792,10 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   if (rc) return rc;
   ctx->host_writes = true;
   ctx->staged = false;
-  // Plans ask for their kernels, and with the first one of a family its module is loaded: only what a batch may take is planned.
-  const int64_t rest = n_rounds % ctx->trace_rounds, most = std::min(n_rounds, ctx->trace_rounds);
-  const int64_t least = n_rounds < ctx->trace_rounds || rest == 0 ? most : rest;  // rounds of the longest and the shortest batch
   PipePlan pipe;
-  if (most >= kPipeMinRounds) rc = plan_pipe(ctx, plan, pipe);
-  if (rc) return rc;
   FusedPlan fused;
   TilePlan tiles;
-  if (most >= 2 && !(pipe.ok && least >= pipe.min_rounds)) {
-    rc = plan_fused(ctx, plan, fused);
-    if (!rc) rc = plan_tiles(ctx, plan, fused, tiles);
-  }
+  rc = plan_call(ctx, plan, n_rounds, pipe, fused, tiles);
   if (rc) return rc;
 
   choose_rings(ctx, n_rounds);
@@ -1798,7 +1814,8 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
     rc = launch_sampler(ctx, (uint64_t)ctx->rounds, batch, ctx->trace, ctx->draws, ctx->rounds % ctx->trace_rounds,
                         ctx->trace_rounds);
     if (rc) return rc;
-    if (pipe.ok && batch >= pipe.min_rounds) {
+    const int kernel = batch_kernel(ctx, plan, pipe, fused, tiles, batch);
+    if (kernel == NETMAX_KERNEL_PIPE) {
       for (int64_t b = 0; b < batch;) {
         const int64_t chunk = std::min({batch - b, pipe.max_rounds, same_high_word((uint64_t)ctx->rounds)});
         rc = launch_pipe(ctx, pipe, p, ctx->x[ctx->cur], ctx->x[ctx->cur ^ 1], (uint64_t)ctx->rounds, (int)chunk,
@@ -1812,7 +1829,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
       done += batch;
       continue;
     }
-    if (plan.short_vectors && tiles.ok && batch >= tiles.min_rounds) {
+    if (plan.short_vectors && kernel == NETMAX_KERNEL_TILES) {
       // short vectors: every round of the batch on shared-memory-resident columns
       ColumnRange all;
       all.nq4 = (ctx->d + 3) / 4;
@@ -1830,7 +1847,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
       done += batch;
       continue;
     }
-    if (plan.short_vectors && ctx->cooperative && batch >= 2) {
+    if (kernel == NETMAX_KERNEL_MULTI_ROUND) {
       // short, L2-resident problem: all rounds of the batch in cooperative launches
       int64_t b = 0;
       while (b < batch) {
@@ -2594,6 +2611,44 @@ int netmax_async_ema(netmax_ctx* ctx, double* ema_out, int64_t* samples_out) {
   if (samples_out) std::memcpy(samples_out, ctx->ema_count.data(), ctx->ema_count.size() * sizeof(int64_t));
   return NETMAX_OK;
 }
+
+int netmax_launch_shape(netmax_ctx* ctx, int64_t n_rounds, netmax_shape* out) try {
+  if (!ctx || !out) return fail(ctx, NETMAX_INVALID_ARG, "ctx or out is NULL");
+  if (n_rounds < 1) return fail(ctx, NETMAX_INVALID_ARG, "n_rounds = %lld < 1", (long long)n_rounds);
+  DeviceGuard guard(ctx->device);
+  RoundPlan plan;
+  PipePlan pipe;
+  FusedPlan fused;
+  TilePlan tiles;
+  int rc = plan_round(ctx, plan, ctx->objective);
+  if (!rc) rc = plan_call(ctx, plan, n_rounds, pipe, fused, tiles);
+  if (rc) return rc;
+  std::memset(out, 0, sizeof *out);
+  out->kernel = batch_kernel(ctx, plan, pipe, fused, tiles, std::min(n_rounds, ctx->trace_rounds));
+  switch (out->kernel) {
+    case NETMAX_KERNEL_PIPE:
+      out->groups = pipe.G;
+      out->rows = pipe.rows;
+      out->warps = pipe.movers + pipe.helpers;
+      break;
+    case NETMAX_KERNEL_TILES:
+      out->groups = tiles.G;
+      out->rows = tiles.rows;
+      out->warps = tiles.threads / 32;
+      out->own_instance = ctx->objective == 1 && tile_shape_of_its_own(tiles.rows, tiles.G, tiles.threads / 32);
+      break;
+    case NETMAX_KERNEL_FUSED:
+      out->groups = fused.threads;
+      out->rows = ctx->M;
+      out->warps = fused.threads / 32;
+      break;
+    default:
+      out->groups = plan.cg;
+      out->rows = (int32_t)((plan.rows_per_group + plan.rl - 1) / plan.rl);
+      out->warps = kThreads / 32;
+  }
+  return NETMAX_OK;
+} NM_CATCH_CTX(ctx)
 
 int netmax_debug_absent_ctas(netmax_ctx* ctx, int32_t n) {
   if (!ctx) return fail(nullptr, NETMAX_INVALID_ARG, "ctx is NULL");
