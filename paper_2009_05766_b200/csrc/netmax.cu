@@ -197,7 +197,6 @@ constexpr int64_t kCutLaps = 16, kCutRounds = 16;  // tiles are cut for up to th
 // (3 x 101,031 elements, 64 x 4,735) tiles are as fast or faster.  Calls of four rounds gain 2 to 15 % up to 64
 // workers (80: -5 %), of eight 8 to 40 %.
 constexpr int kPipeWorkers = 100;
-constexpr int64_t kPipeMinRounds = 4;
 // With more than 36 workers the model knows too little of the telemetry's share from 1,300 cycles on (us per call of 6 and 64 rounds, tiles /
 // here, at 1,498: 57 x 3,783 elements 23.3 / 25.1 and 73.7 / 77.1, 56 x 4,719 23.7 / 25.1 and 73.2 / 68.1; 7 x 30,291 24.4 / 22.7 and
 // 73.4 / 56.3; at 1,224: 98 x 1,538 23.4 / 23.4 and 74.5 / 60.2).
@@ -985,7 +984,7 @@ int plan_pipe_uncached(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& f) {
   f.grid = (int)std::min<int64_t>(f.n_tiles, ctx->sm_count);
   NM_CUDA(ctx, allow_smem((const void*)pick_pipe_kernel(ctx->objective, ctx->L.halves, f.rows), f.smem));
   f.max_rounds = std::min<int64_t>(kMaxRoundsPerLaunch, (int64_t)(kColPartBytes / 16) / f.grid);
-  f.min_rounds = M <= 64 ? kPipeMinRounds : 8;
+  f.min_rounds = M <= 64 ? 4 : 8;
   f.ok = true;
   return NETMAX_OK;
 }
@@ -1756,18 +1755,12 @@ static void choose_rings(netmax_ctx* ctx, int64_t n) {
   std::memset(ctx->on_host.data(), mark, (size_t)(count - first));
 }
 
-// The plans of a call of n_rounds.  Plans ask for their kernels, and with the first one of a family its module is loaded: only what a batch
-// may take is planned.
-static int plan_call(netmax_ctx* ctx, const RoundPlan& plan, int64_t n_rounds, PipePlan& pipe, FusedPlan& fused, TilePlan& tiles) {
-  int rc = NETMAX_OK;
-  const int64_t rest = n_rounds % ctx->trace_rounds, most = std::min(n_rounds, ctx->trace_rounds);
-  const int64_t least = n_rounds < ctx->trace_rounds || rest == 0 ? most : rest;  // rounds of the longest and the shortest batch
-  if (most >= kPipeMinRounds) rc = plan_pipe(ctx, plan, pipe);
-  if (rc) return rc;
-  if (most >= 2 && !(pipe.ok && least >= pipe.min_rounds)) {
-    rc = plan_fused(ctx, plan, fused);
-    if (!rc) rc = plan_tiles(ctx, plan, fused, tiles);
-  }
+// All plans of a context, made by its first call: they ask for their kernels, and with the first one of a family its module is loaded (planning
+// only what the call at hand may take put that into later, longer calls).
+static int plan_call(netmax_ctx* ctx, const RoundPlan& plan, PipePlan& pipe, FusedPlan& fused, TilePlan& tiles) {
+  int rc = plan_fused(ctx, plan, fused);
+  if (!rc) rc = plan_tiles(ctx, plan, fused, tiles);
+  if (!rc) rc = plan_pipe(ctx, plan, pipe);
   return rc;
 }
 
@@ -1795,7 +1788,7 @@ int netmax_round(netmax_ctx* ctx, int64_t n_rounds) try {
   PipePlan pipe;
   FusedPlan fused;
   TilePlan tiles;
-  rc = plan_call(ctx, plan, n_rounds, pipe, fused, tiles);
+  rc = plan_call(ctx, plan, pipe, fused, tiles);
   if (rc) return rc;
 
   choose_rings(ctx, n_rounds);
@@ -2621,7 +2614,7 @@ int netmax_launch_shape(netmax_ctx* ctx, int64_t n_rounds, netmax_shape* out) tr
   FusedPlan fused;
   TilePlan tiles;
   int rc = plan_round(ctx, plan, ctx->objective);
-  if (!rc) rc = plan_call(ctx, plan, n_rounds, pipe, fused, tiles);
+  if (!rc) rc = plan_call(ctx, plan, pipe, fused, tiles);
   if (rc) return rc;
   std::memset(out, 0, sizeof *out);
   out->kernel = batch_kernel(ctx, plan, pipe, fused, tiles, std::min(n_rounds, ctx->trace_rounds));

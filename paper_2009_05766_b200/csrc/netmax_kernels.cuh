@@ -629,7 +629,8 @@ struct FusedParams {
 // launch of 20 rounds, without / with all three: 8 x 11,173,962 elements 2,204 / 2,060, bfloat16 state 2,336 / 2,130, 16 x
 // 8,000,002 3,168 / 3,050, 4 x 8,000,002 912 / 843; eight rounds of 2 x 33,554,435 899 / 802.  Above kStartWorkers the wider
 // table costs rounds per launch, and the one warp per scheduler gains nothing from it (28 x 2,000,002, 8 rounds: 769 before, 765
-// with it, 745 without).
+// with it, 745 without).  It costs them with twelve workers too, eight instead of sixteen, and gains all the same (12 x 4,000,002, 16 and 64
+// rounds, narrow / wide: 1,010 / 978, 3,971 / 3,842; bfloat16 state 1,064 / 1,018, 4,193 / 4,005).
 constexpr int kStartWorkers = 17;
 __host__ __device__ inline uint32_t fused_draw_bytes(int64_t M) { return M <= kStartWorkers ? 16u : 8u; }
 __host__ __device__ inline uint32_t fused_head(int slots, int64_t M, int threads) {

@@ -15,7 +15,7 @@
 // Bound by latency: a round takes the moving warp about 125 cycles with one row per lane (the peer's value by a shuffle,
 // the noise and draws of the next round read under it), a batch about 670 besides.  4 x 4,096 elements, 500 rounds: 281 us
 // with the rows of a tile spread over warps that meet every round (tile_rounds_kernel, 1,106 cycles per round, most of it
-// one warp's chain of noise and then sums), 45 us here.  Above some ten rows of 32 column groups per SM the instructions
+// one warp's chain of noise and then sums), 49 us here.  Above some ten rows of 32 column groups per SM the instructions
 // of the helping warps are what takes the time (95 cycles per such row and SM), and tile_rounds_kernel needs fewer.
 #pragma once
 #include "netmax_tiles.cuh"

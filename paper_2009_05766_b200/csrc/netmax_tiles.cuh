@@ -148,8 +148,10 @@ __host__ __device__ inline size_t tile_smem(int64_t M, int threads, int G, bool 
 // kG, kWarps: column groups per tile and warps per CTA where the instance is made for one shape (0: any).  A thread's addresses are
 // then one register and constants: per row of a column group and scheduler, any shape / its own, 40 workers (32 groups, 4 warps)
 // 214 / 195 cycles, 54 (32, 8) 221 / 208, 64 (32, 8) 207 / 201 (bfloat16 state 216 / 212), 150 (8, 4) 223 / 203, 300 (4, 4) 225 /
-// 208.  The shapes that the plan chooses most have such instances (tile_shape_of_its_own); twelve warps gained 0 to 2 %, six rows per
-// thread lost 2 %.
+// 208.  Shapes that were measured to gain 3 % and more have such instances (tile_shape_of_its_own): four warps of ten rows, which the plan
+// chooses more often than any other, and eight of seven and eight (50 to 64 workers where few tiles fall on a CTA).  Twelve warps gained
+// 0 to 2 %, six rows per thread lost 2 %; four warps of nine and of twelve rows were not measured.  The instances of ten rows spill (12 to 88
+// bytes per thread in fp32, 124 to 144 in bfloat16; any shape's 24 and 84) and gain all the same.
 __host__ __device__ constexpr bool tile_shape_of_its_own(int rows, int G, int warps) {
   return (warps == 4 && rows == 10) || (warps == 8 && G == 32 && (rows == 7 || rows == 8));
 }
