@@ -106,9 +106,10 @@ typedef struct netmax_config {
   void* workspace;               /* device memory for ALL of the context's device buffers, 256-byte
                                     aligned, at least netmax_workspace_size() bytes, owned by the
                                     caller and kept alive until netmax_destroy.  NULL: the library
-                                    allocates with cudaMalloc and frees in netmax_destroy.  (Calls that
-                                    set the policy of many workers borrow more until they return: see
-                                    netmax_set_policy)                                                  */
+                                    allocates with cudaMalloc and frees in netmax_destroy.  Beside it,
+                                    a context whose LINKS have been changed holds the block of that
+                                    search, and creation and other changes of the policy of many
+                                    workers borrow memory until they return: see netmax_set_policy      */
   size_t workspace_bytes;
   int32_t storage;               /* NETMAX_STORAGE_F32 (default) or NETMAX_STORAGE_BF16: see above       */
   int32_t fuse_rounds;           /* rounds that one launch may advance a tile of long vectors while it is
@@ -148,8 +149,9 @@ void netmax_destroy(netmax_ctx* ctx);
  * Replaces P, the link graph and rho between rounds (Algorithm 2: "if received new policy").
  * Arguments as in netmax_config; prob == NULL reruns Algorithm 3; link_speed_gbps == NULL
  * keeps the current graph.  Takes effect from the next round.  With 288 workers and more the work is done on the
- * device, in memory beside the context's own (about 17 M*M bytes, one block) that is given back before the call
- * returns; without that memory it is done on the host.  Creation with 600 workers and more borrows about 9 M*M bytes so.
+ * device, in memory beside the context's workspace: about 17 M*M bytes, one block, which after a change of links the context
+ * keeps for the next one if it is no more than 512 MB (and frees in netmax_destroy); any other call gives what it borrows back
+ * before it returns, creation with 600 workers and more (9 M*M bytes) too.  Without that memory the work is done on the host.
  */
 int netmax_set_policy(netmax_ctx* ctx, const double* link_speed_gbps, const double* prob, double rho);
 

@@ -332,6 +332,7 @@ struct netmax_ctx {
   bool pipe_planned = false;
   PipePlan pipe;
   PhiloxKeys keys;
+  DeviceArena arena;          // of changes of links (many workers)
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
   int sm_count = 148;
@@ -529,7 +530,7 @@ int upload_policy(netmax_ctx* ctx) {
   if (ctx->M >= kDeviceTables) {
     const size_t MM = (size_t)ctx->M * ctx->M;
     DeviceArena arena;
-    if (arena.allocate(DeviceArena::room(MM * sizeof(double)) + MM)) {
+    if (arena.begin(DeviceArena::room(MM * sizeof(double)) + MM)) {
       double* d_P = arena.take<double>(MM);
       uint8_t* d_adj = arena.take<uint8_t>(MM);
       NM_CUDA(ctx, BulkPool::get().to_device(d_P, ctx->P.data(), MM * sizeof(double), ctx->device, ctx->stream));
@@ -1553,12 +1554,12 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
     if (rc) graph_error = g_error;
     return rc;
   });
-  DeviceArena arena;
+  ArenaUse use(ctx->arena);
   double* d_P = nullptr;
   uint8_t* d_adj = nullptr;
   double rho = 0.0;
   const int rc = policy_from_links_device(M, ctx->d, speed, ctx->alpha, ctx->policy_K, ctx->policy_R, ctx->policy_rho_upper,
-                                          ctx->device, ctx->stream, arena, &d_P, &d_adj, &rho);
+                                          ctx->device, ctx->stream, ctx->arena, &d_P, &d_adj, &rho);
   const int graph_rc = graph.get();
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));

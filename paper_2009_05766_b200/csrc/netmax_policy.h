@@ -31,24 +31,33 @@ void set_global_error(const std::string& msg);
 double tridiagonal_top_eigenvalue(const std::vector<double>& alpha, const std::vector<double>& beta);
 void tridiagonal_top_vector(const std::vector<double>& alpha, const std::vector<double>& beta, double lambda, std::vector<double>& z);
 
-// Device memory of one call's work on whole M x M matrices: one allocation on the current device that is carved up (a cudaMalloc or
-// cudaFree costs between half a millisecond and twenty: 19 of them were a third of a policy change of 4,096 workers).  It is given
-// back when the call ends: between calls a context holds no more than its workspace.
+// Device memory for work on whole M x M matrices: one allocation that is carved up.  A cudaMalloc or cudaFree costs between
+// half a millisecond and twenty (19 of them were a third of a policy change of 4,096 workers).  A simulator keeps the block of
+// a change of links for the next one, up to kKept bytes (4,096 workers: 36 ms per change; 44 with one allocation each time); whatever else it
+// borrows is given back when the call ends.  For one caller at a time.
 class DeviceArena {
  public:
+  static constexpr size_t kKept = (size_t)512 << 20;
   DeviceArena() = default;
   DeviceArena(const DeviceArena&) = delete;
   DeviceArena& operator=(const DeviceArena&) = delete;
-  ~DeviceArena() {
-    if (base_) cudaFree(base_);
-  }
-  bool allocate(size_t bytes) {  // (once)
+  ~DeviceArena() { release(); }
+  // Starts over with room for `bytes`; whoever used the block before has finished (its stream has been waited for).
+  bool begin(size_t bytes) {
+    const uint64_t context = context_number();
+    if (base_ && context != context_) base_ = nullptr;  // (it went with its context)
+    used_ = 0;
+    if (base_ && bytes <= size_) return true;
+    release();
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     base_ = (unsigned char*)p;
+    size_ = bytes;
+    context_ = context;
+    cudaGetDevice(&device_);
     return true;
   }
   static size_t room(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
@@ -58,10 +67,32 @@ class DeviceArena {
     used_ += room(count * sizeof(T));
     return at;
   }
+  void end() {
+    if (size_ > kKept) release();
+  }
+  void release() {
+    if (base_) {
+      int now = -1;
+      cudaGetDevice(&now);
+      if (now != device_) cudaSetDevice(device_);
+      if (context_number() == context_) cudaFree(base_);
+      if (now >= 0 && now != device_) cudaSetDevice(now);
+      cudaGetLastError();
+    }
+    base_ = nullptr;
+    size_ = 0;
+  }
 
  private:
   unsigned char* base_ = nullptr;
-  size_t used_ = 0;
+  size_t size_ = 0, used_ = 0;
+  uint64_t context_ = 0;
+  int device_ = 0;
+};
+struct ArenaUse {  // of one call
+  DeviceArena& arena;
+  explicit ArenaUse(DeviceArena& a) : arena(a) {}
+  ~ArenaUse() { arena.end(); }
 };
 
 // A whole policy change on the current device: link speeds (host) -> link graph and iteration times ->
