@@ -333,6 +333,7 @@ struct netmax_ctx {
   PipePlan pipe;
   PhiloxKeys keys;
   DeviceArena arena;          // of changes of links (many workers)
+  HostMatrix t_spare;         // the iteration times of new links, worked out while the policy is searched
   std::vector<double> P;      // policy in force
   std::vector<uint8_t> adj;   // link graph in force
   int sm_count = 148;
@@ -1540,7 +1541,6 @@ void netmax_destroy(netmax_ctx* ctx) {
 static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   const int32_t M = ctx->M;
   std::vector<uint8_t> adj;
-  HostMatrix times;
   std::string graph_error;
   // (a future's destructor waits for its thread, whichever way this function is left; without a thread to be had
   // the work is done at get())
@@ -1548,8 +1548,8 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   std::future<int> graph = std::async(kBeside, [&] {
     int rc = build_adjacency(nullptr, M, speed, adj);  // (its message goes to this thread's g_error)
     if (!rc) {
-      times.resize((size_t)M * M);
-      rc = netmax_iteration_times(M, ctx->d, speed, times.data(), adj.data());  // (the same graph)
+      ctx->t_spare.resize((size_t)M * M);
+      rc = netmax_iteration_times(M, ctx->d, speed, ctx->t_spare.data(), adj.data());  // (the same graph)
     }
     if (rc) graph_error = g_error;
     return rc;
@@ -1564,7 +1564,7 @@ static int set_policy_from_links(netmax_ctx* ctx, const double* speed) {
   if (graph_rc) return fail(ctx, graph_rc, "%s", graph_error.c_str());
   if (rc) return fail(ctx, rc, "%s", netmax_last_error(nullptr));
   ctx->rho = rho;
-  ctx->t_iter.swap(times);
+  ctx->t_iter.swap(ctx->t_spare);
   int done = device_tables(ctx, d_P, d_adj);
   if (!done) {
     const cudaError_t e = BulkPool::get().to_host(ctx->P.data(), d_P, (size_t)M * M * sizeof(double), ctx->device, ctx->stream);
